@@ -514,6 +514,10 @@ int run(gwcp_ctx* c, cudaStream_t s) {
     b.wc_who = get<uint32_t>(c, "wc_who", na, &oom);
     b.wc_row = get<uint32_t>(c, "wc_row", na, &oom);
     b.wc_ep = get<uint32_t>(c, "wc_ep", na, &oom);
+    if (z.grouped) {
+      z.big_cap = z.n_acc / 8 + 65536;  // accesses past it are finished in their own warp
+      b.wc_big = get<uint64_t>(c, "wc_big", z.big_cap, &oom);
+    }
   } else {
     z.n_chunks = uint32_t(check_chunks(z.n_acc));
     const size_t ng = check_group_count(z.n_acc);
@@ -651,7 +655,7 @@ int run(gwcp_ctx* c, cudaStream_t s) {
     b.scan_tmp = get<uint32_t>(c, "scan_tmp", std::max(need2, radix_tmp_need(z.race_cap + 1) + 64), &oom);
     if (oom) return GWCP_ERR_OOM;
     const unsigned long long tests = c->st_host->partner_tests;
-    cudaMemsetAsync(&b.st->n_races, 0, sizeof(unsigned long long), s);
+    cudaMemsetAsync(&b.st->n_races, 0, 2 * sizeof(unsigned long long), s);  // and big_items, next to it
     if (z.sparse_check)
       phaseI_wide_check(b, g, z, s, c->prof);
     else

@@ -49,6 +49,7 @@ struct DevStatus {
   unsigned long long key_or, key_and;    // over access location keys
   unsigned long long lock_or, lock_and;  // over acquire/release lock ids
   unsigned long long n_races;            // races found (may exceed the buffer)
+  unsigned long long big_items;          // partner check: items put aside (may exceed their buffer)
   unsigned long long dep_pool_used;
   unsigned long long partner_tests;
   unsigned long long loop_visits;
@@ -202,6 +203,7 @@ struct Bufs {
   uint32_t* wc_who = nullptr;    // [n_acc] record fields in key order: who, version row, epoch
   uint32_t* wc_row = nullptr;
   uint32_t* wc_ep = nullptr;
+  uint64_t* wc_big = nullptr;    // [big_cap] (position, piece) items of accesses with many partner groups
   // grouped order: hashed bitmap of the locations with a write-class access, and the
   // number of accesses the filter keeps (those whose location's bit is set)
   uint32_t* wl_bits = nullptr;  // [2^wl_log2 / 32]
@@ -367,6 +369,7 @@ struct Sizes {
   uint32_t pool_cap = 0;
   uint32_t n_chunks = 0;
   uint64_t race_cap = 0;
+  uint32_t big_cap = 0;  // partner check: items it may put aside
   uint64_t tile_cap = 0;      // wide clocks: tiles in the pool
   bool cta_barriers = false;  // every block fits one CTA of walkers
   bool hb_only = false;       // versions hold H_t: the check then tests scoped happens-before

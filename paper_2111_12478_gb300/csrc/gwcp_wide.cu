@@ -21,8 +21,8 @@
 // Pool exhaustion sets GWCP_ERR_OOM; the walker then keeps its old tile (the host grows
 // the pool and runs the analysis again).
 //
-// The check for wide clocks enumerates partners per access instead of holding a W-wide
-// table: accesses sorted by location are re-sorted stably by (location, class, agent);
+// The partner check enumerates partners per access instead of holding a W-wide table:
+// accesses sorted by location are re-sorted stably by (location, class, agent);
 // for access b every (class, agent) group of its location whose class conflicts with b
 // is searched for its latest access before b, and an agent is tested once, against its
 // latest conflicting non-exempt access a*: race iff N(a*) > C_b[v] (the paper's check).
@@ -581,6 +581,8 @@ struct WideCheckArgs {
   uint32_t row_words;            // words per entry of rows
   unsigned long long* chunk_ns;  // optional timeline: globaltimer at each block's end
   uint32_t* chunk_races;         // and the races it found
+  uint2* big;         // (position, piece | pieces << 16) items of k_wc_big
+  uint32_t big_cap;   // items it holds
 };
 
 // position j in group gi of the latest member with gs[j] < x (gs ascends within a group:
@@ -629,31 +631,47 @@ __device__ __forceinline__ void emit_race(const WideCheckArgs& a, uint64_t v, ui
   if (at < a.race_cap) a.races[at] = v;
 }
 
-// partner tests of the access at key-order position p; returns how many were made
 // REP: how the clock versions are held (one instantiation each, so that the common
 // representations keep their registers and occupancy)
 enum : int { REP_TILES = 0, REP_DENSE = 1, REP_COMPRESSED = 2 };
 
-template <int REP>
-__device__ uint32_t check_one(const WideCheckArgs& a, uint32_t p, uint32_t* s_cnt, uint64_t* s_buf) {
-  const uint32_t b = a.idx[p];
-  const uint32_t bwho = a.s_who[p];
-  const uint32_t u = who_agent(bwho), cb = who_class(bwho), bu = who_block(bwho);
-  const uint32_t run = a.run_excl[p] + a.flag[p] - 1;
-  const uint32_t* rowtab = a.rows + size_t(a.s_row[p]) * a.row_words;
+// One access to check, and the groups of its location by class.
+struct CheckAcc {
+  uint32_t b, who, run;    // trace index, agent / class / block, location run
+  uint32_t x;              // "earlier than b" in the order gs holds
+  const uint32_t* rowtab;  // b's clock version
+};
+__device__ __forceinline__ CheckAcc check_acc(const WideCheckArgs& a, uint32_t p) {
+  CheckAcc c;
+  c.b = a.idx[p];
+  c.who = a.s_who[p];
+  c.run = a.run_excl[p] + a.flag[p] - 1;
+  c.x = a.grouped ? c.b : p;
+  c.rowtab = a.rows + size_t(a.s_row[p]) * a.row_words;
+  return c;
+}
+// the groups [cur[q], end[q]) of the classes the access may conflict with
+__device__ __forceinline__ void check_lists(const WideCheckArgs& a, const CheckAcc& c, uint32_t (&cur)[4],
+                                            uint32_t (&end)[4]) {
+  const uint32_t cb = who_class(c.who);
   const uint32_t any_mask = conflict_classes(cb, false) | conflict_classes(cb, true);
-  const uint32_t x = a.grouped ? b : p;  // "earlier than b" in the order gs holds
-  uint32_t tests = 0;
-  // The location's groups of each class are sorted by agent: walk the classes' lists
-  // together (a merge by agent), so that each agent is handled once, from the class
-  // holding its latest conflicting access before b (ties: the lower class).
-  uint32_t cur[4], end[4];
 #pragma unroll
   for (uint32_t q = 0; q < 4; ++q) {
     const bool on = (any_mask >> q) & 1u;
-    cur[q] = on ? a.rc_off[(run << 2) | q] : 0u;
-    end[q] = on ? a.rc_off[((run << 2) | q) + 1] : 0u;
+    cur[q] = on ? a.rc_off[(c.run << 2) | q] : 0u;
+    end[q] = on ? a.rc_off[((c.run << 2) | q) + 1] : 0u;
   }
+}
+
+// Partner tests of access c against the groups [cur[q], end[q]); returns how many were made.
+// The location's groups of each class are sorted by agent: walk the classes' lists
+// together (a merge by agent), so that each agent is handled once, from the class
+// holding its latest conflicting access before b (ties: the lower class).
+template <int REP>
+__device__ __forceinline__ uint32_t check_merge(const WideCheckArgs& a, const CheckAcc& c, uint32_t (&cur)[4],
+                                                const uint32_t (&end)[4], uint32_t* s_cnt, uint64_t* s_buf) {
+  const uint32_t u = who_agent(c.who), cb = who_class(c.who), bu = who_block(c.who);
+  uint32_t tests = 0;
   for (;;) {
     uint32_t v = NONE;
 #pragma unroll
@@ -667,7 +685,7 @@ __device__ uint32_t check_one(const WideCheckArgs& a, uint32_t p, uint32_t* s_cn
       if (cur[q] >= end[q] || a.grp_agent[cur[q]] != v) continue;
       const uint32_t gi = cur[q]++;
       if (v == u || !((cm >> q) & 1u)) continue;
-      const uint32_t jq = pred_in_group(a, gi, x);
+      const uint32_t jq = pred_in_group(a, gi, c.x);
       if (jq == NONE) continue;
       const uint32_t pq = a.gs[jq];
       if (pos == NONE || pq > pos) {
@@ -683,21 +701,101 @@ __device__ uint32_t check_one(const WideCheckArgs& a, uint32_t p, uint32_t* s_cn
       const uint32_t na = a.s_ep[qa];
       uint32_t cv;
       if constexpr (REP == REP_COMPRESSED) {
-        cv = cv_entry(rowtab, a.cv_pool, a.cv_cap, v, a.g.apb, cv_group(a.g.gran));
+        cv = cv_entry(c.rowtab, a.cv_pool, a.cv_cap, v, a.g.apb, cv_group(a.g.gran));
       } else if constexpr (REP == REP_DENSE) {
-        cv = __ldg(rowtab + v);
+        cv = __ldg(c.rowtab + v);
       } else {
-        const uint32_t tid = __ldg(rowtab + v / kTileW);
+        const uint32_t tid = __ldg(c.rowtab + v / kTileW);
         cv = tid < a.tile_cap ? __ldg(a.tiles + size_t(tid) * kTileW + v % kTileW) : 0u;
       }
-      if (na > cv) emit_race(a, (uint64_t(b) << 32) | ai, s_cnt, s_buf);  // N(a*) > C_b[v]
+      if (na > cv) emit_race(a, (uint64_t(c.b) << 32) | ai, s_cnt, s_buf);  // N(a*) > C_b[v]
     }
   }
   return tests;
 }
 
+// An access at a location that many agents touched walks up to a group per agent and class,
+// a chain of dependent loads of 1 to 2 us per group: one thread for each such access left a
+// tail of 10 ms after everything else (4M events, 4096 warps: writes to a location that all
+// warps read). Such accesses are cut by agent into parts, one per lane, each walking its own
+// agents' groups: 9.8 -> 0.51 ms there (1.67 -> 0.23 at 512 warps and 2.3M events).
+//   part `part` of `parts`: the longest class list is cut evenly, the other lists at the
+//   same agents (binary searches).
+__device__ __forceinline__ uint32_t group_lower_bound(const WideCheckArgs& a, uint32_t lo, uint32_t hi,
+                                                      uint32_t agent) {
+  while (lo < hi) {
+    const uint32_t mid = (lo + hi) >> 1;
+    if (a.grp_agent[mid] < agent)
+      lo = mid + 1;
+    else
+      hi = mid;
+  }
+  return lo;
+}
+__device__ __forceinline__ void cut_lists(const WideCheckArgs& a, uint32_t part, uint32_t parts, uint32_t (&cur)[4],
+                                          uint32_t (&end)[4]) {
+  uint32_t lo = cur[0], len = end[0] - cur[0];
+#pragma unroll
+  for (uint32_t q = 1; q < 4; ++q) {
+    if (end[q] - cur[q] > len) {
+      len = end[q] - cur[q];
+      lo = cur[q];
+    }
+  }
+  // agents [a0, a1): the part's share of the longest list (the first part also takes the
+  // agents below it, the last part those above). A part with an empty share has a0 == a1.
+  const uint32_t s0 = uint32_t(uint64_t(len) * part / parts), s1 = uint32_t(uint64_t(len) * (part + 1) / parts);
+  const bool first = part == 0, last = part + 1 == parts;
+  const uint32_t a0 = first ? 0u : a.grp_agent[lo + s0], a1 = last ? NONE : a.grp_agent[lo + s1];
+#pragma unroll
+  for (uint32_t q = 0; q < 4; ++q) {
+    const uint32_t c0 = cur[q], c1 = end[q];
+    cur[q] = first ? c0 : group_lower_bound(a, c0, c1, a0);
+    end[q] = last ? c1 : group_lower_bound(a, cur[q], c1, a1);
+  }
+}
+
+// Part `part` of `parts` of the access at position p (out of line: k_wc_check's registers
+// are those of the common walk).
 template <int REP>
-__global__ void __launch_bounds__(kCheckThreads, 8) k_wc_check(WideCheckArgs a) {
+__device__ __noinline__ uint32_t check_part(const WideCheckArgs& a, uint32_t p, uint32_t part, uint32_t parts,
+                                            uint32_t* s_cnt, uint64_t* s_buf) {
+  const CheckAcc c = check_acc(a, p);
+  uint32_t cur[4], end[4];
+  check_lists(a, c, cur, end);
+  cut_lists(a, part, parts, cur, end);
+  return check_merge<REP>(a, c, cur, end, s_cnt, s_buf);
+}
+
+// A lane walks its access's groups itself up to kBigGroups: below, lanes with similar lists
+// are better off each on its own (64 warps, 10M events: the reads of hot locations have ~60
+// groups each; cut by agent, every one of them would pay the searches that place its parts).
+constexpr uint32_t kBigGroups = 192;
+constexpr uint32_t kPieceGroups = 128;  // groups per item of k_wc_big: four per lane
+
+// appends the warp's staged races (one global atomic) and its test count; returns the races found
+__device__ __forceinline__ uint32_t flush_warp(const WideCheckArgs& a, uint32_t tests, uint32_t* s_cnt,
+                                               const uint64_t* s_buf) {
+  const uint32_t lane = threadIdx.x & 31;
+  tests = __reduce_add_sync(0xffffffffu, tests);
+  __syncwarp();
+  const uint32_t found = *s_cnt;
+  const uint32_t n = min(found, kRaceStage);
+  unsigned long long base = 0;
+  if (lane == 0) {
+    if (tests) atomicAdd(&a.st->partner_tests, (unsigned long long)tests);
+    if (n) base = atomicAdd(&a.st->n_races, (unsigned long long)n);
+  }
+  base = __shfl_sync(0xffffffffu, base, 0);
+  for (uint32_t i = lane; i < n; i += 32)
+    if (base + i < a.race_cap) a.races[base + i] = s_buf[i];
+  return found;
+}
+
+// ASIDE: accesses with many groups become items of k_wc_big (those that find no room are
+// walked here); otherwise the lanes of their warp share them (a ranked check keeps its order).
+template <int REP, bool ASIDE>
+__global__ void __launch_bounds__(kCheckThreads, 8) k_wc_check(const __grid_constant__ WideCheckArgs a) {
   constexpr uint32_t kWarps = kCheckThreads / 32;
   __shared__ uint32_t s_cnt[kWarps];
   __shared__ uint64_t s_buf[kWarps][kRaceStage];
@@ -709,28 +807,72 @@ __global__ void __launch_bounds__(kCheckThreads, 8) k_wc_check(WideCheckArgs a) 
   const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
   const uint32_t n_eff = a.n_dev ? min(a.n, *a.n_dev) : a.n;
   uint32_t tests = 0;
-  if (p < n_eff) tests = check_one<REP>(a, p, &s_cnt[warp], s_buf[warp]);
-  tests = __reduce_add_sync(0xffffffffu, tests);
-  __syncwarp();
-  const uint32_t found = s_cnt[warp];
-  const uint32_t n = min(found, kRaceStage);
-  unsigned long long base = 0;
-  if (lane == 0) {
-    if (tests) atomicAdd(&a.st->partner_tests, (unsigned long long)tests);
-    if (n) base = atomicAdd(&a.st->n_races, (unsigned long long)n);
+  bool big = false;
+  {
+    CheckAcc c{};
+    uint32_t cur[4] = {0, 0, 0, 0}, end[4] = {0, 0, 0, 0};
+    if (p < n_eff) {
+      c = check_acc(a, p);
+      check_lists(a, c, cur, end);
+    }
+    uint32_t groups = 0;
+#pragma unroll
+    for (uint32_t q = 0; q < 4; ++q) groups += end[q] - cur[q];
+    big = groups > kBigGroups;
+    if constexpr (ASIDE) {
+      if (big) {
+        const uint32_t pieces = (groups + kPieceGroups - 1) / kPieceGroups;
+        const unsigned long long at = atomicAdd(&a.st->big_items, (unsigned long long)pieces);
+        const bool fits = at + pieces <= a.big_cap;
+        for (unsigned long long i = 0; i < pieces && at + i < a.big_cap; ++i)
+          a.big[at + i] = fits ? make_uint2(p, uint32_t(i) | (pieces << 16)) : make_uint2(NONE, 0);
+        big = fits;
+      }
+    }
+    if (!big) tests = check_merge<REP>(a, c, cur, end, &s_cnt[warp], s_buf[warp]);
   }
-  base = __shfl_sync(0xffffffffu, base, 0);
-  for (uint32_t i = lane; i < n; i += 32)
-    if (base + i < a.race_cap) a.races[base + i] = s_buf[warp][i];
+  if constexpr (!ASIDE) {
+    for (uint32_t m = __ballot_sync(0xffffffffu, big); m; m &= m - 1) {
+      const uint32_t first = blockIdx.x * blockDim.x + warp * 32;
+      tests += check_part<REP>(a, first + (__ffs(m) - 1), lane, 32, &s_cnt[warp], s_buf[warp]);
+      __syncwarp();
+    }
+  }
+  const uint32_t found = flush_warp(a, tests, &s_cnt[warp], s_buf[warp]);
   if (a.chunk_ns && lane == 0) {  // the block's last warp stamps the block's end
     atomicAdd(&s_found, found);
     __threadfence_block();
     if (atomicAdd(&s_done, 1u) == kWarps - 1) {
-      unsigned long long t;
-      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-      a.chunk_ns[blockIdx.x] = t;
+      a.chunk_ns[blockIdx.x] = global_ns();
       a.chunk_races[blockIdx.x] = atomicAdd(&s_found, 0u);
     }
+  }
+}
+
+// The items that k_wc_check put aside, a warp each: piece i of an access's lists, cut into
+// 32 parts per piece. Runs after k_wc_check; the grid strides over the items, so accesses
+// at one hot location (neighbours in the order) spread over all SMs.
+template <int REP>
+__global__ void __launch_bounds__(kCheckThreads, 6) k_wc_big(const __grid_constant__ WideCheckArgs a) {
+  constexpr uint32_t kWarps = kCheckThreads / 32;
+  __shared__ uint32_t s_cnt[kWarps];
+  __shared__ uint64_t s_buf[kWarps][kRaceStage];
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned long long items = min(a.st->big_items, (unsigned long long)a.big_cap);
+  for (unsigned long long t = blockIdx.x * kWarps + warp; t < items; t += gridDim.x * kWarps) {
+    const uint2 it = a.big[t];
+    if (it.x == NONE) continue;
+    if (lane == 0) s_cnt[warp] = 0;
+    __syncwarp();
+    const uint32_t tests =
+        check_part<REP>(a, it.x, (it.y & 0xFFFFu) * 32 + lane, (it.y >> 16) * 32, &s_cnt[warp], s_buf[warp]);
+    __syncwarp();
+    const uint32_t found = flush_warp(a, tests, &s_cnt[warp], s_buf[warp]);
+    if (a.chunk_ns && lane == 0) {  // the item belongs to its access's chunk of the timeline
+      atomicAdd(a.chunk_races + it.x / kCheckThreads, found);
+      atomicMax(a.chunk_ns + it.x / kCheckThreads, global_ns());
+    }
+    __syncwarp();
   }
 }
 
@@ -954,14 +1096,24 @@ void phaseI_wide_check(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t
   a.row_words = z.compress ? g.B : g.RW;
   a.chunk_ns = b.chunk_ns;
   a.chunk_races = b.chunk_races;
+  a.big = reinterpret_cast<uint2*>(b.wc_big);
+  a.big_cap = z.grouped ? z.big_cap : 0;
   p.begin("i_check", double(n) * (4 + 16 + 4 + 4 + 4 + 8));
-  if (z.compress)
-    k_wc_check<REP_COMPRESSED><<<nblk(n, kCheckThreads), kCheckThreads, 0, s>>>(a);
-  else if (g.nT)
-    k_wc_check<REP_TILES><<<nblk(n, kCheckThreads), kCheckThreads, 0, s>>>(a);
-  else
-    k_wc_check<REP_DENSE><<<nblk(n, kCheckThreads), kCheckThreads, 0, s>>>(a);
+  int rep = g.nT ? REP_TILES : REP_DENSE;
+  if (z.compress) rep = REP_COMPRESSED;
+  auto check = rep == REP_TILES ? k_wc_check<REP_TILES, true>
+               : rep == REP_DENSE ? k_wc_check<REP_DENSE, true> : k_wc_check<REP_COMPRESSED, true>;
+  if (!z.grouped)
+    check = rep == REP_TILES ? k_wc_check<REP_TILES, false>
+            : rep == REP_DENSE ? k_wc_check<REP_DENSE, false> : k_wc_check<REP_COMPRESSED, false>;
+  check<<<nblk(n, kCheckThreads), kCheckThreads, 0, s>>>(a);
   count_launch();
+  if (z.grouped && 4 * g.W > kBigGroups) {  // fewer agents have no such access
+    auto big = rep == REP_TILES ? k_wc_big<REP_TILES>
+               : rep == REP_DENSE ? k_wc_big<REP_DENSE> : k_wc_big<REP_COMPRESSED>;
+    big<<<std::min<uint32_t>(nblk(n, 32), 152 * 6), kCheckThreads, 0, s>>>(a);
+    count_launch();
+  }
   p.end();
 }
 
