@@ -150,8 +150,9 @@ int gwcp_load_trace(gwcp_ctx* ctx, const gwcp_event* ev, uint64_t n, const gwcp_
 int gwcp_compute_order(gwcp_ctx* ctx, void* cuda_stream);
 
 /* Waits for the analysis on cuda_stream and copies up to `cap` races into host memory
- * `out` (may be NULL when cap is 0): one DMA into page-locked memory, or through the
- * context's own pinned double buffer into pageable memory. *n_races receives the total
+ * `out` (may be NULL when cap is 0): one DMA into page-locked memory, and into pageable
+ * memory where the GPU reaches it through the host's page tables; elsewhere through the
+ * context's own pinned double buffer. *n_races receives the total
  * number of races.
  * Returns GWCP_ERR_CAPACITY if cap < total, or if a fixed race_capacity was too small
  * (then *n_races is the count required; raise race_capacity and recompute). */

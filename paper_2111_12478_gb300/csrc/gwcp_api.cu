@@ -8,6 +8,7 @@
 #include <string>
 
 #include <nvtx3/nvToolsExt.h>
+#include <unistd.h>
 
 #include "gwcp_internal.cuh"
 
@@ -79,6 +80,7 @@ struct gwcp_ctx {
   cudaStream_t alloc_s = nullptr;  // stream that buffer (re)allocations are ordered on
   void* stage_host = nullptr;       // pinned staging for race copies into pageable memory
   cudaEvent_t stage_ev[2] = {nullptr, nullptr};
+  bool host_pages = false;          // the GPU reaches pageable memory through the host's page tables
   std::vector<float> rank_theta;  // gwcp_set_ranker: the MLP's parameters (empty = off)
   uint32_t clock_mode = GWCP_CLOCKS_AUTO;  // gwcp_set_clock_mode
   uint32_t check_mode = GWCP_CHECK_AUTO;   // gwcp_set_check_mode
@@ -148,15 +150,25 @@ cudaError_t wait_stream(gwcp_ctx* c, cudaStream_t s);
 constexpr size_t kStageChunk = size_t(8) << 20;  // bytes per staging half
 
 // Device -> host copy of `bytes` into caller memory. Page-locked (or registered) memory
-// takes one DMA. Pageable memory goes through the context's own two pinned halves, chunk
-// by chunk (the next chunk's DMA overlaps the host copy of the previous one), instead of
-// the driver's shared staging path.
+// takes one DMA, and so does pageable memory where the GPU reads and writes it through the
+// host's page tables (a coherent host link): measured 163 GB/s at 16 MiB and 185 GB/s at
+// 80 MiB into mapped pages, against 14 GB/s through a staging buffer, whose host copy is
+// the bound. Pages that were never touched are mapped by the host first (one store per page,
+// 2.7 ms for 80 MiB): page faults taken by the copy itself cost up to twice that. On other
+// hosts pageable memory goes through the context's own two pinned halves, chunk by chunk
+// (the next chunk's DMA overlaps the host copy of the previous one).
 int copy_to_host(gwcp_ctx* c, void* out, const void* dev, size_t bytes, cudaStream_t s) {
   cudaPointerAttributes at{};
   const bool pinned = cudaPointerGetAttributes(&at, out) == cudaSuccess &&
                       (at.type == cudaMemoryTypeHost || at.type == cudaMemoryTypeManaged);
   cudaGetLastError();
-  if (pinned || bytes <= 65536) {
+  if (!pinned && c->host_pages && bytes > 65536) {  // the whole range is overwritten below
+    const size_t page = size_t(sysconf(_SC_PAGESIZE));
+    volatile char* p = static_cast<char*>(out);
+    for (size_t i = 0; i < bytes; i += page) p[i] = 0;
+    p[bytes - 1] = 0;
+  }
+  if (pinned || c->host_pages || bytes <= 65536) {
     if (cudaMemcpyAsync(out, dev, bytes, cudaMemcpyDeviceToHost, s) != cudaSuccess) return GWCP_ERR_CUDA;
     return wait_stream(c, s) == cudaSuccess ? GWCP_OK : GWCP_ERR_CUDA;
   }
@@ -740,6 +752,10 @@ int gwcp_create(gwcp_ctx** out, int device, const gwcp_options* opt) {
   auto* c = new gwcp_ctx();
   c->device = device;
   if (opt) c->opt = *opt;
+  int host_pages = 0;
+  if (cudaDeviceGetAttribute(&host_pages, cudaDevAttrPageableMemoryAccessUsesHostPageTables, device) == cudaSuccess)
+    c->host_pages = host_pages != 0;
+  cudaGetLastError();
   if (cudaMallocHost(&c->st_host, sizeof(DevStatus)) != cudaSuccess ||
       cudaMallocHost(&c->cnt_host, 16 * sizeof(uint32_t)) != cudaSuccess ||
       cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess ||
