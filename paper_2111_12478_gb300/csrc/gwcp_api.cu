@@ -1152,23 +1152,25 @@ int gwcp_rank_grad(const float* theta, const float* feat, const float* labels, u
   cudaMemsetAsync(grad, 0, kRankParams * 4, s);
   cudaMemsetAsync(loss, 0, 4, s);
   if (!n) return cuda_rc();
-  return rank_grad(theta, feat, labels, 0, uint32_t(n), pos_weight, 1.0f / float(n), grad, loss, s);
+  return rank_grad(theta, feat, labels, uint32_t(n), pos_weight, grad, loss, s);
 }
 
 int gwcp_rank_train(float* theta, const float* feat, const float* labels, uint64_t n, const gwcp_train_options* o,
                     float* epoch_loss, void* stream) {
   if (!theta || !o || !o->epochs || !o->batch || (n && (!feat || !labels)) || n > kMaxEvents) return GWCP_ERR_ARGS;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // optimizer state, gradient, loss accumulator, per-epoch losses, counters
+  // loss accumulator (64 bits), counters, optimizer state, per-epoch losses; then the
+  // gradient's per-CTA sums, which need no clearing
   float* buf = nullptr;
-  const size_t words = 3 * size_t(kRankParams) + 1 + o->epochs + 2;
-  if (cudaMalloc(&buf, words * 4) != cudaSuccess) {
+  const size_t words = 4 + 2 * size_t(kRankParams) + o->epochs;
+  const size_t part_at = (words + 3) & ~size_t(3);
+  if (cudaMalloc(&buf, (part_at + (n ? rank_part_words(uint32_t(n), o->batch) : 0)) * 4) != cudaSuccess) {
     cudaGetLastError();
     return GWCP_ERR_OOM;
   }
-  float *m = buf, *v = buf + kRankParams, *g = buf + 2 * kRankParams, *acc = buf + 3 * kRankParams;
-  float* losses = acc + 1;
-  auto* ctr = reinterpret_cast<uint32_t*>(losses + o->epochs);
+  auto* acc = reinterpret_cast<double*>(buf);
+  auto* ctr = reinterpret_cast<uint32_t*>(buf + 2);
+  float *m = buf + 4, *v = m + kRankParams, *losses = v + kRankParams, *g = buf + part_at;
   cudaMemsetAsync(buf, 0, words * 4, s);
   int rc = GWCP_OK;
   if (n) {

@@ -476,11 +476,12 @@ void rank_scores(const float* theta, const float* feat, const uint32_t* n_dev, u
 void rank_order(const RankIn& in, const uint32_t* tmp, const float* score, uint64_t* rkey, uint32_t* rval,
                 uint64_t* rkey2, uint32_t* rval2, uint64_t* key_out, uint32_t* idx_out, uint32_t* sort_tmp,
                 cudaStream_t s);
-int rank_grad(const float* theta, const float* feat, const float* y, uint32_t lo, uint32_t hi, float pos_weight,
-              float inv_b, float* grad, float* loss, cudaStream_t s);
-void rank_adam(float* theta, float* m, float* v, float* grad, float lr, float c1, float c2, cudaStream_t s);
+int rank_grad(const float* theta, const float* feat, const float* y, uint32_t n, float pos_weight, float* grad,
+              float* loss, cudaStream_t s);
+// floats of the gradient kernel's per-CTA sums for mini-batches of `batch` of n rows
+size_t rank_part_words(uint32_t n, uint32_t batch);
 int rank_epoch(float* theta, const float* feat, const float* y, uint32_t n, uint32_t batch, float lr,
-               float pos_weight, float* m, float* v, float* grad, float* loss_acc, float* losses, uint32_t* ctr,
+               float pos_weight, float* m, float* v, float* part, double* loss_acc, float* losses, uint32_t* ctr,
                cudaStream_t s);
 // sorted race words (later << 32 | earlier) -> gwcp_race records (gwcp_check.cu)
 void races_to_records(const uint64_t* words, uint64_t n, gwcp_race* out, cudaStream_t s);

@@ -298,137 +298,234 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
-// One thread per sample: forward with the inference roundings, backward with the roundings
-// taken as the identity; gradients summed over the warp, then the block (shared memory),
-// then added to `grad`. Scaled by inv_b (1 / batch size).
-__global__ void __launch_bounds__(128) k_mlp_grad(const float* theta, const float* feat, const float* y, uint32_t lo,
-                                                  uint32_t hi, float pos_weight, float inv_b, float* grad,
-                                                  float* loss) {
-  __shared__ float sW1[NH * NF], sW2[NH * NH], sb1[NH], sb2[NH], sw3[NH];
-  __shared__ float G[N_PARAMS];
-  for (int p = threadIdx.x; p < NH * NF; p += blockDim.x) sW1[p] = bf16r(theta[P_W1 + p]);
-  for (int p = threadIdx.x; p < NH * NH; p += blockDim.x) sW2[p] = bf16r(theta[P_W2 + p]);
-  for (int p = threadIdx.x; p < NH; p += blockDim.x) {
-    sb1[p] = theta[P_B1 + p];
-    sb2[p] = theta[P_B2 + p];
-    sw3[p] = theta[P_W3 + p];
-  }
-  for (int p = threadIdx.x; p < N_PARAMS; p += blockDim.x) G[p] = 0.f;
-  __syncthreads();
-  const uint32_t i = lo + blockIdx.x * blockDim.x + threadIdx.x;
-  const bool valid = i < hi;
-  float x[NF], h1[NH], h2[NH];
-  unsigned long long m1 = 0, m2 = 0;
-#pragma unroll
-  for (int f = 0; f < NF; ++f) x[f] = valid ? bf16r(feat[size_t(i) * NF + f]) : 0.f;
-#pragma unroll
-  for (int k = 0; k < NH; ++k) {
-    float z = sb1[k];
-#pragma unroll
-    for (int f = 0; f < NF; ++f) z = fmaf(sW1[k * NF + f], x[f], z);
-    m1 |= (z > 0.f ? 1ull : 0ull) << k;
-    h1[k] = bf16r(fmaxf(z, 0.f));
-  }
-  float s = theta[P_B3];
-#pragma unroll
-  for (int n = 0; n < NH; ++n) {
-    float z = sb2[n];
-#pragma unroll 16
-    for (int k = 0; k < NH; ++k) z = fmaf(sW2[n * NH + k], h1[k], z);
-    m2 |= (z > 0.f ? 1ull : 0ull) << n;
-    h2[n] = fmaxf(z, 0.f);
-    s = fmaf(h2[n], sw3[n], s);
-  }
-  const float yi = valid ? y[i] : 0.f;
-  const float wt = yi > 0.f ? pos_weight : 1.f;
-  const float sig = 1.f / (1.f + __expf(-s));
-  const float ds = valid ? wt * (sig - yi) * inv_b : 0.f;
-  const float li = valid ? wt * (fmaxf(s, 0.f) + log1pf(__expf(-fabsf(s))) - yi * s) * inv_b : 0.f;
-  const int lane = threadIdx.x & 31;
-  // output layer
+// Loss gradient of samples lo..hi: forward with the inference roundings, backward with the
+// roundings taken as the identity, scaled by inv_b (1 / batch size). PART: each CTA writes its
+// sums (the gradient, then the loss) to its own row of `grad`; else they are added to `grad`
+// and `loss` atomically.
+// A CTA takes GR_ROWS samples at a time (grid-stride) and keeps the sums of its samples in
+// registers: the two weight gradients are outer products over the rows, 4 x 4 (W2) and 1 x 4
+// (W1) entries per thread, every other layer is a matrix product with one output column and
+// four rows per thread, all operands in shared memory. In float throughout (the products of
+// the backward pass are not rounded to bfloat16, so they stay off the tensor cores). Bound
+// by latency at a mini-batch's size: 16 rows per CTA put a batch of 1024 on 64 SMs. One
+// thread per sample, with a warp reduction per weight and sample group, took 8 ms for 40,000
+// samples and 0.55 ms for a batch of 1024; this takes GRAD_BIG and GRAD_BATCH us.
+constexpr int GR_ROWS = 16, GR_THREADS = 256;
+constexpr int GR_WORDS = (N_PARAMS + 1 + 3) & ~3;  // one CTA's sums: the gradient, the loss, padding
+
+template <bool PART>
+__global__ void __launch_bounds__(GR_THREADS, 2) k_mlp_grad(const float* theta, const float* feat, const float* y,
+                                                            uint32_t lo, uint32_t hi, float pos_weight, float inv_b,
+                                                            float* grad, float* loss) {
+  constexpr int LD2 = NH + 1;  // padded rows of W2: read by rows and by columns
+  __shared__ float sW1t[NF * NH];  // [f][k]
+  __shared__ float sW2[NH * LD2];  // [n][k]
+  __shared__ __align__(16) float sX[GR_ROWS * NF], sH1[GR_ROWS * NH], sD2[GR_ROWS * NH], sD1[GR_ROWS * NH];
+  __shared__ float sT[GR_ROWS * (NH + 1)], sDs[GR_ROWS], sW3[NH];
+  const int tid = threadIdx.x, lane = tid & 31;
   {
-    const float t = warp_sum(ds);
-    if (lane == 0) atomicAdd(&G[P_B3], t);
-    const float l = warp_sum(li);
-    if (lane == 0) atomicAdd(loss, l);
-  }
-  for (int n = 0; n < NH; ++n) {
-    const float t = warp_sum(ds * h2[n]);
-    if (lane == 0) atomicAdd(&G[P_W3 + n], t);
-  }
-  // dz2 in place of h2
+    float w1[NH * NF / GR_THREADS], w2[NH * NH / GR_THREADS];  // all loads in flight together
 #pragma unroll
-  for (int n = 0; n < NH; ++n) h2[n] = ((m2 >> n) & 1ull) ? ds * sw3[n] : 0.f;
-  for (int n = 0; n < NH; ++n) {
-    const float dz = h2[n];
-    if (__any_sync(0xffffffffu, dz != 0.f)) {
-      const float t = warp_sum(dz);
-      if (lane == 0) atomicAdd(&G[P_B2 + n], t);
-      for (int k = 0; k < NH; ++k) {
-        const float u = warp_sum(dz * h1[k]);
-        if (lane == 0) atomicAdd(&G[P_W2 + n * NH + k], u);
-      }
+    for (int q = 0; q < NH * NF / GR_THREADS; ++q) w1[q] = theta[P_W1 + q * GR_THREADS + tid];
+#pragma unroll
+    for (int q = 0; q < NH * NH / GR_THREADS; ++q) w2[q] = theta[P_W2 + q * GR_THREADS + tid];
+#pragma unroll
+    for (int q = 0; q < NH * NF / GR_THREADS; ++q) {
+      const int p = q * GR_THREADS + tid;
+      sW1t[(p % NF) * NH + p / NF] = bf16r(w1[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < NH * NH / GR_THREADS; ++q) {
+      const int p = q * GR_THREADS + tid;
+      sW2[(p / NH) * LD2 + p % NH] = bf16r(w2[q]);
     }
   }
-  // dz1 in place of h1
+  const int col = tid & (NH - 1), r0 = (tid / NH) * 4;      // layer outputs: unit col of rows r0..r0+3
+  const int gn = (tid >> 4) * 4, gk = (tid & 15) * 4;       // dW2[gn..gn+3][gk..gk+3]
+  const int hk = tid >> 2, hf = (tid & 3) * 4;              // dW1[hk][hf..hf+3]
+  const float b1 = theta[P_B1 + col], b2 = theta[P_B2 + col], w3 = theta[P_W3 + col], b3 = theta[P_B3];
+  if (tid < NH) sW3[tid] = w3;
+  float g2[4][4] = {}, g1[4] = {}, gb1 = 0.f, gb2 = 0.f, g3 = 0.f, gb3 = 0.f, gl = 0.f;
+  for (uint32_t base = lo + blockIdx.x * GR_ROWS; base < hi; base += gridDim.x * GR_ROWS) {
+    __syncthreads();  // the weights are staged; the previous rows are done with
+    {
+      const uint32_t r = base + tid / NF;  // GR_ROWS * NF == GR_THREADS
+      sX[tid] = r < hi ? bf16r(feat[size_t(r) * NF + tid % NF]) : 0.f;
+    }
+    __syncthreads();
+    // layer 1
+    uint32_t m1 = 0, m2 = 0;
+    float z[4] = {b1, b1, b1, b1};
 #pragma unroll
-  for (int k = 0; k < NH; ++k) {
-    float dh = 0.f;
+    for (int f = 0; f < NF; f += 4) {
+      float w[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) w[q] = sW1t[(f + q) * NH + col];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const float4 x = *reinterpret_cast<const float4*>(sX + (r0 + r) * NF + f);
+        z[r] = fmaf(w[3], x.w, fmaf(w[2], x.z, fmaf(w[1], x.y, fmaf(w[0], x.x, z[r]))));
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      m1 |= (z[r] > 0.f ? 1u : 0u) << r;
+      sH1[(r0 + r) * NH + col] = bf16r(fmaxf(z[r], 0.f));
+      z[r] = b2;
+    }
+    __syncthreads();
+    // layer 2 and the output
+#pragma unroll 4
+    for (int k = 0; k < NH; k += 4) {
+      float w[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) w[q] = sW2[col * LD2 + k + q];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const float4 h = *reinterpret_cast<const float4*>(sH1 + (r0 + r) * NH + k);
+        z[r] = fmaf(w[3], h.w, fmaf(w[2], h.z, fmaf(w[1], h.y, fmaf(w[0], h.x, z[r]))));
+      }
+    }
+    float h2[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      m2 |= (z[r] > 0.f ? 1u : 0u) << r;
+      h2[r] = fmaxf(z[r], 0.f);
+      sT[(r0 + r) * (NH + 1) + col] = h2[r];
+    }
+    __syncthreads();
+    if (tid < GR_ROWS) {
+      const uint32_t i = base + tid;
+      float s = b3;
 #pragma unroll 16
-    for (int n = 0; n < NH; ++n) dh = fmaf(h2[n], sW2[n * NH + k], dh);
-    h1[k] = ((m1 >> k) & 1ull) ? dh : 0.f;
-  }
-  for (int k = 0; k < NH; ++k) {
-    const float dz = h1[k];
-    if (__any_sync(0xffffffffu, dz != 0.f)) {
-      const float t = warp_sum(dz);
-      if (lane == 0) atomicAdd(&G[P_B1 + k], t);
+      for (int n = 0; n < NH; ++n) s = fmaf(sT[tid * (NH + 1) + n], sW3[n], s);
+      float ds = 0.f;
+      if (i < hi) {
+        const float yi = y[i], wt = yi > 0.f ? pos_weight : 1.f;
+        const float sig = 1.f / (1.f + __expf(-s));
+        ds = wt * (sig - yi) * inv_b;
+        gl += wt * (fmaxf(s, 0.f) + log1pf(__expf(-fabsf(s))) - yi * s) * inv_b;
+        gb3 += ds;
+      }
+      sDs[tid] = ds;
+    }
+    __syncthreads();
 #pragma unroll
-      for (int f = 0; f < NF; ++f) {
-        const float u = warp_sum(dz * x[f]);
-        if (lane == 0) atomicAdd(&G[P_W1 + k * NF + f], u);
+    for (int r = 0; r < 4; ++r) {
+      const float ds = sDs[r0 + r];
+      g3 = fmaf(ds, h2[r], g3);
+      const float dz = ((m2 >> r) & 1u) ? ds * w3 : 0.f;
+      gb2 += dz;
+      sD2[(r0 + r) * NH + col] = dz;
+      z[r] = 0.f;
+    }
+    __syncthreads();
+    // back through layer 2
+#pragma unroll 4
+    for (int n = 0; n < NH; n += 4) {
+      float w[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) w[q] = sW2[(n + q) * LD2 + col];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const float4 d = *reinterpret_cast<const float4*>(sD2 + (r0 + r) * NH + n);
+        z[r] = fmaf(d.w, w[3], fmaf(d.z, w[2], fmaf(d.y, w[1], fmaf(d.x, w[0], z[r]))));
       }
     }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const float dz = ((m1 >> r) & 1u) ? z[r] : 0.f;
+      gb1 += dz;
+      sD1[(r0 + r) * NH + col] = dz;
+    }
+    __syncthreads();
+    // weight gradients
+#pragma unroll 4
+    for (int r = 0; r < GR_ROWS; ++r) {
+      const float4 d = *reinterpret_cast<const float4*>(sD2 + r * NH + gn);
+      const float4 h = *reinterpret_cast<const float4*>(sH1 + r * NH + gk);
+      const float dv[4] = {d.x, d.y, d.z, d.w}, hv[4] = {h.x, h.y, h.z, h.w};
+#pragma unroll
+      for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) g2[p][q] = fmaf(dv[p], hv[q], g2[p][q]);
+      const float d1 = sD1[r * NH + hk];
+      const float4 x = *reinterpret_cast<const float4*>(sX + r * NF + hf);
+      g1[0] = fmaf(d1, x.x, g1[0]);
+      g1[1] = fmaf(d1, x.y, g1[1]);
+      g1[2] = fmaf(d1, x.z, g1[2]);
+      g1[3] = fmaf(d1, x.w, g1[3]);
+    }
   }
+  // this CTA's sums; the four row groups of a unit are added in shared memory first
   __syncthreads();
-  for (int p = threadIdx.x; p < N_PARAMS; p += blockDim.x)
-    if (G[p] != 0.f) atomicAdd(grad + p, G[p]);
+  sD2[tid] = gb1;
+  sD1[tid] = gb2;
+  sH1[tid] = g3;
+  __syncthreads();
+  if constexpr (PART) grad += size_t(blockIdx.x) * GR_WORDS;
+  auto out = [&](int p, float v) {
+    if constexpr (PART)
+      grad[p] = v;
+    else
+      atomicAdd(grad + p, v);
+  };
+#pragma unroll
+  for (int p = 0; p < 4; ++p)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) out(P_W2 + (gn + p) * NH + gk + q, g2[p][q]);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) out(P_W1 + hk * NF + hf + q, g1[q]);
+  if (tid < NH) {
+    out(P_B1 + tid, (sD2[tid] + sD2[tid + NH]) + (sD2[tid + 2 * NH] + sD2[tid + 3 * NH]));
+    out(P_B2 + tid, (sD1[tid] + sD1[tid + NH]) + (sD1[tid + 2 * NH] + sD1[tid + 3 * NH]));
+    out(P_W3 + tid, (sH1[tid] + sH1[tid + NH]) + (sH1[tid + 2 * NH] + sH1[tid + 3 * NH]));
+  }
+  if (tid < 32) {
+    gb3 = warp_sum(gb3);
+    gl = warp_sum(gl);
+    if (lane == 0) {
+      out(P_B3, gb3);
+      if constexpr (PART)
+        grad[N_PARAMS] = gl;
+      else
+        atomicAdd(loss, gl);
+    }
+  }
 }
 
-__global__ void k_adam(float* theta, float* m, float* v, float* grad, float lr, float c1, float c2) {
+// Adam on the sum of the gradient kernel's rows (`parts` of them, added in order in 64 bits:
+// the result does not depend on which CTA was first), with the steps of earlier epochs
+// counted in device memory (one epoch of steps is a replayable graph): batch q of an epoch
+// is step t = *step + q + 1; bias corrections 1 / (1 - beta^t). The entry after the last
+// parameter is the loss.
+__global__ void __launch_bounds__(128) k_adam(float* theta, float* m, float* v, const float* grad, uint32_t parts,
+                                              double* loss_acc, float lr, const uint32_t* step, uint32_t q) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= N_PARAMS) return;
-  const float g = grad[p];
-  const float mm = 0.9f * m[p] + 0.1f * g;
-  const float vv = 0.999f * v[p] + 0.001f * g * g;
-  m[p] = mm;
-  v[p] = vv;
-  theta[p] -= lr * (mm * c1) / (sqrtf(vv * c2) + 1e-8f);
-  grad[p] = 0.f;
-}
-
-// Adam with the step count in device memory (one epoch of steps is a replayable graph):
-// step t = *step + 1; bias corrections 1 / (1 - beta^t)
-__global__ void k_adam_dev(float* theta, float* m, float* v, float* grad, float lr, const uint32_t* step) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= N_PARAMS) return;
-  const float t = float(*step + 1);
+  if (p > N_PARAMS) return;
+  double sum = 0;
+#pragma unroll 16
+  for (uint32_t c = 0; c < parts; ++c) sum += double(__ldg(grad + size_t(c) * GR_WORDS + p));
+  if (p == N_PARAMS) {
+    *loss_acc += sum;
+    return;
+  }
+  const float t = float(*step + q + 1);
   const float c1 = 1.f / (1.f - powf(0.9f, t)), c2 = 1.f / (1.f - powf(0.999f, t));
-  const float g = grad[p];
+  const float g = float(sum);
   const float mm = 0.9f * m[p] + 0.1f * g;
   const float vv = 0.999f * v[p] + 0.001f * g * g;
   m[p] = mm;
   v[p] = vv;
   theta[p] -= lr * (mm * c1) / (sqrtf(vv * c2) + 1e-8f);
-  grad[p] = 0.f;
 }
 
-__global__ void k_step_inc(uint32_t* step) { ++*step; }
+__global__ void k_step_add(uint32_t* step, uint32_t n) { *step += n; }
 
 // end of an epoch: its accumulated loss into losses[epoch], then the next epoch
-__global__ void k_epoch_end(float* loss_acc, float* losses, uint32_t* epoch) {
-  losses[*epoch] = *loss_acc;
-  *loss_acc = 0.f;
+__global__ void k_epoch_end(double* loss_acc, float* losses, uint32_t* epoch) {
+  losses[*epoch] = float(*loss_acc);
+  *loss_acc = 0;
   ++*epoch;
 }
 
@@ -535,37 +632,50 @@ void rank_order(const RankIn& in, const uint32_t* tmp, const float* score, uint6
   count_launch();
 }
 
-int rank_grad(const float* theta, const float* feat, const float* y, uint32_t lo, uint32_t hi, float pos_weight,
-              float inv_b, float* grad, float* loss, cudaStream_t s) {
-  if (hi <= lo) return GWCP_OK;
-  k_mlp_grad<<<nblk(hi - lo, 128), 128, 0, s>>>(theta, feat, y, lo, hi, pos_weight, inv_b, grad, loss);
+namespace {
+// CTAs of the gradient kernel over n rows of `rows` or more each: two per SM at most (each
+// writes or adds its 5313 sums once)
+uint32_t grad_ctas(uint32_t n, uint32_t rows) {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return std::min<uint32_t>(nblk(n, rows), uint32_t(sms) * 2);
+}
+}  // namespace
+
+int rank_grad(const float* theta, const float* feat, const float* y, uint32_t n, float pos_weight, float* grad,
+              float* loss, cudaStream_t s) {
+  if (!n) return GWCP_OK;
+  // the CTAs' sums meet in float atomics, each a rounding: 128 rows per CTA keep their number
+  // low (3,001 rows: an error of 0.9e-7 of the norm; with 16 rows per CTA, 2.0e-7)
+  k_mlp_grad<false><<<grad_ctas(n, 128), GR_THREADS, 0, s>>>(theta, feat, y, 0, n, pos_weight, 1.0f / float(n), grad, loss);
   count_launch();
   return cudaGetLastError() == cudaSuccess ? GWCP_OK : GWCP_ERR_CUDA;
 }
 
-// One epoch of training as launches on stream s: per batch the gradient, Adam and the
-// step count; then the epoch's loss. Counters: ctr[0] Adam steps, ctr[1] epochs.
+size_t rank_part_words(uint32_t n, uint32_t batch) { return size_t(grad_ctas(std::min(n, batch), GR_ROWS)) * GR_WORDS; }
+
+// One epoch of training as launches on stream s: per batch the gradient and Adam; then the
+// step count and the epoch's loss. Counters: ctr[0] Adam steps, ctr[1] epochs. part:
+// rank_part_words(n, batch) floats.
 int rank_epoch(float* theta, const float* feat, const float* y, uint32_t n, uint32_t batch, float lr,
-               float pos_weight, float* m, float* v, float* grad, float* loss_acc, float* losses, uint32_t* ctr,
+               float pos_weight, float* m, float* v, float* part, double* loss_acc, float* losses, uint32_t* ctr,
                cudaStream_t s) {
-  const uint32_t nb = (n + batch - 1) / batch;
+  const uint32_t nb = uint32_t((uint64_t(n) + batch - 1) / batch);
   for (uint32_t q = 0; q < nb; ++q) {
-    const uint32_t lo = q * batch, hi = std::min(n, lo + batch);
-    int rc = rank_grad(theta, feat, y, lo, hi, pos_weight, 1.0f / float(hi - lo) / float(nb), grad, loss_acc, s);
-    if (rc) return rc;
-    k_adam_dev<<<nblk(N_PARAMS, 256), 256, 0, s>>>(theta, m, v, grad, lr, ctr);
+    const uint32_t lo = q * batch, hi = uint32_t(std::min<uint64_t>(n, uint64_t(lo) + batch));
+    const uint32_t ctas = grad_ctas(hi - lo, GR_ROWS);
+    k_mlp_grad<true><<<ctas, GR_THREADS, 0, s>>>(theta, feat, y, lo, hi, pos_weight,
+                                                 1.0f / float(hi - lo) / float(nb), part, nullptr);
     count_launch();
-    k_step_inc<<<1, 1, 0, s>>>(ctr);
+    k_adam<<<nblk(N_PARAMS + 1, 128), 128, 0, s>>>(theta, m, v, part, ctas, loss_acc, lr, ctr, q);
     count_launch();
   }
+  k_step_add<<<1, 1, 0, s>>>(ctr, nb);
+  count_launch();
   k_epoch_end<<<1, 1, 0, s>>>(loss_acc, losses, ctr + 1);
   count_launch();
   return cudaGetLastError() == cudaSuccess ? GWCP_OK : GWCP_ERR_CUDA;
-}
-
-void rank_adam(float* theta, float* m, float* v, float* grad, float lr, float c1, float c2, cudaStream_t s) {
-  k_adam<<<nblk(N_PARAMS, 256), 256, 0, s>>>(theta, m, v, grad, lr, c1, c2);
-  count_launch();
 }
 
 }  // namespace gwcp
