@@ -486,6 +486,7 @@ int run(gwcp_ctx* c, cudaStream_t s) {
   }
   b.psnap = get<uint32_t>(c, "psnap", (size_t(z.n_cs) + 1) * g.RW, &oom);
   b.hsnap = get<uint32_t>(c, "hsnap", (size_t(z.n_cs) + 1) * g.RW, &oom);
+  b.jsnap = get<uint32_t>(c, "jsnap", (size_t(z.n_cs) + 1) * g.RW, &oom);
   if (g.nT) {
     // tile pool: a few new tiles per clock version; grown and rerun on exhaustion
     const uint64_t want = 2ull * (uint64_t(z.n_rows) + z.n_cs) + uint64_t(z.n_bar) * (g.apb + 2) + 65536;
@@ -496,17 +497,16 @@ int run(gwcp_ctx* c, cudaStream_t s) {
     // came before
     b.tiles = get_aligned<uint32_t>(c, "tiles", size_t(z.tile_cap) * kTileW, size_t(2) << 20, &oom);
   }
-  b.done = get<uint32_t>(c, "done", size_t(z.n_cs) + 1, &oom);
   b.plan = get<uint4>(c, "plan", 2 * (size_t(z.n_sync) + z.n_incs) + 2, &oom);
+  b.plan2 = get<uint4>(c, "plan2", 2 * (size_t(z.n_sync) + z.n_incs) + 2, &oom);
   b.recmeta = get<uint4>(c, "recmeta", size_t(z.n_cs) + 1, &oom);
   b.flat_off = get<uint32_t>(c, "flat_off", ni1, &oom);
   b.flat = get<uint32_t>(c, "flat", z.pool_cap, &oom);
   b.cursor = get<uint32_t>(c, "cursor", size_t(g.W) * (z.n_locks + 1), &oom);
-  b.jsnap = g.nT ? get<uint32_t>(c, "jsnap", (size_t(z.n_cs) + 1) * g.RW, &oom) : nullptr;
-  const size_t smem = size_t(2) * g.apb * 2 * g.Wp * 4;
-  z.cta_barriers = g.nT ? true : (g.apb <= 32 && smem <= 96 * 1024);
+  z.cta_barriers = g.apb <= 32;  // a block's walkers fit one CTA
   const bool global_bars = !z.cta_barriers || g.gran == GWCP_GRAN_THREAD;
   b.bar_j = get<uint32_t>(c, "bar_j", global_bars ? size_t(z.n_bar) * 2 * g.Wp : 1, &oom);
+  b.bar_jj = get<uint32_t>(c, "bar_jj", global_bars ? size_t(z.n_bar) * g.Wp : 1, &oom);
   b.bar_cnt = get<uint32_t>(c, "bar_cnt", global_bars ? z.n_bar : 1, &oom);
   if (z.sparse_check) {
     const size_t na = size_t(z.n_acc) + 1;
@@ -538,7 +538,6 @@ int run(gwcp_ctx* c, cudaStream_t s) {
   b.races = get<uint64_t>(c, "races", z.race_cap, &oom);
   b.races2 = get<uint64_t>(c, "races2", z.race_cap, &oom);
   if (oom) return GWCP_ERR_OOM;
-  cudaMemsetAsync(b.done, 0, (size_t(z.n_cs) + 1) * 4, s);
   if (g.nT) {  // tile 0 is the zero tile; ids are handed out from 1
     cudaMemsetAsync(b.tiles, 0, kTileW * 4, s);
     const unsigned long long one = 1;
@@ -547,6 +546,7 @@ int run(gwcp_ctx* c, cudaStream_t s) {
   cudaMemsetAsync(b.cursor, 0, size_t(g.W) * (z.n_locks + 1) * 4, s);
   if (global_bars && z.n_bar) {
     cudaMemsetAsync(b.bar_j, 0, size_t(z.n_bar) * 2 * g.Wp * 4, s);
+    cudaMemsetAsync(b.bar_jj, 0, size_t(z.n_bar) * g.Wp * 4, s);
     cudaMemsetAsync(b.bar_cnt, 0, size_t(z.n_bar) * 4, s);
   }
 

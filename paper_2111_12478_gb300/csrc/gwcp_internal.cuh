@@ -165,18 +165,19 @@ struct Bufs {
   uint32_t* ex_dep_cnt = nullptr;
   // phase G: propagation
   uint4* plan = nullptr;        // [2 * (n_sync + n_incs)] one 32-byte entry per clock-changing step
+  uint4* plan2 = nullptr;       // [2 * (n_sync + n_incs)] of in-section accesses: (agent, epoch) per joined release
   uint4* recmeta = nullptr;     // [n_cs + 1] (agent, acquire epoch, release index, scope id)
   uint32_t* flat_off = nullptr; // [n_incs + 1] dependency list of each in-section access
   uint32_t* flat = nullptr;     // [pool_cap]
   uint32_t* rows = nullptr;     // [n_rows * RW], or [n_rows * B] headers of compressed versions
   uint32_t* cv_pool = nullptr;  // compressed versions: [cv_cap] warp words and lane values
-  uint32_t* psnap = nullptr;    // [n_cs * RW]
-  uint32_t* hsnap = nullptr;    // [n_cs * RW]
+  uint32_t* psnap = nullptr;    // [n_cs * RW] P_t published at each release
+  uint32_t* hsnap = nullptr;    // [n_cs * RW] H_t
+  uint32_t* jsnap = nullptr;    // [n_cs * RW] JN_t (the join of the H snapshots in P_t)
   uint32_t* tiles = nullptr;    // wide clocks: [tile_cap * kTileW] tile pool, tile 0 = zeros
-  uint32_t* done = nullptr;     // [n_cs]
   uint32_t* cursor = nullptr;   // [W * n_locks]
-  uint32_t* jsnap = nullptr;    // wide clocks: [n_cs * RW] JN tables published at releases
-  uint32_t* bar_j = nullptr;    // [n_bar * 2 * Wp] global-barrier joins
+  uint32_t* bar_j = nullptr;    // [n_bar * 2 * Wp] global-barrier joins of C and H
+  uint32_t* bar_jj = nullptr;   // [n_bar * Wp] and of JN
   uint32_t* bar_cnt = nullptr;  // [n_bar]
   // forced compression at barriers: barriers by block, their members' records, offsets
   uint64_t *fb_key = nullptr, *fb_key2 = nullptr;  // [n_bar]

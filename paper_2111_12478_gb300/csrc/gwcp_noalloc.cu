@@ -29,13 +29,17 @@ using namespace gwcp;
 
 namespace {
 
-constexpr size_t kScratchBytes = size_t(96) << 20;  // 96 MiB per device
+constexpr size_t kScratchBytes = size_t(96) << 20;  // 96 MiB per device: decides which traces fit
+// Further 32 MiB for the clocks JN_t and the in-section accesses' records. They cannot run
+// out before the first array does: a section takes four clock rows there (two versions, P
+// and H) and one here, a barrier three and one, a step over 200 bytes and 32.
+constexpr size_t kExtraBytes = size_t(32) << 20;
 constexpr uint64_t kMaxEventsNoalloc = uint64_t(1) << 18;
 constexpr uint32_t kMaxAgentsNoalloc = 256;
 
 // Device-side scratch. In host code this name is only a stand-in for the symbol: its
 // device address comes from cudaGetSymbolAddress.
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
+static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes + kExtraBytes];
 
 // Device address of the scratch array in the current device's context. Looked up on
 // every call: an address belongs to a context, and a cached one would go stale after
@@ -55,12 +59,13 @@ int scratch_base(unsigned char** out) {
 
 struct Arena {
   unsigned char* base;
+  size_t bytes_max = kScratchBytes;
   size_t used = 0;
   bool full = false;
   template <typename T>
   T* take(size_t count) {
     const size_t bytes = ((count ? count : 1) * sizeof(T) + 255) & ~size_t(255);
-    if (used + bytes > kScratchBytes) {
+    if (used + bytes > bytes_max) {
       full = true;
       return nullptr;
     }
@@ -86,7 +91,7 @@ int read_back(cudaStream_t s, DevStatus* st_h, const DevStatus* st_d, uint32_t* 
 
 int analyze(const Event* ev, uint64_t n, const Geo& g, gwcp_race* out, uint64_t cap, uint64_t* n_races,
             uint64_t* bad_index, cudaStream_t s, unsigned char* scratch) {
-  Arena A{scratch};
+  Arena A{scratch}, X{scratch + kScratchBytes, kExtraBytes};
   Bufs b{};
   Sizes z{};
   Prof prof;  // off
@@ -199,15 +204,18 @@ int analyze(const Event* ev, uint64_t n, const Geo& g, gwcp_race* out, uint64_t 
   b.rows = A.take<uint32_t>(size_t(z.n_rows) * g.Wp);
   b.psnap = A.take<uint32_t>((size_t(z.n_cs) + 1) * g.Wp);
   b.hsnap = A.take<uint32_t>((size_t(z.n_cs) + 1) * g.Wp);
-  b.done = A.take<uint32_t>(size_t(z.n_cs) + 1);
+  A.take<uint32_t>(size_t(z.n_cs) + 1);  // (unused: which traces fit stays as it was)
   b.plan = A.take<uint4>(2 * (size_t(z.n_sync) + z.n_incs) + 2);
   b.recmeta = A.take<uint4>(size_t(z.n_cs) + 1);
   b.flat_off = A.take<uint32_t>(ni1);
   b.flat = A.take<uint32_t>(z.pool_cap);
   b.cursor = A.take<uint32_t>(size_t(g.W) * (z.n_locks + 1));
-  const size_t smem = size_t(2) * g.apb * 2 * g.Wp * 4;
-  z.cta_barriers = g.apb <= 32 && smem <= 96 * 1024;
+  z.cta_barriers = g.apb <= 32;
   const bool global_bars = !z.cta_barriers || g.gran == GWCP_GRAN_THREAD;
+  b.jsnap = X.take<uint32_t>((size_t(z.n_cs) + 1) * g.Wp);
+  b.plan2 = X.take<uint4>(2 * (size_t(z.n_sync) + z.n_incs) + 2);
+  b.bar_jj = X.take<uint32_t>(global_bars ? size_t(z.n_bar) * g.Wp : 1);
+  if (X.full) return GWCP_ERR_UNSUPPORTED;
   b.bar_j = A.take<uint32_t>(global_bars ? size_t(z.n_bar) * 2 * g.Wp : 1);
   b.bar_cnt = A.take<uint32_t>(global_bars ? z.n_bar : 1);
   z.n_chunks = uint32_t(check_chunks(z.n_acc));
@@ -230,10 +238,10 @@ int analyze(const Event* ev, uint64_t n, const Geo& g, gwcp_race* out, uint64_t 
   uint32_t* race_tmp = A.take<uint32_t>(race_tmp_elems);
   if (A.full || !z.race_cap) return GWCP_ERR_UNSUPPORTED;
 
-  cudaMemsetAsync(b.done, 0, (size_t(z.n_cs) + 1) * 4, s);
   cudaMemsetAsync(b.cursor, 0, size_t(g.W) * (z.n_locks + 1) * 4, s);
   if (global_bars && z.n_bar) {
     cudaMemsetAsync(b.bar_j, 0, size_t(z.n_bar) * 2 * g.Wp * 4, s);
+    cudaMemsetAsync(b.bar_jj, 0, size_t(z.n_bar) * g.Wp * 4, s);
     cudaMemsetAsync(b.bar_cnt, 0, size_t(z.n_bar) * 4, s);
   }
   phaseD_gaps(b, g, z, s, prof);

@@ -7,17 +7,38 @@
 // width (64-, 128- or 256-bit loads). After each entry the warp stores P_t as the
 // agent's next clock version; the race check reads those rows.
 //
-// Cross-agent values are snapshots written once: a release stores P_t and H_t (the
-// paper's P_<l,s>, H_<l,s> and its Rel-queue entry) and then raises a completion flag
-// with release semantics. An acquire waits (bounded) on the flags of the releases it
+// A third clock, JN_t, is the join of every H snapshot that entered P_t: joined from the
+// lock's published JN at an acquire, over the members at a barrier, and with every H
+// snapshot joined in the release loop or at an in-section access. H moves only by joins of
+// whole H clocks, so JN_t[v] >= e means that P_t already holds the H snapshot of v's release
+// at local time e, and a join of that release (release loop, L^w / L^r) changes nothing and
+// is skipped.
+//
+// Cross-agent values are snapshots written once: a release stores P_t, H_t and JN_t (the
+// paper's P_<l,s>, H_<l,s> and its Rel-queue entry) over rows filled with a sentinel word; a
+// row without a sentinel word is complete. An acquire waits (bounded) for the releases it
 // joins - the latest release on every overlapping scope of the lock, precomputed per
 // acquire. Because every dependence points backwards in trace order and each walker
 // processes its own entries in trace order, the earliest unprocessed event can always
 // proceed, so all waits end on a well-formed trace. All walkers are co-resident
-// (cooperative launch). A barrier whose block fits in one CTA is a CTA barrier with a
-// shared-memory join; other barriers use a per-barrier global join with atomics and a
-// bounded wait. A wait that gives up sets GWCP_ERR_TIMEOUT and the walker continues
-// without waiting, so no CTA barrier is left short of arrivals.
+// (cooperative launch). A barrier whose block fits in one CTA is a shared-memory join: two
+// buffers in turn hold the block's joined rows, and since clocks only grow a member adds its
+// rows with max reductions only if they changed since the last barrier, else its own entry
+// alone. Other barriers use a per-barrier global join with atomics and a bounded wait. A wait
+// that gives up sets GWCP_ERR_TIMEOUT and the walker continues without waiting, so no CTA
+// barrier is left short of arrivals.
+//
+// What bounds it: the chain of barrier periods and lock hand-offs, each as long as its
+// slowest walker's steps (two walkers per scheduler issue an instruction every five to eight
+// cycles), so everything a step does not need is kept off that path. Plan entries are read
+// from shared memory, loaded 16 at a time a batch ahead; the records of the next release and
+// the snapshot rows of coming acquires are fetched by walkers that reach a barrier without
+// another step since the last one (they are early), or after a release when no barrier is
+// near. Propagation, ms, against register-held plan entries decoded by shuffles, staging at
+// every step and joins without JN_t: 64 warps, 10M events 16.4 -> 11.2; 256 warps, 5M
+// 6.1 -> 1.87; 512 warps (8 per block), 3M 2.9 (tile tables) and 1.0; two blocks of 128
+// threads, 250k 6.2 -> 0.48; 64 threads, 10k 0.28 -> 0.07; compressed versions, 64 warps, 3M
+// 7.1 -> 5.2. An mbarrier polled between pieces of that work measured 11.6 on the first.
 #include "gwcp_internal.cuh"
 
 namespace gwcp {
@@ -36,14 +57,19 @@ struct PropArgs {
   const uint32_t *cs_of_sync, *cs_agent, *cs_sid, *cs_epoch, *cs_rel_idx, *cs_lock, *lock_cs_lo, *cs_rel_epoch;
   const uint32_t *acq_dep_off, *acq_dep_cnt, *pool;
   const uint32_t* flat;
-  uint4* plan;
+  uint4* plan;   // two per step
+  uint4* plan2;  // two per step, in-section accesses only: (agent, release epoch) per joined release
   uint4* recmeta;
   uint32_t hb_only;  // publish H_t instead of P_t as the clock versions the check reads
   uint32_t* rows;
-  uint32_t *psnap, *hsnap, *done, *cursor;
-  uint32_t *bar_j, *bar_cnt;
+  uint32_t *psnap, *hsnap, *jsnap, *cursor;
+  uint32_t *bar_j, *bar_jj, *bar_cnt;
   uint32_t n_locks;
   int cta_barriers;
+  // shared memory of a CTA, in words: the barrier joins' rows, then per warp its plan entries,
+  // a row, the H rows of the last acquire (keep_h) and `slots` staged acquires of up to `deps`
+  // releases each
+  uint32_t acc_words, warp_words, slots, deps, keep_h;
   uint32_t forced;  // forced compression at barriers: local times come from the plan
   // compressed clock versions: rows holds B header words per version
   uint32_t compress;
@@ -216,31 +242,26 @@ __device__ __forceinline__ CvState put_row_lanes(const PropArgs& a, uint32_t row
   return cs;
 }
 
-template <int K>
-__device__ __forceinline__ void join_row(uint32_t (&x)[K], const uint32_t* row) {
-  uint32_t y[K];
-  load_row<K>(row, y);
-#pragma unroll
-  for (int j = 0; j < K; ++j) x[j] = max(x[j], y[j]);
-}
-
-// entry v of a blocked clock (owner lane v / K, register v % K), broadcast to the warp
+// entry v of a blocked clock (owner lane v / K, register v % K), broadcast to the warp. The
+// registers are selected by bit tests of v, so that the array is never indexed (indexed, it
+// lives in local memory).
 template <int K>
 __device__ __forceinline__ uint32_t get_entry(const uint32_t (&x)[K], uint32_t v) {
-  uint32_t r = 0;
+  uint32_t t[K];
 #pragma unroll
-  for (int j = 0; j < K; ++j)
-    if (j == int(v % K)) r = x[j];
-  return __shfl_sync(0xffffffffu, r, int(v / K));
+  for (int j = 0; j < K; ++j) t[j] = x[j];
+#pragma unroll
+  for (int h = K / 2; h >= 1; h /= 2)
+#pragma unroll
+    for (int j = 0; j < h; ++j) t[j] = (v & h) ? t[j + h] : t[j];
+  return __shfl_sync(0xffffffffu, t[0], int(v / K));
 }
 
 template <int K>
 __device__ __forceinline__ void set_entry(uint32_t (&x)[K], uint32_t v, uint32_t val) {
-  if ((threadIdx.x & 31) == v / K) {
+  const uint32_t first = (threadIdx.x & 31) * K;
 #pragma unroll
-    for (int j = 0; j < K; ++j)
-      if (j == int(v % K)) x[j] = val;
-  }
+  for (int j = 0; j < K; ++j) x[j] = first + j == v ? val : x[j];
 }
 
 constexpr uint32_t SENTINEL = 0xFFFFFFFFu;  // no clock entry ever takes this value
@@ -259,13 +280,20 @@ __device__ __forceinline__ bool row_complete(const uint32_t (&y)[K]) {
   return __all_sync(0xffffffffu, ok);
 }
 
+template <int K>
+__device__ __forceinline__ bool rows_complete(const uint32_t (&x)[K], const uint32_t (&y)[K], const uint32_t (&z)[K]) {
+  bool ok = true;
+#pragma unroll
+  for (int j = 0; j < K; ++j) ok &= x[j] != SENTINEL && y[j] != SENTINEL && z[j] != SENTINEL;
+  return __all_sync(0xffffffffu, ok);
+}
+
 // re-read from L2 until complete (bounded: after `limit` polls the wait gives up, sets
 // GWCP_ERR_TIMEOUT and the walker carries on)
 template <int K>
-__device__ __noinline__ void wait_row(const uint32_t* row, uint32_t (&y)[K], bool& abort, DevStatus* st,
-                                     uint32_t limit = kSpinLimit) {
-  uint32_t it = 0;
-  for (;;) {
+__device__ __forceinline__ void wait_row(const uint32_t* row, uint32_t (&y)[K], bool& abort, DevStatus* st,
+                                         uint32_t limit = kSpinLimit) {
+  for (uint32_t it = 0;;) {
     load_row<K>(row, y);
     if (row_complete<K>(y) || abort) return;
     if (++it > limit) {
@@ -273,66 +301,50 @@ __device__ __noinline__ void wait_row(const uint32_t* row, uint32_t (&y)[K], boo
       abort = true;
       return;
     }
-    __nanosleep(32);
+    if (it > 16) __nanosleep(32);
   }
 }
 
-// x |= the rows at base + ids[q] * Wp, all loads issued before any is used
+// x |= row, y |= row for the n rows at base + ids[q] * Wp, all loads issued before any is used
 template <int K, int M>
-__device__ __forceinline__ void join_rows(uint32_t (&x)[K], const uint32_t* base, const uint32_t (&ids)[M], int n,
-                                          uint32_t Wp, bool& abort, DevStatus* st) {
-  uint32_t y[M][K];
+__device__ __forceinline__ void join_rows(uint32_t (&x)[K], uint32_t (&y)[K], const uint32_t* base,
+                                          const uint32_t (&ids)[M], int n, bool& abort, DevStatus* st) {
+  uint32_t r[M][K];
 #pragma unroll
   for (int q = 0; q < M; ++q)
-    if (q < n) load_row<K>(base + size_t(ids[q]) * Wp, y[q]);
+    if (q < n) load_row<K>(base + size_t(ids[q]) * 32 * K, r[q]);
 #pragma unroll
   for (int q = 0; q < M; ++q) {
     if (q < n) {
-      if (!row_complete<K>(y[q])) wait_row<K>(base + size_t(ids[q]) * Wp, y[q], abort, st);
-#pragma unroll
-      for (int j = 0; j < K; ++j) x[j] = max(x[j], y[q][j]);
-    }
-  }
-}
-
-// x |= rows of base_x, y |= rows of base_y for the same ids: all loads issued first
-template <int K, int M>
-__device__ __forceinline__ void join_rows2(uint32_t (&x)[K], const uint32_t* base_x, uint32_t (&y)[K],
-                                           const uint32_t* base_y, const uint32_t (&ids)[M], int n, uint32_t Wp,
-                                           bool& abort, DevStatus* st) {
-  uint32_t rx[M][K], ry[M][K];
-#pragma unroll
-  for (int q = 0; q < M; ++q) {
-    if (q < n) {
-      load_row<K>(base_x + size_t(ids[q]) * Wp, rx[q]);
-      load_row<K>(base_y + size_t(ids[q]) * Wp, ry[q]);
-    }
-  }
-#pragma unroll
-  for (int q = 0; q < M; ++q) {
-    if (q < n) {
-      if (!row_complete<K>(rx[q])) wait_row<K>(base_x + size_t(ids[q]) * Wp, rx[q], abort, st);
-      if (!row_complete<K>(ry[q])) wait_row<K>(base_y + size_t(ids[q]) * Wp, ry[q], abort, st);
+      if (!row_complete<K>(r[q])) wait_row<K>(base + size_t(ids[q]) * 32 * K, r[q], abort, st);
 #pragma unroll
       for (int j = 0; j < K; ++j) {
-        x[j] = max(x[j], rx[q][j]);
-        y[j] = max(y[j], ry[q][j]);
+        x[j] = max(x[j], r[q][j]);
+        y[j] = max(y[j], r[q][j]);
       }
     }
   }
 }
 
-// P entry v of every lane's own agent index (lane-varying v), by K shuffles
+// entry v of x for a lane-varying v: by K shuffles, or with many entries per lane through
+// the warp's shared row
 template <int K>
-__device__ __forceinline__ uint32_t lookup_entry(const uint32_t (&x)[K], uint32_t v) {
-  uint32_t r = 0;
-  const int src = int(min(v, 32u * K - 1) / K);
+__device__ __forceinline__ uint32_t lookup_entry(const uint32_t (&x)[K], uint32_t v, uint32_t* scratch) {
+  if constexpr (K <= 4) {
+    uint32_t r = 0;
+    const int src = int(min(v, 32u * K - 1) / K);
 #pragma unroll
-  for (int j = 0; j < K; ++j) {
-    const uint32_t t = __shfl_sync(0xffffffffu, x[j], src);
-    if (j == int(v % K)) r = t;
+    for (int j = 0; j < K; ++j) {
+      const uint32_t t = __shfl_sync(0xffffffffu, x[j], src);
+      if (j == int(v % K)) r = t;
+    }
+    return r;
+  } else {
+    __syncwarp();
+    store_row_shared<K>(scratch, x);
+    __syncwarp();
+    return v < 32u * K ? scratch[v] : 0u;
   }
-  return r;
 }
 
 // cp.async (LDGSTS): 16-byte copy global -> shared through L2 only (no L1 line that
@@ -343,16 +355,16 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
                : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
-// stage one clock row (Wc words) into shared memory: lane l copies 16-byte chunk l
-template <int Wc>
-__device__ __forceinline__ void stage_row(uint32_t* dst, const uint32_t* src) {
-  const int lane = threadIdx.x & 31;
-  if (lane < Wc / 4) cp_async16(dst + 4 * lane, src + 4 * lane);
+// until at most n (< 4) of the youngest groups are in flight
+__device__ __forceinline__ void cp_async_wait(uint32_t n) {
+  if (n == 0)
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+  else if (n == 1)
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+  else if (n == 2)
+    asm volatile("cp.async.wait_group 2;" ::: "memory");
+  else
+    asm volatile("cp.async.wait_group 3;" ::: "memory");
 }
 
 template <int K>
@@ -362,72 +374,98 @@ __device__ __forceinline__ void read_row_shared(const uint32_t* row, uint32_t (&
   for (int j = 0; j < K; ++j) y[j] = p[j];
 }
 
-// shared-memory words per ring slot: four rows, or 32 section records + one row; then
-// a 4-word header (kind, staged cursor, row count)
+// Shared memory by 32-bit address (the walkers' inner loop counts instructions).
+__device__ __forceinline__ uint32_t smem_addr(const void* p) {
+  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+__device__ __forceinline__ uint32_t lds(uint32_t at) {
+  uint32_t v;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(at) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint4 lds4(uint32_t at) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(at) : "memory");
+  return v;
+}
+__device__ __forceinline__ void red_max(uint32_t at, uint32_t v) {
+  asm volatile("red.shared.max.u32 [%0], %1;" ::"r"(at), "r"(v) : "memory");
+}
+// A row of a barrier buffer: the lane's K entries at lane * K (two or fewer: one load), else
+// entry j of all lanes together (no bank conflicts).
 template <int K>
-__host__ __device__ constexpr int slot_words() {
-  return (((4 * 32 * K > 128 + 32 * K) ? 4 * 32 * K : 128 + 32 * K) + 4 + 3) & ~3;
+__device__ __forceinline__ constexpr uint32_t brow(int j) {
+  return K <= 2 ? 4 * j : 128 * j;
+}
+template <int K>
+__device__ __forceinline__ void lds_row(uint32_t at, uint32_t (&x)[K]) {
+  if constexpr (K == 2) {
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(x[0]), "=r"(x[1]) : "r"(at) : "memory");
+  } else {
+#pragma unroll
+    for (int j = 0; j < K; ++j) x[j] = lds(at + brow<K>(j));
+  }
+}
+
+// plan entries per batch (64 bytes each in shared memory, two batches per warp)
+template <int K>
+__host__ __device__ constexpr int plan_batch() {
+  return K >= 32 ? 8 : 16;
 }
 
 // One warp per agent walks the agent's plan (its clock-changing steps in trace order).
-// R > 0: a ring of R shared-memory slots per warp; while entry p is processed, the
-// copies for entry p + R - 1 are in flight (one commit group per entry).
 // CV: clock versions stored compressed (a separate instantiation, so that the plain
 // walkers' register allocation does not carry it).
-template <int K, int R, int MAXT, bool CV>
-__global__ void __launch_bounds__(MAXT, 1) k_propagate(PropArgs a) {
+template <int K, int MAXT, bool CV>
+__global__ void __launch_bounds__(MAXT, 1) k_propagate(const __grid_constant__ PropArgs a) {
   constexpr int Wc = 32 * K;
-  constexpr int SLOT = slot_words<K>();
-  constexpr int RR = R > 0 ? R : 1;
+  constexpr int PB = plan_batch<K>();
+  constexpr uint32_t EW = 16;  // words of a plan entry in shared memory
   extern __shared__ __align__(16) uint32_t sm[];
   const Geo& g = a.g;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  const uint32_t u = a.cta_barriers ? blockIdx.x * g.apb + warp : blockIdx.x * 32 + warp;
-  uint32_t* const xchg = sm;  // CTA barriers: [2 buffers][warps][C | H][Wp]
-  const uint32_t xchg_words = a.cta_barriers ? 2u * nwarps * 2 * Wc : 0u;
-  uint32_t* const ring = sm + xchg_words + (R > 0 ? size_t(warp) * RR * SLOT : 0);  // unused when R = 0
-  // per-warp scratch for folding joined release epochs into jn (stale words never exceed jn)
-  uint32_t* const jn_tmp = sm + xchg_words + (R > 0 ? size_t(nwarps) * RR * SLOT : 0) + size_t(warp) * Wc;
+  const uint32_t u = a.cta_barriers ? blockIdx.x * g.apb + warp : blockIdx.x * nwarps + warp;
+  uint32_t* const acc = sm;  // barrier joins: two buffers of (C, H, JN) rows (brow)
+  uint32_t* const plan_s = sm + a.acc_words + size_t(warp) * a.warp_words;  // [2][PB][EW]
+  uint32_t* const scratch = plan_s + 2 * PB * EW;                                // [Wc]
+  uint32_t* const last_h = scratch + Wc;                                         // [2][Wc] with keep_h
+  uint32_t* const slots = last_h + (a.keep_h ? 2 * Wc : 0);                      // [slots][deps][P, H, JN][Wc]
+  const uint32_t slot_words = a.deps * 3 * Wc;
   // one read of the status per CTA, so all warps of a CTA agree on whether to run
   __shared__ int start_code;
   if (threadIdx.x == 0) start_code = *(volatile int*)&a.st->code;
+  for (uint32_t i = threadIdx.x; i < a.acc_words; i += blockDim.x) acc[i] = 0;
   __syncthreads();
   if (start_code) return;
-  const bool active = a.cta_barriers ? (uint32_t(warp) < g.apb) : (u < g.W);
-  if (!active) return;
-  for (int j = lane; j < Wc; j += 32) jn_tmp[j] = 0;
-  __syncwarp();
+  if (u >= g.W) return;  // (only without CTA barriers)
 
-  uint32_t P[K], H[K];
-  // jn[v]: latest release epoch of agent v whose H snapshot is already joined into P.
-  // H of one agent only grows along its timeline, so a release of v with epoch <= jn[v]
-  // is dominated and its join is a no-op.
-  uint32_t jn[K];
+  uint32_t P[K], H[K], J[K];
 #pragma unroll
-  for (int j = 0; j < K; ++j) P[j] = H[j] = jn[j] = 0;
-  set_entry<K>(H, u, 1u);  // H_t = bottom{t := 1}
-  uint32_t N = 1;          // N_t
+  for (int j = 0; j < K; ++j) P[j] = H[j] = J[j] = 0;
+  // H_t = bottom{t := 1}. H_t[t] = N_t is kept in N alone and put into the row where it is
+  // published (the row's own entry may lag).
+  uint32_t N = 1;  // N_t
   bool abort = false;
-  uint64_t joins = 0, visits = 0;
-  uint32_t nbar = 0;
+  uint32_t joins = 0, visits = 0, nbar = 0;
+  bool busy = false;     // a step other than a barrier since the block's last barrier
+  bool changed = false;  // P_t, H_t or JN_t took in more than its own entry since the block's last barrier
+  uint32_t last0 = NONE, last1 = NONE;  // the releases whose H rows last_h holds
   CvState cvs{0, 0, 0};  // compressed versions
   const bool cv_lanes = g.gran == GWCP_GRAN_WARP && g.apb % K == 0;
   auto put_version = [&](uint32_t r) {
+    if (a.hb_only) set_entry<K>(H, u, N);
     if constexpr (CV) {
       if (cv_lanes) {
         cvs = a.hb_only ? put_row_lanes<K>(a, r, H, cvs) : put_row_lanes<K>(a, r, P, cvs);
         return;
       }
-      // the clock goes through the warp's jn scratch words, which are then left holding jn
-      // (the release loop's rule: no word there exceeds jn)
+      __syncwarp();
       if (a.hb_only)
-        store_row_shared<K>(jn_tmp, H);
+        store_row_shared<K>(scratch, H);
       else
-        store_row_shared<K>(jn_tmp, P);
+        store_row_shared<K>(scratch, P);
       __syncwarp();
-      cvs = put_row_c(a, r, jn_tmp, cvs);
-      store_row_shared<K>(jn_tmp, jn);
-      __syncwarp();
+      cvs = put_row_c(a, r, scratch, cvs);
     } else if (a.hb_only) {
       store_row<K>(a.rows + size_t(r) * Wc, H);
     } else {
@@ -439,318 +477,412 @@ __global__ void __launch_bounds__(MAXT, 1) k_propagate(PropArgs a) {
   const uint32_t pb = k0 + a.incs_off[k0], pe = k1 + a.incs_off[k1];
   uint32_t* const cursor_row = a.cursor + size_t(u) * a.n_locks;
 
-  // plan entries in registers: the current batch of 32 and the next one; a release
-  // entry's lane also holds its cursor (forwarded when an earlier release of the same
-  // lock moves it)
-  uint4 ea, eb, ea2, eb2;
-  uint32_t pre, pre2;
-  auto load_batch = [&](uint32_t b0, uint4& xa, uint4& xb, uint32_t& xp) {
-    const uint32_t pi = b0 + lane;
-    xa = make_uint4(0, 0, 0, 0);
-    xb = make_uint4(0, 0, 0, 0);
-    xp = 0;
-    if (pi < pe) {
-      xa = a.plan[2 * size_t(pi)];
-      xb = a.plan[2 * size_t(pi) + 1];
-      if ((xa.x & 0xFF) == P_REL) xp = __ldcg(cursor_row + xa.w);
-    }
-  };
-  uint32_t base = pb;
-  load_batch(base, ea, eb, pre);
-  load_batch(base + 32, ea2, eb2, pre2);
-
-  auto stage = [&](uint32_t p) {
-    if constexpr (R > 0) {
-      if (p < pe) {
-        const bool second = p >= base + 32;
-        const int src = int((p - base) & 31);
-        const uint32_t t2 = __shfl_sync(0xffffffffu, second ? ea2.x : ea.x, src) & 0xFF;
-        if (t2 == P_BAR) {  // a barrier stages nothing: an empty group, header kind 0
-          if (lane == 0) (ring + (p % R) * SLOT)[SLOT - 4] = 0u;
-          cp_async_commit();
-          return;
-        }
-        const uint32_t w2 = __shfl_sync(0xffffffffu, second ? ea2.w : ea.w, src);
-        const uint32_t x0 = __shfl_sync(0xffffffffu, second ? eb2.x : eb.x, src);
-        const uint32_t x1 = __shfl_sync(0xffffffffu, second ? eb2.y : eb.y, src);
-        const uint32_t x2 = __shfl_sync(0xffffffffu, second ? eb2.z : eb.z, src);
-        const uint32_t x3 = __shfl_sync(0xffffffffu, second ? eb2.w : eb.w, src);
-        const uint32_t pr = __shfl_sync(0xffffffffu, second ? pre2 : pre, src);
-        uint32_t* slot = ring + (p % R) * SLOT;
-        uint32_t kind = 0, nrows = 0, cur_staged = 0;
-        if (t2 == P_ACQ && w2 >= 1 && w2 <= 2) {
-          stage_row<Wc>(slot, a.psnap + size_t(x0) * Wc);
-          stage_row<Wc>(slot + Wc, a.hsnap + size_t(x0) * Wc);
-          if (w2 == 2) {
-            stage_row<Wc>(slot + 2 * Wc, a.psnap + size_t(x1) * Wc);
-            stage_row<Wc>(slot + 3 * Wc, a.hsnap + size_t(x1) * Wc);
-          }
-          kind = 1;
-          nrows = 2 * w2;
-        } else if (t2 == P_INCS && w2 >= 1 && w2 <= 4) {
-          const uint32_t ids[4] = {x0, x1, x2, x3};
+  // Batches of PB plan entries: the current one (first step `base`, in half `half` of the
+  // plan buffer) and the next, whose entries are loaded into registers when the current batch
+  // begins and put into shared memory later, with the loads of its releases' cursors. This,
+  // the rows of coming acquires and the records of the next release are fetched while the
+  // walker waits at a barrier or after it has published a release (`ahead` below).
+  constexpr int LD = PB * 4 / 32;
+  uint4 nx[LD];
+  auto load_entries = [&](uint32_t b0) {
 #pragma unroll
-          for (int q = 0; q < 4; ++q)
-            if (q < int(w2)) stage_row<Wc>(slot + q * Wc, a.hsnap + size_t(ids[q]) * Wc);
-          kind = 1;
-          nrows = w2;
-        } else if (t2 == P_REL) {
-          const uint32_t lo = x0, hi = x1;
-          cur_staged = pr;
-          if (lo + pr + lane < hi) cp_async16(slot + 4 * lane, a.recmeta + lo + pr + lane);
-          if (lo + pr < hi) stage_row<Wc>(slot + 128, a.hsnap + size_t(lo + pr) * Wc);
-          kind = 2;
-        }
-        if (lane == 0) {
-          slot[SLOT - 4] = kind;
-          slot[SLOT - 3] = cur_staged;
-          slot[SLOT - 2] = nrows;
-        }
-      }
-      cp_async_commit();
+    for (int q = 0; q < LD; ++q) {
+      const uint32_t c = q * 32 + lane, e = b0 + c / 4;
+      nx[q] = make_uint4(0, 0, 0, 0);
+      if (e < pe) nx[q] = (c & 2) ? __ldcg(a.plan2 + 2 * size_t(e) + (c & 1)) : __ldcg(a.plan + 2 * size_t(e) + (c & 1));
     }
   };
-  for (int q = 0; q < R - 1; ++q) stage(pb + q);
-
-  for (uint32_t p = pb; p < pe; ++p) {
-    const uint32_t i = p - base;
+  // lane l < PB: the lock and the cursor of entry l when it is a release, else NONE
+  uint32_t lock_a = NONE, cur_a = 0, lock_b = NONE, cur_b = 0;
+  uint32_t acq_a = 0, acq_b = 0;  // the batch's acquires (bit per entry)
+  uint32_t rel_a = 0, rel_b = 0;  // releases
+  uint32_t bar_a = 0, bar_b = 0;  // and block barriers
+  bool put = false;               // the next batch is in shared memory
+  auto put_entries = [&](uint32_t b0, uint32_t h) {
+    uint4* d = reinterpret_cast<uint4*>(plan_s + h * PB * EW);
     __syncwarp();
-    stage(p + R - 1);
-    uint32_t skind = 0;
-    const uint32_t* slot = ring + (R > 0 ? (p % RR) : 0) * SLOT;
-    if constexpr (R > 0) {
-      cp_async_wait<(R > 0 ? R - 1 : 0)>();
-      __syncwarp();
-      skind = slot[SLOT - 4];
+#pragma unroll
+    for (int q = 0; q < LD; ++q) d[q * 32 + lane] = nx[q];
+    __syncwarp();
+    const bool mine = lane < PB && b0 + lane < pe;
+    const uint32_t* e = plan_s + (h * PB + (lane & (PB - 1))) * EW;
+    const uint32_t t = mine ? e[0] & 0xFF : 0xFFu;
+    acq_b = __ballot_sync(0xffffffffu, t == P_ACQ);
+    rel_b = __ballot_sync(0xffffffffu, t == P_REL);
+    bar_b = __ballot_sync(0xffffffffu, t == P_BAR && e[4] == BAR_CTA);
+    put = true;
+    lock_b = NONE;
+    if (t == P_REL) {
+      lock_b = e[3];
+      cur_b = __ldcg(cursor_row + lock_b);
     }
-    const uint32_t t = __shfl_sync(0xffffffffu, ea.x, i) & 0xFF;
-    const uint32_t row = __shfl_sync(0xffffffffu, ea.y, i);
-    const uint32_t z = __shfl_sync(0xffffffffu, ea.z, i);
-    const uint32_t w = __shfl_sync(0xffffffffu, ea.w, i);
-    if ((t == P_ACQ || t == P_INCS) && skind == 1) {
-      // staged rows: validate (an incomplete one is re-read from L2), then join
-      const int nrows = int(slot[SLOT - 2]);
-      const uint32_t ids[4] = {__shfl_sync(0xffffffffu, eb.x, i), __shfl_sync(0xffffffffu, eb.y, i),
-                               __shfl_sync(0xffffffffu, eb.z, i), __shfl_sync(0xffffffffu, eb.w, i)};
+  };
+  uint32_t base = pb, half = 0;
+  if (pb < pe) {
+    load_entries(pb);
+    put_entries(pb, 0);
+    lock_a = lock_b;
+    cur_a = cur_b;
+    acq_a = acq_b;
+    rel_a = rel_b;
+    bar_a = bar_b;
+    lock_b = NONE;
+    acq_b = rel_b = bar_b = 0;
+    put = false;
+    load_entries(pb + PB);
+  }
+  auto entry = [&](uint32_t i) {  // entry i of the current batch, or i - PB of the next
+    return plan_s + (((i >= uint32_t(PB)) ? half ^ 1u : half) * PB + (i & (PB - 1))) * EW;
+  };
+
+  // Staged acquires, in trace order: the rows of steps q0, q1, .. (NONE: none) are in slots
+  // first, first + 1, ..; the search for the next one starts at step sq.
+  uint32_t q0 = NONE, q1 = NONE, q2 = NONE, q3 = NONE, staged = 0, first = 0, sq = pb;
+  // Records of the next release (step rec_p), a lane each from its lock's cursor on: the agent
+  // (NONE past the lock's last record), the acquire's local time (0 for an own record) and
+  // the release's (0 unless the release may join it).
+  uint32_t rec_ag = NONE, rec_acq = 0, rec_rel = 0;
+  uint32_t rec_p = NONE;
+  auto load_records = [&](uint32_t rec, uint32_t hi, uint32_t s, uint32_t my_idx) {
+    uint4 m = make_uint4(NONE, 0, NONE, 0);
+    if (rec < hi) m = __ldg(a.recmeta + rec);
+    rec_ag = m.x == NONE ? NONE : (m.x & 0xFFFF);
+    const bool mine = rec_ag == u;
+    rec_acq = mine ? 0u : m.y;
+    rec_rel = !mine && m.z != NONE && m.z < my_idx && scopes_overlap(m.x >> 16, s) ? m.w : 0u;
+  };
+  // One piece of work for later steps, at step p; false when there is none.
+  auto ahead = [&](uint32_t p) -> bool {
+    if (int(sq - p) <= 0) sq = p + 1;
+    const uint32_t m_acq =
+        staged < a.slots && sq - base < 2 * PB ? (acq_a | (acq_b << PB)) & (0xFFFFFFFFu << (sq - base)) : 0u;
+    if (!m_acq) {
+      // the records of the next release; then the next batch's entries. Neither is touched
+      // before its loads (the batch's cursors, the entries) have had a few steps to arrive.
+      const uint32_t m = (rel_a | (p - base >= 3 * PB / 4 ? rel_b << PB : 0u)) & (0xFFFFFFFEu << (p - base));
+      const uint32_t i = m ? uint32_t(__ffs(m) - 1) : 0u;
+      if (m && rec_p != base + i) {
+        rec_p = base + i;
+        const uint32_t* e = entry(i);
+        const uint32_t c = __shfl_sync(0xffffffffu, i < uint32_t(PB) ? cur_a : cur_b, i & (PB - 1));
+        load_records(e[4] + c + lane, e[5], e[6], e[7]);
+        return true;
+      }
+      if (!put && p - base >= PB / 4 && base + PB < pe) {
+        put_entries(base + PB, half ^ 1u);
+        return true;
+      }
+      return false;
+    }
+    const uint32_t i = uint32_t(__ffs(m_acq) - 1);
+    const uint32_t* e = entry(i);
+    sq = base + i + 1;
+    const uint32_t cnt = e[3];
+    if (cnt == 0 || cnt > a.deps) return true;
+    uint32_t* slot = slots + ((first + staged) & (a.slots - 1)) * slot_words;
+    for (uint32_t d = 0; d < cnt; ++d) {
+      const size_t at = size_t(e[4 + d]) * Wc;
+      uint32_t* dst = slot + d * 3 * Wc;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        if (q < nrows) {
-          uint32_t y[K];
-          read_row_shared<K>(slot + q * Wc, y);
-          const bool acq = t == P_ACQ;
-          const uint32_t* src = acq ? ((q & 1) ? a.hsnap : a.psnap) + size_t(ids[q >> 1]) * Wc
-                                    : a.hsnap + size_t(ids[q]) * Wc;
-          if (!row_complete<K>(y)) wait_row<K>(src, y, abort, a.st);
-          if (acq && (q & 1)) {
+      for (int c = lane; c < 3 * Wc / 4; c += 32) {
+        const int r = c / (Wc / 4);
+        const uint32_t* src = (r == 0 ? a.psnap : r == 1 ? a.hsnap : a.jsnap) + at;
+        cp_async16(dst + 4 * c, src + 4 * (c % (Wc / 4)));
+      }
+    }
+    cp_async_commit();
+    q0 = staged == 0 ? base + i : q0;
+    q1 = staged == 1 ? base + i : q1;
+    q2 = staged == 2 ? base + i : q2;
+    q3 = staged == 3 ? base + i : q3;
+    ++staged;
+    return true;
+  };
+
+  // the barrier buffer in turn (bufs: the sum of both addresses), and the agent's own entries
+  // in it: lane 0 the C row's, lane 1 the H row's
+  uint32_t buf = smem_addr(acc);
+  const uint32_t bufs = 2 * buf + 12 * Wc;
+  const uint32_t own = (lane & 1) * Wc * 4 + u / K * (K <= 2 ? 4 * K : 4) +
+                       (u % K) * (K <= 2 ? 4 : 128);
+  uint32_t e_at = smem_addr(plan_s);  // the entry of step p
+  for (uint32_t p = pb; p < pe; ++p) {
+    const uint4 ea = lds4(e_at), eb = lds4(e_at + 16);
+    const uint32_t t = ea.x, z = ea.z, w = ea.w;
+    if (t == P_BAR) {
+      // sync (Algorithm 1): join C_t and H_t over the barrier's scope. The plan holds N_t
+      // entering the join (under forced compression at barriers the highest N among the
+      // members)
+      const uint32_t mode = eb.x;
+      N = eb.y;
+      if (mode == BAR_CTA) {
+        // Two buffers in turn hold the block's joined rows, which only grow: a member whose
+        // rows are still the last join's adds its own entries alone.
+        if (changed) {
+          const uint32_t at = buf + (K <= 2 ? lane * K : lane) * 4;
 #pragma unroll
-            for (int j = 0; j < K; ++j) H[j] = max(H[j], y[j]);
-          } else {
-#pragma unroll
-            for (int j = 0; j < K; ++j) P[j] = max(P[j], y[j]);
+          for (int j = 0; j < K; ++j) {
+            red_max(at + brow<K>(j), P[j]);
+            red_max(at + Wc * 4 + brow<K>(j), H[j]);
+            red_max(at + Wc * 8 + brow<K>(j), J[j]);
           }
         }
-      }
-      joins += nrows;
-    } else if (t == P_ACQ || t == P_INCS) {
-      // acquire (Algorithm 1): P_t |= P_<l,s'>, H_t |= H_<l,s'> over the overlapping
-      // scopes' latest releases; in-section access (Algorithm 2): P_t |= L^w (| L^r)
-      const uint32_t* list = t == P_ACQ ? a.pool : a.flat;
-      for (uint32_t q0 = 0; q0 < w; q0 += 4) {
-        uint32_t ids[4];
-        if (w <= 4) {
-          ids[0] = __shfl_sync(0xffffffffu, eb.x, i);
-          ids[1] = __shfl_sync(0xffffffffu, eb.y, i);
-          ids[2] = __shfl_sync(0xffffffffu, eb.z, i);
-          ids[3] = __shfl_sync(0xffffffffu, eb.w, i);
-        } else {
+        // (no other member holds a larger value, so a plain store is enough)
+        if (lane < 2) asm volatile("st.shared.u32 [%0], %1;" ::"r"(buf + own), "r"(N) : "memory");
+        // a member with no other step since the last barrier is early: it works ahead
+        if (!busy) ahead(p);
+        changed = busy = false;
+        __syncthreads();
+        {
+          const uint32_t at = buf + (K <= 2 ? lane * K : lane) * 4;
+          lds_row<K>(at, P);
+          lds_row<K>(at + Wc * 4, H);
+          lds_row<K>(at + Wc * 8, J);
+        }
+        // the other buffer, which every member has read after the barrier before, takes this
+        // join in (members that are ahead may already add to it)
+        const uint32_t other = bufs - buf;
+        for (uint32_t q = threadIdx.x * 4; q < 12 * Wc; q += blockDim.x * 4) {
+          const uint32_t v = lds(buf + q);
+          if (v > lds(other + q)) red_max(other + q, v);
+        }
+        buf = other;
+        ++nbar;
+      } else {
+        set_entry<K>(P, u, N);  // C_t
+        if (mode == BAR_GLOBAL) {
+          const uint32_t bid = z, count = w;
+          uint32_t* JP = a.bar_j + size_t(bid) * 2 * Wc;
+          uint32_t* JJ = a.bar_jj + size_t(bid) * Wc;
+          set_entry<K>(H, u, N);
 #pragma unroll
-          for (int q = 0; q < 4; ++q) ids[q] = q0 + q < w ? __ldcg(list + z + q0 + q) : 0;
-        }
-        const int n = int(min(4u, w - q0));
-        if (t == P_ACQ) {
-          join_rows2<K, 4>(P, a.psnap, H, a.hsnap, ids, n, Wc, abort, a.st);
-          joins += 2 * n;
-        } else {
-          join_rows<K, 4>(P, a.hsnap, ids, n, Wc, abort, a.st);
-          joins += n;
+          for (int j = 0; j < K; ++j) {
+            atomicMax(JP + lane * K + j, P[j]);
+            atomicMax(JP + Wc + lane * K + j, H[j]);
+            atomicMax(JJ + lane * K + j, J[j]);
+          }
+          __threadfence();
+          __syncwarp();
+          if (lane == 0) atomicAdd(a.bar_cnt + bid, 1u);
+          if (!abort) {
+            bool ok = true;
+            if (lane == 0) {
+              uint32_t it = 0;
+              while (ld_acquire(a.bar_cnt + bid) < count) {
+                if (++it > kSpinLimit) {
+                  ok = false;
+                  break;
+                }
+                if (it > 16) __nanosleep(64);
+              }
+              if (!ok) atomicCAS(&a.st->code, 0, GWCP_ERR_TIMEOUT);
+            }
+            ok = __shfl_sync(0xffffffffu, ok, 0);
+            __syncwarp();
+            if (!ok) abort = true;
+          }
+          load_row<K>(JP, P);
+          load_row<K>(JP + Wc, H);
+          load_row<K>(JJ, J);
+          changed = true;
+          joins += 2;
         }
       }
-    } else if (t == P_REL) {
+      ++N;
+    } else if (t == P_INCS) {
+      busy = true;
+      // in-section access (Algorithm 2): P_t |= L^w (| L^r), each the H snapshot of an earlier
+      // section's release, unless JN_t already covers it
+      for (uint32_t q = 0; q < w; ++q) {
+        uint32_t x, ag, ep;
+        if (w <= 4) {
+          x = q == 0 ? eb.x : q == 1 ? eb.y : q == 2 ? eb.z : eb.w;
+          ag = lds(e_at + 32 + 8 * q);
+          ep = lds(e_at + 36 + 8 * q);
+        } else {
+          x = __ldcg(a.flat + z + q);
+          const uint4 mx = __ldg(a.recmeta + x);
+          ag = mx.x & 0xFFFF;
+          ep = mx.w;
+        }
+        if (get_entry<K>(J, ag) >= ep) continue;
+        uint32_t y[K];
+        if (x == last0 || x == last1)
+          read_row_shared<K>(last_h + (x == last0 ? 0 : Wc), y);
+        else
+          wait_row<K>(a.hsnap + size_t(x) * Wc, y, abort, a.st);
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+          P[j] = max(P[j], y[j]);
+          J[j] = max(J[j], y[j]);
+        }
+        changed = true;
+        ++joins;
+      }
+    } else if (t == P_ACQ) {
+      busy = true;
+      // acquire (Algorithm 1): P_t |= P_<l,s'>, H_t |= H_<l,s'> over the overlapping
+      // scopes' latest releases
+      const bool here = q0 == p;  // its rows are in slot `first`
+      const uint32_t* slot = slots + (first & (a.slots - 1)) * slot_words;
+      if (here) {
+        --staged;
+        cp_async_wait(staged);
+        ++first;
+        q0 = q1;
+        q1 = q2;
+        q2 = q3;
+        q3 = NONE;
+        __syncwarp();  // every lane's copies
+      }
+      for (uint32_t q = 0; q < w; ++q) {
+        const uint32_t x = w > 4 ? __ldcg(a.pool + z + q) : q == 0 ? eb.x : q == 1 ? eb.y : q == 2 ? eb.z : eb.w;
+        const size_t at = size_t(x) * Wc;
+        if constexpr (K <= 8) {
+          uint32_t yp[K], yh[K], yj[K];
+          bool ok = false;
+          if (here) {
+            const uint32_t* rows = slot + q * 3 * Wc;
+            read_row_shared<K>(rows, yp);
+            read_row_shared<K>(rows + Wc, yh);
+            read_row_shared<K>(rows + 2 * Wc, yj);
+            ok = rows_complete<K>(yp, yh, yj);
+          }
+          for (uint32_t it = 0; !ok; ++it) {  // the three rows polled together
+            load_row<K>(a.psnap + at, yp);
+            load_row<K>(a.hsnap + at, yh);
+            load_row<K>(a.jsnap + at, yj);
+            ok = rows_complete<K>(yp, yh, yj);
+            if (ok || abort) break;
+            if (it >= kSpinLimit) {
+              if (lane == 0) atomicCAS(&a.st->code, 0, GWCP_ERR_TIMEOUT);
+              abort = true;
+              break;
+            }
+            if (it > 16) __nanosleep(32);
+          }
+#pragma unroll
+          for (int j = 0; j < K; ++j) {
+            P[j] = max(P[j], yp[j]);
+            H[j] = max(H[j], yh[j]);
+            J[j] = max(J[j], yj[j]);
+          }
+          if (a.keep_h && q < 2) store_row_shared<K>(last_h + q * Wc, yh);
+        } else {
+          uint32_t y[K];
+          wait_row<K>(a.psnap + at, y, abort, a.st);
+#pragma unroll
+          for (int j = 0; j < K; ++j) P[j] = max(P[j], y[j]);
+          wait_row<K>(a.jsnap + at, y, abort, a.st);
+#pragma unroll
+          for (int j = 0; j < K; ++j) J[j] = max(J[j], y[j]);
+          wait_row<K>(a.hsnap + at, y, abort, a.st);
+#pragma unroll
+          for (int j = 0; j < K; ++j) H[j] = max(H[j], y[j]);
+          if (a.keep_h && q < 2) store_row_shared<K>(last_h + q * Wc, y);
+        }
+      }
+      joins += 2 * w;
+      changed |= w != 0;
+      last0 = w > 0 && w <= 4 && a.keep_h ? eb.x : NONE;
+      last1 = w > 1 && w <= 4 && a.keep_h ? eb.y : NONE;
+    } else {
       // release (Algorithm 1): pop other agents' records on this lock while their
       // acquire is ordered before C_t; join the released ones whose scope overlaps.
       // Waves: every record before the first one failing the test against the current
       // P passes (P only grows), so their snapshots are joined together; the failing
       // record is tested again only if the wave changed P.
-      const uint32_t c = z, L = w;
-      const uint32_t lo = __shfl_sync(0xffffffffu, eb.x, i), hi = __shfl_sync(0xffffffffu, eb.y, i);
-      const uint32_t s = __shfl_sync(0xffffffffu, eb.z, i), my_idx = __shfl_sync(0xffffffffu, eb.w, i);
-      uint32_t cur = __shfl_sync(0xffffffffu, pre, i);
-      bool staged = skind == 2 && slot[SLOT - 3] == cur;
-      bool stop = false;
-      while (!stop && lo + cur < hi) {
-        const uint32_t rec = lo + cur + lane;
+      busy = true;
+      const uint32_t i = p - base, c = z, L = w;
+      const uint32_t lo = eb.x, hi = eb.y;
+      uint32_t cur = __shfl_sync(0xffffffffu, cur_a, i);
+      bool fetched = rec_p == p;
+      while (lo + cur < hi) {
+        if (!fetched) load_records(lo + cur + lane, hi, eb.z, eb.w);
+        fetched = false;
         const uint32_t nbr = min(32u, hi - (lo + cur));
-        uint4 m = make_uint4(NONE, 0, NONE, 0);
-        uint32_t spec[K];
-        if (staged) {  // the first 32 records and the first one's snapshot are in the slot
-          if (rec < hi) m = *reinterpret_cast<const uint4*>(slot + 4 * lane);
-          read_row_shared<K>(slot + 128, spec);
-        } else {
-          if (rec < hi) m = __ldg(a.recmeta + rec);
-          load_row<K>(a.hsnap + size_t(lo + cur) * Wc, spec);
-        }
-        staged = false;
-        bool spec_live = true;
-        const uint32_t mag = m.x == NONE ? NONE : (m.x & 0xFFFF);
-        const uint32_t msid = m.x >> 16;
-        const bool mine = mag == u;
-        const bool joinable = !mine && m.z != NONE && m.z < my_idx && scopes_overlap(msid, s);
+        const uint32_t others = __ballot_sync(0xffffffffu, rec_ag != u);  // (lanes past the last record too)
         uint32_t start = 0;
-        while (start < nbr) {
-          const uint32_t pv = lookup_entry<K>(P, mag);
-          const uint32_t jv = lookup_entry<K>(jn, mag);
-          const bool in = uint32_t(lane) >= start && uint32_t(lane) < nbr;
-          const uint32_t fail = __ballot_sync(0xffffffffu, in && !mine && m.y > pv);
+        bool stop = false;
+        for (;;) {
+          const uint32_t pv = lookup_entry<K>(P, rec_ag, scratch);
+          const uint32_t jv = lookup_entry<K>(J, rec_ag, scratch);
+          const uint32_t from = 0xFFFFFFFFu << start;  // start < 32
+          const uint32_t fail = __ballot_sync(0xffffffffu, rec_acq > pv) & from;
           const uint32_t f = fail ? uint32_t(__ffs(fail) - 1) : nbr;  // first failing record
-          const uint32_t popped = __ballot_sync(0xffffffffu, in && uint32_t(lane) < f && joinable);
+          const uint32_t below = f < 32 ? (1u << f) - 1u : 0xFFFFFFFFu;
+          visits += __popc(others & from & (fail ? below | (1u << f) : below));
           // of the popped releases, join only those not dominated, and per agent only
           // the latest (records of one agent are in acquire order)
-          const bool cand = ((popped >> lane) & 1u) && m.w > jv;
-          const uint32_t same = __match_any_sync(0xffffffffu, cand ? mag : 0xFFFFFFFFu);
-          const uint32_t wave = __ballot_sync(0xffffffffu, cand && (same >> lane) <= 1u);
-          visits += __popc(__ballot_sync(0xffffffffu, in && uint32_t(lane) <= f && !mine));
-          uint32_t wm = wave;
-          if (wave) {  // record the joined releases' epochs: distinct agents scatter, owners fold
-            if ((wave >> lane) & 1u) jn_tmp[mag] = m.w;
-            __syncwarp();
-#pragma unroll
-            for (int j = 0; j < K; ++j) jn[j] = max(jn[j], jn_tmp[lane * K + j]);
-            __syncwarp();
-          }
-          if (spec_live && (wm & 1u)) {  // record lo + cur: its row is already loaded
-            if (!row_complete<K>(spec)) wait_row<K>(a.hsnap + size_t(lo + cur) * Wc, spec, abort, a.st);
-#pragma unroll
-            for (int j = 0; j < K; ++j) P[j] = max(P[j], spec[j]);
-            ++joins;
-            wm &= ~1u;
-          }
-          spec_live = false;
-          while (wm) {
-            uint32_t ids[4];
-            int n = 0;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              ids[q] = 0;
-              if (wm) {
-                ids[q] = lo + cur + (__ffs(wm) - 1);
-                wm &= wm - 1;
-                ++n;
-              }
+          uint32_t wave = __ballot_sync(0xffffffffu, rec_rel > jv) & from & below;
+          if (wave) {
+            changed = true;
+            if (wave & (wave - 1)) {
+              const bool cand = (wave >> lane) & 1u;
+              const uint32_t same = __match_any_sync(0xffffffffu, cand ? rec_ag : 0xFFFFFFFFu);
+              wave = __ballot_sync(0xffffffffu, cand && (same >> lane) <= 1u);
             }
-            join_rows<K, 4>(P, a.hsnap, ids, n, Wc, abort, a.st);
-            joins += n;
+            constexpr int M = K <= 4 ? 4 : K <= 8 ? 2 : 1;
+            for (uint32_t wm = wave; wm;) {
+              uint32_t ids[M];
+              int n = 0;
+#pragma unroll
+              for (int q = 0; q < M; ++q) {
+                ids[q] = 0;
+                if (wm) {
+                  ids[q] = lo + cur + (__ffs(wm) - 1);
+                  wm &= wm - 1;
+                  ++n;
+                }
+              }
+              join_rows<K, M>(P, J, a.hsnap, ids, n, abort, a.st);
+              joins += n;
+            }
           }
-          if (f == nbr) {
-            start = nbr;
-          } else if (wave) {
-            start = f;  // P grew: test the failing record again
-          } else {
+          start = f;
+          if (!fail) break;
+          if (!wave) {
             stop = true;  // P unchanged: the record stays unordered
-            start = f;
             break;
           }
+          // P grew: test the failing record again
         }
         cur += start;
+        if (stop) break;
       }
+      set_entry<K>(H, u, N);  // H_t[t] = N_t
+      const size_t at = size_t(c) * Wc;
+      store_row<K>(a.psnap + at, P);
+      store_row<K>(a.hsnap + at, H);
+      store_row<K>(a.jsnap + at, J);
       if (lane == 0) __stcg(cursor_row + L, cur);
       // later releases of L, in this batch and the next, start from the new cursor
-      if (lane > int(i) && (ea.x & 0xFF) == P_REL && ea.w == L) pre = cur;
-      if ((ea2.x & 0xFF) == P_REL && ea2.w == L) pre2 = cur;
-      store_row<K>(a.psnap + size_t(c) * Wc, P);
-      store_row<K>(a.hsnap + size_t(c) * Wc, H);
-      set_entry<K>(H, u, N + 1);  // H_t[t]++ (H_t[t] = N_t)
-      ++N;
-    } else {
-      // sync (Algorithm 1): join C_t and H_t over the barrier's scope
-      const uint32_t mode = __shfl_sync(0xffffffffu, eb.x, i);
-      // under forced compression at barriers the agent enters the join with the highest
-      // N among the members (otherwise the plan holds N_t itself)
-      if (a.forced) {
-        const uint32_t Nb = __shfl_sync(0xffffffffu, eb.y, i);
-        if (Nb != N) {
-          N = Nb;
-          set_entry<K>(H, u, N);
-        }
-      }
-      uint32_t C[K];
-#pragma unroll
-      for (int j = 0; j < K; ++j) C[j] = P[j];
-      set_entry<K>(C, u, N);
-      if (mode == BAR_SINGLE) {
-#pragma unroll
-        for (int j = 0; j < K; ++j) P[j] = C[j];
-      } else if (mode == BAR_CTA) {
-        uint32_t* buf = xchg + size_t(nbar & 1) * nwarps * 2 * Wc;
-        store_row_shared<K>(buf + size_t(warp) * 2 * Wc, C);
-        store_row_shared<K>(buf + size_t(warp) * 2 * Wc + Wc, H);
-        __syncthreads();
-#pragma unroll
-        for (int j = 0; j < K; ++j) P[j] = H[j] = 0;
-        for (int wv = 0; wv < nwarps; ++wv) {
-          const uint32_t* srcp = buf + size_t(wv) * 2 * Wc + lane * K;
-#pragma unroll
-          for (int j = 0; j < K; ++j) {
-            P[j] = max(P[j], srcp[j]);
-            H[j] = max(H[j], srcp[Wc + j]);
-          }
-        }
-        joins += 2;  // this member's C_t and H_t joined into the block's
-        ++nbar;
-      } else {
-        const uint32_t bid = z, count = w;
-        uint32_t* J = a.bar_j + size_t(bid) * 2 * Wc;
-#pragma unroll
-        for (int j = 0; j < K; ++j) {
-          atomicMax(J + lane * K + j, C[j]);
-          atomicMax(J + Wc + lane * K + j, H[j]);
-        }
-        __threadfence();
-        __syncwarp();
-        if (lane == 0) atomicAdd(a.bar_cnt + bid, 1u);
-        if (!abort) {
-          bool ok = true;
-          if (lane == 0) {
-            uint32_t it = 0;
-            while (ld_acquire(a.bar_cnt + bid) < count) {
-              if (++it > kSpinLimit) {
-                ok = false;
-                break;
-              }
-              __nanosleep(64);
-            }
-            if (!ok) atomicCAS(&a.st->code, 0, GWCP_ERR_TIMEOUT);
-          }
-          ok = __shfl_sync(0xffffffffu, ok, 0);
-          __syncwarp();
-          if (!ok) abort = true;
-        }
-        load_row<K>(J, P);
-        load_row<K>(J + Wc, H);
-        joins += 2;
-      }
-      set_entry<K>(H, u, N + 1);
-      ++N;
+      if (lane > int(i) && lock_a == L) cur_a = cur;
+      if (lock_b == L) cur_b = cur;
+      ++N;  // H_t[t]++
+      // a barrier later in the batch has time for the work ahead; otherwise a piece is done here
+      if (!(bar_a >> i)) ahead(p);
     }
-    put_version(row);
-    if (i == 31) {  // next batch
-      base += 32;
-      ea = ea2;
-      eb = eb2;
-      pre = pre2;
-      load_batch(base + 32, ea2, eb2, pre2);
+    put_version(ea.y);
+    e_at += EW * 4;
+    if (p + 1 - base == PB) {  // next batch
+      if (!put) put_entries(base + PB, half ^ 1u);
+      base += PB;
+      half ^= 1u;
+      e_at = smem_addr(plan_s) + half * PB * EW * 4;
+      lock_a = lock_b;
+      cur_a = cur_b;
+      acq_a = acq_b;
+      rel_a = rel_b;
+      bar_a = bar_b;
+      lock_b = NONE;
+      acq_b = rel_b = bar_b = 0;
+      put = false;
+      load_entries(base + PB);
     }
   }
-  if constexpr (R > 0) cp_async_wait<0>();
+  joins += 2 * nbar;  // at a block barrier each member's C_t and H_t enter the block's
+  asm volatile("cp.async.wait_all;" ::: "memory");
   if (lane == 0) {
     atomicAdd(&a.st->joins, (unsigned long long)joins);
     atomicAdd(&a.st->loop_visits, (unsigned long long)visits);
@@ -841,49 +973,68 @@ __global__ void k_plan_incs(PropArgs a, const uint32_t* incs_k, const uint32_t* 
   const size_t p = size_t(k) + 1 + r;
   const uint32_t off = flat_off[r], cnt = flat_off[r + 1] - off;
   a.plan[2 * p] = make_uint4(P_INCS, a.rowbase[u] + incs_ver[r], off, cnt);
-  a.plan[2 * p + 1] = cnt <= 4 ? make_uint4(cnt > 0 ? a.flat[off] : 0, cnt > 1 ? a.flat[off + 1] : 0,
-                                            cnt > 2 ? a.flat[off + 2] : 0, cnt > 3 ? a.flat[off + 3] : 0)
-                               : make_uint4(0, 0, 0, 0);
+  uint32_t id[4] = {0, 0, 0, 0}, meta[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  if (cnt <= 4) {
+#pragma unroll
+    for (uint32_t q = 0; q < 4; ++q) {
+      if (q >= cnt) break;
+      id[q] = a.flat[off + q];
+      const uint4 m = a.recmeta[id[q]];
+      meta[2 * q] = m.x & 0xFFFF;  // the releasing agent and its local time at the release
+      meta[2 * q + 1] = m.w;
+    }
+  }
+  a.plan[2 * p + 1] = make_uint4(id[0], id[1], id[2], id[3]);
+  a.plan2[2 * p] = make_uint4(meta[0], meta[1], meta[2], meta[3]);
+  a.plan2[2 * p + 1] = make_uint4(meta[4], meta[5], meta[6], meta[7]);
 }
 
-template <int K, int R, int MAXT, bool CV = false>
-int launch(const PropArgs& a, uint32_t grid, uint32_t threads, size_t smem_xchg, cudaStream_t s) {
-  auto kern = k_propagate<K, R, MAXT, CV>;
-  const size_t smem = smem_xchg + (R > 0 ? size_t(threads / 32) * R * slot_words<K>() * 4 : 0) +
-                     size_t(threads / 32) * 32 * K * 4;
-  if (smem > 48 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)))
-    return GWCP_ERR_UNSUPPORTED;
-  int dev = 0, sms = 0, per_sm = 0;
+// Launches the walkers with the most staging that fits a CTA's shared memory and keeps all
+// CTAs co-resident.
+template <int K, int MAXT, bool CV>
+int launch(const PropArgs& args, uint32_t grid, uint32_t threads, cudaStream_t s) {
+  auto kern = k_propagate<K, MAXT, CV>;
+  constexpr uint32_t Wc = 32 * K;
+  const uint32_t warps = threads / 32;
+  int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, int(threads), smem) != cudaSuccess)
-    return GWCP_ERR_CUDA;
-  if (uint64_t(per_sm) * sms < grid) return GWCP_ERR_UNSUPPORTED;  // walkers must be co-resident
-  PropArgs copy = a;
-  void* args[] = {&copy};
-  if (cudaLaunchCooperativeKernel(reinterpret_cast<void*>(kern), dim3(grid), dim3(threads), args, smem, s) !=
-      cudaSuccess)
-    return GWCP_ERR_CUDA;
-  count_launch();
-  return GWCP_OK;
+  // (slots, releases per staged acquire, keep the acquired H rows)
+  constexpr uint32_t kShapes[6][3] = {{4, 2, 1}, {2, 2, 1}, {2, 1, 1}, {1, 1, 1}, {0, 0, 1}, {0, 0, 0}};
+  for (const auto& sh : kShapes) {
+    if (sh[0] && K > 8) continue;  // three rows at a time do not fit the registers
+    PropArgs a = args;
+    a.slots = sh[0];
+    a.deps = sh[1];
+    a.keep_h = sh[2];
+    a.acc_words = a.cta_barriers && a.g.apb > 1 ? 6 * Wc : 0;
+    a.warp_words = 2 * plan_batch<K>() * 16 + Wc + (a.keep_h ? 2 * Wc : 0) + a.slots * a.deps * 3 * Wc;
+    const size_t smem = (size_t(a.acc_words) + size_t(warps) * a.warp_words) * 4;
+    if (smem > 200 * 1024) continue;
+    if (smem > 48 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)))
+      return GWCP_ERR_UNSUPPORTED;
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, int(threads), smem) != cudaSuccess)
+      return GWCP_ERR_CUDA;
+    if (uint64_t(per_sm) * sms < grid) continue;  // walkers must be co-resident
+    void* kargs[] = {&a};
+    if (cudaLaunchCooperativeKernel(reinterpret_cast<void*>(kern), dim3(grid), dim3(threads), kargs, smem, s) !=
+        cudaSuccess)
+      return GWCP_ERR_CUDA;
+    count_launch();
+    return GWCP_OK;
+  }
+  return GWCP_ERR_UNSUPPORTED;
 }
 
-// ring depth: deepest that keeps a CTA's shared memory within budget
+// CTAs of up to eight and sixteen walkers have the registers of 256 and 512 threads
 template <int K>
-int launch_k(const PropArgs& a, uint32_t grid, uint32_t threads, size_t smem_xchg, cudaStream_t s) {
-  const size_t per_slot = size_t(threads / 32) * slot_words<K>() * 4;
-  const size_t kBudget = 160 * 1024 - size_t(threads / 32) * 32 * K * 4;
-  // compressed versions: the same shapes, instantiated with the compressing store
-  if constexpr (K <= 4) {
-    if (threads <= 256 && smem_xchg + 8 * per_slot <= kBudget)
-      return a.compress ? launch<K, 8, 256, true>(a, grid, threads, smem_xchg, s)
-                        : launch<K, 8, 256>(a, grid, threads, smem_xchg, s);
-    if (smem_xchg + 2 * per_slot <= kBudget)
-      return a.compress ? launch<K, 2, 1024, true>(a, grid, threads, smem_xchg, s)
-                        : launch<K, 2, 1024>(a, grid, threads, smem_xchg, s);
-  }
-  return a.compress ? launch<K, 0, 1024, true>(a, grid, threads, smem_xchg, s)
-                    : launch<K, 0, 1024>(a, grid, threads, smem_xchg, s);
+int launch_k(const PropArgs& a, uint32_t grid, uint32_t threads, cudaStream_t s) {
+  if (threads <= 256)
+    return a.compress ? launch<K, 256, true>(a, grid, threads, s) : launch<K, 256, false>(a, grid, threads, s);
+  if (threads <= 512)
+    return a.compress ? launch<K, 512, true>(a, grid, threads, s) : launch<K, 512, false>(a, grid, threads, s);
+  return a.compress ? launch<K, 1024, true>(a, grid, threads, s) : launch<K, 1024, false>(a, grid, threads, s);
 }
 
 // failure-detection test: one warp waits, with the walkers' bounded wait, on a clock row
@@ -948,14 +1099,16 @@ int phaseG_propagate(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s
   a.rows = b.rows;
   a.psnap = b.psnap;
   a.hsnap = b.hsnap;
-  a.done = b.done;
+  a.jsnap = b.jsnap;
   a.cursor = b.cursor;
   a.bar_j = b.bar_j;
+  a.bar_jj = b.bar_jj;
   a.bar_cnt = b.bar_cnt;
   a.n_locks = z.n_locks;
   a.cta_barriers = z.cta_barriers;
   a.flat = b.flat;
   a.plan = b.plan;
+  a.plan2 = b.plan2;
   a.recmeta = b.recmeta;
   a.hb_only = z.hb_only;
   a.forced = z.forced_barrier;
@@ -973,7 +1126,7 @@ int phaseG_propagate(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s
     // snapshot rows start as SENTINEL: a reader accepts a row once none is left
     cudaMemsetAsync(b.psnap, 0xFF, size_t(z.n_cs) * g.RW * 4, s);
     cudaMemsetAsync(b.hsnap, 0xFF, size_t(z.n_cs) * g.RW * 4, s);
-    if (g.nT) cudaMemsetAsync(b.jsnap, 0xFF, size_t(z.n_cs) * g.RW * 4, s);
+    cudaMemsetAsync(b.jsnap, 0xFF, size_t(z.n_cs) * g.RW * 4, s);
   }
   if (z.n_incs) {
     k_flatcount<<<(z.n_incs + 255) / 256, 256, 0, s>>>(z.n_incs, b.exp_off, b.ex_dep_cnt, b.flat_off, b.st);
@@ -997,26 +1150,20 @@ int phaseG_propagate(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s
     p.end();
     return rc;
   }
-  uint32_t grid, threads;
-  size_t smem = 0;
-  if (z.cta_barriers) {
-    grid = g.B;
-    threads = g.apb * 32;
-    smem = size_t(2) * g.apb * 2 * g.Wp * 4;
-  } else {
-    grid = (g.W + 31) / 32;
-    threads = 1024;
-  }
+  // a CTA per block of the traced program; without CTA barriers the walkers are spread eight
+  // to a CTA over the SMs
+  const uint32_t threads = z.cta_barriers ? g.apb * 32 : 256;
+  const uint32_t grid = z.cta_barriers ? g.B : (g.W + 7) / 8;
   // algorithmic bytes: each clock version written once, each join reads a row
   p.begin("g_propagate", double(z.n_rows) * g.Wp * 4 + double(z.n_cs) * 2 * g.Wp * 4);
   int rc;
   switch (g.K) {
-    case 1: rc = launch_k<1>(a, grid, threads, smem, s); break;
-    case 2: rc = launch_k<2>(a, grid, threads, smem, s); break;
-    case 4: rc = launch_k<4>(a, grid, threads, smem, s); break;
-    case 8: rc = launch_k<8>(a, grid, threads, smem, s); break;
-    case 16: rc = launch_k<16>(a, grid, threads, smem, s); break;
-    case 32: rc = launch_k<32>(a, grid, threads, smem, s); break;
+    case 1: rc = launch_k<1>(a, grid, threads, s); break;
+    case 2: rc = launch_k<2>(a, grid, threads, s); break;
+    case 4: rc = launch_k<4>(a, grid, threads, s); break;
+    case 8: rc = launch_k<8>(a, grid, threads, s); break;
+    case 16: rc = launch_k<16>(a, grid, threads, s); break;
+    case 32: rc = launch_k<32>(a, grid, threads, s); break;
     default: rc = GWCP_ERR_UNSUPPORTED;
   }
   p.end();
