@@ -253,7 +253,7 @@ int gwcp_counters_ex(const gwcp_ctx* ctx, uint64_t* out, uint32_t n);
  * that must not call cudaMalloc/cudaFree because those can synchronise the device).
  * Same analysis and same results as gwcp_load_trace(ev_is_device = 1) +
  * gwcp_compute_order + gwcp_report_races, but every intermediate buffer comes from one
- * file-scope __device__ scratch array: 96 MiB, which decide what fits, and 32 MiB for buffers
+ * file-scope __device__ scratch array: 96 MiB, which decide what fits, and 40 MiB for buffers
  * that cannot run out before them. The call itself allocates nothing (no
  * cudaMalloc, cudaFree or allocating library routine). The array is reserved on a device
  * when the library's device code is loaded there: under CUDA's lazy module loading that

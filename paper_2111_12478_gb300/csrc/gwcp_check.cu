@@ -327,7 +327,7 @@ size_t check_group_count(uint32_t n_acc) { return (check_chunks(n_acc) + GRP - 1
 
 void phaseH_sort(Bufs& b, const Geo& g, const Sizes& z, uint64_t key_mask, uint32_t* tmp, cudaStream_t s, Prof& p) {
   (void)g;
-  p.begin("h_sort", double(z.n_acc) * 12 * 3 * radix_windows(key_mask).size(), s);
+  p.begin("h_sort", double(z.n_acc) * 12 * 3 * radix_passes(key_mask), s);
   RadixKeep keep;
   if (z.wl_log2) {  // the written-location filter of the grouped order, in the first pass
     keep.bits = b.wl_bits;
@@ -335,7 +335,7 @@ void phaseH_sort(Bufs& b, const Geo& g, const Sizes& z, uint64_t key_mask, uint3
     keep.shift = 15;
     keep.n_out = b.n_kept;
   }
-  if (radix_sort_pairs(b.acc_key, b.acc_idx, b.acc_key2, b.acc_idx2, z.n_acc, key_mask, tmp, s, nullptr, keep)) {
+  if (radix_sort_pairs(b.acc_key, b.acc_idx, b.acc_key2, b.acc_idx2, z.n_acc, key_mask, tmp, s, nullptr, keep, b.st)) {
     std::swap(b.acc_key, b.acc_key2);
     std::swap(b.acc_idx, b.acc_idx2);
   }
@@ -410,7 +410,7 @@ bool phaseI_sort_races(const Bufs& b, const Sizes& z, uint64_t n_races, cudaStre
   for (uint64_t v = z.N; v; v >>= 1) mask = (mask << 1) | 1;
   mask |= mask << 32;
   p.begin("i_race_sort", double(n) * 8 * 2);
-  bool second = radix_sort_pairs(b.races, nullptr, b.races2, nullptr, n, mask, b.scan_tmp, s);
+  bool second = radix_sort_pairs(b.races, nullptr, b.races2, nullptr, n, mask, b.scan_tmp, s, nullptr, {}, b.st);
   p.end();
   return second;
 }

@@ -224,11 +224,27 @@ void count_launch();
 // Exclusive scan of n u32 values (in may equal out); writes the total to *total_dev
 // when non-null. tmp must hold scan_tmp_need(n) elements.
 size_t scan_tmp_need(size_t n);
+// Several independent scans that are all small (scan_is_small) in one launch, a block each.
+struct ScanJob {
+  const uint32_t* in;
+  uint32_t* out;
+  uint32_t* total;  // or null
+  uint32_t n;       // may be 0
+};
+constexpr int kScanJobs = 8;
+struct ScanBatch {
+  ScanJob job[kScanJobs];
+};
+bool scan_is_small(size_t n);
+void scan_small(const ScanBatch& b, int jobs, cudaStream_t s);
 void scan_exclusive(const uint32_t* in, uint32_t* out, size_t n, uint32_t* total_dev, uint32_t* tmp,
                     cudaStream_t s);
+// the batch's scans, small or not
+void scan_all(const ScanBatch& b, int jobs, uint32_t* tmp, cudaStream_t s);
 // Stable LSD radix sort of (key, val) pairs on the bits set in `mask`, 8-bit digits.
 // Ping-pongs between (k0, v0) and (k1, v1); returns true if the result is in (k1, v1).
-// tmp must hold radix_tmp_need(n) u32. With n_dev, only the first min(n, *n_dev) pairs are
+// tmp must hold radix_tmp_need(n) u32. st (or null) gets GWCP_ERR_TIMEOUT if a bounded wait
+// between tiles gives up. With n_dev, only the first min(n, *n_dev) pairs are
 // sorted (a count known on the device only; n bounds it).
 // With keep.bits, the first pass keeps only the pairs whose bit wl_bit(key >> keep.shift,
 // keep.log2) is set in keep.bits (a stable filter folded into the sort); the kept count is
@@ -240,9 +256,10 @@ struct RadixKeep {
 };
 size_t radix_tmp_need(size_t n);
 bool radix_sort_pairs(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, size_t n, uint64_t mask,
-                      uint32_t* tmp, cudaStream_t s, const uint32_t* n_dev = nullptr, RadixKeep keep = {});
-// Digit windows covering the bits of `mask` (low bit of each window).
-std::vector<int> radix_windows(uint64_t mask);
+                      uint32_t* tmp, cudaStream_t s, const uint32_t* n_dev = nullptr, RadixKeep keep = {},
+                      DevStatus* st = nullptr);
+// passes a sort on the bits of `mask` takes
+int radix_passes(uint64_t mask);
 
 // ---- device helpers -----------------------------------------------------------------
 __device__ __forceinline__ void set_error(DevStatus* st, int code, unsigned long long idx) {

@@ -30,10 +30,11 @@ using namespace gwcp;
 namespace {
 
 constexpr size_t kScratchBytes = size_t(96) << 20;  // 96 MiB per device: decides which traces fit
-// Further 32 MiB for the clocks JN_t and the in-section accesses' records. They cannot run
-// out before the first array does: a section takes four clock rows there (two versions, P
-// and H) and one here, a barrier three and one, a step over 200 bytes and 32.
-constexpr size_t kExtraBytes = size_t(32) << 20;
+// Further 40 MiB for the clocks JN_t, the in-section accesses' records and the sorts' scratch.
+// They cannot run out before the first array does: a section takes four clock rows there
+// (two versions, P and H) and one here, a barrier three and one, a step over 200 bytes and
+// 32; the sorts' scratch is below 4 MB for 2^18 events and the races that fit.
+constexpr size_t kExtraBytes = size_t(40) << 20;
 constexpr uint64_t kMaxEventsNoalloc = uint64_t(1) << 18;
 constexpr uint32_t kMaxAgentsNoalloc = 256;
 
@@ -89,6 +90,13 @@ int read_back(cudaStream_t s, DevStatus* st_h, const DevStatus* st_d, uint32_t* 
   return cudaGetLastError() == cudaSuccess ? GWCP_OK : GWCP_ERR_CUDA;
 }
 
+// words the first array sets aside per sort of n pairs (which traces fit depends on it; the
+// sorts' own scratch is in the second)
+size_t sort_words(size_t n) {
+  const size_t t = 256 * ((n + 2047) / 2048);
+  return t + scan_tmp_need(t) + 1;
+}
+
 int analyze(const Event* ev, uint64_t n, const Geo& g, gwcp_race* out, uint64_t cap, uint64_t* n_races,
             uint64_t* bad_index, cudaStream_t s, unsigned char* scratch) {
   Arena A{scratch}, X{scratch + kScratchBytes, kExtraBytes};
@@ -104,10 +112,10 @@ int analyze(const Event* ev, uint64_t n, const Geo& g, gwcp_race* out, uint64_t 
   b.st = A.take<DevStatus>(1);
   b.hist_a = A.take<uint32_t>(size_t(g.W) * z.ntA + 1);
   b.tile_cnt = A.take<uint32_t>(3 * (size_t(z.ntA) + 1));
-  const size_t scan_need = std::max({scan_tmp_need(size_t(g.W) * z.ntA + 1), radix_tmp_need(n + 1),
+  const size_t scan_need = std::max({scan_tmp_need(size_t(g.W) * z.ntA + 1), sort_words(n + 1),
                                      scan_tmp_need(n + 1)}) + 64;
-  uint32_t* scan1 = A.take<uint32_t>(scan_need);
-  b.scan_tmp = scan1;
+  A.take<uint32_t>(scan_need);
+  b.scan_tmp = X.take<uint32_t>(std::max(scan_need, radix_tmp_need(n + 1) + 64));
   if (A.full) return GWCP_ERR_UNSUPPORTED;
   DevStatus init{};
   init.bad_index = ~0ull;
@@ -226,17 +234,19 @@ int analyze(const Event* ev, uint64_t n, const Geo& g, gwcp_race* out, uint64_t 
   const size_t left = kScratchBytes - A.used;
   z.race_cap = left / (2 * sizeof(uint64_t) + 8) > 4096 ? left / (2 * sizeof(uint64_t) + 8) - 4096 : 0;
   const size_t ex_bound = size_t(z.n_incs) * kMaxNest + 1;
-  const size_t need2 = std::max({scan_need, radix_tmp_need(ex_bound), scan_tmp_need(ex_bound)}) + 64;
-  if (need2 > scan_need) b.scan_tmp = A.take<uint32_t>(need2);
-  size_t race_tmp_elems = radix_tmp_need(z.race_cap + 1) + 64;
+  const size_t need2 = std::max({scan_need, sort_words(ex_bound), scan_tmp_need(ex_bound)}) + 64;
+  if (need2 > scan_need) A.take<uint32_t>(need2);
+  b.scan_tmp = X.take<uint32_t>(std::max({need2, radix_tmp_need(ex_bound) + 64, radix_tmp_need(n + 1) + 64}));
+  size_t race_tmp_elems = sort_words(z.race_cap + 1) + 64;
   while (z.race_cap && A.used + 2 * ((z.race_cap * 8 + 255) & ~size_t(255)) + race_tmp_elems * 4 + 512 > kScratchBytes) {
     z.race_cap -= z.race_cap / 8 + 1;
-    race_tmp_elems = radix_tmp_need(z.race_cap + 1) + 64;
+    race_tmp_elems = sort_words(z.race_cap + 1) + 64;
   }
   b.races = A.take<uint64_t>(z.race_cap);
   b.races2 = A.take<uint64_t>(z.race_cap);
-  uint32_t* race_tmp = A.take<uint32_t>(race_tmp_elems);
-  if (A.full || !z.race_cap) return GWCP_ERR_UNSUPPORTED;
+  A.take<uint32_t>(race_tmp_elems);
+  uint32_t* race_tmp = X.take<uint32_t>(radix_tmp_need(z.race_cap + 1) + 64);
+  if (A.full || X.full || !z.race_cap) return GWCP_ERR_UNSUPPORTED;
 
   cudaMemsetAsync(b.cursor, 0, size_t(g.W) * (z.n_locks + 1) * 4, s);
   if (global_bars && z.n_bar) {

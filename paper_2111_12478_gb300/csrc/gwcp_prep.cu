@@ -1144,10 +1144,12 @@ void phaseA_count(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, P
     k_aw_count<<<blocks(z.ntA, 8), 256, 0, s>>>(b.ev, z.N, g, z.TA, z.ntA, b.tile_cnt, b.st, vec);
     count_launch();
     p.end();
+    ScanBatch sb{};
     for (int q = 0; q < 4; ++q) {  // in-place exclusive scans of the per-tile counts
       uint32_t* t = b.tile_cnt + q * (z.ntA + 1);
-      scan_exclusive(t, t, z.ntA, t + z.ntA, b.scan_tmp, s);
+      sb.job[q] = ScanJob{t, t, t + z.ntA, z.ntA};
     }
+    scan_all(sb, 4, b.scan_tmp, s);
     return;
   }
   const uint32_t aw = a_warps(g);
@@ -1156,10 +1158,18 @@ void phaseA_count(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, P
   count_launch();
   p.end();
   // in-place exclusive scans: agent histogram and the three per-tile counts
-  scan_exclusive(b.hist_a, b.hist_a, size_t(g.W) * z.ntA, b.hist_a + size_t(g.W) * z.ntA, b.scan_tmp, s);
+  ScanBatch sb{};
   for (int q = 0; q < 3; ++q) {
     uint32_t* t = b.tile_cnt + q * (z.ntA + 1);
-    scan_exclusive(t, t, z.ntA, t + z.ntA, b.scan_tmp, s);
+    sb.job[q] = ScanJob{t, t, t + z.ntA, z.ntA};
+  }
+  const size_t nh = size_t(g.W) * z.ntA;
+  sb.job[3] = ScanJob{b.hist_a, b.hist_a, b.hist_a + nh, uint32_t(nh)};
+  if (scan_is_small(nh)) {
+    scan_all(sb, 4, b.scan_tmp, s);
+  } else {
+    scan_all(sb, 3, b.scan_tmp, s);
+    scan_exclusive(b.hist_a, b.hist_a, nh, b.hist_a + nh, b.scan_tmp, s);
   }
 }
 
@@ -1176,7 +1186,7 @@ void phaseA_scatter(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s,
     while ((1u << ab) < g.W) ++ab;
     const uint64_t mask = ((1ull << ab) - 1) << 32;
     const uint64_t* sorted =
-        radix_sort_pairs(b.s_key, nullptr, b.s_key2, nullptr, z.nS, mask, b.s_tmp, s) ? b.s_key2 : b.s_key;
+        radix_sort_pairs(b.s_key, nullptr, b.s_key2, nullptr, z.nS, mask, b.s_tmp, s, nullptr, {}, b.st) ? b.s_key2 : b.s_key;
     if (z.nS) {
       k_aw_extract<<<blocks(z.nS, 256), 256, 0, s>>>(sorted, z.nS, b.S);
       count_launch();
@@ -1221,8 +1231,10 @@ void phaseC_walk(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, Pr
                                                            b.sy_relk, b.incs_cnt, b.vcount, b.sy_agent, b.st);
   count_launch();
   p.end();
-  scan_exclusive(b.incs_cnt, b.incs_cnt, z.n_sync + 1, nullptr, b.scan_tmp, s);
-  scan_exclusive(b.vcount, b.vcount, g.W + 1, nullptr, b.scan_tmp, s);
+  ScanBatch sb{};
+  sb.job[0] = ScanJob{b.incs_cnt, b.incs_cnt, nullptr, z.n_sync + 1};
+  sb.job[1] = ScanJob{b.vcount, b.vcount, nullptr, g.W + 1};
+  scan_all(sb, 2, b.scan_tmp, s);
 }
 
 void phaseC_forced(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, Prof& p) {
@@ -1233,7 +1245,7 @@ void phaseC_forced(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, 
   count_launch();
   uint64_t mask = 0;  // keys 0..B (B: one-member barriers, left out of the walk)
   while (mask < g.B) mask = (mask << 1) | 1;
-  const bool second = radix_sort_pairs(b.fb_key, b.fb_val, b.fb_key2, b.fb_val2, n, mask, b.scan_tmp, s);
+  const bool second = radix_sort_pairs(b.fb_key, b.fb_val, b.fb_key2, b.fb_val2, n, mask, b.scan_tmp, s, nullptr, {}, b.st);
   const uint64_t* skey = second ? b.fb_key2 : b.fb_key;
   const uint32_t* spos = second ? b.fb_val2 : b.fb_val;
   k_fb_rank<<<blocks(uint64_t(n) + 1, 256), 256, 0, s>>>(b.ev, g, b.bar, skey, spos, n, b.fb_rank, b.fb_off,
@@ -1285,7 +1297,7 @@ void phaseE_locks(Bufs& b, const Geo& g, const Sizes& z, uint64_t lock_mask, cud
   const uint32_t n = z.n_acqrel;
   if (!n) return;
   p.begin("e_sort", double(n) * 24);
-  if (radix_sort_pairs(b.lk_key, b.lk_k, b.lk_key2, b.lk_k2, n, lock_mask, b.scan_tmp, s)) {
+  if (radix_sort_pairs(b.lk_key, b.lk_k, b.lk_key2, b.lk_k2, n, lock_mask, b.scan_tmp, s, nullptr, {}, b.st)) {
     std::swap(b.lk_key, b.lk_key2);
     std::swap(b.lk_k, b.lk_k2);
   }
@@ -1357,7 +1369,7 @@ void phaseF_walk(Bufs& bb, const Geo& g, const Sizes& z, uint64_t key_mask, cuda
     uint64_t mask = stage == 0 ? idx_mask : stage == 1 ? key_mask : 0;
     if (stage == 2)
       for (uint64_t v = z.n_locks; v; v >>= 1) mask = (mask << 1) | 1;
-    if (radix_sort_pairs(bb.ex_key, bb.ex_val, bb.ex_key2, bb.ex_val2, n, mask, bb.scan_tmp, s)) {
+    if (radix_sort_pairs(bb.ex_key, bb.ex_val, bb.ex_key2, bb.ex_val2, n, mask, bb.scan_tmp, s, nullptr, {}, b.st)) {
       std::swap(bb.ex_key, bb.ex_key2);
       std::swap(bb.ex_val, bb.ex_val2);
     }

@@ -1024,7 +1024,7 @@ void phaseI_wide_group(Bufs& b, const Geo& g, Sizes& z, uint32_t* tmp, cudaStrea
   while ((1ull << rb) < n) ++rb;
   while ((1u << ab) < g.W) ++ab;
   const uint64_t mask = (((1ull << rb) - 1) << 15) | (3ull << 13) | ((1ull << ab) - 1);
-  if (radix_sort_pairs(b.wc_key, b.wc_val, b.wc_key2, b.wc_val2, n, mask, tmp, s, n_kept)) {
+  if (radix_sort_pairs(b.wc_key, b.wc_val, b.wc_key2, b.wc_val2, n, mask, tmp, s, n_kept, {}, b.st)) {
     std::swap(b.wc_key, b.wc_key2);
     std::swap(b.wc_val, b.wc_val2);
   }
@@ -1052,8 +1052,10 @@ void phaseI_grouped(Bufs& b, const Geo& g, Sizes& z, uint32_t* tmp, cudaStream_t
   p.begin("i_wide_group", double(n) * (8 + 4 * 4 + 16 + 12 + 16), s);  // ~ per access
   k_gr_flags<<<nblk(n, 256), 256, 0, s>>>(b.acc_key, n, b.n_kept, b.wc_flag, b.wc_gflag);
   count_launch();
-  scan_exclusive(b.wc_flag, b.wc_run, n, b.wc_run + n, tmp, s);
-  scan_exclusive(b.wc_gflag, b.wc_gexcl, n, b.wc_gexcl + n, tmp, s);
+  ScanBatch sb{};
+  sb.job[0] = ScanJob{b.wc_flag, b.wc_run, b.wc_run + n, n};
+  sb.job[1] = ScanJob{b.wc_gflag, b.wc_gexcl, b.wc_gexcl + n, n};
+  scan_all(sb, 2, tmp, s);
   k_gr_groups<<<nblk(n, 256), 256, 0, s>>>(b.acc_key, b.wc_flag, b.wc_run, b.wc_gflag, b.wc_gexcl, b.n_kept,
                                           b.wc_grp_lo, b.wc_grp_agent, b.wc_rc);
   count_launch();
