@@ -70,6 +70,7 @@ struct gwcp_ctx {
   bool acc_info_partial = false;         // last compute wrote the kept accesses' records only
   uint64_t clock_words[3] = {};  // last compute: tiles, pool words taken, words written
   uint64_t tile_cap_hint = 0;  // wide clocks: pool size that the last run needed
+  bool tiles_if_oom = false;   // dense by choice, tiles when the device memory runs out
   bool compressed = false;     // GWCP_CLOCKS_COMPRESSED was in force at gwcp_load_trace
   uint64_t cv_cap_hint = 0;    // compressed versions: pool words that the last run needed
   uint64_t alloc_limit = 0;    // gwcp_debug_alloc_limit: cap on the cached buffers' bytes (0 = none)
@@ -489,7 +490,8 @@ int run(gwcp_ctx* c, cudaStream_t s) {
   b.jsnap = get<uint32_t>(c, "jsnap", (size_t(z.n_cs) + 1) * g.RW, &oom);
   if (g.nT) {
     // tile pool: a few new tiles per clock version; grown and rerun on exhaustion
-    const uint64_t want = 2ull * (uint64_t(z.n_rows) + z.n_cs) + uint64_t(z.n_bar) * (g.apb + 2) + 65536;
+    const uint64_t want = 2ull * (uint64_t(z.n_rows) + z.n_cs) + uint64_t(z.n_bar) * (g.apb + 2) +
+                          std::max<uint64_t>(65536, 16ull * g.W + 32768);  // each walker holds up to two chunks of 8
     z.tile_cap = std::max<uint64_t>(c->tile_cap_hint, want);
     // 2 MB aligned: the walkers' time depended by ~3% on where the pool landed after the
     // buffers allocated before it (77 vs 79.5 ms on the 8192-warp, 200M-event workload
@@ -772,6 +774,29 @@ int gwcp_create(gwcp_ctx** out, int device, const gwcp_options* opt) {
   return GWCP_OK;
 }
 
+namespace {
+Geo make_geo(const gwcp_geometry& geo, bool tiles) {
+  Geo g{};
+  g.W = geo.num_agents;
+  g.apb = geo.agents_per_block;
+  g.B = g.W / g.apb;
+  g.gran = geo.granularity;
+  uint32_t k = 1;
+  while (k * 32 < g.W) k <<= 1;
+  g.K = k;
+  g.Wp = 32 * k;
+  g.nT = 0;
+  g.RW = g.Wp;
+  if (tiles) {
+    g.nT = (g.W + kTileW - 1) / kTileW;
+    g.Wp = g.nT * kTileW;
+    g.K = g.Wp / 32;
+    g.RW = kTabW;
+  }
+  return g;
+}
+}  // namespace
+
 int gwcp_load_trace(gwcp_ctx* c, const gwcp_event* ev, uint64_t n, const gwcp_geometry* geo, int ev_is_device,
                     void* stream) {
   if (!c || !geo || (!ev && n)) return GWCP_ERR_ARGS;
@@ -785,29 +810,15 @@ int gwcp_load_trace(gwcp_ctx* c, const gwcp_event* ev, uint64_t n, const gwcp_ge
   if (geo->num_agents > kMaxAgents && !tiles_ok) return GWCP_ERR_UNSUPPORTED;
   if (c->clock_mode == GWCP_CLOCKS_TILES && !tiles_ok) return GWCP_ERR_UNSUPPORTED;
   if (c->clock_mode == GWCP_CLOCKS_COMPRESSED && geo->num_agents > kMaxAgents) return GWCP_ERR_UNSUPPORTED;
-  // automatic: tiles from kTilesFromAgents agents on (measured faster from there on GB300)
+  const bool choose = c->clock_mode == GWCP_CLOCKS_AUTO && tiles_ok;
   const bool tiles = geo->num_agents > kMaxAgents || c->clock_mode == GWCP_CLOCKS_TILES ||
-                     (c->clock_mode == GWCP_CLOCKS_AUTO && tiles_ok && geo->num_agents >= kTilesFromAgents);
+                     (choose && tiles_preferred(geo->num_agents, geo->agents_per_block));
+  // tiles hold less: the widest clocks that are dense by choice have them to fall back on
+  c->tiles_if_oom = choose && !tiles && geo->num_agents >= 512;
   cudaSetDevice(c->device);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   use_stream(c, s);
-  Geo g{};
-  g.W = geo->num_agents;
-  g.apb = geo->agents_per_block;
-  g.B = g.W / g.apb;
-  g.gran = geo->granularity;
-  uint32_t k = 1;
-  while (k * 32 < g.W) k <<= 1;
-  g.K = k;
-  g.Wp = 32 * k;
-  g.nT = 0;
-  g.RW = g.Wp;
-  if (tiles) {
-    g.nT = (g.W + kTileW - 1) / kTileW;
-    g.Wp = g.nT * kTileW;
-    g.K = g.Wp / 32;
-    g.RW = kTabW;
-  }
+  const Geo g = make_geo(*geo, tiles);
   c->g = g;
   c->compressed = c->clock_mode == GWCP_CLOCKS_COMPRESSED;
   c->n = n;
@@ -852,6 +863,15 @@ int gwcp_compute_order(gwcp_ctx* c, void* stream) {
   int rc = run(c, static_cast<cudaStream_t>(stream));
   for (int attempt = 0; rc == kRerun && attempt < 6; ++attempt) rc = run(c, static_cast<cudaStream_t>(stream));
   if (rc == kRerun) rc = GWCP_ERR_OOM;
+  if (rc == GWCP_ERR_OOM && c->tiles_if_oom) {
+    c->tiles_if_oom = false;
+    cudaStreamSynchronize(static_cast<cudaStream_t>(stream));
+    for (auto& kv : c->allocs)  // what the dense attempt holds
+      if (kv.second.first) cudaFreeAsync(kv.second.first, c->alloc_s);
+    c->allocs.clear();
+    c->g = make_geo(gwcp_geometry{c->g.W, c->g.apb, c->g.gran, 0}, true);
+    return gwcp_compute_order(c, stream);
+  }
   c->computed = true;
   c->compute_rc = rc;
   return rc;

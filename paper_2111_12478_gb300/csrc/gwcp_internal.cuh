@@ -17,9 +17,17 @@ constexpr uint32_t kMaxAgents = 1024;      // clocks held in registers
 constexpr uint32_t kMaxAgentsWide = 8192;  // clocks as tables of copy-on-write tiles
 constexpr uint32_t kTileW = 256;           // entries per clock tile
 constexpr uint32_t kTabW = 32;             // words per published tile table (nT <= 32)
-constexpr uint32_t kTilesFromAgents = 512;  // automatic clock mode: tiles from this width on
+// Automatic clock mode: tiles above 512 agents, and above 256 where a block has more than 16
+// (its walkers' CTA then leaves 64 registers per thread, and a clock of 16 words per lane
+// spills). Propagation, dense and tiles, ms: 512 agents in blocks of 8 (4M events) 1.29 and
+// 2.21, of 16 2.85 and 3.94, of 32 9.2 and 6.5; 600 in blocks of 8 2.46 and 2.20; 1024 in blocks
+// of 16 (3M) 3.06 and 1.80; 384 in blocks of 24 (2M) 4.5 and 3.2; 256 in blocks of 32 5.45 and 5.54.
+inline bool tiles_preferred(uint32_t agents, uint32_t per_block) {
+  return agents > 512 || (agents > 256 && per_block > 16);
+}
 constexpr uint32_t kSparseCheckFromAgents = 1;  // automatic check mode: partner groups (measured faster)
 constexpr uint32_t kMaxEvents = (1u << 30) - 1;
+constexpr size_t kMaxDynamicSmem = 200 * 1024;  // shared memory a walker's CTA may ask for
 // distinct scope ids one lock may be used with: 64, or 320 when the trace has more than
 // 63 blocks (a block-scoped lock may be used in every block)
 constexpr int kLockScopesSmall = 64, kLockScopesLarge = 320;

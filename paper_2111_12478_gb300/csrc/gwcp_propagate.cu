@@ -999,6 +999,9 @@ int launch(const PropArgs& args, uint32_t grid, uint32_t threads, cudaStream_t s
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  // (one limit for every launch: other threads may be launching with another size)
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kMaxDynamicSmem)) != cudaSuccess)
+    return GWCP_ERR_CUDA;
   // (slots, releases per staged acquire, keep the acquired H rows)
   constexpr uint32_t kShapes[6][3] = {{4, 2, 1}, {2, 2, 1}, {2, 1, 1}, {1, 1, 1}, {0, 0, 1}, {0, 0, 0}};
   for (const auto& sh : kShapes) {
@@ -1010,9 +1013,7 @@ int launch(const PropArgs& args, uint32_t grid, uint32_t threads, cudaStream_t s
     a.acc_words = a.cta_barriers && a.g.apb > 1 ? 6 * Wc : 0;
     a.warp_words = 2 * plan_batch<K>() * 16 + Wc + (a.keep_h ? 2 * Wc : 0) + a.slots * a.deps * 3 * Wc;
     const size_t smem = (size_t(a.acc_words) + size_t(warps) * a.warp_words) * 4;
-    if (smem > 200 * 1024) continue;
-    if (smem > 48 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)))
-      return GWCP_ERR_UNSUPPORTED;
+    if (smem > kMaxDynamicSmem) continue;
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, int(threads), smem) != cudaSuccess)
       return GWCP_ERR_CUDA;

@@ -35,6 +35,8 @@ namespace gwcp {
 namespace {
 
 constexpr uint32_t kSpinLimitW = 1u << 23;
+constexpr uint32_t kPlanBatch = 16;
+constexpr unsigned long long kBarrierLimitNs = 60ull * 1000 * 1000 * 1000;
 constexpr uint32_t SENT = 0xFFFFFFFFu;
 enum : uint32_t { P_ACQ = 0, P_REL = 1, P_BAR = 2, P_INCS = 3 };
 enum : uint32_t { BAR_SINGLE = 0, BAR_CTA = 1, BAR_GLOBAL = 2 };
@@ -68,14 +70,6 @@ __device__ __forceinline__ void prefetch_tile(const WideArgs& a, uint32_t id) {
 #pragma unroll
   for (int q = 0; q < 8; ++q) asm volatile("prefetch.global.L1 [%0];" ::"l"(p + q * 128));
 }
-// the tiles a merge of `src` into the table `my` will read (lane T: tile T of each)
-__device__ __forceinline__ void prefetch_merge(const WideArgs& a, uint32_t my, uint32_t src) {
-  if ((threadIdx.x & 31) < int(a.g.nT) && src != 0 && src != my && my != 0) {
-    prefetch_tile(a, my);
-    prefetch_tile(a, src);
-  }
-}
-
 __device__ __forceinline__ const uint4* tile_src(const WideArgs& a, uint32_t id) {
   return reinterpret_cast<const uint4*>(a.tiles + size_t(id) * kTileW) + (threadIdx.x & 31) * 2;
 }
@@ -85,23 +79,6 @@ __device__ __forceinline__ uint4* tile_dst(const WideArgs& a, uint32_t id) {
 
 // A lane holds 8 consecutive entries of a tile as (x0, x1). These update entry c (0..7)
 // with register selects only, so the pair is never addressed through memory.
-__device__ __forceinline__ uint32_t sel_raise(uint32_t x, bool hit, uint32_t val, bool& up) {
-  const bool h = hit && x < val;
-  up |= h;
-  return h ? val : x;
-}
-__device__ __forceinline__ bool raise8(uint4& x0, uint4& x1, uint32_t c, uint32_t val) {
-  bool up = false;
-  x0.x = sel_raise(x0.x, c == 0, val, up);
-  x0.y = sel_raise(x0.y, c == 1, val, up);
-  x0.z = sel_raise(x0.z, c == 2, val, up);
-  x0.w = sel_raise(x0.w, c == 3, val, up);
-  x1.x = sel_raise(x1.x, c == 4, val, up);
-  x1.y = sel_raise(x1.y, c == 5, val, up);
-  x1.z = sel_raise(x1.z, c == 6, val, up);
-  x1.w = sel_raise(x1.w, c == 7, val, up);
-  return up;
-}
 __device__ __forceinline__ void set8(uint4& x0, uint4& x1, uint32_t c, uint32_t val) {
   x0.x = c == 0 ? val : x0.x;
   x0.y = c == 1 ? val : x0.y;
@@ -114,10 +91,13 @@ __device__ __forceinline__ void set8(uint4& x0, uint4& x1, uint32_t c, uint32_t 
 }
 
 // Tile ids are handed to each warp kTileChunk at a time (one atomic per chunk instead of
-// one per tile on a single counter); the warp-uniform state lives in the walker.
+// one per tile on a single counter); the warp-uniform state lives in the walker. The next
+// chunk is asked for when the current one is begun, so that its atomic's latency is over
+// when it is needed.
 constexpr uint32_t kTileChunk = 8;
 struct TileAlloc {
   uint32_t next = 0, end = 0;  // ids [next, end) are the warp's; both clamped to the pool size
+  unsigned long long ahead = 0;  // lane 0: the next chunk's first id
   uint32_t* cnt = nullptr;     // shared words: tiles read, tiles written (lane 0 adds)
   __device__ __forceinline__ void count(uint32_t rd, uint32_t wr) const {
     if ((threadIdx.x & 31) == 0) {
@@ -126,13 +106,15 @@ struct TileAlloc {
     }
   }
 };
+__device__ __forceinline__ void ask_chunk(const WideArgs& a, TileAlloc& ta) {
+  if ((threadIdx.x & 31) == 0) ta.ahead = atomicAdd(a.tile_ctr, (unsigned long long)kTileChunk);
+}
 
 // a fresh tile id (warp-uniform); 0 when the pool is exhausted (GWCP_ERR_OOM set)
 __device__ __forceinline__ uint32_t alloc_tile(const WideArgs& a, TileAlloc& ta) {
   if (ta.next == ta.end) {
-    unsigned long long base = 0;
-    if ((threadIdx.x & 31) == 0) base = atomicAdd(a.tile_ctr, (unsigned long long)kTileChunk);
-    base = __shfl_sync(0xffffffffu, base, 0);
+    const unsigned long long base = __shfl_sync(0xffffffffu, ta.ahead, 0);
+    ask_chunk(a, ta);
     ta.next = uint32_t(min(base, a.tile_cap));
     ta.end = uint32_t(min(base + kTileChunk, a.tile_cap));
     if (ta.next == ta.end) {
@@ -143,48 +125,177 @@ __device__ __forceinline__ uint32_t alloc_tile(const WideArgs& a, TileAlloc& ta)
   return ta.next++;
 }
 
-// my |= src, tile by tile (lane T < nT holds the ids of tile T)
-__device__ __noinline__ void merge_table(const WideArgs& a, uint32_t& my, uint32_t src, bool& dirty, TileAlloc& ta) {
+// max of tiles ia and ib by the whole warp: an input's id when the result equals it, else that
+// of a new tile (ia when the pool is exhausted)
+__device__ __forceinline__ uint32_t merge_one(const WideArgs& a, uint32_t ia, uint32_t ib, bool& fresh,
+                                              TileAlloc& ta) {
+  const uint4* pa = tile_src(a, ia);
+  const uint4* pb = tile_src(a, ib);
+  const uint4 x0 = __ldca(pa), x1 = __ldca(pa + 1), y0 = __ldca(pb), y1 = __ldca(pb + 1);
+  const uint4 r0 = max4(x0, y0), r1 = max4(x1, y1);
+  fresh = false;
+  if (__all_sync(0xffffffffu, eq4(r0, x0) && eq4(r1, x1))) return ia;
+  if (__all_sync(0xffffffffu, eq4(r0, y0) && eq4(r1, y1))) return ib;
+  const uint32_t nid = alloc_tile(a, ta);
+  if (!nid) return ia;
+  uint4* d = tile_dst(a, nid);
+  d[0] = r0;
+  d[1] = r1;
+  fresh = true;
+  return nid;
+}
+
+// A merge of whole tables is up to 32 merges of tiles per table, each a chain of loads, votes,
+// an id and stores: 1,400 cycles, and 65 us for the three tables of an acquire with 8192 warps
+// when one warp walks them, while the other walkers of its CTA mostly wait at the block's
+// barrier. So a walker posts its merges in shared memory, and walkers that wait (at a barrier,
+// or for a release) take them one by one, as does the walker itself. Propagation, with the
+// plan ring and the members' own entries raised from shared memory (the barrier join 35,000
+// -> 17,000 cycles): 8192 warps, 50M events 16.7 -> 9.5 ms; 4096 warps, 4M 4.2 -> 1.86; 512
+// warps, 2.3M 2.2 -> 1.3. (The pairs of eight merges copied to shared memory ahead of the
+// one walker: 13.5 and 3.0 ms; four tiles per warp at a time: slower than one.)
+// A post is open while `next` is below kClosed; it is reused only after all its merges are
+// done, and opened by the store to `next` after everything else is written, so a helper that
+// comes late finds either no merge or one of the new post.
+struct Post {
+  uint32_t next, total, done, pad;  // merge to take next; merges; merges done
+  uint32_t ida[96], idb[96];        // the merges: my tile (then the result), the source's
+};
+constexpr uint32_t kClosed = 0x40000000u;
+constexpr uint32_t kPosts = 4;  // per CTA; a walker that finds none free walks its merges alone
+
+struct __align__(16) Shared {  // a CTA's posts
+  uint32_t open;     // posts with merges left (bit each)
+  uint32_t arrived;  // walkers that have reached a block barrier, all barriers together
+  uint32_t used;     // posts taken (bit each)
+  uint32_t pad;
+  Post post[kPosts];
+};
+
+// takes one merge of post b, if one is left
+__device__ __forceinline__ bool take_merge(const WideArgs& a, Shared& sh, int b, TileAlloc& ta) {
   const int lane = threadIdx.x & 31;
-  bool need = lane < int(a.g.nT) && src != 0 && src != my;
-  if (need && my == 0) {
-    my = src;
-    need = false;
+  Post& q = sh.post[b];
+  uint32_t j = 0;
+  if (lane == 0) j = atomicAdd(&q.next, 1u);
+  j = __shfl_sync(0xffffffffu, j, 0);
+  const uint32_t total = *(volatile uint32_t*)&q.total;
+  if (j >= kClosed || j >= total) return false;
+  if (j + 1 == total && lane == 0) atomicAnd(&sh.open, ~(1u << b));
+  bool fresh;
+  const uint32_t id = merge_one(a, *(volatile uint32_t*)&q.ida[j], *(volatile uint32_t*)&q.idb[j], fresh, ta);
+  ta.count(2, fresh ? 1u : 0u);
+  // (the tile is ordered before `done`, and the poster fences before it publishes a table)
+  __syncwarp();
+  if (lane == 0) {
+    *(volatile uint32_t*)&q.ida[j] = id;
+    __threadfence_block();
+    atomicAdd(&q.done, 1u);
   }
-  if (need) {
-    prefetch_tile(a, my);
-    prefetch_tile(a, src);
+  return true;
+}
+
+// (posts with merges left, arrivals at block barriers): one load, the same for all lanes. The
+// waiting walkers poll it, up to 62 on an SM beside the ones that work, so a poll is few
+// instructions and polls are kWaitNs apart.
+constexpr uint32_t kWaitNs = 300;
+__device__ __forceinline__ uint2 look(const Shared& sh) {
+  uint2 v;
+  asm volatile("ld.volatile.shared.v2.u32 {%0, %1}, [%2];"
+               : "=r"(v.x), "=r"(v.y)
+               : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(&sh.open)))
+               : "memory");
+  return make_uint2(__shfl_sync(0xffffffffu, v.x, 0), __shfl_sync(0xffffffffu, v.y, 0));
+}
+__device__ __noinline__ void help(const WideArgs& a, Shared& sh, uint32_t open, TileAlloc& ta) {
+  take_merge(a, sh, __ffs(open) - 1, ta);
+}
+
+// my[q] |= src[q] tile by tile for the tables q < NT (lane T < nT holds the ids of tile T)
+template <int NT>
+__device__ __noinline__ void merge_tables(const WideArgs& a, uint32_t (&my)[NT], const uint32_t (&src)[NT], bool& dirty,
+                                          TileAlloc& ta, Shared& sh) {
+  const int lane = threadIdx.x & 31;
+  uint32_t total = 0, at[NT];
+  const uint32_t lt = lanemask_lt();
+#pragma unroll
+  for (int q = 0; q < NT; ++q) {
+    bool need = lane < int(a.g.nT) && src[q] != 0 && src[q] != my[q];
+    if (need && my[q] == 0) {
+      my[q] = src[q];
+      need = false;
+    }
+    const uint32_t m = __ballot_sync(0xffffffffu, need);
+    at[q] = need ? total + __popc(m & lt) : NONE;  // the merge's place in the post
+    total += __popc(m);
   }
-  uint32_t m = __ballot_sync(0xffffffffu, need);
-  while (m) {
-    const int T = __ffs(m) - 1;
-    m &= m - 1;
-    const uint32_t ia = __shfl_sync(0xffffffffu, my, T), ib = __shfl_sync(0xffffffffu, src, T);
-    const uint4* pa = tile_src(a, ia);
-    const uint4* pb = tile_src(a, ib);
-    const uint4 x0 = __ldca(pa), x1 = __ldca(pa + 1), y0 = __ldca(pb), y1 = __ldca(pb + 1);
-    const uint4 r0 = max4(x0, y0), r1 = max4(x1, y1);
-    uint32_t nid;
-    if (__all_sync(0xffffffffu, eq4(r0, x0) && eq4(r1, x1))) {
-      nid = ia;
-      ta.count(2, 0);
-    } else if (__all_sync(0xffffffffu, eq4(r0, y0) && eq4(r1, y1))) {
-      nid = ib;
-      ta.count(2, 0);
-    } else {
-      nid = alloc_tile(a, ta);
-      ta.count(2, 1);
-      if (nid) {
-        uint4* d = tile_dst(a, nid);
-        d[0] = r0;
-        d[1] = r1;
-        dirty = true;
-      } else {
-        nid = ia;
+  if (!total) return;
+  int b = -1;
+  if (total > 1 && blockDim.x > 32) {
+    if (lane == 0) {
+      const uint32_t left = ~*(volatile uint32_t*)&sh.used & ((1u << kPosts) - 1u);
+      if (left) {
+        const int q = __ffs(left) - 1;
+        if (!(atomicOr(&sh.used, 1u << q) & (1u << q))) b = q;
       }
     }
-    if (lane == T) my = nid;
+    b = __shfl_sync(0xffffffffu, b, 0);
   }
+  if (b < 0) {  // alone
+#pragma unroll
+    for (int q = 0; q < NT; ++q) {
+      if (at[q] != NONE) {
+        prefetch_tile(a, my[q]);
+        prefetch_tile(a, src[q]);
+      }
+      for (uint32_t m = __ballot_sync(0xffffffffu, at[q] != NONE); m; m &= m - 1) {
+        const int T = __ffs(m) - 1;
+        bool fresh;
+        const uint32_t id = merge_one(a, __shfl_sync(0xffffffffu, my[q], T), __shfl_sync(0xffffffffu, src[q], T),
+                                      fresh, ta);
+        if (lane == T) my[q] = id;
+        ta.count(2, fresh ? 1u : 0u);
+        dirty |= fresh;
+      }
+    }
+    return;
+  }
+  Post& post = sh.post[b];
+#pragma unroll
+  for (int q = 0; q < NT; ++q) {
+    if (at[q] != NONE) {
+      post.ida[at[q]] = my[q];
+      post.idb[at[q]] = src[q];
+    }
+  }
+  if (lane == 0) {
+    post.total = total;
+    post.done = 0;
+  }
+  __threadfence_block();
+  __syncwarp();
+  if (lane == 0) {
+    atomicOr(&sh.open, 1u << b);  // (before the first merge can be taken: the last one taken clears it)
+    __threadfence_block();
+    atomicExch(&post.next, 0u);
+  }
+  while (take_merge(a, sh, b, ta)) {
+  }
+  // helpers finish what they took (they wait for nothing meanwhile); bounded all the same
+  for (uint32_t it = 0; it < kSpinLimitW; ++it) {
+    if (__all_sync(0xffffffffu, *(volatile uint32_t*)&post.done >= total)) break;
+    if (it + 1 == kSpinLimitW && lane == 0) atomicCAS(&a.st->code, 0, GWCP_ERR_TIMEOUT);
+  }
+  __threadfence_block();
+#pragma unroll
+  for (int q = 0; q < NT; ++q)
+    if (at[q] != NONE) my[q] = *(volatile uint32_t*)&post.ida[at[q]];
+  __syncwarp();
+  if (lane == 0) {
+    atomicExch(&post.next, kClosed);
+    atomicAnd(&sh.used, ~(1u << b));
+  }
+  dirty = true;
 }
 
 // copy of tile `id` with entry e set to val; returns the new id (warp-uniform)
@@ -213,14 +324,19 @@ __device__ __forceinline__ void set_entry_w(const WideArgs& a, uint32_t& my, uin
 }
 
 // a published table: wait (bounded) until none of its nT words is SENTINEL
-__device__ __forceinline__ uint32_t read_table(const WideArgs& a, const uint32_t* tab, bool& abort) {
+__device__ __forceinline__ uint32_t read_table(const WideArgs& a, const uint32_t* tab, bool& abort, Shared& sh,
+                                               TileAlloc& ta) {
   const int lane = threadIdx.x & 31;
   const bool act = lane < int(a.g.nT);
   uint32_t v = act ? __ldcg(tab + lane) : 0;
   if (__all_sync(0xffffffffu, v != SENT)) return v;
   uint32_t it = 0;
   while (!abort) {
-    __nanosleep(64);
+    const uint32_t open = look(sh).x;
+    if (open)
+      help(a, sh, open, ta);
+    else
+      __nanosleep(64);
     v = act ? __ldcg(tab + lane) : 0;
     if (__all_sync(0xffffffffu, v != SENT)) return v;
     if (++it > kSpinLimitW) {
@@ -246,47 +362,69 @@ __device__ __forceinline__ uint32_t entry_of(const WideArgs& a, uint32_t my, uin
 }
 
 // Join of one tile over a CTA's members (lane m holds member m's id for the tile), with
-// the members' own entries raised to their local times (C_m[u_m] = N_m; H_m[u_m] = N_m,
-// which the walker keeps implicit). One pass over the distinct input tiles keeps the
+// the members' own entries raised to their local times nbuf[m] (C_m[u_m] = N_m; H_m[u_m] =
+// N_m, which the walker keeps implicit). One pass over the distinct input tiles keeps the
 // running maximum and which input equals it so far (an input equals the final maximum
 // iff it is >= every other input); the result keeps that input's id when the own
 // entries raise nothing, else it is written as a new tile.
-__device__ __noinline__ uint32_t join_members(const WideArgs& a, uint32_t idm, uint32_t nm, uint32_t apb, uint32_t first,
-                                 uint32_t T, bool own, bool& dirty, TileAlloc& ta) {
+__device__ __noinline__ uint32_t join_members(const WideArgs& a, uint32_t idm, const uint32_t* nbuf, uint32_t apb,
+                                              uint32_t first, uint32_t T, bool own, bool& dirty, TileAlloc& ta) {
   const int lane = threadIdx.x & 31;
   const bool act = uint32_t(lane) < apb && idm != 0;
-  const uint32_t same = __match_any_sync(0xffffffffu, act ? idm : 0xFFFFFFFFu);
-  const uint32_t leaders = __ballot_sync(0xffffffffu, act && (__ffs(same) - 1) == lane);
+  const uint32_t any = __ballot_sync(0xffffffffu, act);
   // members whose own entry lies in tile T
-  const uint32_t lo = T * kTileW, hi = lo + kTileW;
-  const bool own_here = own && uint32_t(lane) < apb && first + lane >= lo && first + lane < hi;
-  const uint32_t ovm = __ballot_sync(0xffffffffu, own_here);
-  if (!ovm && __popc(leaders) <= 1) return leaders ? __shfl_sync(0xffffffffu, idm, __ffs(leaders) - 1) : 0u;
+  const uint32_t lo = T * kTileW;
+  const bool own_here = own && first < lo + kTileW && first + apb > lo;
+  // the usual case: one tile, shared since the last barrier, and no own entries
+  const uint32_t id0 = __shfl_sync(0xffffffffu, idm, any ? __ffs(any) - 1 : 0);
+  uint32_t leaders = any & (0u - any);
+  if (!__all_sync(0xffffffffu, !act || idm == id0)) {
+    const uint32_t same = __match_any_sync(0xffffffffu, act ? idm : 0xFFFFFFFFu);
+    leaders = __ballot_sync(0xffffffffu, act && (__ffs(same) - 1) == lane);
+  }
+  if (!own_here && !(leaders & (leaders - 1))) return any ? id0 : 0u;
   uint4 r0 = make_uint4(0, 0, 0, 0), r1 = r0;
   bool have = leaders == 0;  // no input: the zero tile (id 0) equals the maximum so far
   uint32_t cid = 0;          // id of an input equal to the maximum so far (when have)
-  for (uint32_t m = leaders; m; m &= m - 1) {
-    const uint32_t id = __shfl_sync(0xffffffffu, idm, __ffs(m) - 1);
-    const uint4* p = tile_src(a, id);
-    const uint4 x0 = __ldca(p), x1 = __ldca(p + 1);
-    const bool le = __all_sync(0xffffffffu, eq4(max4(r0, x0), r0) && eq4(max4(r1, x1), r1));  // x <= r
-    const bool ge = __all_sync(0xffffffffu, eq4(max4(r0, x0), x0) && eq4(max4(r1, x1), x1));  // x >= r
-    r0 = max4(r0, x0);
-    r1 = max4(r1, x1);
+  auto take = [&](uint32_t id, const uint4& x0, const uint4& x1) {
+    const uint4 m0 = max4(r0, x0), m1 = max4(r1, x1);
+    const bool le = __all_sync(0xffffffffu, eq4(m0, r0) && eq4(m1, r1));  // x <= r
+    const bool ge = __all_sync(0xffffffffu, eq4(m0, x0) && eq4(m1, x1));  // x >= r
+    r0 = m0;
+    r1 = m1;
     if (!(le && have)) cid = id;
     have = (le && have) || ge;
+  };
+  for (uint32_t m = leaders; m;) {  // two inputs' loads at a time
+    const uint32_t ia = __shfl_sync(0xffffffffu, idm, __ffs(m) - 1);
+    m &= m - 1;
+    const uint32_t ib = __shfl_sync(0xffffffffu, idm, m ? __ffs(m) - 1 : 0);
+    const uint4* p = tile_src(a, ia);
+    const uint4* q = tile_src(a, m ? ib : ia);
+    const uint4 x0 = __ldca(p), x1 = __ldca(p + 1), y0 = __ldca(q), y1 = __ldca(q + 1);
+    take(ia, x0, x1);
+    if (m) take(ib, y0, y1);
+    m &= m - 1;
   }
   bool raised = false;
-  for (uint32_t m = ovm; m; m &= m - 1) {
-    const int mm = __ffs(m) - 1;
-    const uint32_t e = first + mm - lo, val = __shfl_sync(0xffffffffu, nm, mm);
-    if (lane == int(e >> 3)) raised |= raise8(r0, r1, e & 7, val);
+  if (own_here) {  // the lane's entries lo + 8 lane + c are those of members lo + 8 lane + c - first
+    const int m0 = int(lo + 8 * lane) - int(first);
+    if (m0 > -8 && m0 < int(apb)) {
+      auto raise = [&](uint32_t x, int c) {
+        const int m = m0 + c;
+        const uint32_t v = m >= 0 && m < int(apb) ? nbuf[m] : 0u;
+        raised |= v > x;
+        return max(x, v);
+      };
+      r0 = make_uint4(raise(r0.x, 0), raise(r0.y, 1), raise(r0.z, 2), raise(r0.w, 3));
+      r1 = make_uint4(raise(r1.x, 4), raise(r1.y, 5), raise(r1.z, 6), raise(r1.w, 7));
+    }
   }
   const bool keep = have && !__any_sync(0xffffffffu, raised);
   ta.count(__popc(leaders), keep ? 0u : 1u);
   if (keep) return cid;
   const uint32_t nid = alloc_tile(a, ta);
-  if (!nid) return leaders ? __shfl_sync(0xffffffffu, idm, __ffs(leaders) - 1) : 0u;
+  if (!nid) return any ? id0 : 0u;
   uint4* d = tile_dst(a, nid);
   d[0] = r0;
   d[1] = r1;
@@ -297,19 +435,28 @@ __device__ __noinline__ uint32_t join_members(const WideArgs& a, uint32_t idm, u
 // One warp per agent, one CTA per block of the traced program (agents_per_block <= 32).
 // MINB = CTAs of 1024 threads that must share an SM for all blocks to be co-resident.
 template <int MINB>
-__global__ void __launch_bounds__(1024, MINB) k_prop_wide(WideArgs a) {
-  extern __shared__ uint32_t sm[];
+__global__ void __launch_bounds__(1024, MINB) k_prop_wide(const __grid_constant__ WideArgs a) {
+  extern __shared__ __align__(16) uint32_t sm[];
+  __shared__ Shared sh;
   const Geo& g = a.g;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t apb = g.apb;
   const uint32_t first = blockIdx.x * apb;
   const uint32_t u = first + warp;
-  uint32_t* tabs = sm;                  // [apb][3][32] member tables (P, H, JN)
-  uint32_t* nbuf = sm + apb * 96;       // [apb] member epochs
+  uint32_t* const ring = sm + warp * 2 * kPlanBatch * 8;  // [apb][2][kPlanBatch] plan entries
+  uint32_t* tabs = sm + apb * 2 * kPlanBatch * 8;         // [apb][3][32] member tables (P, H, JN)
+  uint32_t* nbuf = tabs + apb * 96;     // [apb] member epochs
   uint32_t* J = nbuf + 32;              // [3][32] joined tables
   uint32_t* tcnt = J + 96 + warp * 2;   // [apb][2] tiles this warp read and wrote (lane 0 counts)
   __shared__ int start_code;
-  if (threadIdx.x == 0) start_code = *(volatile int*)&a.st->code;
+  if (threadIdx.x == 0) {
+    start_code = *(volatile int*)&a.st->code;
+    sh.used = sh.open = sh.arrived = 0;
+    for (uint32_t q = 0; q < kPosts; ++q) {
+      sh.post[q].next = kClosed;
+      sh.post[q].total = 0;
+    }
+  }
   __syncthreads();
   if (start_code) return;
   const bool act = lane < int(g.nT);
@@ -317,6 +464,7 @@ __global__ void __launch_bounds__(1024, MINB) k_prop_wide(WideArgs a) {
   TileAlloc ta;
   ta.cnt = tcnt;
   if (lane == 0) tcnt[0] = tcnt[1] = 0;
+  ask_chunk(a, ta);
   // H_t = bottom{t := 1}: the table starts at bottom and H_t[t] = N_t is kept implicit (in
   // N), so no tile is copied when it increments; a release snapshot writes it out
   // JN_t (jid): the join of every H snapshot joined into P_t, carried along with P_t (joined
@@ -325,22 +473,33 @@ __global__ void __launch_bounds__(1024, MINB) k_prop_wide(WideArgs a) {
   // at epoch e: such a join (release loop, in-section access) changes nothing and is skipped.
   uint32_t pid = 0, hid = 0, jid = 0;
   uint32_t N = 1;
+  uint32_t arrivals = 0;  // arrivals that complete the block barrier at hand
   unsigned long long joins = 0, visits = 0;
   if (act) a.rows[size_t(a.rowbase[u]) * kTabW + lane] = a.hb_only ? hid : 0u;
   const uint32_t k0 = a.sy_start[u], k1 = a.sy_start[u + 1];
   const uint32_t pb = k0 + a.incs_off[k0], pe = k1 + a.incs_off[k1];
   uint32_t* const cursor_row = a.cursor + size_t(u) * a.n_locks;
-  uint4 na = make_uint4(0, 0, 0, 0), nb = na;
-  if (pb < pe) {
-    na = a.plan[2 * size_t(pb)];
-    nb = a.plan[2 * size_t(pb) + 1];
-  }
+  // plan entries, 16 at a time in two halves of the warp's ring: the next ones are copied in
+  // while these are walked (read one step ahead they were 1,900 cycles of memory latency each)
+  auto fetch = [&](uint32_t b0, uint32_t half) {
+    const uint32_t e = b0 + lane / 2;
+    if (e < pe)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<uint32_t>(
+                       __cvta_generic_to_shared(ring + half * kPlanBatch * 8 + lane * 4))),
+                   "l"(a.plan + 2 * size_t(b0) + lane)
+                   : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  fetch(pb, 0);
   for (uint32_t p = pb; p < pe; ++p) {
-    const uint4 ea = na, eb = nb;
-    if (p + 1 < pe) {  // the next entry's loads overlap this one
-      na = a.plan[2 * size_t(p + 1)];
-      nb = a.plan[2 * size_t(p + 1) + 1];
+    const uint32_t i = (p - pb) % kPlanBatch, half = ((p - pb) / kPlanBatch) & 1u;
+    if (i == 0) {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncwarp();
+      fetch(p + kPlanBatch, half ^ 1u);
     }
+    const uint4 ea = *reinterpret_cast<const uint4*>(ring + (half * kPlanBatch + i) * 8),
+                eb = *reinterpret_cast<const uint4*>(ring + (half * kPlanBatch + i) * 8 + 4);
     const uint32_t t = ea.x & 0xFF, row = ea.y;
     if (t == P_ACQ || t == P_INCS) {
       // acquire: P_t |= P_<l,s'>, H_t |= H_<l,s'>; in-section access: P_t |= L^w (| L^r)
@@ -354,29 +513,32 @@ __global__ void __launch_bounds__(1024, MINB) k_prop_wide(WideArgs a) {
           x = __ldcg(list + off + q);
         if (t == P_ACQ) {
           // the three published tables are loaded together (a table still being written is
-          // then waited for), and every tile the three merges read is prefetched first
+          // then waited for)
           uint32_t sp = lane < int(g.nT) ? __ldcg(a.psnap + size_t(x) * kTabW + lane) : 0;
-          uint32_t sh = lane < int(g.nT) ? __ldcg(a.hsnap + size_t(x) * kTabW + lane) : 0;
+          uint32_t sq = lane < int(g.nT) ? __ldcg(a.hsnap + size_t(x) * kTabW + lane) : 0;
           uint32_t sj = lane < int(g.nT) ? __ldcg(a.jsnap + size_t(x) * kTabW + lane) : 0;
-          if (!__all_sync(0xffffffffu, sp != SENT && sh != SENT && sj != SENT)) {
-            sp = read_table(a, a.psnap + size_t(x) * kTabW, abort);
-            sh = read_table(a, a.hsnap + size_t(x) * kTabW, abort);
-            sj = read_table(a, a.jsnap + size_t(x) * kTabW, abort);
+          if (!__all_sync(0xffffffffu, sp != SENT && sq != SENT && sj != SENT)) {
+            sp = read_table(a, a.psnap + size_t(x) * kTabW, abort, sh, ta);
+            sq = read_table(a, a.hsnap + size_t(x) * kTabW, abort, sh, ta);
+            sj = read_table(a, a.jsnap + size_t(x) * kTabW, abort, sh, ta);
           }
-          prefetch_merge(a, hid, sh);
-          prefetch_merge(a, jid, sj);
-          merge_table(a, pid, sp, dirty, ta);
-          merge_table(a, hid, sh, dirty, ta);
-          merge_table(a, jid, sj, dirty, ta);
+          uint32_t mine[3] = {pid, hid, jid};
+          const uint32_t theirs[3] = {sp, sq, sj};
+          merge_tables<3>(a, mine, theirs, dirty, ta, sh);
+          pid = mine[0];
+          hid = mine[1];
+          jid = mine[2];
           joins += 2;
         } else {
           // L^w / L^r: the H snapshot of section x's release, unless JN_t already covers it
           const uint4 mx = __ldg(a.recmeta + x);
           if (entry_of(a, jid, mx.x & 0xFFFF) < mx.w) {
-            const uint32_t sx = read_table(a, a.hsnap + size_t(x) * kTabW, abort);
-            prefetch_merge(a, jid, sx);
-            merge_table(a, pid, sx, dirty, ta);
-            merge_table(a, jid, sx, dirty, ta);
+            const uint32_t sx = read_table(a, a.hsnap + size_t(x) * kTabW, abort, sh, ta);
+            uint32_t mine[2] = {pid, jid};
+            const uint32_t theirs[2] = {sx, sx};
+            merge_tables<2>(a, mine, theirs, dirty, ta, sh);
+            pid = mine[0];
+            jid = mine[1];
             joins += 1;
           }
         }
@@ -412,10 +574,12 @@ __global__ void __launch_bounds__(1024, MINB) k_prop_wide(WideArgs a) {
           visits += __popc(__ballot_sync(0xffffffffu, in && uint32_t(lane) <= f && !mine));
           for (uint32_t wm = wave; wm; wm &= wm - 1) {
             const uint32_t r = lo + cur + (__ffs(wm) - 1);
-            const uint32_t sx = read_table(a, a.hsnap + size_t(r) * kTabW, abort);
-            prefetch_merge(a, jid, sx);
-            merge_table(a, pid, sx, dirty, ta);
-            merge_table(a, jid, sx, dirty, ta);
+            const uint32_t sx = read_table(a, a.hsnap + size_t(r) * kTabW, abort, sh, ta);
+            uint32_t mine[2] = {pid, jid};
+            const uint32_t theirs[2] = {sx, sx};
+            merge_tables<2>(a, mine, theirs, dirty, ta, sh);
+            pid = mine[0];
+            jid = mine[1];
             ++joins;
           }
           if (f == nbr) {
@@ -452,28 +616,43 @@ __global__ void __launch_bounds__(1024, MINB) k_prop_wide(WideArgs a) {
           tabs[(warp * 3 + 2) * 32 + lane] = jid;
         }
         if (lane == 0) nbuf[warp] = N;
-        __syncthreads();
+        // all members have arrived when the count says so; until then merges of others are
+        // taken. The members' own waits are bounded and always end in an arrival; the time
+        // limit here only backs them up.
         const uint32_t nw = blockDim.x >> 5;
-        bool wrote = false;
-        for (uint32_t T = warp; T < g.nT; T += nw) {
-          const bool mem = uint32_t(lane) < apb;
-          const uint32_t cm = mem ? tabs[(lane * 3) * 32 + T] : 0, hm = mem ? tabs[(lane * 3 + 1) * 32 + T] : 0;
-          const uint32_t jm = mem ? tabs[(lane * 3 + 2) * 32 + T] : 0;
-          const uint32_t nm = mem ? nbuf[lane] : 0;
-          if (cm) prefetch_tile(a, cm);
-          if (hm) prefetch_tile(a, hm);
-          if (jm) prefetch_tile(a, jm);
-          const uint32_t jc = join_members(a, cm, nm, apb, first, T, true, wrote, ta);
-          const uint32_t jh = join_members(a, hm, nm, apb, first, T, true, wrote, ta);
-          const uint32_t jj = join_members(a, jm, nm, apb, first, T, false, wrote, ta);
-          if (lane == 0) {
-            J[T] = jc;
-            J[32 + T] = jh;
-            J[64 + T] = jj;
+        arrivals += nw;
+        __threadfence_block();
+        __syncwarp();
+        if (lane == 0) atomicAdd(&sh.arrived, 1u);
+        unsigned long long t0 = 0;
+        for (uint32_t it = 1; !abort; ++it) {
+          const uint2 seen = look(sh);
+          if (int(seen.y - arrivals) >= 0) break;
+          if (seen.x)
+            help(a, sh, seen.x, ta);
+          else
+            __nanosleep(kWaitNs);
+          if ((it & 0xFFFFu) == 0) {
+            const unsigned long long now = global_ns();
+            if (!t0) t0 = now;
+            if (__any_sync(0xffffffffu, now - t0 > kBarrierLimitNs)) {
+              if (lane == 0) atomicCAS(&a.st->code, 0, GWCP_ERR_TIMEOUT);
+              abort = true;
+            }
           }
         }
-        if (wrote) __threadfence();  // members may publish the joined tiles at once
+        __threadfence_block();
+        bool wrote = false;  // (members fence before they publish the joined tiles)
+        // (table, tile) pairs over the warps (asking for their inputs with L1 prefetches first
+        // measured 8% slower)
+        for (uint32_t job = warp; job < 3 * g.nT; job += nw) {
+          const uint32_t tab = job / g.nT, T = job - tab * g.nT;
+          const uint32_t id = uint32_t(lane) < apb ? tabs[(lane * 3 + tab) * 32 + T] : 0;
+          const uint32_t j = join_members(a, id, nbuf, apb, first, T, tab < 2, wrote, ta);
+          if (lane == 0) J[tab * 32 + T] = j;
+        }
         __syncthreads();
+        dirty = true;
         pid = act ? J[lane] : 0;
         hid = act ? J[32 + lane] : 0;
         jid = act ? J[64 + lane] : 0;
@@ -963,7 +1142,8 @@ int phaseG_wide(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s) {
   a.n_locks = z.n_locks;
   a.hb_only = z.hb_only;
   const uint32_t threads = g.apb * 32;
-  const size_t smem = (size_t(g.apb) * 96 + 32 + 96 + 2 * size_t(g.apb)) * 4;
+  // member tables, epochs, joined tables, tile counts, plan rings
+  const size_t smem = (size_t(g.apb) * 96 + 32 + 96 + 2 * size_t(g.apb) + size_t(g.apb) * 2 * kPlanBatch * 8) * 4;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -973,6 +1153,8 @@ int phaseG_wide(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s) {
   void* order[2] = {reinterpret_cast<void*>(k_prop_wide<1>), reinterpret_cast<void*>(k_prop_wide<2>)};
   if (z.pack_walkers) std::swap(order[0], order[1]);
   for (void* k : order) {
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kMaxDynamicSmem)) != cudaSuccess)
+      return GWCP_ERR_CUDA;
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, int(threads), smem) != cudaSuccess)
       return GWCP_ERR_CUDA;
