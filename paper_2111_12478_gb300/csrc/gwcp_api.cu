@@ -433,7 +433,7 @@ int run(gwcp_ctx* c, cudaStream_t s) {
   z.n_cs = z.n_acqrel ? c->cnt_host[2] : 0;
   z.n_locks = z.n_acqrel ? c->cnt_host[3] : 0;
   z.n_exp = c->cnt_host[4];
-  const uint32_t slots = std::min<uint32_t>(g.B + 1, lock_scope_cap(g.B));
+  const uint32_t slots = lock_stride(g);
   z.pool_cap = z.n_cs * slots + z.n_exp * 2 * slots + 64;
   b.dep_pool = get<uint32_t>(c, "dep_pool", z.pool_cap, &oom);
   z.race_cap = c->opt.race_capacity ? c->opt.race_capacity : std::max<uint64_t>(1u << 20, z.N);

@@ -35,6 +35,10 @@ __host__ __device__ inline uint32_t lock_scope_cap(uint32_t blocks) {
   return blocks + 1 <= uint32_t(kLockScopesSmall) ? kLockScopesSmall : kLockScopesLarge;
 }
 
+// most scope ids one lock can have: an acquire joins at most one release per scope
+struct Geo;
+inline uint32_t lock_stride(const Geo& g);
+
 // S entry kinds (agent-sorted event stream), packed as (kind << 30) | trace index
 enum : uint32_t { K_ACCESS = 0, K_ACQ = 1, K_REL = 2, K_BAR = 3 };
 __host__ __device__ inline uint32_t s_kind(uint32_t s) { return s >> 30; }
@@ -79,6 +83,11 @@ struct Geo {
   uint32_t nT;  // wide clocks: tiles of kTileW entries (0: clocks in registers)
   uint32_t RW;  // words per published clock: Wp, or kTabW tile ids when nT > 0
 };
+
+inline uint32_t lock_stride(const Geo& g) {
+  const uint32_t cap = lock_scope_cap(g.B);
+  return g.B + 1 < cap ? g.B + 1 : cap;
+}
 
 // Per-access record consumed by the check (indexed by trace index).
 struct AccInfo {

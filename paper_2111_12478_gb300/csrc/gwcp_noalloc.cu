@@ -186,7 +186,7 @@ int analyze(const Event* ev, uint64_t n, const Geo& g, gwcp_race* out, uint64_t 
   z.n_cs = z.n_acqrel ? v[2] : 0;
   z.n_locks = z.n_acqrel ? v[3] : 0;
   z.n_exp = v[4];
-  const uint32_t slots = std::min<uint32_t>(g.B + 1, lock_scope_cap(g.B));
+  const uint32_t slots = lock_stride(g);
   z.pool_cap = z.n_cs * slots + z.n_exp * 2 * slots + 64;
   b.dep_pool = A.take<uint32_t>(z.pool_cap);
   if (A.full) return GWCP_ERR_UNSUPPORTED;
