@@ -258,14 +258,17 @@ int run(gwcp_ctx* c, cudaStream_t s) {
   // many agents: S by a sort on the agent (a per-warp count table of Wp words would leave
   // phase A a few warps per SM)
   z.agent_sort = g.Wp > 2048;
-  z.TA = g.Wp <= 256 || z.agent_sort ? 2048 : 8192;
-  if (!z.agent_sort)
-    while (uint64_t(g.W) * ((z.N + z.TA - 1) / z.TA) > (1ull << 26)) z.TA <<= 1;  // bounded agent histogram
+  z.TA = phaseA_tile(g, z.N, z.agent_sort);
   z.ntA = uint32_t((z.N + z.TA - 1) / z.TA);
+  // phase D's index: windows of 2^d_shift events, at most 2^23 entries over all agents
+  z.d_shift = 8;
+  while (uint64_t(g.W) * ((z.N >> z.d_shift) + 2) > (1ull << 23)) ++z.d_shift;
+  z.d_nw = uint32_t((z.N >> z.d_shift) + 2);
   const size_t hist_words = z.agent_sort ? 1 : size_t(g.W) * z.ntA + 1;
   b.ev = c->ev_dev;
   b.st = get<DevStatus>(c, "st", 1, &oom);
-  b.hist_a = get<uint32_t>(c, "hist_a", hist_words, &oom);
+  // phase A's agent histogram, later phase D's index
+  b.hist_a = b.d_index = get<uint32_t>(c, "d_index", std::max(hist_words, size_t(g.W) * z.d_nw), &oom);
   b.tile_cnt = get<uint32_t>(c, "tile_cnt", 4 * (size_t(z.ntA) + 1), &oom);
   const size_t scan_need = std::max({scan_tmp_need(hist_words), radix_tmp_need(z.N + 1),
                                      scan_tmp_need(z.N + 1)}) + 64;
@@ -349,11 +352,6 @@ int run(gwcp_ctx* c, cudaStream_t s) {
   b.sy_match = get<uint32_t>(c, "sy_match", ns1, &oom);
   b.sy_relk = get<uint32_t>(c, "sy_relk", ns1, &oom);
   b.sy_agent = get<uint32_t>(c, "sy_agent", ns1, &oom);
-  // phase D's index: windows of 2^d_shift events, at most 2^23 entries over all agents
-  z.d_shift = 8;
-  while (uint64_t(g.W) * ((z.N >> z.d_shift) + 2) > (1ull << 23)) ++z.d_shift;
-  z.d_nw = uint32_t((z.N >> z.d_shift) + 2);
-  b.d_index = get<uint32_t>(c, "d_index", size_t(g.W) * z.d_nw, &oom);
   b.incs_cnt = get<uint32_t>(c, "incs_cnt", ns1, &oom);
   b.vcount = get<uint32_t>(c, "vcount", g.W + 1, &oom);
   const size_t na1 = size_t(z.n_acqrel) + 1;

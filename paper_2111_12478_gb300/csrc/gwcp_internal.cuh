@@ -465,6 +465,7 @@ struct Prof {
   void end();
 };
 
+uint32_t phaseA_tile(const Geo& g, uint64_t n, bool agent_sort);  // events per tile (a warp's)
 void phaseA_count(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, Prof& p);
 void phaseA_scatter(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, Prof& p);
 void phaseB_sync(const Bufs& b, const Geo& g, Sizes& z, cudaStream_t s, Prof& p);

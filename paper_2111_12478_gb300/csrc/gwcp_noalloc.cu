@@ -106,6 +106,7 @@ int analyze(const Event* ev, uint64_t n, const Geo& g, gwcp_race* out, uint64_t 
   DevStatus st{};
   uint32_t v[8] = {};
   z.N = n;
+  // (the first array sets aside tiles of 2048 events: which traces fit depends on it)
   z.TA = 2048;
   z.ntA = uint32_t((n + z.TA - 1) / z.TA);
   b.ev = ev;
@@ -115,8 +116,21 @@ int analyze(const Event* ev, uint64_t n, const Geo& g, gwcp_race* out, uint64_t 
   const size_t scan_need = std::max({scan_tmp_need(size_t(g.W) * z.ntA + 1), sort_words(n + 1),
                                      scan_tmp_need(n + 1)}) + 64;
   A.take<uint32_t>(scan_need);
-  b.scan_tmp = X.take<uint32_t>(std::max(scan_need, radix_tmp_need(n + 1) + 64));
-  if (A.full) return GWCP_ERR_UNSUPPORTED;
+  // smaller tiles, where their counts fit what the second array has left: phase A is done
+  // with them before anything else is carved from it
+  const uint32_t ta = phaseA_tile(g, n, false);
+  const size_t nt = size_t((n + ta - 1) / ta), fine = size_t(g.W) * nt + 1;
+  b.scan_tmp = X.take<uint32_t>(std::max({scan_need, scan_tmp_need(fine) + 64, radix_tmp_need(n + 1) + 64}));
+  if (A.full || X.full) return GWCP_ERR_UNSUPPORTED;
+  Arena T = X;
+  uint32_t* const hist = T.take<uint32_t>(fine);
+  uint32_t* const cnt = T.take<uint32_t>(4 * (nt + 1));
+  if (ta < z.TA && !T.full) {
+    z.TA = ta;
+    z.ntA = uint32_t(nt);
+    b.hist_a = hist;
+    b.tile_cnt = cnt;
+  }
   DevStatus init{};
   init.bad_index = ~0ull;
   init.key_and = ~0ull;

@@ -1210,6 +1210,26 @@ inline uint32_t a_warps(const Geo& g) {
 
 }  // namespace
 
+// A tile is a warp's serial work, so tiles are small while there are few of them: 256 events
+// (two loads of 128) until there are 10,240 tiles (64 or so per SM: one warp per tile fills
+// it), and until the agent histogram has 4M words (a tile reads and writes a word per agent,
+// each in a sector of its own). Phase A with its scans, by tile size:
+//   10k events, 64 agents     256: 0.063 ms   2048: 0.132
+//   1M, 64                    128: 0.113      256: 0.102     2048: 0.221
+//   10M, 64                   512: 0.371      1024: 0.360    2048: 0.391
+//   5M, 256                   256: 0.288      512: 0.236     2048: 0.281
+//   2.3M, 512                 256: 0.183      512: 0.161     8192: 0.669
+//   3M, 1024                  512: 0.236      1024: 0.202    8192: 0.681
+uint32_t phaseA_tile(const Geo& g, uint64_t n, bool agent_sort) {
+  const uint32_t most = g.Wp <= 256 || agent_sort ? 2048 : 8192;
+  uint32_t t = 256;
+  auto tiles = [&] { return (n + t - 1) / t; };
+  while (t < most && (tiles() > 10240 || (!agent_sort && g.W * tiles() > (4u << 20)))) t <<= 1;
+  if (!agent_sort)
+    while (g.W * tiles() > (1ull << 26)) t <<= 1;  // bounded agent histogram
+  return t;
+}
+
 void phaseA_count(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, Prof& p) {
   p.begin("a_count", double(z.N) * 16);
   const bool vec = (reinterpret_cast<uintptr_t>(b.ev) & 15) == 0;
