@@ -434,7 +434,12 @@ int run(gwcp_ctx* c, cudaStream_t s) {
   const uint32_t slots = lock_stride(g);
   z.pool_cap = z.n_cs * slots + z.n_exp * 2 * slots + 64;
   b.dep_pool = get<uint32_t>(c, "dep_pool", z.pool_cap, &oom);
-  z.race_cap = c->opt.race_capacity ? c->opt.race_capacity : std::max<uint64_t>(1u << 20, z.N);
+  // automatic capacity: at least what the race buffers of an earlier pass hold (a trace with
+  // more races than events would run its check twice on every pass)
+  z.race_cap = c->opt.race_capacity ? c->opt.race_capacity
+                                    : std::max<uint64_t>({1u << 20, z.N,
+                                                          std::min(c->allocs["races"].second,
+                                                                   c->allocs["races2"].second) / 8});
   // scratch for every later scan and sort (the stream is idle here, so it may move)
   const size_t ex_bound = size_t(z.n_incs) * kMaxNest + 1;
   const size_t need2 = std::max({scan_need, radix_tmp_need(ex_bound), radix_tmp_need(z.race_cap + 1),
@@ -483,13 +488,28 @@ int run(gwcp_ctx* c, cudaStream_t s) {
     z.cv_cap = std::min<uint64_t>(c->cv_cap_hint ? c->cv_cap_hint : want, kCvMaxWords);
     b.cv_pool = get<uint32_t>(c, "cv_pool", z.cv_cap, &oom);
   }
-  b.psnap = get<uint32_t>(c, "psnap", (size_t(z.n_cs) + 1) * g.RW, &oom);
+  b.races = get<uint64_t>(c, "races", z.race_cap, &oom);
+  b.races2 = get<uint64_t>(c, "races2", z.race_cap, &oom);
+  // what only the propagation reads and writes lies in the race sort's second buffer, as far
+  // as that reaches
+  size_t late_used = 0;
+  auto late = [&](const char* name, size_t bytes) -> void* {
+    const size_t at = late_used, end = (at + bytes + 255) & ~size_t(255);
+    if (oom || end > z.race_cap * sizeof(uint64_t)) return get<unsigned char>(c, name, bytes, &oom);
+    late_used = end;
+    return reinterpret_cast<unsigned char*>(b.races2) + at;
+  };
+  const size_t plan_bytes = (2 * (size_t(z.n_sync) + z.n_incs) + 2) * sizeof(uint4);
+  const size_t snap_bytes = (size_t(z.n_cs) + 1) * g.RW * sizeof(uint32_t);
+  b.plan = static_cast<uint4*>(late("plan", plan_bytes));
+  b.plan2 = static_cast<uint4*>(late("plan2", plan_bytes));
+  b.jsnap = static_cast<uint32_t*>(late("jsnap", snap_bytes));
+  b.psnap = static_cast<uint32_t*>(late("psnap", snap_bytes));
   b.hsnap = get<uint32_t>(c, "hsnap", (size_t(z.n_cs) + 1) * g.RW, &oom);
-  b.jsnap = get<uint32_t>(c, "jsnap", (size_t(z.n_cs) + 1) * g.RW, &oom);
   if (g.nT) {
     // tile pool: a few new tiles per clock version; grown and rerun on exhaustion
     const uint64_t want = 2ull * (uint64_t(z.n_rows) + z.n_cs) + uint64_t(z.n_bar) * (g.apb + 2) +
-                          std::max<uint64_t>(65536, 16ull * g.W + 32768);  // each walker holds up to two chunks of 8
+                          65536;  // each walker holds up to two chunks of 4
     z.tile_cap = std::max<uint64_t>(c->tile_cap_hint, want);
     // 2 MB aligned: the walkers' time depended by ~3% on where the pool landed after the
     // buffers allocated before it (77 vs 79.5 ms on the 8192-warp, 200M-event workload
@@ -497,8 +517,6 @@ int run(gwcp_ctx* c, cudaStream_t s) {
     // came before
     b.tiles = get_aligned<uint32_t>(c, "tiles", size_t(z.tile_cap) * kTileW, size_t(2) << 20, &oom);
   }
-  b.plan = get<uint4>(c, "plan", 2 * (size_t(z.n_sync) + z.n_incs) + 2, &oom);
-  b.plan2 = get<uint4>(c, "plan2", 2 * (size_t(z.n_sync) + z.n_incs) + 2, &oom);
   b.recmeta = get<uint4>(c, "recmeta", size_t(z.n_cs) + 1, &oom);
   b.flat_off = get<uint32_t>(c, "flat_off", ni1, &oom);
   b.flat = get<uint32_t>(c, "flat", z.pool_cap, &oom);
@@ -526,17 +544,11 @@ int run(gwcp_ctx* c, cudaStream_t s) {
     b.wc_who = get<uint32_t>(c, "wc_who", na, &oom);
     b.wc_row = get<uint32_t>(c, "wc_row", na, &oom);
     b.wc_ep = get<uint32_t>(c, "wc_ep", na, &oom);
-    if (z.grouped) {
-      z.big_cap = z.n_acc / 8 + 65536;  // accesses past it are finished in their own warp
-      b.wc_big = get<uint64_t>(c, "wc_big", z.big_cap, &oom);
-    }
   } else {
     z.n_chunks = uint32_t(check_chunks(z.n_acc));
     const size_t ng = check_group_count(z.n_acc);
     b.tails = get<uint32_t>(c, "tails", (size_t(z.n_chunks) + ng) * 4 * g.Wp * 2 + ng + 8, &oom);
   }
-  b.races = get<uint64_t>(c, "races", z.race_cap, &oom);
-  b.races2 = get<uint64_t>(c, "races2", z.race_cap, &oom);
   if (oom) return GWCP_ERR_OOM;
   if (g.nT) {  // tile 0 is the zero tile; ids are handed out from 1
     cudaMemsetAsync(b.tiles, 0, kTileW * 4, s);
@@ -620,6 +632,10 @@ int run(gwcp_ctx* c, cudaStream_t s) {
               : phaseI_wide_group(b, g, z, side_tmp, c->side, c->prof);
   else
     phaseI_carry(b, g, z, c->side, c->prof);
+  if (z.grouped) {  // in the access sort's other buffer; an access that finds no room is walked by its own thread
+    z.big_cap = std::min(z.n_acc, z.n_acc / 8 + 65536);
+    b.wc_big = b.acc_key2;
+  }
   int prc = phaseG_propagate(b, g, z, s, c->prof);
   side.join();
   if (prc) return prc;

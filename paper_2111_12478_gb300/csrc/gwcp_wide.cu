@@ -94,7 +94,7 @@ __device__ __forceinline__ void set8(uint4& x0, uint4& x1, uint32_t c, uint32_t 
 // one per tile on a single counter); the warp-uniform state lives in the walker. The next
 // chunk is asked for when the current one is begun, so that its atomic's latency is over
 // when it is needed.
-constexpr uint32_t kTileChunk = 8;
+constexpr uint32_t kTileChunk = 4;
 struct TileAlloc {
   uint32_t next = 0, end = 0;  // ids [next, end) are the warp's; both clamped to the pool size
   unsigned long long ahead = 0;  // lane 0: the next chunk's first id
