@@ -17,7 +17,6 @@ unsigned long long launch_count();
 size_t check_chunks(uint32_t n_acc);
 size_t check_group_count(uint32_t n_acc);
 void phaseE_scan(const Bufs& b, const Sizes& z, cudaStream_t s, Prof& p);
-void phaseF_deps(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, Prof& p);
 
 cudaEvent_t Prof::ev() {
   if (used == pool.size()) {
@@ -467,17 +466,12 @@ int run(gwcp_ctx* c, cudaStream_t s) {
   b.incs_k = get<uint32_t>(c, "incs_k", ni1, &oom);
   b.incs_key = get<uint64_t>(c, "incs_key", ni1, &oom);
   b.incs_wr = get<uint32_t>(c, "incs_wr", ni1, &oom);
-  b.exp_off = get<uint32_t>(c, "exp_off", ni1, &oom);
-  // expanded records: sized by the bound (depth <= kMaxNest), sorted by the exact count
-  const size_t ne1 = std::max<size_t>(size_t(z.n_exp), size_t(z.n_incs) * kMaxNest) + 1;
+  const size_t ne1 = size_t(z.n_exp) + 1;
   b.ex_key = get<uint64_t>(c, "ex_key", ne1, &oom);
   b.ex_val = get<uint32_t>(c, "ex_val", ne1, &oom);
   b.ex_key2 = get<uint64_t>(c, "ex_key2", ne1, &oom);
   b.ex_val2 = get<uint32_t>(c, "ex_val2", ne1, &oom);
-  b.ex_rec = get<uint32_t>(c, "ex_rec", ne1, &oom);
-  b.ex_cs = get<uint32_t>(c, "ex_cs", ne1, &oom);
-  b.ex_flags = get<uint32_t>(c, "ex_flags", ne1, &oom);
-  b.ex_group = get<uint32_t>(c, "ex_group", ne1 + 1, &oom);
+  b.ex_info = get<uint2>(c, "ex_info", ne1, &oom);
   b.ex_dep_off = get<uint32_t>(c, "ex_dep_off", ne1, &oom);
   b.ex_dep_cnt = get<uint32_t>(c, "ex_dep_cnt", ne1, &oom);
   b.rows = get<uint32_t>(c, "rows", size_t(z.n_rows) * (z.compress ? g.B : g.RW), &oom);
@@ -595,10 +589,8 @@ int run(gwcp_ctx* c, cudaStream_t s) {
     b.chunk_races = nullptr;
   }
   if (oom) return GWCP_ERR_OOM;
-  phaseF_incs(b, g, z, key_mask, s, c->prof);
-  phaseF_walk(b, g, z, key_mask, s, c->prof);
-  z.n_groups = z.n_exp;  // upper bound; the kernel reads the exact count on the device
-  phaseF_deps(b, g, z, s, c->prof);
+  phaseF_expand(b, z, s, c->prof);
+  phaseF_deps(b, g, z, key_mask, s, c->prof);
   cudaStreamWaitEvent(c->side, c->fork2, 0);
   if (z.grouped) {
     // the main stream has phases D-F queued; the sort has usually finished by now

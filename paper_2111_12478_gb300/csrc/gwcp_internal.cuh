@@ -169,15 +169,13 @@ struct Bufs {
   uint32_t* acq_dep_cnt = nullptr;
   uint32_t* dep_pool = nullptr;     // [pool_cap]
   // phase F: in-section dependencies
-  uint32_t* exp_off = nullptr;   // [n_incs + 1]
+  uint32_t* cs_exp = nullptr;    // [n_cs] the section's first (access, held section) record
+  uint32_t* cs_r0 = nullptr;     // [n_cs] its first in-section access
   uint64_t* ex_key = nullptr;    // [n_exp] (+ alt)
   uint32_t* ex_val = nullptr;
   uint64_t* ex_key2 = nullptr;
   uint32_t* ex_val2 = nullptr;
-  uint32_t* ex_rec = nullptr;    // [n_exp] in-section record of each expanded record
-  uint32_t* ex_cs = nullptr;     // [n_exp] held critical section
-  uint32_t* ex_flags = nullptr;  // [n_exp + 1]
-  uint32_t* ex_group = nullptr;  // [n_groups + 1]
+  uint2* ex_info = nullptr;      // [n_exp] (held critical section, its lock << 1 | write class)
   uint32_t* ex_dep_off = nullptr;  // [n_exp]
   uint32_t* ex_dep_cnt = nullptr;
   // phase G: propagation
@@ -400,7 +398,7 @@ struct Sizes {
   uint32_t ntA = 0, TA = 0;
   uint32_t nS = 0, n_acc = 0, n_acqrel = 0, n_bar = 0;
   uint32_t ntS = 0;
-  uint32_t n_sync = 0, n_incs = 0, n_rows = 0, n_cs = 0, n_locks = 0, n_exp = 0, n_groups = 0;
+  uint32_t n_sync = 0, n_incs = 0, n_rows = 0, n_cs = 0, n_locks = 0, n_exp = 0;
   uint32_t pool_cap = 0;
   uint32_t n_chunks = 0;
   uint64_t race_cap = 0;
@@ -476,9 +474,9 @@ void phaseD_gaps(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, Pr
 // records of the others are then left unwritten)
 void phaseD_trace(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, bool filtered);
 void phaseE_locks(Bufs& b, const Geo& g, const Sizes& z, uint64_t lock_mask, cudaStream_t s, Prof& p);
-void phaseE_walk(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, Prof& p);
-void phaseF_incs(const Bufs& b, const Geo& g, const Sizes& z, uint64_t key_mask, cudaStream_t s, Prof& p);
-void phaseF_walk(Bufs& b, const Geo& g, const Sizes& z, uint64_t key_mask, cudaStream_t s, Prof& p);
+void phaseE_walk(Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, Prof& p);
+void phaseF_expand(const Bufs& b, const Sizes& z, cudaStream_t s, Prof& p);
+void phaseF_deps(Bufs& b, const Geo& g, const Sizes& z, uint64_t key_mask, cudaStream_t s, Prof& p);
 int phaseG_propagate(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, Prof& p);
 // failure detection test: the walkers' bounded wait on a row nothing completes
 int wait_probe(uint32_t limit, int* code);

@@ -20,7 +20,6 @@
 
 namespace gwcp {
 void phaseE_scan(const Bufs& b, const Sizes& z, cudaStream_t s, Prof& p);
-void phaseF_deps(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, Prof& p);
 size_t check_chunks(uint32_t n_acc);
 size_t check_group_count(uint32_t n_acc);
 }  // namespace gwcp
@@ -215,18 +214,24 @@ int analyze(const Event* ev, uint64_t n, const Geo& g, gwcp_race* out, uint64_t 
   const size_t ni1 = size_t(z.n_incs) + 1;
   const size_t ne1 = std::max<size_t>(size_t(z.n_exp), size_t(z.n_incs) * kMaxNest) + 1;
   b.acc_info = A.take<AccInfo>(z.N);
-  uint32_t** inc[] = {&b.incs_idx, &b.incs_ver, &b.incs_k, &b.incs_wr, &b.exp_off};
+  uint32_t** inc[] = {&b.incs_idx, &b.incs_ver, &b.incs_k, &b.incs_wr};
   for (uint32_t** q : inc) *q = A.take<uint32_t>(ni1);
+  // (sizes marked "unused" stay: which traces fit depends on them)
+  A.take<uint32_t>(ni1);  // unused
   b.incs_key = A.take<uint64_t>(ni1);
   b.ex_key = A.take<uint64_t>(ne1);
   b.ex_key2 = A.take<uint64_t>(ne1);
-  uint32_t** ex[] = {&b.ex_val, &b.ex_val2, &b.ex_rec, &b.ex_cs, &b.ex_flags, &b.ex_dep_off, &b.ex_dep_cnt};
+  uint32_t** ex[] = {&b.ex_val, &b.ex_val2, &b.ex_dep_off, &b.ex_dep_cnt};
   for (uint32_t** q : ex) *q = A.take<uint32_t>(ne1);
-  b.ex_group = A.take<uint32_t>(ne1 + 1);
+  uint32_t* const info = A.take<uint32_t>(ne1);  // ex_info: this and the next
+  A.take<uint32_t>(ne1);
+  b.ex_info = reinterpret_cast<uint2*>(info);
+  A.take<uint32_t>(ne1);      // unused
+  A.take<uint32_t>(ne1 + 1);  // unused
   b.rows = A.take<uint32_t>(size_t(z.n_rows) * g.Wp);
   b.psnap = A.take<uint32_t>((size_t(z.n_cs) + 1) * g.Wp);
   b.hsnap = A.take<uint32_t>((size_t(z.n_cs) + 1) * g.Wp);
-  A.take<uint32_t>(size_t(z.n_cs) + 1);  // (unused: which traces fit stays as it was)
+  A.take<uint32_t>(size_t(z.n_cs) + 1);  // unused
   b.plan = A.take<uint4>(2 * (size_t(z.n_sync) + z.n_incs) + 2);
   b.recmeta = A.take<uint4>(size_t(z.n_cs) + 1);
   b.flat_off = A.take<uint32_t>(ni1);
@@ -269,10 +274,8 @@ int analyze(const Event* ev, uint64_t n, const Geo& g, gwcp_race* out, uint64_t 
     cudaMemsetAsync(b.bar_cnt, 0, size_t(z.n_bar) * 4, s);
   }
   phaseD_gaps(b, g, z, s, prof);
-  phaseF_incs(b, g, z, key_mask, s, prof);
-  phaseF_walk(b, g, z, key_mask, s, prof);
-  z.n_groups = z.n_exp;
-  phaseF_deps(b, g, z, s, prof);
+  phaseF_expand(b, z, s, prof);
+  phaseF_deps(b, g, z, key_mask, s, prof);
   phaseH_sort(b, g, z, key_mask, b.scan_tmp, s, prof);
   if (int rc = phaseG_propagate(b, g, z, s, prof)) return rc;
   phaseI_carry(b, g, z, s, prof);

@@ -52,7 +52,7 @@ struct PropArgs {
   const Event* ev;
   DevStatus* st;
   const uint32_t *sy_start, *sy_idx, *sy_kind, *sy_N, *sy_ver, *sy_aux, *sy_agent;
-  const uint32_t *incs_off, *incs_ver, *incs_k, *exp_off, *ex_dep_off, *ex_dep_cnt;
+  const uint32_t *incs_off, *incs_ver, *incs_k, *sy_inner, *cs_parent, *cs_exp, *cs_r0, *ex_dep_off, *ex_dep_cnt;
   const uint32_t* rowbase;
   const uint32_t *cs_of_sync, *cs_agent, *cs_sid, *cs_epoch, *cs_rel_idx, *cs_lock, *lock_cs_lo, *cs_rel_epoch;
   const uint32_t *acq_dep_off, *acq_dep_cnt, *pool;
@@ -893,38 +893,19 @@ __global__ void __launch_bounds__(MAXT, 1) k_propagate(const __grid_constant__ P
 // ---- plan construction -------------------------------------------------------------
 
 
-// section record as the release loop reads it: (agent | scope id << 16, acquire epoch,
-// release index, release epoch)
-__global__ void k_recmeta(uint32_t n_cs, const uint32_t* cs_agent, const uint32_t* cs_epoch,
-                          const uint32_t* cs_rel_idx, const uint32_t* cs_sid, const uint32_t* cs_rel_epoch,
-                          uint4* recmeta) {
-  const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c < n_cs) recmeta[c] = make_uint4(cs_agent[c] | (cs_sid[c] << 16), cs_epoch[c], cs_rel_idx[c], cs_rel_epoch[c]);
-}
-
-// (both flattening kernels stand down after an error: the per-record lists are then
-// incomplete)
-__global__ void k_flatcount(uint32_t n_incs, const uint32_t* exp_off, const uint32_t* ex_dep_cnt, uint32_t* cnt,
-                            const DevStatus* st) {
-  const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= n_incs) return;
-  if (st->code) {
-    cnt[r] = 0;
-    return;
-  }
+// Per section, its record as the release loop reads it: (agent | scope id << 16, acquire
+// epoch, release index, release epoch). Per in-section access, the number of releases it
+// joins, over the sections that it is held in.
+__global__ void k_plan_counts(PropArgs a, uint32_t n_cs, const uint32_t* cs_epoch, const uint32_t* cs_rel_epoch,
+                              uint32_t n_incs, uint32_t* cnt) {
+  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n_cs) a.recmeta[i] = make_uint4(a.cs_agent[i] | (a.cs_sid[i] << 16), cs_epoch[i], a.cs_rel_idx[i], cs_rel_epoch[i]);
+  if (i >= n_incs) return;
   uint32_t t = 0;
-  for (uint32_t e = exp_off[r]; e < exp_off[r + 1]; ++e) t += ex_dep_cnt[e];
-  cnt[r] = t;
-}
-
-__global__ void k_flatfill(uint32_t n_incs, const uint32_t* exp_off, const uint32_t* ex_dep_off,
-                           const uint32_t* ex_dep_cnt, const uint32_t* pool, const uint32_t* flat_off,
-                           uint32_t* flat, const DevStatus* st) {
-  const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= n_incs || st->code) return;
-  uint32_t o = flat_off[r];
-  for (uint32_t e = exp_off[r]; e < exp_off[r + 1]; ++e)
-    for (uint32_t q = 0; q < ex_dep_cnt[e]; ++q) flat[o++] = pool[ex_dep_off[e] + q];
+  if (!a.st->code)  // (after an error the lists are incomplete)
+    for (uint32_t c = a.cs_of_sync[a.sy_inner[a.incs_k[i]]]; c != NONE; c = a.cs_parent[c])
+      t += a.ex_dep_cnt[a.cs_exp[c] + (i - a.cs_r0[c])];
+  cnt[i] = t;
 }
 
 __global__ void k_plan_sync(PropArgs a, const uint32_t* sy_kind_, const uint32_t* sy_ver, const uint32_t* sy_match,
@@ -964,21 +945,28 @@ __global__ void k_plan_sync(PropArgs a, const uint32_t* sy_kind_, const uint32_t
   a.plan[2 * p + 1] = eb;
 }
 
-__global__ void k_plan_incs(PropArgs a, const uint32_t* incs_k, const uint32_t* incs_ver, const uint32_t* flat_off,
-                            uint32_t n_incs) {
+// the flattened list of an in-section access (its sections from the inside out), its entry
+__global__ void k_plan_incs(PropArgs a, const uint32_t* flat_off, uint32_t* flat, uint32_t n_incs) {
   const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= n_incs) return;
-  const uint32_t k = incs_k[r];
+  if (r >= n_incs || a.st->code) return;
+  const uint32_t k = a.incs_k[r];
   const uint32_t u = a.sy_agent[k];
   const size_t p = size_t(k) + 1 + r;
   const uint32_t off = flat_off[r], cnt = flat_off[r + 1] - off;
-  a.plan[2 * p] = make_uint4(P_INCS, a.rowbase[u] + incs_ver[r], off, cnt);
+  uint32_t o = off;
+  if (cnt)
+    for (uint32_t c = a.cs_of_sync[a.sy_inner[k]]; c != NONE; c = a.cs_parent[c]) {
+      const uint32_t e = a.cs_exp[c] + (r - a.cs_r0[c]);
+      const uint32_t* list = a.pool + a.ex_dep_off[e];
+      for (uint32_t q = 0; q < a.ex_dep_cnt[e]; ++q) flat[o++] = list[q];
+    }
+  a.plan[2 * p] = make_uint4(P_INCS, a.rowbase[u] + a.incs_ver[r], off, cnt);
   uint32_t id[4] = {0, 0, 0, 0}, meta[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   if (cnt <= 4) {
 #pragma unroll
     for (uint32_t q = 0; q < 4; ++q) {
       if (q >= cnt) break;
-      id[q] = a.flat[off + q];
+      id[q] = flat[off + q];
       const uint4 m = a.recmeta[id[q]];
       meta[2 * q] = m.x & 0xFFFF;  // the releasing agent and its local time at the release
       meta[2 * q + 1] = m.w;
@@ -1082,7 +1070,10 @@ int phaseG_propagate(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s
   a.incs_off = b.incs_cnt;
   a.incs_ver = b.incs_ver;
   a.incs_k = b.incs_k;
-  a.exp_off = b.exp_off;
+  a.sy_inner = b.sy_inner;
+  a.cs_parent = b.cs_parent;
+  a.cs_exp = b.cs_exp;
+  a.cs_r0 = b.cs_r0;
   a.ex_dep_off = b.ex_dep_off;
   a.ex_dep_cnt = b.ex_dep_cnt;
   a.rowbase = b.vcount;
@@ -1121,8 +1112,8 @@ int phaseG_propagate(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s
   // plan: per-agent stream of clock-changing steps with their static data resolved
   p.begin("g_plan", double(z.n_sync + z.n_incs) * 64 + double(z.n_cs) * 2 * g.RW * 4);
   if (z.n_cs) {
-    k_recmeta<<<(z.n_cs + 255) / 256, 256, 0, s>>>(z.n_cs, b.cs_agent, b.cs_epoch, b.cs_rel_idx, b.cs_sid,
-                                                    b.cs_rel_epoch, b.recmeta);
+    const uint32_t most = std::max(z.n_cs, z.n_incs);
+    k_plan_counts<<<(most + 255) / 256, 256, 0, s>>>(a, z.n_cs, b.cs_epoch, b.cs_rel_epoch, z.n_incs, b.flat_off);
     count_launch();
     // snapshot rows start as SENTINEL: a reader accepts a row once none is left
     cudaMemsetAsync(b.psnap, 0xFF, size_t(z.n_cs) * g.RW * 4, s);
@@ -1130,13 +1121,8 @@ int phaseG_propagate(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s
     cudaMemsetAsync(b.jsnap, 0xFF, size_t(z.n_cs) * g.RW * 4, s);
   }
   if (z.n_incs) {
-    k_flatcount<<<(z.n_incs + 255) / 256, 256, 0, s>>>(z.n_incs, b.exp_off, b.ex_dep_cnt, b.flat_off, b.st);
-    count_launch();
     scan_exclusive(b.flat_off, b.flat_off, size_t(z.n_incs) + 1, nullptr, b.scan_tmp, s);
-    k_flatfill<<<(z.n_incs + 255) / 256, 256, 0, s>>>(z.n_incs, b.exp_off, b.ex_dep_off, b.ex_dep_cnt, b.dep_pool,
-                                                       b.flat_off, b.flat, b.st);
-    count_launch();
-    k_plan_incs<<<(z.n_incs + 255) / 256, 256, 0, s>>>(a, b.incs_k, b.incs_ver, b.flat_off, z.n_incs);
+    k_plan_incs<<<(z.n_incs + 255) / 256, 256, 0, s>>>(a, b.flat_off, b.flat, z.n_incs);
     count_launch();
   }
   if (z.n_sync) {
