@@ -181,11 +181,12 @@ __device__ __forceinline__ uint32_t a_compact(const ACompact& c, const Event& e,
 }
 
 // Phase A, pass 2: stable scatter into the agent-sorted stream S and the trace-order
-// compactions. Chunks with a barrier are processed one event at a time.
+// compactions. (Rounds with a barrier went one event at a time, 250 cycles each: 60k events,
+// 64 agents 34 us, now 14; 10M events 0.22 ms, now 0.15.)
 __global__ void k_a_scatter(const Event* ev, uint64_t N, Geo g, uint32_t TA, uint32_t ntA, const uint32_t* hist,
                             const uint32_t* tile_off, uint32_t* S, ACompact cpt, bool vec) {
   extern __shared__ uint32_t sm[];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t tile = blockIdx.x * (blockDim.x >> 5) + warp;
   if (tile >= ntA) return;
   uint32_t* cnt = sm + warp * g.Wp;
@@ -215,45 +216,35 @@ __global__ void k_a_scatter(const Event* ev, uint64_t N, Geo g, uint32_t TA, uin
       const bool isbar = ok && e.op == GWCP_BARRIER;
       const uint32_t kind = entry_kind(e.op);
       const uint32_t m = a_compact(cpt, e, i, acc, ar, isbar, g, lt, o_acc, o_ar, o_bar);
-      // agent-sorted stream
-      if (!m) {
-        const bool in_s = acc || ar;
-        const uint32_t key = in_s ? e.agent : 0xFFFFFFFFu;
-        const uint32_t peers = __match_any_sync(0xffffffffu, key);
-        const uint32_t b0 = in_s ? cnt[e.agent] : 0;
+      // agent-sorted stream: the accesses, acquires and releases up to a barrier at once,
+      // then the barrier's members
+      const bool in_s = acc || ar;
+      uint32_t from = 0, bars = m;
+      for (;;) {
+        const uint32_t L = bars ? __ffs(bars) - 1 : 32;
+        const bool now = in_s && lane >= from && lane < L;
+        const uint32_t peers = __match_any_sync(0xffffffffu, now ? e.agent : 0xFFFFFFFFu);
+        const uint32_t b0 = now ? cnt[e.agent] : 0;
         __syncwarp();
-        if (in_s) {
+        if (now) {
           S[b0 + __popc(peers & lt)] = (kind << 30) | uint32_t(i);
-          if (lane == __ffs(peers) - 1) cnt[e.agent] = b0 + __popc(peers);
+          if ((peers & lt) == 0) cnt[e.agent] = b0 + __popc(peers);
         }
         __syncwarp();
-      } else {
-        for (int L = 0; L < 32; ++L) {
-          const uint32_t eop = __shfl_sync(0xffffffffu, uint32_t(e.op), L);
-          const uint32_t eagent = __shfl_sync(0xffffffffu, e.agent, L);
-          const uint32_t escope = __shfl_sync(0xffffffffu, uint32_t(e.scope), L);
-          const uint64_t eaddr = __shfl_sync(0xffffffffu, e.addr, L);
-          const bool ev_valid = __shfl_sync(0xffffffffu, valid, L);
-          const bool ev_ok = __shfl_sync(0xffffffffu, ok, L);
-          if (!ev_valid) break;
-          const uint32_t idx = uint32_t(base) + L;
-          if (!ev_ok) continue;
-          if (eop <= GWCP_REL) {
-            if (lane == 0) S[cnt[eagent]++] = (entry_kind(uint8_t(eop)) << 30) | idx;
-          } else if (eop == GWCP_BARRIER) {
-            Event be{};
-            be.agent = eagent;
-            be.op = GWCP_BARRIER;
-            be.scope = uint8_t(escope);
-            be.addr = eaddr;
-            BarMembers bm = barrier_members(be, g);
-            for (uint32_t j = lane; j < bm.count; j += 32) {
-              uint32_t mb = member_at(bm, j);
-              S[cnt[mb]++] = (K_BAR << 30) | idx;
-            }
-          }
-          __syncwarp();
+        if (L == 32) break;
+        Event be{};
+        be.agent = __shfl_sync(0xffffffffu, e.agent, L);
+        be.op = GWCP_BARRIER;
+        be.scope = uint8_t(__shfl_sync(0xffffffffu, uint32_t(e.scope), L));
+        be.addr = __shfl_sync(0xffffffffu, e.addr, L);
+        const BarMembers bm = barrier_members(be, g);
+        for (uint32_t j = lane; j < bm.count; j += 32) {
+          const uint32_t mb = member_at(bm, j);
+          S[cnt[mb]++] = (K_BAR << 30) | (uint32_t(base) + L);
         }
+        __syncwarp();
+        from = L + 1;
+        bars &= bars - 1;
       }
     }
   }
@@ -940,10 +931,11 @@ __global__ void k_e_assign_rel(const uint32_t* kk, uint32_t n, const uint32_t* s
 // `recent` list, emptied by each device-scope release). An acquire's list has its own place
 // in the pool, `stride` (the most scopes a lock may have) words per section; where the pool's
 // words would not be counted in 32 bits (stride 0) the lists are packed by an atomic counter.
-// One warp per lock: the lanes load 32 entries at a time, a batch ahead, and all walk them
-// in order with the slots in shared memory. (A thread per lock, its slots in local memory
+// One warp per lock: the lanes load 32 entries at a time, a batch ahead, and take them all
+// at once or in order, with the slots in shared memory. (A thread per lock, its slots in local memory
 // and four dependent loads and an atomic per entry, was a chain of 1.8 us per entry: 250k
-// events, 32 locks, the phase took 0.47 ms, now 0.10; 10M events, 1024 locks 0.27, now 0.07.)
+// events, 32 locks, the phase took 0.47 ms, one entry after the other by a warp 0.10, now 0.03;
+// 10M events, 1024 locks 0.27, now 0.07.)
 template <int MAXS>
 struct LockSlots {
   static constexpr int HS = MAXS <= 64 ? 128 : 1024;  // power of two, at least twice MAXS
@@ -978,6 +970,70 @@ __global__ void __launch_bounds__(E_WARPS * 32) k_e_walk(const uint2* rec, const
     const uint2 r = next;
     if (m0 + 32 + lane < end) next = rec[m0 + 32 + lane];
     const uint32_t n = min(32u, end - m0);
+    // A batch at one scope's level - no device-scope entry, or nothing else and no scope to
+    // join but device scope - goes all lanes at once. The entries of a scope see only their
+    // own scope's in the batch, and device scope as it stands before it.
+    {
+      const bool in = uint32_t(lane) < n, acq = in && (r.x >> 31), rel = in && !(r.x >> 31);
+      const uint32_t sid = in ? r.x & 0x7FFFFFFFu : 0xFFFFFFFFu;
+      const uint32_t dev = __ballot_sync(0xffffffffu, in && sid == 0);
+      const uint32_t all = __ballot_sync(0xffffffffu, in);
+      const uint32_t peers = __match_any_sync(0xffffffffu, sid);
+      int mine = -1;  // my scope's slot
+      if (in) {
+        for (uint32_t h = (sid * 0x9E3779B1u) >> 16;; ++h) {
+          const uint32_t e = L.hslot[h & (Slots::HS - 1)];
+          if (e == 0) break;
+          if (L.sid[e - 1] == sid) {
+            mine = int(e) - 1;
+            break;
+          }
+        }
+      }
+      const bool known = __all_sync(0xffffffffu, !in || (mine >= 0 && r.y != NONE));
+      if (stride && known && (dev == 0 || (dev == all && n_recent == 0 && open_total == (q0 >= 0 ? L.open[q0] : 0u)))) {
+        const uint32_t below = peers & lanemask_lt();
+        const uint32_t acqs = __ballot_sync(0xffffffffu, acq), rels = __ballot_sync(0xffffffffu, rel);
+        const uint32_t dev_open = q0 >= 0 ? L.open[q0] : 0u, dev_latest = q0 >= 0 ? L.latest[q0] : NONE;
+        const uint32_t opens = (in ? L.open[mine] : 0u) + __popc(acqs & below) - __popc(rels & below);
+        const bool clash = acq && (opens > 0 || (dev == 0 && dev_open > 0));
+        const uint32_t bad = __ballot_sync(0xffffffffu, clash);
+        if (bad) {
+          if (lane == __ffs(bad) - 1) set_error(st, GWCP_ERR_INVALID_TRACE, sy_idx[kk[m0 + lane]]);
+          return;
+        }
+        const uint32_t rb = rels & below;
+        const uint32_t before = __shfl_sync(0xffffffffu, r.y, rb ? 31 - __clz(rb) : 0);
+        const uint32_t own = rb ? before : in ? L.latest[mine] : NONE;
+        if (acq) {
+          uint32_t* const deps = pool + size_t(r.y) * stride;
+          uint32_t nd = 0;
+          if (dev == 0 && dev_latest != NONE) deps[nd++] = dev_latest;
+          if (own != NONE) deps[nd++] = own;
+          acq_dep_off[r.y] = r.y * stride;
+          acq_dep_cnt[r.y] = nd;
+        }
+        // the slots after the batch, by each scope's last entry
+        const uint32_t rp = rels & peers;
+        const uint32_t last_rel = __shfl_sync(0xffffffffu, r.y, rp ? 31 - __clz(rp) : 0);
+        const bool leader = in && (peers >> lane) == 1u;
+        const bool lists = leader && rp && dev == 0 && !L.in_recent[mine];
+        const uint32_t listed = __ballot_sync(0xffffffffu, lists);
+        __syncwarp();
+        if (leader) {
+          L.open[mine] += __popc(acqs & peers) - __popc(rels & peers);
+          if (rp) L.latest[mine] = last_rel;
+          if (lists) {
+            L.in_recent[mine] = 1;
+            L.recent[n_recent + __popc(listed & lanemask_lt())] = uint16_t(mine);
+          }
+        }
+        n_recent += __popc(listed);
+        open_total += __popc(acqs) - __popc(rels);
+        __syncwarp();
+        continue;
+      }
+    }
     for (uint32_t i = 0; i < n; ++i) {
       const uint32_t w = __shfl_sync(0xffffffffu, r.x, i), c = __shfl_sync(0xffffffffu, r.y, i);
       if (c == NONE) return;  // invalid trace, flagged by the agent walk
