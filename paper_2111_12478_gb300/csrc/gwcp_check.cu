@@ -1,7 +1,7 @@
 // Access grouping and the per-location race check of libgwcp.
 //
 // Accesses are sorted by (location key, trace index) with the library's radix sort,
-// then cut into fixed chunks of CH entries; one warp checks one chunk in order. The
+// then cut into chunks of a fixed length; one warp checks one chunk in order. The
 // warp keeps, for every agent v (lane l owns agents [l*K, l*K+K)) and access class
 // (read, write, block-scoped atomic, device-scoped atomic), the latest access by v to
 // the current location as (index << 32 | epoch) - the R_x / W_x state of the paper's
@@ -17,7 +17,6 @@ namespace gwcp {
 
 namespace {
 
-constexpr uint32_t CH = 512;       // accesses per chunk (one warp)
 constexpr uint32_t GRP = 32;       // chunks per first-level scan group
 constexpr int CHK_WARPS = 4;
 
@@ -27,6 +26,7 @@ struct ChunkArgs {
   const AccInfo* info;
   uint32_t n;
   uint32_t n_chunks;
+  uint32_t ch;          // accesses per chunk (one warp)
   uint64_t* T;          // [n_chunks][4 * Wp] packed (index << 32 | epoch), 0 = none
   const uint32_t* rows;
   uint64_t* races;
@@ -40,7 +40,7 @@ struct ChunkArgs {
 __device__ __forceinline__ bool chunk_continues(const ChunkArgs& a, uint32_t c) {
   // the last location of chunk c goes on into chunk c + 1
   if (c + 1 >= a.n_chunks) return false;
-  const uint32_t e = (c + 1) * CH;
+  const uint32_t e = (c + 1) * a.ch;
   return a.key[e - 1] == a.key[e];
 }
 
@@ -66,7 +66,7 @@ __global__ void k_tail(ChunkArgs a) {
 #pragma unroll
     for (int j = 0; j < K; ++j) last[q][j] = 0;
   if (chunk_continues(a, c)) {
-    const uint32_t lo = c * CH, hi = min(lo + CH, a.n);
+    const uint32_t lo = c * a.ch, hi = min(lo + a.ch, a.n);
     const uint64_t tk = a.key[hi - 1];
     for (uint32_t b0 = lo; b0 < hi; b0 += 32) {
       const uint32_t p = b0 + lane;
@@ -99,26 +99,38 @@ __global__ void k_tail(ChunkArgs a) {
 // continues into c and chunk c holds only that location
 __device__ __forceinline__ bool linked(const ChunkArgs& a, uint32_t c) {
   if (c == 0 || !chunk_continues(a, c - 1)) return false;
-  const uint32_t lo = c * CH, hi = min(lo + CH, a.n);
+  const uint32_t lo = c * a.ch, hi = min(lo + a.ch, a.n);
   return a.key[lo] == a.key[hi - 1];
+}
+
+// the links of a group's chunks, a bit each (a chunk's keys are loaded once, not per column)
+__device__ __forceinline__ uint32_t group_links(const ChunkArgs& a, uint32_t g0, uint32_t g1) {
+  const uint32_t c = g0 + (threadIdx.x & 31);
+  return __ballot_sync(0xffffffffu, c < g1 && linked(a, c));
 }
 
 __global__ void k_scan1(ChunkArgs a, uint64_t* gagg, uint32_t* gfull) {
   const uint32_t cols = 4 * a.g.Wp;
   const uint32_t g0 = blockIdx.x * GRP, g1 = min(g0 + GRP, a.n_chunks);
-  const bool first_linked = linked(a, g0);
-  bool full = first_linked;
-  for (uint32_t c = g0 + 1; c < g1; ++c) full = full && linked(a, c);
+  const uint32_t links = group_links(a, g0, g1);
+  const bool full = links == (g1 - g0 == 32 ? 0xffffffffu : (1u << (g1 - g0)) - 1);
   for (uint32_t col = threadIdx.x; col < cols; col += blockDim.x) {
     uint64_t acc = 0;
-    for (uint32_t c = g0; c < g1; ++c) {
-      uint64_t v = a.T[size_t(c) * cols + col];
-      acc = (c > g0 && linked(a, c)) ? max(acc, v) : v;
-      a.T[size_t(c) * cols + col] = acc;
+    for (uint32_t c0 = g0; c0 < g1; c0 += 8) {
+      uint64_t v[8];
+#pragma unroll
+      for (uint32_t q = 0; q < 8; ++q) v[q] = c0 + q < g1 ? a.T[size_t(c0 + q) * cols + col] : 0;
+#pragma unroll
+      for (uint32_t q = 0; q < 8; ++q) {
+        const uint32_t c = c0 + q;
+        if (c >= g1) break;
+        acc = (c > g0 && ((links >> (c - g0)) & 1)) ? max(acc, v[q]) : v[q];
+        a.T[size_t(c) * cols + col] = acc;
+      }
     }
     gagg[size_t(blockIdx.x) * cols + col] = acc;
   }
-  if (threadIdx.x == 0) gfull[blockIdx.x] = uint32_t(full) | (uint32_t(first_linked) << 1);
+  if (threadIdx.x == 0) gfull[blockIdx.x] = uint32_t(full) | ((links & 1) << 1);
 }
 
 __global__ void k_scan2(ChunkArgs a, uint32_t ngroups, uint64_t* gagg, const uint32_t* gfull) {
@@ -150,10 +162,13 @@ __global__ void k_scan2(ChunkArgs a, uint32_t ngroups, uint64_t* gagg, const uin
 __global__ void k_scan3(ChunkArgs a, const uint64_t* gagg) {
   const uint32_t cols = 4 * a.g.Wp;
   const uint32_t g0 = blockIdx.x * GRP, g1 = min(g0 + GRP, a.n_chunks);
+  const uint32_t links = group_links(a, g0, g1);
+  const uint32_t n = min(g1 - g0, links == 0xffffffffu ? 32u : uint32_t(__ffs(~links)) - 1);  // chunks the carry reaches
   for (uint32_t col = threadIdx.x; col < cols; col += blockDim.x) {
     const uint64_t carry = gagg[size_t(blockIdx.x) * cols + col];
     if (!carry) continue;
-    for (uint32_t c = g0; c < g1 && linked(a, c); ++c) {
+#pragma unroll 8
+    for (uint32_t c = g0; c < g0 + n; ++c) {
       uint64_t& v = a.T[size_t(c) * cols + col];
       v = max(v, carry);
     }
@@ -179,7 +194,7 @@ __global__ void __launch_bounds__(CHK_WARPS * 32) k_check(ChunkArgs a) {
   if (c >= a.n_chunks) return;
   const Geo& g = a.g;
   const uint32_t Wp = g.Wp;
-  const uint32_t lo = c * CH, hi = min(lo + CH, a.n);
+  const uint32_t lo = c * a.ch, hi = min(lo + a.ch, a.n);
   const uint32_t lt = lanemask_lt();
   uint64_t last[4][K];
   if (c > 0 && chunk_continues(a, c - 1)) {
@@ -322,8 +337,8 @@ void run_check(const ChunkArgs& a, cudaStream_t s, Prof& p, double bytes_per) {
 
 }  // namespace
 
-size_t check_chunks(uint32_t n_acc) { return (n_acc + CH - 1) / CH; }
-size_t check_group_count(uint32_t n_acc) { return (check_chunks(n_acc) + GRP - 1) / GRP; }
+size_t check_chunks(uint32_t n_acc, uint32_t ch) { return (size_t(n_acc) + ch - 1) / ch; }
+size_t check_group_count(uint32_t n_acc, uint32_t ch) { return (check_chunks(n_acc, ch) + GRP - 1) / GRP; }
 
 void phaseH_sort(Bufs& b, const Geo& g, const Sizes& z, uint64_t key_mask, uint32_t* tmp, cudaStream_t s, Prof& p) {
   (void)g;
@@ -349,6 +364,7 @@ static ChunkArgs chunk_args(const Bufs& b, const Geo& g, const Sizes& z) {
   a.info = b.acc_info;
   a.n = z.n_acc;
   a.n_chunks = z.n_chunks;
+  a.ch = z.check_ch;
   a.T = reinterpret_cast<uint64_t*>(b.tails);
   a.rows = b.rows;
   a.races = b.races;
@@ -364,7 +380,7 @@ void phaseI_carry(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, P
   if (!z.n_acc) return;
   const ChunkArgs a = chunk_args(b, g, z);
   uint64_t* gagg = a.T + size_t(z.n_chunks) * 4 * g.Wp;
-  uint32_t* gfull = reinterpret_cast<uint32_t*>(gagg + size_t(check_group_count(z.n_acc)) * 4 * g.Wp);
+  uint32_t* gfull = reinterpret_cast<uint32_t*>(gagg + check_group_count(z.n_acc, z.check_ch) * 4 * g.Wp);
   switch (g.K) {
     case 1: run_carry<1>(a, gagg, gfull, s, p); break;
     case 2: run_carry<2>(a, gagg, gfull, s, p); break;

