@@ -14,8 +14,8 @@
 
 namespace gwcp {
 unsigned long long launch_count();
-size_t check_chunks(uint32_t n_acc);
-size_t check_group_count(uint32_t n_acc);
+size_t check_chunks(uint32_t n_acc, uint32_t ch);
+size_t check_group_count(uint32_t n_acc, uint32_t ch);
 void phaseE_scan(const Bufs& b, const Sizes& z, cudaStream_t s, Prof& p);
 
 cudaEvent_t Prof::ev() {
@@ -539,8 +539,8 @@ int run(gwcp_ctx* c, cudaStream_t s) {
     b.wc_row = get<uint32_t>(c, "wc_row", na, &oom);
     b.wc_ep = get<uint32_t>(c, "wc_ep", na, &oom);
   } else {
-    z.n_chunks = uint32_t(check_chunks(z.n_acc));
-    const size_t ng = check_group_count(z.n_acc);
+    z.n_chunks = uint32_t(check_chunks(z.n_acc, z.check_ch));
+    const size_t ng = check_group_count(z.n_acc, z.check_ch);
     b.tails = get<uint32_t>(c, "tails", (size_t(z.n_chunks) + ng) * 4 * g.Wp * 2 + ng + 8, &oom);
   }
   if (oom) return GWCP_ERR_OOM;
@@ -625,7 +625,7 @@ int run(gwcp_ctx* c, cudaStream_t s) {
   else
     phaseI_carry(b, g, z, c->side, c->prof);
   if (z.grouped) {  // in the access sort's other buffer; an access that finds no room is walked by its own thread
-    z.big_cap = std::min(z.n_acc, z.n_acc / 8 + 65536);
+    z.big_cap = z.n_acc;
     b.wc_big = b.acc_key2;
   }
   int prc = phaseG_propagate(b, g, z, s, c->prof);

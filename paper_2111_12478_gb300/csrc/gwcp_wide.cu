@@ -762,6 +762,7 @@ struct WideCheckArgs {
   uint32_t* chunk_races;         // and the races it found
   uint2* big;         // (position, piece | pieces << 16) items of k_wc_big
   uint32_t big_cap;   // items it holds
+  uint32_t big_groups;  // most groups that a lane walks itself
 };
 
 // position j in group gi of the latest member with gs[j] < x (gs ascends within a group:
@@ -946,10 +947,21 @@ __device__ __noinline__ uint32_t check_part(const WideCheckArgs& a, uint32_t p, 
   return check_merge<REP>(a, c, cur, end, s_cnt, s_buf);
 }
 
-// A lane walks its access's groups itself up to kBigGroups: below, lanes with similar lists
-// are better off each on its own (64 warps, 10M events: the reads of hot locations have ~60
-// groups each; cut by agent, every one of them would pay the searches that place its parts).
-constexpr uint32_t kBigGroups = 192;
+// A lane walks its access's groups itself up to a limit (big_groups): below, lanes with
+// similar lists are better off each on its own (the reads of a hot location, whose group
+// count grows with the trace: cut by agent, every one of them would pay the searches that
+// place its parts). In a short trace the longest walk is the check's time, so the limit is
+// low there. The check (ms), by limit:
+//   accesses, agents    48      64      96      192
+//   200k, 256           0.045   0.045   0.061   0.111
+//   1M, 64              0.05    0.11    0.19    0.20
+//   1M, 64, ranked      0.047   0.074   0.172   0.172   (the lanes of the access's own warp)
+//   2M, 128             0.092   0.104   0.123   0.471
+//   2.3M, 512           0.424   0.141   0.154   0.217
+//   5M, 256             1.145   0.850   0.274   0.344
+//   10M, 64             2.156   0.467   0.528   0.555
+//   5M, 512 threads     0.331   0.316   0.306   0.231
+inline uint32_t big_groups(uint32_t n) { return n <= (1u << 21) ? 48 : 96; }
 constexpr uint32_t kPieceGroups = 128;  // groups per item of k_wc_big: four per lane
 
 // appends the warp's staged races (one global atomic) and its test count; returns the races found
@@ -997,7 +1009,7 @@ __global__ void __launch_bounds__(kCheckThreads, 8) k_wc_check(const __grid_cons
     uint32_t groups = 0;
 #pragma unroll
     for (uint32_t q = 0; q < 4; ++q) groups += end[q] - cur[q];
-    big = groups > kBigGroups;
+    big = groups > a.big_groups;
     if constexpr (ASIDE) {
       if (big) {
         const uint32_t pieces = (groups + kPieceGroups - 1) / kPieceGroups;
@@ -1280,6 +1292,7 @@ void phaseI_wide_check(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t
   a.row_words = z.compress ? g.B : g.RW;
   a.chunk_ns = b.chunk_ns;
   a.chunk_races = b.chunk_races;
+  a.big_groups = big_groups(n);
   a.big = reinterpret_cast<uint2*>(b.wc_big);
   a.big_cap = z.grouped ? z.big_cap : 0;
   p.begin("i_check", double(n) * (4 + 16 + 4 + 4 + 4 + 8));
@@ -1292,7 +1305,7 @@ void phaseI_wide_check(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t
             : rep == REP_DENSE ? k_wc_check<REP_DENSE, false> : k_wc_check<REP_COMPRESSED, false>;
   check<<<nblk(n, kCheckThreads), kCheckThreads, 0, s>>>(a);
   count_launch();
-  if (z.grouped && 4 * g.W > kBigGroups) {  // fewer agents have no such access
+  if (z.grouped && 4 * g.W > a.big_groups) {  // fewer agents have no such access
     auto big = rep == REP_TILES ? k_wc_big<REP_TILES>
                : rep == REP_DENSE ? k_wc_big<REP_DENSE> : k_wc_big<REP_COMPRESSED>;
     big<<<std::min<uint32_t>(nblk(n, 32), 152 * 6), kCheckThreads, 0, s>>>(a);
