@@ -217,9 +217,10 @@ cudaError_t wait_stream(gwcp_ctx* c, cudaStream_t s) {
 }
 
 int read_status(gwcp_ctx* c, cudaStream_t s, const uint32_t* const* extra, int n_extra) {
-  cudaMemcpyAsync(c->st_host, c->b.st, sizeof(DevStatus), cudaMemcpyDeviceToHost, s);
-  for (int i = 0; i < n_extra; ++i)
-    cudaMemcpyAsync(c->cnt_host + i, extra[i], sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
+  // one kernel that writes the pinned words (a copy each took 2 to 3 us, 12 of them per pass)
+  ReadBack r{};
+  for (r.n = 0; r.n < n_extra; ++r.n) r.word[r.n] = extra[r.n];
+  read_back_to(c->b.st, r, c->st_host, c->cnt_host, s);
   if (wait_stream(c, s) != cudaSuccess) return GWCP_ERR_CUDA;
   return cuda_rc();
 }
@@ -277,7 +278,8 @@ int run(gwcp_ctx* c, cudaStream_t s) {
   init.bad_index = ~0ull;
   init.key_and = ~0ull;
   init.lock_and = ~0ull;
-  cudaMemcpyAsync(b.st, &init, sizeof(init), cudaMemcpyHostToDevice, s);
+  if (g.nT) init.spare[2] = 1;  // the tile pool's counter
+  status_init(b.st, init, s);
   c->prof.on = c->opt.profile != 0;
   c->prof.s = s;
   c->prof.recs.clear();
@@ -348,8 +350,8 @@ int run(gwcp_ctx* c, cudaStream_t s) {
   b.sy_depth = get<uint32_t>(c, "sy_depth", ns1, &oom);
   b.sy_inner = get<uint32_t>(c, "sy_inner", ns1, &oom);
   b.sy_ver = get<uint32_t>(c, "sy_ver", ns1, &oom);
-  b.sy_match = get<uint32_t>(c, "sy_match", ns1, &oom);
-  b.sy_relk = get<uint32_t>(c, "sy_relk", ns1, &oom);
+  b.sy_match = get<uint32_t>(c, "sy_match", 2 * ns1, &oom);  // with sy_relk; both are phase D's packed entries later
+  b.sy_relk = b.sy_match + ns1;
   b.sy_agent = get<uint32_t>(c, "sy_agent", ns1, &oom);
   b.incs_cnt = get<uint32_t>(c, "incs_cnt", ns1, &oom);
   b.vcount = get<uint32_t>(c, "vcount", g.W + 1, &oom);
@@ -409,8 +411,6 @@ int run(gwcp_ctx* c, cudaStream_t s) {
     cudaEventRecord(c->kept_ev, c->side);
   }
   phaseB_sync(b, g, z, s, c->prof);
-  cudaMemsetAsync(b.vcount, 0, size_t(g.W + 1) * 4, s);
-  cudaMemsetAsync(b.cs_of_sync, 0xFF, ns1 * 4, s);
   phaseC_walk(b, g, z, s, c->prof);
   // forced compression at barriers renumbers the local times; barriers are validated in
   // phase A, so an invalid trace skips it
@@ -419,7 +419,7 @@ int run(gwcp_ctx* c, cudaStream_t s) {
   phaseE_scan(b, z, s, c->prof);
   {
     const uint32_t* ex[5] = {b.incs_cnt + z.n_sync, b.vcount + g.W, b.lk_csid + z.n_acqrel,
-                             b.lk_flags + z.n_acqrel, reinterpret_cast<const uint32_t*>(&b.st->spare[1])};
+                             b.lk_k2 + z.n_acqrel, reinterpret_cast<const uint32_t*>(&b.st->spare[1])};
     int rc = read_status(c, s, ex, 5);
     if (rc) return rc;
   }
@@ -495,9 +495,9 @@ int run(gwcp_ctx* c, cudaStream_t s) {
   };
   const size_t plan_bytes = (2 * (size_t(z.n_sync) + z.n_incs) + 2) * sizeof(uint4);
   const size_t snap_bytes = (size_t(z.n_cs) + 1) * g.RW * sizeof(uint32_t);
-  b.plan = static_cast<uint4*>(late("plan", plan_bytes));
-  b.plan2 = static_cast<uint4*>(late("plan2", plan_bytes));
   b.jsnap = static_cast<uint32_t*>(late("jsnap", snap_bytes));
+  b.plan2 = static_cast<uint4*>(late("plan2", plan_bytes));
+  b.plan = static_cast<uint4*>(late("plan", plan_bytes));
   b.psnap = static_cast<uint32_t*>(late("psnap", snap_bytes));
   b.hsnap = get<uint32_t>(c, "hsnap", (size_t(z.n_cs) + 1) * g.RW, &oom);
   if (g.nT) {
@@ -544,17 +544,6 @@ int run(gwcp_ctx* c, cudaStream_t s) {
     b.tails = get<uint32_t>(c, "tails", (size_t(z.n_chunks) + ng) * 4 * g.Wp * 2 + ng + 8, &oom);
   }
   if (oom) return GWCP_ERR_OOM;
-  if (g.nT) {  // tile 0 is the zero tile; ids are handed out from 1
-    cudaMemsetAsync(b.tiles, 0, kTileW * 4, s);
-    const unsigned long long one = 1;
-    cudaMemcpyAsync(&b.st->spare[2], &one, sizeof(one), cudaMemcpyHostToDevice, s);
-  }
-  cudaMemsetAsync(b.cursor, 0, size_t(g.W) * (z.n_locks + 1) * 4, s);
-  if (global_bars && z.n_bar) {
-    cudaMemsetAsync(b.bar_j, 0, size_t(z.n_bar) * 2 * g.Wp * 4, s);
-    cudaMemsetAsync(b.bar_jj, 0, size_t(z.n_bar) * g.Wp * 4, s);
-    cudaMemsetAsync(b.bar_cnt, 0, size_t(z.n_bar) * 4, s);
-  }
 
   phaseD_gaps(b, g, z, s, c->prof);
   c->acc_info_partial = z.wl_log2 != 0;

@@ -251,6 +251,29 @@ struct ScanBatch {
   ScanJob job[kScanJobs];
 };
 bool scan_is_small(size_t n);
+// Several buffers filled in one launch (256-byte aligned, whole words).
+struct FillJob {
+  void* ptr;
+  size_t words;
+  uint32_t value;
+};
+constexpr int kFillJobs = 8;
+struct FillBatch {
+  FillJob job[kFillJobs];
+  int n = 0;
+  void add(void* ptr, size_t words, uint32_t value) {
+    if (words) job[n++] = FillJob{ptr, words, value};
+  }
+};
+void fill_all(const FillBatch& b, cudaStream_t s);
+// The status and up to eight device words to st_out and val_out (either device memory or
+// pinned host memory) in one launch; the status's first value, likewise.
+struct ReadBack {
+  const uint32_t* word[8];
+  int n;
+};
+void read_back_to(const DevStatus* st, const ReadBack& r, DevStatus* st_out, uint32_t* val_out, cudaStream_t s);
+void status_init(DevStatus* st, const DevStatus& v, cudaStream_t s);
 void scan_small(const ScanBatch& b, int jobs, cudaStream_t s);
 void scan_exclusive(const uint32_t* in, uint32_t* out, size_t n, uint32_t* total_dev, uint32_t* tmp,
                     cudaStream_t s);

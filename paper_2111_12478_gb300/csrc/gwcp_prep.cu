@@ -184,13 +184,17 @@ __device__ __forceinline__ uint32_t a_compact(const ACompact& c, const Event& e,
 // compactions. (Rounds with a barrier went one event at a time, 250 cycles each: 60k events,
 // 64 agents 34 us, now 14; 10M events 0.22 ms, now 0.15.)
 __global__ void k_a_scatter(const Event* ev, uint64_t N, Geo g, uint32_t TA, uint32_t ntA, const uint32_t* hist,
-                            const uint32_t* tile_off, uint32_t* S, ACompact cpt, bool vec) {
+                            const uint32_t* tile_off, uint32_t* S, uint32_t nS, uint32_t* seg, ACompact cpt, bool vec) {
   extern __shared__ uint32_t sm[];
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t tile = blockIdx.x * (blockDim.x >> 5) + warp;
   if (tile >= ntA) return;
   uint32_t* cnt = sm + warp * g.Wp;
   for (uint32_t u = lane; u < g.W; u += 32) cnt[u] = hist[size_t(u) * ntA + tile];
+  if (tile == 0) {  // the agents' segments of S
+    for (uint32_t u = lane; u < g.W; u += 32) seg[u] = cnt[u];
+    if (lane == 0) seg[g.W] = nS;
+  }
   __syncwarp();
   uint32_t o_acc = tile_off[tile], o_ar = tile_off[ntA + 1 + tile], o_bar = tile_off[2 * (ntA + 1) + tile];
   const uint32_t lt = lanemask_lt();
@@ -390,12 +394,6 @@ __global__ void k_aw_seg(const uint64_t* key, uint32_t n, uint32_t W, uint32_t* 
   seg[u] = lo;
 }
 
-__global__ void k_a_segments(const uint32_t* hist, uint32_t W, uint32_t ntA, uint32_t nS, uint32_t* seg) {
-  uint32_t u = blockIdx.x * blockDim.x + threadIdx.x;
-  if (u < W) seg[u] = hist[size_t(u) * ntA];
-  if (u == W) seg[W] = nS;
-}
-
 template <typename T>
 __device__ __forceinline__ uint32_t lower_bound_dev(const T* a, uint32_t n, T x) {
   uint32_t lo = 0, hi = n;
@@ -428,10 +426,8 @@ __global__ void k_b_count(const uint32_t* S, uint32_t nS, uint32_t n_chunks, uin
   if (lane == 0) cnt[chunk] = c;
 }
 
-__global__ void k_b_scatter(const Event* ev, const uint32_t* S, uint32_t nS, uint32_t n_chunks, const uint32_t* off,
-                            const uint32_t* bar, uint32_t n_bar, const uint32_t* acqrel, uint32_t n_acqrel,
-                            uint32_t* sy_spos, uint32_t* sy_idx, uint32_t* sy_kind, uint32_t* sy_aux,
-                            uint64_t* lk_key, uint32_t* lk_k) {
+__global__ void k_b_scatter(const uint32_t* S, uint32_t nS, uint32_t n_chunks, const uint32_t* off, uint32_t* sy_spos,
+                            uint32_t* sy_idx, uint32_t* sy_kind, uint32_t* sy_relk, uint32_t* cs_of_sync) {
   const uint32_t chunk = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (chunk >= n_chunks) return;
   const uint32_t base = chunk * B_CHUNK;
@@ -451,25 +447,36 @@ __global__ void k_b_scatter(const Event* ev, const uint32_t* S, uint32_t nS, uin
     const uint32_t m = __ballot_sync(0xffffffffu, sy);
     if (sy) {
       const uint32_t k = run + __popc(m & lt);
-      const uint32_t idx = s_idx(s), kind = s_kind(s);
       sy_spos[k] = p;
-      sy_idx[k] = idx;
-      sy_kind[k] = kind;
-      sy_aux[k] = kind == K_BAR ? lower_bound_dev(bar, n_bar, idx) : NONE;
-      if (kind != K_BAR) {
-        uint32_t q = lower_bound_dev(acqrel, n_acqrel, idx);
-        lk_key[q] = ev[idx].addr;
-        lk_k[q] = k;
-      }
+      sy_idx[k] = s_idx(s);
+      sy_kind[k] = s_kind(s);
+      sy_relk[k] = NONE;  // (set by the agent walk and the lock phases)
+      cs_of_sync[k] = NONE;
     }
     run += __popc(m);
   }
 }
 
-__global__ void k_b_starts(const uint32_t* seg, uint32_t W, const uint32_t* sy_spos, uint32_t n_sync,
-                           uint32_t* sy_start) {
-  uint32_t u = blockIdx.x * blockDim.x + threadIdx.x;
-  if (u <= W) sy_start[u] = lower_bound_dev(sy_spos, n_sync, seg[u]);
+// The searches of phase B: an agent's first entry, a barrier's position among the barriers,
+// an acquire's or release's among its kind. A thread per entry: inside the compaction, where
+// a warp's few entries searched round after round, they took 15 of its 19 us at 60k events
+// over 64 agents and 23 of 31 at 1M.
+__global__ void k_b_search(const Event* ev, const uint32_t* seg, uint32_t W, const uint32_t* sy_spos, uint32_t n_sync,
+                           uint32_t* sy_start, const uint32_t* sy_idx, const uint32_t* sy_kind, const uint32_t* bar,
+                           uint32_t n_bar, const uint32_t* acqrel, uint32_t n_acqrel, uint32_t* sy_aux,
+                           uint64_t* lk_key, uint32_t* lk_k) {
+  const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k <= W) sy_start[k] = lower_bound_dev(sy_spos, n_sync, seg[k]);
+  if (k >= n_sync) return;
+  const uint32_t idx = sy_idx[k];
+  if (sy_kind[k] == K_BAR) {
+    sy_aux[k] = lower_bound_dev(bar, n_bar, idx);
+  } else {
+    sy_aux[k] = NONE;
+    const uint32_t q = lower_bound_dev(acqrel, n_acqrel, idx);
+    lk_key[q] = ev[idx].addr;
+    lk_k[q] = k;
+  }
 }
 
 // Phase C: one warp per agent over its synchronisation entries.
@@ -613,11 +620,25 @@ __global__ void k_c_walk(const Event* ev, Geo g, const uint32_t* seg, const uint
 // Phase D's index: table[u * nw + w] is agent u's first synchronisation entry at or after
 // trace position w << shift (sy_start[u + 1] when there is none), so an access at i
 // searches only the entries of its own window, [table[w], table[w + 1]). One thread per
-// entry fills the windows from after its predecessor's window up to its own.
+// entry fills the windows from after its predecessor's window up to its own, and packs what
+// an access after the entry needs, (N, version | in a section), into one load. (Three loads from
+// three arrays per kept access: 50M events over 8192 agents, the phase 1.10 ms, now 0.87.)
+// The blocks from tail_from on fill the windows after an agent's last entry (all of them when
+// it has none), a warp per agent.
 __global__ void k_d_index(const uint32_t* sy_idx, const uint32_t* sy_agent, const uint32_t* sy_start, uint32_t n_sync,
-                          uint32_t shift, uint32_t nw, uint32_t* table) {
+                          uint32_t W, uint32_t shift, uint32_t nw, uint32_t* table, uint32_t tail_from,
+                          const uint32_t* sy_N, const uint32_t* sy_depth, const uint32_t* sy_ver, uint2* sy_pack) {
+  if (blockIdx.x >= tail_from) {
+    const uint32_t u = ((blockIdx.x - tail_from) * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (u >= W) return;
+    const uint32_t k0 = sy_start[u], k1 = sy_start[u + 1];
+    uint32_t* row = table + size_t(u) * nw;
+    for (uint32_t w = (k1 > k0 ? (sy_idx[k1 - 1] >> shift) + 1 : 0) + lane; w < nw; w += 32) row[w] = k1;
+    return;
+  }
   const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n_sync) return;
+  sy_pack[k] = make_uint2(sy_N[k], sy_ver[k] | (sy_depth[k] ? 0x80000000u : 0u));
   const uint32_t u = sy_agent[k];
   const uint32_t wk = sy_idx[k] >> shift;
   const uint32_t w0 = k > sy_start[u] ? (sy_idx[k - 1] >> shift) + 1 : 0;
@@ -625,20 +646,9 @@ __global__ void k_d_index(const uint32_t* sy_idx, const uint32_t* sy_agent, cons
   for (uint32_t w = w0; w <= wk; ++w) row[w] = k;
 }
 
-// the windows after an agent's last entry (all of them when it has none): a warp per agent
-__global__ void k_d_index_tail(const uint32_t* sy_idx, const uint32_t* sy_start, uint32_t W, uint32_t shift,
-                               uint32_t nw, uint32_t* table) {
-  const uint32_t u = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (u >= W) return;
-  const uint32_t k0 = sy_start[u], k1 = sy_start[u + 1];
-  const uint32_t w0 = k1 > k0 ? (sy_idx[k1 - 1] >> shift) + 1 : 0;
-  uint32_t* row = table + size_t(u) * nw;
-  for (uint32_t w = w0 + lane; w < nw; w += 32) row[w] = k1;
-}
-
 __global__ void k_d_trace(const Event* ev, uint64_t N, Geo g, const uint32_t* sy_start, const uint32_t* sy_idx,
-                          const uint32_t* table, uint32_t shift, uint32_t nw, const uint32_t* sy_N,
-                          const uint32_t* sy_depth, const uint32_t* sy_ver, const uint32_t* rowbase, AccInfo* acc_info,
+                          const uint32_t* table, uint32_t shift, uint32_t nw, const uint2* sy_pack,
+                          const uint32_t* rowbase, AccInfo* acc_info,
                           const DevStatus* st, bool vec, const uint32_t* wl_bits, uint32_t wl_log2,
                           uint32_t comp_lo, uint32_t comp_span) {
   const uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -665,24 +675,27 @@ __global__ void k_d_trace(const Event* ev, uint64_t N, Geo g, const uint32_t* sy
   }
   uint32_t epoch = 1, ver = 0;
   if (a > k0) {
-    const uint32_t k = a - 1;
-    if (sy_depth[k] > 0) return;  // in a critical section: the gap walk below
-    epoch = sy_N[k];
-    ver = sy_ver[k];
+    const uint2 e = sy_pack[a - 1];
+    if (e.y >> 31) return;  // in a critical section: the gap walk below
+    epoch = e.x;
+    ver = e.y;
   }
   acc_info[i] = AccInfo{epoch, rowbase[u] + ver, make_who(u, access_class(e), u / g.apb), 0};
 }
 
-// Phase D, accesses inside critical sections: one warp per gap after a synchronisation
-// entry at nesting depth > 0 (each access there has a clock version of its own).
+// Phase D, accesses inside critical sections: eight lanes per gap after a synchronisation
+// entry at nesting depth > 0 (each access there has a clock version of its own; most gaps
+// have a few accesses, and most entries are not in a section: with a warp per entry, 1.5M
+// entries took 0.22 ms, a quarter of the phase).
+constexpr uint32_t D_LANES = 8;
 __global__ void k_d_fill(const Event* ev, Geo g, uint32_t n_sync, const uint32_t* S, const uint32_t* seg,
                          const uint32_t* sy_start, const uint32_t* sy_agent, const uint32_t* sy_spos,
                          const uint32_t* sy_N,
                          const uint32_t* sy_depth, const uint32_t* sy_ver, const uint32_t* incs_off,
                          const uint32_t* rowbase, AccInfo* acc_info, uint32_t* incs_idx, uint32_t* incs_ver,
                          uint32_t* incs_k, uint64_t* incs_key, uint32_t* incs_wr, const DevStatus* st) {
-  const int lane = threadIdx.x & 31;
-  const uint64_t gid = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+  const uint32_t lane = threadIdx.x & (D_LANES - 1);
+  const uint64_t gid = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) / D_LANES;
   if (gid >= n_sync || st->code) return;
   const uint32_t k = uint32_t(gid);
   if (sy_depth[k] == 0) return;
@@ -691,7 +704,7 @@ __global__ void k_d_fill(const Event* ev, Geo g, uint32_t n_sync, const uint32_t
   const uint32_t hi = (k + 1 < sy_start[u + 1]) ? sy_spos[k + 1] : seg[u + 1];
   const uint32_t epoch = sy_N[k], vbase = sy_ver[k];
   const uint32_t rb = rowbase[u];
-  for (uint32_t p = lo + lane; p < hi; p += 32) {
+  for (uint32_t p = lo + lane; p < hi; p += D_LANES) {
     const uint32_t j = p - lo + 1;
     const uint32_t idx = s_idx(S[p]);
     const Event e = ev[idx];
@@ -1331,9 +1344,7 @@ void phaseA_scatter(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s,
   }
   const uint32_t aw = a_warps(g);
   k_a_scatter<<<blocks(z.ntA, aw), aw * 32, aw * g.Wp * 4, s>>>(b.ev, z.N, g, z.TA, z.ntA, b.hist_a, b.tile_cnt,
-                                                                b.S, cpt, vec);
-  count_launch();
-  k_a_segments<<<blocks(g.W + 1, 256), 256, 0, s>>>(b.hist_a, g.W, z.ntA, z.nS, b.seg);
+                                                                b.S, z.nS, b.seg, cpt, vec);
   count_launch();
   p.end();
 }
@@ -1346,19 +1357,18 @@ void phaseB_sync(const Bufs& b, const Geo& g, Sizes& z, cudaStream_t s, Prof& p)
     count_launch();
     scan_exclusive(b.sy_cnt, b.sy_cnt, z.ntS, b.sy_cnt + z.ntS, b.scan_tmp, s);
     k_b_scatter<<<blocks(uint64_t(z.ntS) * 32, B_THREADS), B_THREADS, 0, s>>>(
-        b.ev, b.S, z.nS, z.ntS, b.sy_cnt, b.bar, z.n_bar, b.acqrel, z.n_acqrel, b.sy_spos, b.sy_idx, b.sy_kind,
-        b.sy_aux, b.lk_key, b.lk_k);
+        b.S, z.nS, z.ntS, b.sy_cnt, b.sy_spos, b.sy_idx, b.sy_kind, b.sy_relk, b.cs_of_sync);
     count_launch();
   }
-  k_b_starts<<<blocks(g.W + 1, 256), 256, 0, s>>>(b.seg, g.W, b.sy_spos, z.n_sync, b.sy_start);
+  k_b_search<<<blocks(std::max(g.W + 1, z.n_sync), 256), 256, 0, s>>>(b.ev, b.seg, g.W, b.sy_spos, z.n_sync, b.sy_start,
+                                                                      b.sy_idx, b.sy_kind, b.bar, z.n_bar, b.acqrel,
+                                                                      z.n_acqrel, b.sy_aux, b.lk_key, b.lk_k);
   count_launch();
   p.end();
 }
 
 void phaseC_walk(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, Prof& p) {
   p.begin("c_walk", double(z.n_sync) * 40);
-  cudaMemsetAsync(b.sy_relk, 0xFF, size_t(z.n_sync + 1) * 4, s);
-  cudaMemsetAsync(b.incs_cnt, 0, size_t(z.n_sync + 1) * 4, s);
   k_c_walk<<<blocks(uint64_t(g.W) * 32, 128), 128, 0, s>>>(b.ev, g, b.seg, b.sy_start, b.sy_spos, b.sy_idx, b.sy_kind,
                                                            b.sy_N, b.sy_depth, b.sy_inner, b.sy_ver, b.sy_match,
                                                            b.sy_relk, b.incs_cnt, b.vcount, b.sy_agent, b.st);
@@ -1399,7 +1409,7 @@ void phaseC_forced(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, 
 // the trace-order pass of phase D; filtered: only accesses the grouped order keeps
 void phaseD_trace(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, bool filtered) {
   k_d_trace<<<blocks(z.N, 256), 256, 0, s>>>(b.ev, z.N, g, b.sy_start, b.sy_idx, b.d_index, z.d_shift, z.d_nw,
-                                              b.sy_N, b.sy_depth, b.sy_ver, b.vcount, b.acc_info, b.st,
+                                              reinterpret_cast<const uint2*>(b.sy_match), b.vcount, b.acc_info, b.st,
                                               (reinterpret_cast<uintptr_t>(b.ev) & 15) == 0, b.wl_bits,
                                               filtered ? z.wl_log2 : 0u, z.comp_lo, z.comp_span);
   count_launch();
@@ -1407,17 +1417,14 @@ void phaseD_trace(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, b
 
 void phaseD_gaps(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, Prof& p) {
   p.begin("d_gaps", double(z.n_acc) * (4 + 16 + 16), s);
-  if (z.n_sync) {
-    k_d_index<<<blocks(z.n_sync, 256), 256, 0, s>>>(b.sy_idx, b.sy_agent, b.sy_start, z.n_sync, z.d_shift, z.d_nw,
-                                                    b.d_index);
-    count_launch();
-  }
-  k_d_index_tail<<<blocks(uint64_t(g.W) * 32, 256), 256, 0, s>>>(b.sy_idx, b.sy_start, g.W, z.d_shift, z.d_nw,
-                                                                 b.d_index);
+  const uint32_t tail_from = blocks(z.n_sync, 256);
+  k_d_index<<<tail_from + blocks(uint64_t(g.W) * 32, 256), 256, 0, s>>>(b.sy_idx, b.sy_agent, b.sy_start, z.n_sync, g.W,
+                                                                        z.d_shift, z.d_nw, b.d_index, tail_from, b.sy_N, b.sy_depth,
+                                                                        b.sy_ver, reinterpret_cast<uint2*>(b.sy_match));
   count_launch();
   phaseD_trace(b, g, z, s, true);
   if (z.n_sync) {
-    k_d_fill<<<blocks(uint64_t(z.n_sync) * 32, 256), 256, 0, s>>>(
+    k_d_fill<<<blocks(uint64_t(z.n_sync) * D_LANES, 256), 256, 0, s>>>(
         b.ev, g, z.n_sync, b.S, b.seg, b.sy_start, b.sy_agent, b.sy_spos, b.sy_N, b.sy_depth, b.sy_ver, b.incs_cnt,
         b.vcount, b.acc_info, b.incs_idx, b.incs_ver, b.incs_k, b.incs_key, b.incs_wr, b.st);
     count_launch();
@@ -1440,13 +1447,16 @@ void phaseE_locks(Bufs& b, const Geo& g, const Sizes& z, uint64_t lock_mask, cud
 }
 
 // lk_csid = exclusive scan of the acquire flags (critical-section ids, grouped by lock
-// and in acquire order within a lock); lk_flags then holds the scan of new-lock flags.
+// and in acquire order within a lock); lk_k2, the sort's other buffer, the scan of the
+// new-lock flags.
 void phaseE_scan(const Bufs& b, const Sizes& z, cudaStream_t s, Prof& p) {
   const uint32_t n = z.n_acqrel;
   if (!n) return;
   p.begin("e_scan", double(n) * 16);
-  scan_exclusive(b.lk_flags, b.lk_csid, n, b.lk_csid + n, b.scan_tmp, s);
-  scan_exclusive(b.lk_rank, b.lk_flags, n, b.lk_flags + n, b.scan_tmp, s);
+  ScanBatch sb{};
+  sb.job[0] = ScanJob{b.lk_flags, b.lk_csid, b.lk_csid + n, n};
+  sb.job[1] = ScanJob{b.lk_rank, b.lk_k2, b.lk_k2 + n, n};
+  scan_all(sb, 2, b.scan_tmp, s);
   p.end();
 }
 
@@ -1457,7 +1467,7 @@ void phaseE_walk(Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, Prof& p)
   b.cs_r0 = b.cs_exp + n;
   p.begin("e_walk", double(n) * 32);
   const uint32_t* newflag = b.lk_rank;
-  const uint32_t* newscan = b.lk_flags;
+  const uint32_t* newscan = b.lk_k2;
   k_e_assign<<<blocks(n, 256), 256, 0, s>>>(b.ev, g, b.lk_k, n, newflag, b.lk_csid, newscan, b.sy_kind, b.sy_idx,
                                             b.sy_N, b.sy_relk, b.cs_of_sync, b.cs_agent, b.cs_sid, b.cs_epoch,
                                             b.cs_rel_idx, b.cs_rel_epoch, b.cs_lock, b.lock_first, b.lock_cs_lo, b.incs_cnt,

@@ -497,6 +497,44 @@ void scan_small(const ScanBatch& b, int jobs, cudaStream_t s) {
   k_scan_one<<<jobs, SC_ONE_THREADS, 0, s>>>(b);
   count_launch();
 }
+
+namespace {
+__global__ void __launch_bounds__(256) k_fill(const __grid_constant__ FillBatch b) {
+  const size_t t = size_t(blockIdx.x) * blockDim.x + threadIdx.x, all = size_t(gridDim.x) * blockDim.x;
+  for (int j = 0; j < b.n; ++j) {
+    const uint32_t v = b.job[j].value;
+    const size_t n = b.job[j].words;
+    uint4* const q = static_cast<uint4*>(b.job[j].ptr);
+    for (size_t i = t; i < n / 4; i += all) q[i] = make_uint4(v, v, v, v);
+    if (t < n % 4) static_cast<uint32_t*>(b.job[j].ptr)[n / 4 * 4 + t] = v;
+  }
+}
+__global__ void k_read_back(const DevStatus* st, const __grid_constant__ ReadBack r, DevStatus* st_out, uint32_t* val_out) {
+  const int t = threadIdx.x;
+  constexpr int words = sizeof(DevStatus) / 4;
+  static_assert(sizeof(DevStatus) % 4 == 0 && words + 8 <= 64);
+  if (t < words) reinterpret_cast<uint32_t*>(st_out)[t] = reinterpret_cast<const uint32_t*>(st)[t];
+  if (t < r.n) val_out[t] = *r.word[t];
+}
+__global__ void k_status_init(DevStatus* st, const __grid_constant__ DevStatus v) { *st = v; }
+}  // namespace
+
+void fill_all(const FillBatch& b, cudaStream_t s) {
+  size_t most = 0;
+  for (int j = 0; j < b.n; ++j) most = std::max(most, b.job[j].words);
+  if (!b.n) return;
+  k_fill<<<unsigned(std::min<size_t>((most + 1023) / 1024, 152 * 8)), 256, 0, s>>>(b);
+  count_launch();
+}
+void read_back_to(const DevStatus* st, const ReadBack& r, DevStatus* st_out, uint32_t* val_out, cudaStream_t s) {
+  k_read_back<<<1, 64, 0, s>>>(st, r, st_out, val_out);
+  count_launch();
+}
+void status_init(DevStatus* st, const DevStatus& v, cudaStream_t s) {
+  k_status_init<<<1, 1, 0, s>>>(st, v);
+  count_launch();
+}
+
 bool scan_is_small(size_t n) { return n <= size_t(SC_ONE); }
 
 void scan_exclusive(const uint32_t* in, uint32_t* out, size_t n, uint32_t* total_dev, uint32_t* tmp,

@@ -908,10 +908,8 @@ __global__ void k_plan_counts(PropArgs a, uint32_t n_cs, const uint32_t* cs_epoc
   cnt[i] = t;
 }
 
-__global__ void k_plan_sync(PropArgs a, const uint32_t* sy_kind_, const uint32_t* sy_ver, const uint32_t* sy_match,
-                            uint32_t n_sync) {
-  const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n_sync) return;
+// the entry of synchronisation entry k
+__device__ __forceinline__ void plan_sync(const PropArgs& a, const uint32_t* sy_kind_, const uint32_t* sy_ver, uint32_t k) {
   const Geo& g = a.g;
   const uint32_t u = a.sy_agent[k];
   const uint32_t row = a.rowbase[u] + sy_ver[k];
@@ -939,15 +937,17 @@ __global__ void k_plan_sync(PropArgs a, const uint32_t* sy_kind_, const uint32_t
     eb.x = mode;
     eb.y = a.sy_N[k] - 1;  // N_t entering the join (after the barrier, N_t = eb.y + 1)
   }
-  (void)sy_match;
   const size_t p = size_t(k) + a.incs_off[k];
   a.plan[2 * p] = ea;
   a.plan[2 * p + 1] = eb;
 }
 
-// the flattened list of an in-section access (its sections from the inside out), its entry
-__global__ void k_plan_incs(PropArgs a, const uint32_t* flat_off, uint32_t* flat, uint32_t n_incs) {
+// The plan's entries: per synchronisation entry, and per in-section access with its flattened
+// list (its sections from the inside out).
+__global__ void k_plan(const __grid_constant__ PropArgs a, const uint32_t* sy_kind_, const uint32_t* sy_ver, uint32_t n_sync,
+                       const uint32_t* flat_off, uint32_t* flat, uint32_t n_incs) {
   const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
+  if (r < n_sync) plan_sync(a, sy_kind_, sy_ver, r);
   if (r >= n_incs || a.st->code) return;
   const uint32_t k = a.incs_k[r];
   const uint32_t u = a.sy_agent[k];
@@ -1115,18 +1115,24 @@ int phaseG_propagate(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s
     const uint32_t most = std::max(z.n_cs, z.n_incs);
     k_plan_counts<<<(most + 255) / 256, 256, 0, s>>>(a, z.n_cs, b.cs_epoch, b.cs_rel_epoch, z.n_incs, b.flat_off);
     count_launch();
-    // snapshot rows start as SENTINEL: a reader accepts a row once none is left
-    cudaMemsetAsync(b.psnap, 0xFF, size_t(z.n_cs) * g.RW * 4, s);
-    cudaMemsetAsync(b.hsnap, 0xFF, size_t(z.n_cs) * g.RW * 4, s);
-    cudaMemsetAsync(b.jsnap, 0xFF, size_t(z.n_cs) * g.RW * 4, s);
   }
+  FillBatch f;
+  // snapshot rows start as SENTINEL: a reader accepts a row once none is left
+  for (uint32_t* snap : {b.psnap, b.hsnap, b.jsnap}) f.add(snap, size_t(z.n_cs) * g.RW, 0xFFFFFFFFu);
+  f.add(b.cursor, size_t(g.W) * (z.n_locks + 1), 0);
+  if ((!z.cta_barriers || g.gran == GWCP_GRAN_THREAD) && z.n_bar) {  // barriers joined in global memory
+    f.add(b.bar_j, size_t(z.n_bar) * 2 * g.Wp, 0);
+    f.add(b.bar_jj, size_t(z.n_bar) * g.Wp, 0);
+    f.add(b.bar_cnt, z.n_bar, 0);
+  }
+  if (g.nT) f.add(b.tiles, kTileW, 0);  // tile 0 is the zero tile; ids are handed out from 1
+  fill_all(f, s);
   if (z.n_incs) {
     scan_exclusive(b.flat_off, b.flat_off, size_t(z.n_incs) + 1, nullptr, b.scan_tmp, s);
-    k_plan_incs<<<(z.n_incs + 255) / 256, 256, 0, s>>>(a, b.flat_off, b.flat, z.n_incs);
-    count_launch();
   }
-  if (z.n_sync) {
-    k_plan_sync<<<(z.n_sync + 255) / 256, 256, 0, s>>>(a, b.sy_kind, b.sy_ver, b.sy_match, z.n_sync);
+  if (z.n_sync) {  // (no in-section access without a synchronisation entry)
+    const uint32_t most = std::max(z.n_sync, z.n_incs);
+    k_plan<<<(most + 255) / 256, 256, 0, s>>>(a, b.sy_kind, b.sy_ver, z.n_sync, b.flat_off, b.flat, z.n_incs);
     count_launch();
   }
   p.end();
