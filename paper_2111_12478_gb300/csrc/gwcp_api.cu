@@ -436,7 +436,7 @@ int run(gwcp_ctx* c, cudaStream_t s) {
   // automatic capacity: at least what the race buffers of an earlier pass hold (a trace with
   // more races than events would run its check twice on every pass)
   z.race_cap = c->opt.race_capacity ? c->opt.race_capacity
-                                    : std::max<uint64_t>({1u << 20, z.N,
+                                    : std::max<uint64_t>({(1u << 20) - (1u << 15), z.N,
                                                           std::min(c->allocs["races"].second,
                                                                    c->allocs["races2"].second) / 8});
   // scratch for every later scan and sort (the stream is idle here, so it may move)
@@ -446,17 +446,22 @@ int run(gwcp_ctx* c, cudaStream_t s) {
   b.scan_tmp = get<uint32_t>(c, "scan_tmp", need2, &oom);
   if (oom) return GWCP_ERR_OOM;
   phaseE_walk(b, g, z, s, c->prof);  // W3; runs on invalid traces too, for the first bad index
-  {
-    // the last validation (W3) and the acquires' dependency lists are done: no later phase
-    // runs on an invalid trace or after an error (their inputs would be incomplete)
-    int rc = read_status(c, s, nullptr, 0);
+  // The last validation (W3) and the acquires' dependency lists are done: no later phase runs
+  // on an invalid trace or after an error (their inputs would be incomplete). In the grouped
+  // order the kernels that follow see to that themselves and the host goes on without waiting
+  // (10 to 15 us); where the rest does not fit, the trace's own error comes first.
+  auto invalid = [&]() -> int {
+    const int rc = read_status(c, s, nullptr, 0);
     if (rc) return rc;
-  }
-  code = c->st_host->code;
-  if (code) {
-    c->bad_index = c->st_host->bad_index;
-    return code;
-  }
+    if (c->st_host->code) c->bad_index = c->st_host->bad_index;
+    return c->st_host->code;
+  };
+  auto out_of_memory = [&]() -> int {
+    const int rc = invalid();
+    return rc ? rc : GWCP_ERR_OOM;
+  };
+  if (code || !z.grouped)
+    if (int rc = invalid()) return rc;
 
   // ---- remaining buffers ------------------------------------------------------------
   const size_t ni1 = size_t(z.n_incs) + 1;
@@ -543,7 +548,7 @@ int run(gwcp_ctx* c, cudaStream_t s) {
     const size_t ng = check_group_count(z.n_acc, z.check_ch);
     b.tails = get<uint32_t>(c, "tails", (size_t(z.n_chunks) + ng) * 4 * g.Wp * 2 + ng + 8, &oom);
   }
-  if (oom) return GWCP_ERR_OOM;
+  if (oom) return out_of_memory();
 
   phaseD_gaps(b, g, z, s, c->prof);
   c->acc_info_partial = z.wl_log2 != 0;
@@ -577,7 +582,7 @@ int run(gwcp_ctx* c, cudaStream_t s) {
     b.chunk_ns = nullptr;
     b.chunk_races = nullptr;
   }
-  if (oom) return GWCP_ERR_OOM;
+  if (oom) return out_of_memory();
   phaseF_expand(b, z, s, c->prof);
   phaseF_deps(b, g, z, key_mask, s, c->prof);
   cudaStreamWaitEvent(c->side, c->fork2, 0);
@@ -619,7 +624,10 @@ int run(gwcp_ctx* c, cudaStream_t s) {
   }
   int prc = phaseG_propagate(b, g, z, s, c->prof);
   side.join();
-  if (prc) return prc;
+  if (prc) {
+    const int rc = invalid();
+    return rc ? rc : prc;
+  }
   if (b.chunk_ns) stamp_now(&b.st->spare[5], s);  // the check's start, for the timeline
   if (z.sparse_check)
     phaseI_wide_check(b, g, z, s, c->prof);

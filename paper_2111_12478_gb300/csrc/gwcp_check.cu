@@ -55,6 +55,7 @@ __device__ __forceinline__ void put_slot(uint64_t (&last)[4][K], int lane, uint3
 // State of the chunk's last location over the chunk's entries.
 template <int K>
 __global__ void k_tail(ChunkArgs a) {
+  if (a.st->code) return;  // (the access records are incomplete)
   const int lane = threadIdx.x & 31;
   const uint32_t c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (c >= a.n_chunks) return;
@@ -189,6 +190,7 @@ __device__ __forceinline__ uint32_t conflict_mask(uint32_t cb, bool same) {
 
 template <int K>
 __global__ void __launch_bounds__(CHK_WARPS * 32) k_check(ChunkArgs a) {
+  if (a.st->code) return;
   const int lane = threadIdx.x & 31;
   const uint32_t c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (c >= a.n_chunks) return;

@@ -218,11 +218,19 @@ int analyze(const Event* ev, uint64_t n, const Geo& g, gwcp_race* out, uint64_t 
   // the last validity check (W3) needs only the buffers carved so far: an invalid trace is
   // reported with its first bad index before the rest of the scratch is sized
   phaseE_walk(b, g, z, s, prof);
-  if (int rc = read_back(s, &st, b.st, v, nullptr, 0)) return rc;
-  if (st.code) {  // no later phase runs on an invalid trace or after an error
-    if (bad_index) *bad_index = st.bad_index;
+  // no later phase runs on an invalid trace or after an error: the kernels that follow see to
+  // it themselves, so the host waits here only when it has such a trace or refuses this one
+  auto invalid = [&]() -> int {
+    if (int rc = read_back(s, &st, b.st, v, nullptr, 0)) return rc;
+    if (st.code && bad_index) *bad_index = st.bad_index;
     return st.code;
-  }
+  };
+  auto refused = [&]() -> int {
+    const int rc = invalid();
+    return rc ? rc : GWCP_ERR_UNSUPPORTED;
+  };
+  if (code)
+    if (int rc = invalid()) return rc;
   const size_t ni1 = size_t(z.n_incs) + 1;
   const size_t ne1 = std::max<size_t>(size_t(z.n_exp), size_t(z.n_incs) * kMaxNest) + 1;
   b.acc_info = A.take<AccInfo>(z.N);
@@ -254,13 +262,13 @@ int analyze(const Event* ev, uint64_t n, const Geo& g, gwcp_race* out, uint64_t 
   b.jsnap = X.take<uint32_t>((size_t(z.n_cs) + 1) * g.Wp);
   b.plan2 = X.take<uint4>(2 * (size_t(z.n_sync) + z.n_incs) + 2);
   b.bar_jj = X.take<uint32_t>(global_bars ? size_t(z.n_bar) * g.Wp : 1);
-  if (X.full) return GWCP_ERR_UNSUPPORTED;
+  if (X.full) return refused();
   b.bar_j = A.take<uint32_t>(global_bars ? size_t(z.n_bar) * 2 * g.Wp : 1);
   b.bar_cnt = A.take<uint32_t>(global_bars ? z.n_bar : 1);
   z.n_chunks = uint32_t(check_chunks(z.n_acc, z.check_ch));
   const size_t ng = check_group_count(z.n_acc, z.check_ch);
   b.tails = A.take<uint32_t>((size_t(z.n_chunks) + ng) * 4 * g.Wp * 2 + ng + 8);
-  if (A.full) return GWCP_ERR_UNSUPPORTED;
+  if (A.full) return refused();
   // races: the rest of the scratch, split in two sort buffers and their sort scratch
   const size_t left = kScratchBytes - A.used;
   z.race_cap = left / (2 * sizeof(uint64_t) + 8) > 4096 ? left / (2 * sizeof(uint64_t) + 8) - 4096 : 0;
@@ -277,7 +285,7 @@ int analyze(const Event* ev, uint64_t n, const Geo& g, gwcp_race* out, uint64_t 
   b.races2 = A.take<uint64_t>(z.race_cap);
   A.take<uint32_t>(race_tmp_elems);
   uint32_t* race_tmp = X.take<uint32_t>(radix_tmp_need(z.race_cap + 1) + 64);
-  if (A.full || X.full || !z.race_cap) return GWCP_ERR_UNSUPPORTED;
+  if (A.full || X.full || !z.race_cap) return refused();
   // A chunk is a warp's serial work, about 1 us per access: chunks are cut down to 32 accesses
   // while there are at most 4096 and their states fit the race sort's second buffer, which is
   // not in use before the check is done (60k events, 64 agents: states, their scan and the
@@ -294,7 +302,10 @@ int analyze(const Event* ev, uint64_t n, const Geo& g, gwcp_race* out, uint64_t 
   phaseF_expand(b, z, s, prof);
   phaseF_deps(b, g, z, key_mask, s, prof);
   phaseH_sort(b, g, z, key_mask, b.scan_tmp, s, prof);
-  if (int rc = phaseG_propagate(b, g, z, s, prof)) return rc;
+  if (int rc = phaseG_propagate(b, g, z, s, prof)) {
+    const int bad = invalid();
+    return bad ? bad : rc;
+  }
   phaseI_carry(b, g, z, s, prof);
   phaseI_check(b, g, z, s, prof);
   if (int rc = read_back(s, &st, b.st, v, nullptr, 0)) return rc;

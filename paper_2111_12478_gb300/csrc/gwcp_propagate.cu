@@ -947,8 +947,9 @@ __device__ __forceinline__ void plan_sync(const PropArgs& a, const uint32_t* sy_
 __global__ void k_plan(const __grid_constant__ PropArgs a, const uint32_t* sy_kind_, const uint32_t* sy_ver, uint32_t n_sync,
                        const uint32_t* flat_off, uint32_t* flat, uint32_t n_incs) {
   const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
+  if (a.st->code) return;  // (the lists are incomplete, the walkers stand down)
   if (r < n_sync) plan_sync(a, sy_kind_, sy_ver, r);
-  if (r >= n_incs || a.st->code) return;
+  if (r >= n_incs) return;
   const uint32_t k = a.incs_k[r];
   const uint32_t u = a.sy_agent[k];
   const size_t p = size_t(k) + 1 + r;

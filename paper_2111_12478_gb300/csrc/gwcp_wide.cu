@@ -987,6 +987,7 @@ __device__ __forceinline__ uint32_t flush_warp(const WideCheckArgs& a, uint32_t 
 // walked here); otherwise the lanes of their warp share them (a ranked check keeps its order).
 template <int REP, bool ASIDE>
 __global__ void __launch_bounds__(kCheckThreads, 8) k_wc_check(const __grid_constant__ WideCheckArgs a) {
+  if (a.st->code) return;  // (the access records or clocks are incomplete)
   constexpr uint32_t kWarps = kCheckThreads / 32;
   __shared__ uint32_t s_cnt[kWarps];
   __shared__ uint64_t s_buf[kWarps][kRaceStage];
@@ -1045,6 +1046,7 @@ __global__ void __launch_bounds__(kCheckThreads, 8) k_wc_check(const __grid_cons
 // at one hot location (neighbours in the order) spread over all SMs.
 template <int REP>
 __global__ void __launch_bounds__(kCheckThreads, 6) k_wc_big(const __grid_constant__ WideCheckArgs a) {
+  if (a.st->code) return;  // (the access records or clocks are incomplete)
   constexpr uint32_t kWarps = kCheckThreads / 32;
   __shared__ uint32_t s_cnt[kWarps];
   __shared__ uint64_t s_buf[kWarps][kRaceStage];

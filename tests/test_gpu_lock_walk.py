@@ -96,3 +96,30 @@ def test_lists_placed_by_a_counter(gw):
         races = c.report_races()
         assert np.array_equal(races, want.races)
     assert len(races)
+
+
+def test_invalid_trace_comes_before_lack_of_memory(gw):
+    # a section that interleaves with an overlapping one, under a limit that leaves no room for
+    # the arrays after the lock walk
+    ev, geo = sections(5, 8, 8, 4000, 3, 0.3)
+    bad = np.concatenate([ev, np.array([(0, TG.ACQ, TG.DEVICE, 0, 0, 1), (9, TG.ACQ, TG.CTA, 0, 0, 1)], dtype=ev.dtype)])
+
+    def result(events, limit):
+        with gw.Context(0) as c:
+            c.debug_alloc_limit(limit)
+            c.load_trace(events, *geo.astuple())
+            try:
+                c.compute_order()
+            except gw.GwcpError as e:
+                return e.code, e.bad_index if e.code == gw.ERR_INVALID_TRACE else None
+            return 0, None
+
+    assert result(ev, 1 << 40)[0] == 0
+    assert result(bad, 1 << 40) == (gw.ERR_INVALID_TRACE, len(ev) + 1)
+    lo, hi = 0, 1 << 30  # the smallest limit that the valid trace fits
+    while hi - lo > 1 << 12:
+        mid = (lo + hi) // 2
+        lo, hi = (lo, mid) if result(ev, mid)[0] == 0 else (mid, hi)
+    code = result(ev, lo)[0]
+    assert code != 0 and code != gw.ERR_INVALID_TRACE
+    assert result(bad, lo) == (gw.ERR_INVALID_TRACE, len(ev) + 1)
