@@ -1081,11 +1081,13 @@ namespace {
 // location order rebuilt from the trace (the grouped order leaves read-only locations
 // out): the accesses' (location key, trace index) pairs in trace order, then a stable sort
 __global__ void k_lf_flag(const Event* ev, uint64_t N, uint32_t* flag) {
+  grid_begin();
   const uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i < N) flag[i] = ev[i].op <= GWCP_ATOMIC ? 1u : 0u;
 }
 __global__ void k_lf_acc(const Event* ev, uint64_t N, uint32_t apb, const uint32_t* flag, const uint32_t* pos,
                          uint64_t* k, uint32_t* v) {
+  grid_begin();
   const uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i < N && flag[i]) {
     k[pos[i]] = location_key(ev[i], apb);
@@ -1127,10 +1129,10 @@ int gwcp_location_features(gwcp_ctx* c, float* feat, uint64_t* keys, uint64_t ca
     uint32_t* st2 = get<uint32_t>(c, "lf_tmp", std::max(radix_tmp_need(n + 1), scan_tmp_need(z.N)) + 64, &oom);
     if (oom) return GWCP_ERR_OOM;
     const uint32_t nbN = uint32_t((z.N + 255) / 256);
-    k_lf_flag<<<nbN, 256, 0, s>>>(b.ev, z.N, flag);
+    launch(k_lf_flag, nbN, 256, 0, s)(b.ev, z.N, flag);
     count_launch();
     scan_exclusive(flag, pos, z.N, nullptr, st2, s);
-    k_lf_acc<<<nbN, 256, 0, s>>>(b.ev, z.N, c->g.apb, flag, pos, k0, v0);
+    launch(k_lf_acc, nbN, 256, 0, s)(b.ev, z.N, c->g.apb, flag, pos, k0, v0);
     count_launch();
     if (radix_sort_pairs(k0, v0, k1, v1, n, c->key_mask, st2, s)) {
       std::swap(k0, k1);

@@ -55,6 +55,7 @@ __device__ __forceinline__ void put_slot(uint64_t (&last)[4][K], int lane, uint3
 // State of the chunk's last location over the chunk's entries.
 template <int K>
 __global__ void k_tail(ChunkArgs a) {
+  grid_begin();
   if (a.st->code) return;  // (the access records are incomplete)
   const int lane = threadIdx.x & 31;
   const uint32_t c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -111,6 +112,7 @@ __device__ __forceinline__ uint32_t group_links(const ChunkArgs& a, uint32_t g0,
 }
 
 __global__ void k_scan1(ChunkArgs a, uint64_t* gagg, uint32_t* gfull) {
+  grid_begin();
   const uint32_t cols = 4 * a.g.Wp;
   const uint32_t g0 = blockIdx.x * GRP, g1 = min(g0 + GRP, a.n_chunks);
   const uint32_t links = group_links(a, g0, g1);
@@ -135,6 +137,7 @@ __global__ void k_scan1(ChunkArgs a, uint64_t* gagg, uint32_t* gfull) {
 }
 
 __global__ void k_scan2(ChunkArgs a, uint32_t ngroups, uint64_t* gagg, const uint32_t* gfull) {
+  grid_begin();
   // gagg[g] becomes the carry into group g. The loads of a window of groups are issued
   // together; only the running value is carried from group to group.
   constexpr int U = 8;
@@ -161,6 +164,7 @@ __global__ void k_scan2(ChunkArgs a, uint32_t ngroups, uint64_t* gagg, const uin
 }
 
 __global__ void k_scan3(ChunkArgs a, const uint64_t* gagg) {
+  grid_begin();
   const uint32_t cols = 4 * a.g.Wp;
   const uint32_t g0 = blockIdx.x * GRP, g1 = min(g0 + GRP, a.n_chunks);
   const uint32_t links = group_links(a, g0, g1);
@@ -190,6 +194,7 @@ __device__ __forceinline__ uint32_t conflict_mask(uint32_t cb, bool same) {
 
 template <int K>
 __global__ void __launch_bounds__(CHK_WARPS * 32) k_check(ChunkArgs a) {
+  grid_begin();
   if (a.st->code) return;
   const int lane = threadIdx.x & 31;
   const uint32_t c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -317,13 +322,13 @@ void run_carry(const ChunkArgs& a, uint64_t* gagg, uint32_t* gfull, cudaStream_t
   const uint32_t cols = 4 * a.g.Wp;
   const uint32_t ng = blocks(nw, GRP);
   p.begin("i_carry", double(nw) * cols * 8 * 3, s);
-  k_tail<K><<<blocks(uint64_t(nw) * 32, CHK_WARPS * 32), CHK_WARPS * 32, 0, s>>>(a);
+  launch(k_tail<K>, blocks(uint64_t(nw) * 32, CHK_WARPS * 32), CHK_WARPS * 32, 0, s)(a);
   count_launch();
-  k_scan1<<<ng, 256, 0, s>>>(a, gagg, gfull);
+  launch(k_scan1, ng, 256, 0, s)(a, gagg, gfull);
   count_launch();
-  k_scan2<<<blocks(cols, 256), 256, 0, s>>>(a, ng, gagg, gfull);
+  launch(k_scan2, blocks(cols, 256), 256, 0, s)(a, ng, gagg, gfull);
   count_launch();
-  k_scan3<<<ng, 256, 0, s>>>(a, gagg);
+  launch(k_scan3, ng, 256, 0, s)(a, gagg);
   count_launch();
   p.end();
 }
@@ -332,7 +337,7 @@ template <int K>
 void run_check(const ChunkArgs& a, cudaStream_t s, Prof& p, double bytes_per) {
   const uint32_t nw = a.n_chunks;
   p.begin("i_check", double(a.n) * bytes_per, s);
-  k_check<K><<<blocks(uint64_t(nw) * 32, CHK_WARPS * 32), CHK_WARPS * 32, 0, s>>>(a);
+  launch(k_check<K>, blocks(uint64_t(nw) * 32, CHK_WARPS * 32), CHK_WARPS * 32, 0, s)(a);
   count_launch();
   p.end();
 }
@@ -410,6 +415,7 @@ void phaseI_check(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, P
 
 namespace {
 __global__ void k_race_records(const uint64_t* w, uint64_t n, gwcp_race* out) {
+  grid_begin();
   const uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i < n) out[i] = gwcp_race{w[i] & 0xFFFFFFFFull, w[i] >> 32};
 }
@@ -417,7 +423,7 @@ __global__ void k_race_records(const uint64_t* w, uint64_t n, gwcp_race* out) {
 
 void races_to_records(const uint64_t* words, uint64_t n, gwcp_race* out, cudaStream_t s) {
   if (!n) return;
-  k_race_records<<<unsigned((n + 255) / 256), 256, 0, s>>>(words, n, out);
+  launch(k_race_records, unsigned((n + 255) / 256), 256, 0, s)(words, n, out);
   count_launch();
 }
 

@@ -76,6 +76,7 @@ struct Arena {
 };
 
 __global__ void k_races_out(const uint64_t* keys, uint64_t n, gwcp_race* out) {
+  grid_begin();
   const uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i < n) out[i] = gwcp_race{keys[i] & 0xFFFFFFFFull, keys[i] >> 32};
 }
@@ -320,7 +321,7 @@ int analyze(const Event* ev, uint64_t n, const Geo& g, gwcp_race* out, uint64_t 
   const bool second = phaseI_sort_races(b, z, total, s, prof);
   const uint64_t m = std::min<uint64_t>(total, cap);
   if (m) {
-    k_races_out<<<uint32_t((m + 255) / 256), 256, 0, s>>>(second ? b.races2 : b.races, m, out);
+    launch(k_races_out, uint32_t((m + 255) / 256), 256, 0, s)(second ? b.races2 : b.races, m, out);
     count_launch();
   }
   if (cudaStreamSynchronize(s) != cudaSuccess || cudaGetLastError() != cudaSuccess) return GWCP_ERR_CUDA;

@@ -69,6 +69,7 @@ __device__ __forceinline__ Event load_event(const Event* ev, uint64_t i, bool ve
 // Phase A, pass 1: per (agent, tile) entry counts and per-tile compaction counts.
 __global__ void k_a_count(const Event* ev, uint64_t N, Geo g, uint32_t TA, uint32_t ntA, uint32_t* hist,
                           uint32_t* tile_cnt, DevStatus* st, bool vec) {
+  grid_begin();
   extern __shared__ uint32_t sm[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t tile = blockIdx.x * (blockDim.x >> 5) + warp;
@@ -185,6 +186,7 @@ __device__ __forceinline__ uint32_t a_compact(const ACompact& c, const Event& e,
 // 64 agents 34 us, now 14; 10M events 0.22 ms, now 0.15.)
 __global__ void k_a_scatter(const Event* ev, uint64_t N, Geo g, uint32_t TA, uint32_t ntA, const uint32_t* hist,
                             const uint32_t* tile_off, uint32_t* S, uint32_t nS, uint32_t* seg, ACompact cpt, bool vec) {
+  grid_begin();
   extern __shared__ uint32_t sm[];
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t tile = blockIdx.x * (blockDim.x >> 5) + warp;
@@ -261,6 +263,7 @@ __global__ void k_a_scatter(const Event* ev, uint64_t N, Geo g, uint32_t TA, uin
 // 256-thread blocks per SM (64 registers; 80 allowed three): 0.9 ms faster per 200M events.
 __global__ void __launch_bounds__(256, 4) k_aw_count(const Event* ev, uint64_t N, Geo g, uint32_t TA, uint32_t ntA, uint32_t* tile_cnt,
                            DevStatus* st, bool vec) {
+  grid_begin();
   const int lane = threadIdx.x & 31;
   const uint32_t tile = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (tile >= ntA) return;
@@ -329,6 +332,7 @@ __global__ void __launch_bounds__(256, 4) k_aw_count(const Event* ev, uint64_t N
 // gives S (each agent's entries in trace order).
 __global__ void __launch_bounds__(256, 4) k_aw_scatter(const Event* ev, uint64_t N, Geo g, uint32_t TA, uint32_t ntA, const uint32_t* tile_off,
                              uint64_t* skey, ACompact cpt, bool vec) {
+  grid_begin();
   const int lane = threadIdx.x & 31;
   const uint32_t tile = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (tile >= ntA) return;
@@ -374,12 +378,14 @@ __global__ void __launch_bounds__(256, 4) k_aw_scatter(const Event* ev, uint64_t
 }
 
 __global__ void k_aw_extract(const uint64_t* key, uint32_t n, uint32_t* S) {
+  grid_begin();
   const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p < n) S[p] = uint32_t(key[p]);
 }
 
 // seg[u]: the first S position of agent u (seg[W] = n)
 __global__ void k_aw_seg(const uint64_t* key, uint32_t n, uint32_t W, uint32_t* seg) {
+  grid_begin();
   const uint32_t u = blockIdx.x * blockDim.x + threadIdx.x;
   if (u > W) return;
   const uint64_t x = uint64_t(u) << 32;
@@ -413,6 +419,7 @@ __device__ __forceinline__ uint32_t lower_bound_dev(const T* a, uint32_t n, T x)
 constexpr int B_THREADS = 256, B_ROUNDS = 16, B_CHUNK = 32 * B_ROUNDS;
 
 __global__ void k_b_count(const uint32_t* S, uint32_t nS, uint32_t n_chunks, uint32_t* cnt) {
+  grid_begin();
   const uint32_t chunk = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (chunk >= n_chunks) return;
   const uint32_t base = chunk * B_CHUNK;
@@ -428,6 +435,7 @@ __global__ void k_b_count(const uint32_t* S, uint32_t nS, uint32_t n_chunks, uin
 
 __global__ void k_b_scatter(const uint32_t* S, uint32_t nS, uint32_t n_chunks, const uint32_t* off, uint32_t* sy_spos,
                             uint32_t* sy_idx, uint32_t* sy_kind, uint32_t* sy_relk, uint32_t* cs_of_sync) {
+  grid_begin();
   const uint32_t chunk = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (chunk >= n_chunks) return;
   const uint32_t base = chunk * B_CHUNK;
@@ -465,6 +473,7 @@ __global__ void k_b_search(const Event* ev, const uint32_t* seg, uint32_t W, con
                            uint32_t* sy_start, const uint32_t* sy_idx, const uint32_t* sy_kind, const uint32_t* bar,
                            uint32_t n_bar, const uint32_t* acqrel, uint32_t n_acqrel, uint32_t* sy_aux,
                            uint64_t* lk_key, uint32_t* lk_k) {
+  grid_begin();
   const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k <= W) sy_start[k] = lower_bound_dev(sy_spos, n_sync, seg[k]);
   if (k >= n_sync) return;
@@ -485,6 +494,7 @@ __global__ void k_c_walk(const Event* ev, Geo g, const uint32_t* seg, const uint
                          uint32_t* sy_depth, uint32_t* sy_inner, uint32_t* sy_ver, uint32_t* sy_match,
                          uint32_t* sy_relk, uint32_t* incs_cnt, uint32_t* vcount, uint32_t* sy_agent,
                          DevStatus* st) {
+  grid_begin();
   const int lane = threadIdx.x & 31;
   const uint32_t u = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (u >= g.W) return;
@@ -628,6 +638,7 @@ __global__ void k_c_walk(const Event* ev, Geo g, const uint32_t* seg, const uint
 __global__ void k_d_index(const uint32_t* sy_idx, const uint32_t* sy_agent, const uint32_t* sy_start, uint32_t n_sync,
                           uint32_t W, uint32_t shift, uint32_t nw, uint32_t* table, uint32_t tail_from,
                           const uint32_t* sy_N, const uint32_t* sy_depth, const uint32_t* sy_ver, uint2* sy_pack) {
+  grid_begin();
   if (blockIdx.x >= tail_from) {
     const uint32_t u = ((blockIdx.x - tail_from) * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (u >= W) return;
@@ -651,6 +662,7 @@ __global__ void k_d_trace(const Event* ev, uint64_t N, Geo g, const uint32_t* sy
                           const uint32_t* rowbase, AccInfo* acc_info,
                           const DevStatus* st, bool vec, const uint32_t* wl_bits, uint32_t wl_log2,
                           uint32_t comp_lo, uint32_t comp_span) {
+  grid_begin();
   const uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i >= N || st->code) return;
   const Event e = load_event(ev, i, vec);
@@ -694,6 +706,7 @@ __global__ void k_d_fill(const Event* ev, Geo g, uint32_t n_sync, const uint32_t
                          const uint32_t* sy_depth, const uint32_t* sy_ver, const uint32_t* incs_off,
                          const uint32_t* rowbase, AccInfo* acc_info, uint32_t* incs_idx, uint32_t* incs_ver,
                          uint32_t* incs_k, uint64_t* incs_key, uint32_t* incs_wr, const DevStatus* st) {
+  grid_begin();
   const uint32_t lane = threadIdx.x & (D_LANES - 1);
   const uint64_t gid = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) / D_LANES;
   if (gid >= n_sync || st->code) return;
@@ -734,6 +747,7 @@ __global__ void k_d_fill(const Event* ev, Geo g, uint32_t n_sync, const uint32_t
 // barrier -> (its block, or B for a one-member barrier; its trace-order position)
 __global__ void k_fb_keys(const Event* ev, Geo g, const uint32_t* bar, uint32_t n_bar, uint64_t* key,
                           uint32_t* val) {
+  grid_begin();
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n_bar) return;
   const Event e = ev[bar[i]];
@@ -745,6 +759,7 @@ __global__ void k_fb_keys(const Event* ev, Geo g, const uint32_t* bar, uint32_t 
 // position r of the block-sorted order: inverse map, member count, block starts
 __global__ void k_fb_rank(const Event* ev, Geo g, const uint32_t* bar, const uint64_t* skey, const uint32_t* spos,
                           uint32_t n_bar, uint32_t* rank, uint32_t* cnt, uint32_t* blo) {
+  grid_begin();
   const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r > n_bar) return;
   const uint32_t blk = r < n_bar ? uint32_t(skey[r]) : g.B;
@@ -767,6 +782,7 @@ __global__ void k_fb_rank(const Event* ev, Geo g, const uint32_t* bar, const uin
 __global__ void k_fb_records(const Event* ev, Geo g, uint32_t n_sync, uint32_t n_bar, const uint32_t* sy_agent,
                              const uint32_t* sy_kind, const uint32_t* sy_idx, const uint32_t* sy_aux,
                              const uint32_t* sy_N, const uint32_t* rank, const uint32_t* off, uint4* rec) {
+  grid_begin();
   const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n_sync || sy_kind[k] != K_BAR) return;
   const uint32_t u = sy_agent[k];
@@ -781,6 +797,7 @@ constexpr uint32_t FB_STAGE = 1024;  // records staged in shared memory at a tim
 
 __global__ void __launch_bounds__(32) k_fb_walk(Geo g, uint32_t n_sync, const uint32_t* blo, const uint32_t* off,
                                                 const uint4* rec, uint32_t* boff, DevStatus* st) {
+  grid_begin();
   __shared__ uint32_t off_s[1024];  // per member of the block (agents_per_block <= 1024)
   __shared__ uint4 rec_s[FB_STAGE];
   const uint32_t lane = threadIdx.x, b = blockIdx.x;
@@ -853,6 +870,7 @@ __global__ void __launch_bounds__(32) k_fb_walk(Geo g, uint32_t n_sync, const ui
 
 // N after each entry += the offset of the agent's latest barrier entry at or before it
 __global__ void k_fb_apply(Geo g, const uint32_t* sy_start, const uint32_t* boff, uint32_t* sy_N) {
+  grid_begin();
   const uint32_t lane = threadIdx.x & 31;
   const uint32_t u = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (u >= g.W) return;
@@ -874,6 +892,7 @@ __global__ void k_fb_apply(Geo g, const uint32_t* sy_start, const uint32_t* boff
 // Phase E
 __global__ void k_e_flags(const uint64_t* key, const uint32_t* kk, uint32_t n, const uint32_t* sy_kind,
                           uint32_t* is_acq, uint32_t* is_new) {
+  grid_begin();
   uint32_t m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= n) return;
   is_acq[m] = sy_kind[kk[m]] == K_ACQ;
@@ -887,6 +906,7 @@ __global__ void k_e_assign(const Event* ev, Geo g, const uint32_t* kk, uint32_t 
                            uint32_t* cs_rel_idx, uint32_t* cs_rel_epoch, uint32_t* cs_lock, uint32_t* lock_first,
                            uint32_t* lock_cs_lo, const uint32_t* incs_off, const uint32_t* sy_start,
                            uint32_t* cs_exp, uint32_t* cs_r0) {
+  grid_begin();
   uint32_t m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= n) return;
   const uint32_t k = kk[m];
@@ -918,6 +938,7 @@ __global__ void k_e_assign(const Event* ev, Geo g, const uint32_t* kk, uint32_t 
 // rec[m], the lock walk's input in lock order: (scope id | 1 << 31 for an acquire, section)
 __global__ void k_e_assign_rel(const uint32_t* kk, uint32_t n, const uint32_t* sy_kind, const uint32_t* sy_match,
                                uint32_t* cs_of_sync, const uint32_t* cs_sid, uint32_t* cs_parent, uint2* rec) {
+  grid_begin();
   uint32_t m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= n) return;
   const uint32_t k = kk[m];
@@ -965,6 +986,7 @@ __global__ void __launch_bounds__(E_WARPS * 32) k_e_walk(const uint2* rec, const
                                                          uint32_t* acq_dep_off, uint32_t* acq_dep_cnt, uint32_t* pool,
                                                          uint32_t stride, uint32_t pool_cap, uint32_t n_cs,
                                                          DevStatus* st) {
+  grid_begin();
   using Slots = LockSlots<MAXS>;
   __shared__ Slots all[E_WARPS];
   const int lane = threadIdx.x & 31;
@@ -1150,6 +1172,7 @@ __global__ void k_f_expand(const uint32_t* incs_k, uint32_t n_incs, const uint64
                            const uint32_t* sy_inner, const uint32_t* cs_of_sync, const uint32_t* cs_parent,
                            const uint32_t* cs_lock, const uint32_t* cs_exp, const uint32_t* cs_r0, uint2* ex_info,
                            uint64_t* key, uint32_t* val, const DevStatus* st) {
+  grid_begin();
   const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= n_incs || st->code) return;
   const uint64_t loc = incs_key[r];
@@ -1174,6 +1197,7 @@ template <int MAXS>
 __global__ void k_f_walk(const uint64_t* key, const uint32_t* val, uint32_t n, const uint2* ex_info,
                          const uint32_t* cs_sid, const uint32_t* cs_rel_idx, uint32_t* ex_dep_off,
                          uint32_t* ex_dep_cnt, uint32_t* pool, uint32_t pool_cap, DevStatus* st) {
+  grid_begin();
   uint32_t m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= n || st->code) return;
   const uint64_t loc = key[m];
@@ -1287,7 +1311,7 @@ void phaseA_count(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, P
   p.begin("a_count", double(z.N) * 16);
   const bool vec = (reinterpret_cast<uintptr_t>(b.ev) & 15) == 0;
   if (z.agent_sort) {
-    k_aw_count<<<blocks(z.ntA, 8), 256, 0, s>>>(b.ev, z.N, g, z.TA, z.ntA, b.tile_cnt, b.st, vec);
+    launch(k_aw_count, blocks(z.ntA, 8), 256, 0, s)(b.ev, z.N, g, z.TA, z.ntA, b.tile_cnt, b.st, vec);
     count_launch();
     p.end();
     ScanBatch sb{};
@@ -1299,7 +1323,7 @@ void phaseA_count(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, P
     return;
   }
   const uint32_t aw = a_warps(g);
-  k_a_count<<<blocks(z.ntA, aw), aw * 32, aw * g.Wp * 4, s>>>(b.ev, z.N, g, z.TA, z.ntA, b.hist_a,
+  launch(k_a_count, blocks(z.ntA, aw), aw * 32, aw * g.Wp * 4, s)(b.ev, z.N, g, z.TA, z.ntA, b.hist_a,
                                                                           b.tile_cnt, b.st, vec);
   count_launch();
   p.end();
@@ -1326,7 +1350,7 @@ void phaseA_scatter(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s,
   const ACompact cpt{b.acc_key, b.acc_idx, b.acqrel, b.bar, z.grouped ? z.comp_lo : 0u,
                      z.grouped ? z.comp_span : 0u, b.wl_bits, z.wl_log2};
   if (z.agent_sort) {
-    k_aw_scatter<<<blocks(z.ntA, 8), 256, 0, s>>>(b.ev, z.N, g, z.TA, z.ntA, b.tile_cnt, b.s_key, cpt, vec);
+    launch(k_aw_scatter, blocks(z.ntA, 8), 256, 0, s)(b.ev, z.N, g, z.TA, z.ntA, b.tile_cnt, b.s_key, cpt, vec);
     count_launch();
     uint32_t ab = 0;
     while ((1u << ab) < g.W) ++ab;
@@ -1334,16 +1358,16 @@ void phaseA_scatter(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s,
     const uint64_t* sorted =
         radix_sort_pairs(b.s_key, nullptr, b.s_key2, nullptr, z.nS, mask, b.s_tmp, s, nullptr, {}, b.st) ? b.s_key2 : b.s_key;
     if (z.nS) {
-      k_aw_extract<<<blocks(z.nS, 256), 256, 0, s>>>(sorted, z.nS, b.S);
+      launch(k_aw_extract, blocks(z.nS, 256), 256, 0, s)(sorted, z.nS, b.S);
       count_launch();
     }
-    k_aw_seg<<<blocks(g.W + 1, 256), 256, 0, s>>>(sorted, z.nS, g.W, b.seg);
+    launch(k_aw_seg, blocks(g.W + 1, 256), 256, 0, s)(sorted, z.nS, g.W, b.seg);
     count_launch();
     p.end();
     return;
   }
   const uint32_t aw = a_warps(g);
-  k_a_scatter<<<blocks(z.ntA, aw), aw * 32, aw * g.Wp * 4, s>>>(b.ev, z.N, g, z.TA, z.ntA, b.hist_a, b.tile_cnt,
+  launch(k_a_scatter, blocks(z.ntA, aw), aw * 32, aw * g.Wp * 4, s)(b.ev, z.N, g, z.TA, z.ntA, b.hist_a, b.tile_cnt,
                                                                 b.S, z.nS, b.seg, cpt, vec);
   count_launch();
   p.end();
@@ -1353,14 +1377,14 @@ void phaseB_sync(const Bufs& b, const Geo& g, Sizes& z, cudaStream_t s, Prof& p)
   z.ntS = blocks(z.nS, B_CHUNK);  // chunks of S, one warp each
   p.begin("b_sync", double(z.nS) * 8);
   if (z.ntS) {
-    k_b_count<<<blocks(uint64_t(z.ntS) * 32, B_THREADS), B_THREADS, 0, s>>>(b.S, z.nS, z.ntS, b.sy_cnt);
+    launch(k_b_count, blocks(uint64_t(z.ntS) * 32, B_THREADS), B_THREADS, 0, s)(b.S, z.nS, z.ntS, b.sy_cnt);
     count_launch();
     scan_exclusive(b.sy_cnt, b.sy_cnt, z.ntS, b.sy_cnt + z.ntS, b.scan_tmp, s);
-    k_b_scatter<<<blocks(uint64_t(z.ntS) * 32, B_THREADS), B_THREADS, 0, s>>>(
+    launch(k_b_scatter, blocks(uint64_t(z.ntS) * 32, B_THREADS), B_THREADS, 0, s)(
         b.S, z.nS, z.ntS, b.sy_cnt, b.sy_spos, b.sy_idx, b.sy_kind, b.sy_relk, b.cs_of_sync);
     count_launch();
   }
-  k_b_search<<<blocks(std::max(g.W + 1, z.n_sync), 256), 256, 0, s>>>(b.ev, b.seg, g.W, b.sy_spos, z.n_sync, b.sy_start,
+  launch(k_b_search, blocks(std::max(g.W + 1, z.n_sync), 256), 256, 0, s)(b.ev, b.seg, g.W, b.sy_spos, z.n_sync, b.sy_start,
                                                                       b.sy_idx, b.sy_kind, b.bar, z.n_bar, b.acqrel,
                                                                       z.n_acqrel, b.sy_aux, b.lk_key, b.lk_k);
   count_launch();
@@ -1369,7 +1393,7 @@ void phaseB_sync(const Bufs& b, const Geo& g, Sizes& z, cudaStream_t s, Prof& p)
 
 void phaseC_walk(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, Prof& p) {
   p.begin("c_walk", double(z.n_sync) * 40);
-  k_c_walk<<<blocks(uint64_t(g.W) * 32, 128), 128, 0, s>>>(b.ev, g, b.seg, b.sy_start, b.sy_spos, b.sy_idx, b.sy_kind,
+  launch(k_c_walk, blocks(uint64_t(g.W) * 32, 128), 128, 0, s)(b.ev, g, b.seg, b.sy_start, b.sy_spos, b.sy_idx, b.sy_kind,
                                                            b.sy_N, b.sy_depth, b.sy_inner, b.sy_ver, b.sy_match,
                                                            b.sy_relk, b.incs_cnt, b.vcount, b.sy_agent, b.st);
   count_launch();
@@ -1384,31 +1408,31 @@ void phaseC_forced(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, 
   const uint32_t n = z.n_bar;
   if (!n) return;
   p.begin("c_forced", double(n) * 40 + double(z.n_sync) * 24);
-  k_fb_keys<<<blocks(n, 256), 256, 0, s>>>(b.ev, g, b.bar, n, b.fb_key, b.fb_val);
+  launch(k_fb_keys, blocks(n, 256), 256, 0, s)(b.ev, g, b.bar, n, b.fb_key, b.fb_val);
   count_launch();
   uint64_t mask = 0;  // keys 0..B (B: one-member barriers, left out of the walk)
   while (mask < g.B) mask = (mask << 1) | 1;
   const bool second = radix_sort_pairs(b.fb_key, b.fb_val, b.fb_key2, b.fb_val2, n, mask, b.scan_tmp, s, nullptr, {}, b.st);
   const uint64_t* skey = second ? b.fb_key2 : b.fb_key;
   const uint32_t* spos = second ? b.fb_val2 : b.fb_val;
-  k_fb_rank<<<blocks(uint64_t(n) + 1, 256), 256, 0, s>>>(b.ev, g, b.bar, skey, spos, n, b.fb_rank, b.fb_off,
+  launch(k_fb_rank, blocks(uint64_t(n) + 1, 256), 256, 0, s)(b.ev, g, b.bar, skey, spos, n, b.fb_rank, b.fb_off,
                                                           b.fb_blo);
   count_launch();
   scan_exclusive(b.fb_off, b.fb_off, size_t(n) + 1, nullptr, b.scan_tmp, s);
   cudaMemsetAsync(b.fb_boff, 0xFF, size_t(z.n_sync + 1) * 4, s);
-  k_fb_records<<<blocks(z.n_sync, 256), 256, 0, s>>>(b.ev, g, z.n_sync, n, b.sy_agent, b.sy_kind, b.sy_idx, b.sy_aux,
+  launch(k_fb_records, blocks(z.n_sync, 256), 256, 0, s)(b.ev, g, z.n_sync, n, b.sy_agent, b.sy_kind, b.sy_idx, b.sy_aux,
                                                      b.sy_N, b.fb_rank, b.fb_off, b.fb_rec);
   count_launch();
-  k_fb_walk<<<g.B, 32, 0, s>>>(g, z.n_sync, b.fb_blo, b.fb_off, b.fb_rec, b.fb_boff, b.st);
+  launch(k_fb_walk, g.B, 32, 0, s)(g, z.n_sync, b.fb_blo, b.fb_off, b.fb_rec, b.fb_boff, b.st);
   count_launch();
-  k_fb_apply<<<blocks(uint64_t(g.W) * 32, 128), 128, 0, s>>>(g, b.sy_start, b.fb_boff, b.sy_N);
+  launch(k_fb_apply, blocks(uint64_t(g.W) * 32, 128), 128, 0, s)(g, b.sy_start, b.fb_boff, b.sy_N);
   count_launch();
   p.end();
 }
 
 // the trace-order pass of phase D; filtered: only accesses the grouped order keeps
 void phaseD_trace(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, bool filtered) {
-  k_d_trace<<<blocks(z.N, 256), 256, 0, s>>>(b.ev, z.N, g, b.sy_start, b.sy_idx, b.d_index, z.d_shift, z.d_nw,
+  launch(k_d_trace, blocks(z.N, 256), 256, 0, s)(b.ev, z.N, g, b.sy_start, b.sy_idx, b.d_index, z.d_shift, z.d_nw,
                                               reinterpret_cast<const uint2*>(b.sy_match), b.vcount, b.acc_info, b.st,
                                               (reinterpret_cast<uintptr_t>(b.ev) & 15) == 0, b.wl_bits,
                                               filtered ? z.wl_log2 : 0u, z.comp_lo, z.comp_span);
@@ -1418,13 +1442,13 @@ void phaseD_trace(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, b
 void phaseD_gaps(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, Prof& p) {
   p.begin("d_gaps", double(z.n_acc) * (4 + 16 + 16), s);
   const uint32_t tail_from = blocks(z.n_sync, 256);
-  k_d_index<<<tail_from + blocks(uint64_t(g.W) * 32, 256), 256, 0, s>>>(b.sy_idx, b.sy_agent, b.sy_start, z.n_sync, g.W,
+  launch(k_d_index, tail_from + blocks(uint64_t(g.W) * 32, 256), 256, 0, s)(b.sy_idx, b.sy_agent, b.sy_start, z.n_sync, g.W,
                                                                         z.d_shift, z.d_nw, b.d_index, tail_from, b.sy_N, b.sy_depth,
                                                                         b.sy_ver, reinterpret_cast<uint2*>(b.sy_match));
   count_launch();
   phaseD_trace(b, g, z, s, true);
   if (z.n_sync) {
-    k_d_fill<<<blocks(uint64_t(z.n_sync) * D_LANES, 256), 256, 0, s>>>(
+    launch(k_d_fill, blocks(uint64_t(z.n_sync) * D_LANES, 256), 256, 0, s)(
         b.ev, g, z.n_sync, b.S, b.seg, b.sy_start, b.sy_agent, b.sy_spos, b.sy_N, b.sy_depth, b.sy_ver, b.incs_cnt,
         b.vcount, b.acc_info, b.incs_idx, b.incs_ver, b.incs_k, b.incs_key, b.incs_wr, b.st);
     count_launch();
@@ -1441,7 +1465,7 @@ void phaseE_locks(Bufs& b, const Geo& g, const Sizes& z, uint64_t lock_mask, cud
     std::swap(b.lk_key, b.lk_key2);
     std::swap(b.lk_k, b.lk_k2);
   }
-  k_e_flags<<<blocks(n, 256), 256, 0, s>>>(b.lk_key, b.lk_k, n, b.sy_kind, b.lk_flags, b.lk_rank);
+  launch(k_e_flags, blocks(n, 256), 256, 0, s)(b.lk_key, b.lk_k, n, b.sy_kind, b.lk_flags, b.lk_rank);
   count_launch();
   p.end();
 }
@@ -1468,20 +1492,20 @@ void phaseE_walk(Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, Prof& p)
   p.begin("e_walk", double(n) * 32);
   const uint32_t* newflag = b.lk_rank;
   const uint32_t* newscan = b.lk_k2;
-  k_e_assign<<<blocks(n, 256), 256, 0, s>>>(b.ev, g, b.lk_k, n, newflag, b.lk_csid, newscan, b.sy_kind, b.sy_idx,
+  launch(k_e_assign, blocks(n, 256), 256, 0, s)(b.ev, g, b.lk_k, n, newflag, b.lk_csid, newscan, b.sy_kind, b.sy_idx,
                                             b.sy_N, b.sy_relk, b.cs_of_sync, b.cs_agent, b.cs_sid, b.cs_epoch,
                                             b.cs_rel_idx, b.cs_rel_epoch, b.cs_lock, b.lock_first, b.lock_cs_lo, b.incs_cnt,
                                             b.sy_start, b.cs_exp, b.cs_r0);
   count_launch();
   // (the sorted lock ids were last read for the new-lock flags)
   auto* rec = reinterpret_cast<uint2*>(b.lk_key);
-  k_e_assign_rel<<<blocks(n, 256), 256, 0, s>>>(b.lk_k, n, b.sy_kind, b.sy_match, b.cs_of_sync, b.cs_sid, b.cs_parent,
+  launch(k_e_assign_rel, blocks(n, 256), 256, 0, s)(b.lk_k, n, b.sy_kind, b.sy_match, b.cs_of_sync, b.cs_sid, b.cs_parent,
                                                 rec);
   count_launch();
   const uint64_t words = uint64_t(lock_stride(g)) * (z.n_cs + 2 * uint64_t(z.n_exp)) + 64;
   const uint32_t stride = words == z.pool_cap ? lock_stride(g) : 0;
   auto ew = lock_scope_cap(g.B) == kLockScopesSmall ? k_e_walk<kLockScopesSmall> : k_e_walk<kLockScopesLarge>;
-  ew<<<blocks(z.n_locks, E_WARPS), E_WARPS * 32, 0, s>>>(rec, b.lk_k, b.lock_first, z.n_locks, b.sy_idx, b.acq_dep_off,
+  launch(ew, blocks(z.n_locks, E_WARPS), E_WARPS * 32, 0, s)(rec, b.lk_k, b.lock_first, z.n_locks, b.sy_idx, b.acq_dep_off,
                                                          b.acq_dep_cnt, b.dep_pool, stride, z.pool_cap, z.n_cs, b.st);
   count_launch();
   p.end();
@@ -1491,7 +1515,7 @@ void phaseF_expand(const Bufs& b, const Sizes& z, cudaStream_t s, Prof& p) {
   if (!z.n_incs || !z.n_exp) return;
   p.begin("f_expand", double(z.n_incs) * 24 + double(z.n_exp) * 20);
   scan_exclusive(b.cs_exp, b.cs_exp, z.n_cs, nullptr, b.scan_tmp, s);
-  k_f_expand<<<blocks(z.n_incs, 256), 256, 0, s>>>(b.incs_k, z.n_incs, b.incs_key, b.incs_wr, b.sy_inner,
+  launch(k_f_expand, blocks(z.n_incs, 256), 256, 0, s)(b.incs_k, z.n_incs, b.incs_key, b.incs_wr, b.sy_inner,
                                                    b.cs_of_sync, b.cs_parent, b.cs_lock, b.cs_exp, b.cs_r0, b.ex_info,
                                                    b.ex_key, b.ex_val, b.st);
   count_launch();
@@ -1509,7 +1533,7 @@ void phaseF_deps(Bufs& b, const Geo& g, const Sizes& z, uint64_t key_mask, cudaS
   p.end();
   p.begin("f_deps", double(n) * 32);
   auto fw = lock_scope_cap(g.B) == kLockScopesSmall ? k_f_walk<kLockScopesSmall> : k_f_walk<kLockScopesLarge>;
-  fw<<<blocks(n, 128), 128, 0, s>>>(b.ex_key, b.ex_val, n, b.ex_info, b.cs_sid, b.cs_rel_idx, b.ex_dep_off,
+  launch(fw, blocks(n, 128), 128, 0, s)(b.ex_key, b.ex_val, n, b.ex_info, b.cs_sid, b.cs_rel_idx, b.ex_dep_off,
                                     b.ex_dep_cnt, b.dep_pool, z.pool_cap, b.st);
   count_launch();
   p.end();

@@ -74,6 +74,7 @@ __device__ __forceinline__ void store_items(uint32_t* out, size_t base, size_t n
 }
 
 __global__ void __launch_bounds__(SC_ONE_THREADS) k_scan_one(ScanBatch b) {
+  grid_begin();
   const ScanJob job = b.job[blockIdx.x];
   const size_t base = size_t(threadIdx.x) * SC_ONE_ITEMS;
   uint32_t v[SC_ONE_ITEMS], s = 0;
@@ -93,6 +94,7 @@ __global__ void __launch_bounds__(SC_ONE_THREADS) k_scan_one(ScanBatch b) {
 }
 
 __global__ void __launch_bounds__(SC_THREADS) k_scan_reduce(const uint32_t* in, size_t n, uint32_t* sums) {
+  grid_begin();
   const size_t base = size_t(blockIdx.x) * SC_TILE + size_t(threadIdx.x) * SC_ITEMS;
   uint32_t v[SC_ITEMS], s = 0;
   load_items<SC_ITEMS>(in, base, n, v);
@@ -104,6 +106,7 @@ __global__ void __launch_bounds__(SC_THREADS) k_scan_reduce(const uint32_t* in, 
 }
 
 __global__ void __launch_bounds__(SC_ONE_THREADS) k_scan_sums(uint32_t* sums, uint32_t nb, uint32_t* total) {
+  grid_begin();
   __shared__ uint32_t tot;
   uint32_t carry = 0;
   for (uint32_t base = 0; base < nb; base += SC_ONE_THREADS) {
@@ -121,6 +124,7 @@ __global__ void __launch_bounds__(SC_ONE_THREADS) k_scan_sums(uint32_t* sums, ui
 // block writes the total
 __global__ void __launch_bounds__(SC_THREADS) k_scan_apply(const uint32_t* in, uint32_t* out, size_t n,
                                                            const uint32_t* sums, bool scanned, uint32_t* total) {
+  grid_begin();
   __shared__ uint32_t tot, before;
   uint32_t prefix;
   if (scanned) {
@@ -191,6 +195,7 @@ constexpr int HI_THREADS = 512;
 __global__ void __launch_bounds__(HI_THREADS) k_sweep_hist(const uint64_t* keys, size_t n, const uint32_t* n_dev,
                                                            const __grid_constant__ SweepPlan pl, uint32_t* hist, uint4* status,
                                                            size_t status_quads, RadixKeep kp) {
+  grid_begin();
   __shared__ uint32_t h[kMaxPasses * 256];
   for (int i = threadIdx.x; i < pl.passes * 256; i += HI_THREADS) h[i] = 0;
   const size_t first = size_t(blockIdx.x) * HI_THREADS + threadIdx.x, step = size_t(gridDim.x) * HI_THREADS;
@@ -266,6 +271,7 @@ constexpr size_t sweep_smem() {
 // of one digit's run.
 template <int THREADS, int ITEMS>
 __global__ void __launch_bounds__(THREADS, ITEMS <= 4 ? 6 : 4) k_sweep(const __grid_constant__ SweepArgs a) {
+  grid_begin();
   constexpr int WARPS = THREADS / 32, TILE = THREADS * ITEMS;
   static_assert(THREADS >= 256, "a thread per digit");
   extern __shared__ __align__(16) unsigned char dyn[];
@@ -397,6 +403,7 @@ constexpr int ONE_THREADS = 1024, ONE_ITEMS = 4, ONE_MAX = ONE_THREADS * ONE_ITE
 __global__ void __launch_bounds__(ONE_THREADS) k_sort_one(const uint64_t* kin, const uint32_t* vin, uint64_t* kout,
                                                           uint32_t* vout, uint32_t n, const uint32_t* n_dev,
                                                           const __grid_constant__ SweepPlan pl, RadixKeep kp) {
+  grid_begin();
   constexpr int WARPS = ONE_THREADS / 32;
   extern __shared__ __align__(16) unsigned char dyn[];
   uint64_t* const sk = reinterpret_cast<uint64_t*>(dyn);
@@ -485,7 +492,7 @@ void launch_sweep(const SweepArgs& a, uint32_t tiles, cudaStream_t s) {
   constexpr size_t smem = sweep_smem<THREADS, ITEMS>();
   if (smem > 48 * 1024)
     cudaFuncSetAttribute(k_sweep<THREADS, ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-  k_sweep<THREADS, ITEMS><<<tiles, THREADS, smem, s>>>(a);
+  launch(k_sweep<THREADS, ITEMS>, tiles, THREADS, smem, s)(a);
   count_launch();
 }
 
@@ -494,12 +501,13 @@ void launch_sweep(const SweepArgs& a, uint32_t tiles, cudaStream_t s) {
 size_t scan_tmp_need(size_t n) { return (n + SC_TILE - 1) / SC_TILE + 1; }
 
 void scan_small(const ScanBatch& b, int jobs, cudaStream_t s) {
-  k_scan_one<<<jobs, SC_ONE_THREADS, 0, s>>>(b);
+  launch(k_scan_one, jobs, SC_ONE_THREADS, 0, s)(b);
   count_launch();
 }
 
 namespace {
 __global__ void __launch_bounds__(256) k_fill(const __grid_constant__ FillBatch b) {
+  grid_begin();
   const size_t t = size_t(blockIdx.x) * blockDim.x + threadIdx.x, all = size_t(gridDim.x) * blockDim.x;
   for (int j = 0; j < b.n; ++j) {
     const uint32_t v = b.job[j].value;
@@ -510,28 +518,29 @@ __global__ void __launch_bounds__(256) k_fill(const __grid_constant__ FillBatch 
   }
 }
 __global__ void k_read_back(const DevStatus* st, const __grid_constant__ ReadBack r, DevStatus* st_out, uint32_t* val_out) {
+  grid_begin();
   const int t = threadIdx.x;
   constexpr int words = sizeof(DevStatus) / 4;
   static_assert(sizeof(DevStatus) % 4 == 0 && words + 8 <= 64);
   if (t < words) reinterpret_cast<uint32_t*>(st_out)[t] = reinterpret_cast<const uint32_t*>(st)[t];
   if (t < r.n) val_out[t] = *r.word[t];
 }
-__global__ void k_status_init(DevStatus* st, const __grid_constant__ DevStatus v) { *st = v; }
+__global__ void k_status_init(DevStatus* st, const __grid_constant__ DevStatus v) { grid_begin(); *st = v; }
 }  // namespace
 
 void fill_all(const FillBatch& b, cudaStream_t s) {
   size_t most = 0;
   for (int j = 0; j < b.n; ++j) most = std::max(most, b.job[j].words);
   if (!b.n) return;
-  k_fill<<<unsigned(std::min<size_t>((most + 1023) / 1024, 152 * 8)), 256, 0, s>>>(b);
+  launch(k_fill, unsigned(std::min<size_t>((most + 1023) / 1024, 152 * 8)), 256, 0, s)(b);
   count_launch();
 }
 void read_back_to(const DevStatus* st, const ReadBack& r, DevStatus* st_out, uint32_t* val_out, cudaStream_t s) {
-  k_read_back<<<1, 64, 0, s>>>(st, r, st_out, val_out);
+  launch(k_read_back, 1, 64, 0, s)(st, r, st_out, val_out);
   count_launch();
 }
 void status_init(DevStatus* st, const DevStatus& v, cudaStream_t s) {
-  k_status_init<<<1, 1, 0, s>>>(st, v);
+  launch(k_status_init, 1, 1, 0, s)(st, v);
   count_launch();
 }
 
@@ -550,14 +559,14 @@ void scan_exclusive(const uint32_t* in, uint32_t* out, size_t n, uint32_t* total
     return;
   }
   const uint32_t nb = uint32_t((n + SC_TILE - 1) / SC_TILE);
-  k_scan_reduce<<<nb, SC_THREADS, 0, s>>>(in, n, tmp);
+  launch(k_scan_reduce, nb, SC_THREADS, 0, s)(in, n, tmp);
   count_launch();
   const bool own_sums = nb <= SC_SUMS;
   if (!own_sums) {
-    k_scan_sums<<<1, SC_ONE_THREADS, 0, s>>>(tmp, nb, total_dev);
+    launch(k_scan_sums, 1, SC_ONE_THREADS, 0, s)(tmp, nb, total_dev);
     count_launch();
   }
-  k_scan_apply<<<nb, SC_THREADS, 0, s>>>(in, out, n, tmp, !own_sums, total_dev);
+  launch(k_scan_apply, nb, SC_THREADS, 0, s)(in, out, n, tmp, !own_sums, total_dev);
   count_launch();
 }
 
@@ -621,7 +630,7 @@ bool radix_sort_pairs(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, si
   if (n <= size_t(ONE_MAX)) {
     constexpr size_t smem = size_t(ONE_MAX) * 12 + size_t(ONE_THREADS / 32) * 256 * 4;
     cudaFuncSetAttribute(k_sort_one, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    k_sort_one<<<1, ONE_THREADS, smem, s>>>(k0, v0, k1, v1, uint32_t(n), n_dev, pl, keep);
+    launch(k_sort_one, 1, ONE_THREADS, smem, s)(k0, v0, k1, v1, uint32_t(n), n_dev, pl, keep);
     count_launch();
     return true;
   }
@@ -632,7 +641,7 @@ bool radix_sort_pairs(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, si
   auto* status = reinterpret_cast<unsigned long long*>((reinterpret_cast<uintptr_t>(tmp + kSweepHead) + 15) & ~uintptr_t(15));
   cudaMemsetAsync(tmp, 0, kSweepHead * 4, s);
   const uint32_t hist_blocks = uint32_t(std::min<size_t>((n + 2047) / 2048, 152 * 4));
-  k_sweep_hist<<<hist_blocks, HI_THREADS, 0, s>>>(k0, n, n_dev, pl, hist, reinterpret_cast<uint4*>(status),
+  launch(k_sweep_hist, hist_blocks, HI_THREADS, 0, s)(k0, n, n_dev, pl, hist, reinterpret_cast<uint4*>(status),
                                                  size_t(tiles) * 128, keep);
   count_launch();
   bool in_second = false;

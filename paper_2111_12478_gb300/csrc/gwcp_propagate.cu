@@ -898,6 +898,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_propagate(const __grid_constant__ P
 // joins, over the sections that it is held in.
 __global__ void k_plan_counts(PropArgs a, uint32_t n_cs, const uint32_t* cs_epoch, const uint32_t* cs_rel_epoch,
                               uint32_t n_incs, uint32_t* cnt) {
+  grid_begin();
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n_cs) a.recmeta[i] = make_uint4(a.cs_agent[i] | (a.cs_sid[i] << 16), cs_epoch[i], a.cs_rel_idx[i], cs_rel_epoch[i]);
   if (i >= n_incs) return;
@@ -946,6 +947,7 @@ __device__ __forceinline__ void plan_sync(const PropArgs& a, const uint32_t* sy_
 // list (its sections from the inside out).
 __global__ void k_plan(const __grid_constant__ PropArgs a, const uint32_t* sy_kind_, const uint32_t* sy_ver, uint32_t n_sync,
                        const uint32_t* flat_off, uint32_t* flat, uint32_t n_incs) {
+  grid_begin();
   const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
   if (a.st->code) return;  // (the lists are incomplete, the walkers stand down)
   if (r < n_sync) plan_sync(a, sy_kind_, sy_ver, r);
@@ -1114,7 +1116,7 @@ int phaseG_propagate(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s
   p.begin("g_plan", double(z.n_sync + z.n_incs) * 64 + double(z.n_cs) * 2 * g.RW * 4);
   if (z.n_cs) {
     const uint32_t most = std::max(z.n_cs, z.n_incs);
-    k_plan_counts<<<(most + 255) / 256, 256, 0, s>>>(a, z.n_cs, b.cs_epoch, b.cs_rel_epoch, z.n_incs, b.flat_off);
+    launch(k_plan_counts, (most + 255) / 256, 256, 0, s)(a, z.n_cs, b.cs_epoch, b.cs_rel_epoch, z.n_incs, b.flat_off);
     count_launch();
   }
   FillBatch f;
@@ -1133,7 +1135,7 @@ int phaseG_propagate(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s
   }
   if (z.n_sync) {  // (no in-section access without a synchronisation entry)
     const uint32_t most = std::max(z.n_sync, z.n_incs);
-    k_plan<<<(most + 255) / 256, 256, 0, s>>>(a, b.sy_kind, b.sy_ver, z.n_sync, b.flat_off, b.flat, z.n_incs);
+    launch(k_plan, (most + 255) / 256, 256, 0, s)(a, b.sy_kind, b.sy_ver, z.n_sync, b.flat_off, b.flat, z.n_incs);
     count_launch();
   }
   p.end();

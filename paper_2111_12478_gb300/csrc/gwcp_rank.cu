@@ -36,17 +36,20 @@ enum { A_N, A_R, A_W, A_A, A_CTA, A_DEV, A_INS, A_INSW, A_FIRST, A_SW, A_CSW, A_
 inline uint32_t nblk(uint64_t n, uint32_t t) { return uint32_t((n + t - 1) / t); }
 
 __global__ void k_rk_incs(const uint32_t* incs_idx, uint32_t n_incs, uint32_t* bits) {
+  grid_begin();
   const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r < n_incs) atomicOr(bits + (incs_idx[r] >> 5), 1u << (incs_idx[r] & 31));
 }
 
 __global__ void k_rk_flags(const uint64_t* key, uint32_t n, uint32_t* flag) {
+  grid_begin();
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) flag[i] = (i == 0 || key[i] != key[i - 1]) ? 1u : 0u;
   if (i == n) flag[n] = 0u;  // so that the scan's total counts the locations
 }
 
 __global__ void k_rk_starts(const uint32_t* flag, const uint32_t* excl, uint32_t n, uint32_t* loc_start) {
+  grid_begin();
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n && flag[i]) loc_start[excl[i]] = i;
   if (i == 0) loc_start[excl[n]] = n;  // excl[n] = number of locations
@@ -67,6 +70,7 @@ struct AccArgs {
 // location inside the warp; a run that the warp holds whole is stored, one that crosses
 // a warp boundary is added atomically.
 __global__ void k_rk_acc(AccArgs a) {
+  grid_begin();
   const uint32_t lane = threadIdx.x & 31;
   const uint32_t base = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32;
   if (base >= a.n) return;
@@ -168,6 +172,7 @@ struct FinalArgs {
 };
 
 __global__ void k_rk_final(FinalArgs a) {
+  grid_begin();
   const uint32_t L = blockIdx.x * blockDim.x + threadIdx.x;
   if (L >= *a.n_loc) return;
   const uint32_t lo = a.loc_start[L], hi = a.loc_start[L + 1];
@@ -226,6 +231,7 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1
 // rows), layer 3 a dot product over the accumulator fragments and the 4 lanes of a row.
 __global__ void __launch_bounds__(256) k_mlp_fwd(const float* theta, const float* feat, const uint32_t* n_dev,
                                                  uint32_t n_host, float* score) {
+  grid_begin();
   __shared__ uint32_t sW1[NH * NF / 2];  // bf16 pairs, row-major [64][16]
   __shared__ uint32_t sW2[NH * NH / 2];  // [64][64]
   __shared__ float sb1[NH], sb2[NH], sw3[NH];
@@ -317,6 +323,7 @@ template <bool PART>
 __global__ void __launch_bounds__(GR_THREADS, 2) k_mlp_grad(const float* theta, const float* feat, const float* y,
                                                             uint32_t lo, uint32_t hi, float pos_weight, float inv_b,
                                                             float* grad, float* loss) {
+  grid_begin();
   constexpr int LD2 = NH + 1;  // padded rows of W2: read by rows and by columns
   __shared__ float sW1t[NF * NH];  // [f][k]
   __shared__ float sW2[NH * LD2];  // [n][k]
@@ -501,6 +508,7 @@ __global__ void __launch_bounds__(GR_THREADS, 2) k_mlp_grad(const float* theta, 
 // parameter is the loss.
 __global__ void __launch_bounds__(128) k_adam(float* theta, float* m, float* v, const float* grad, uint32_t parts,
                                               double* loss_acc, float lr, const uint32_t* step, uint32_t q) {
+  grid_begin();
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p > N_PARAMS) return;
   double sum = 0;
@@ -520,10 +528,11 @@ __global__ void __launch_bounds__(128) k_adam(float* theta, float* m, float* v, 
   theta[p] -= lr * (mm * c1) / (sqrtf(vv * c2) + 1e-8f);
 }
 
-__global__ void k_step_add(uint32_t* step, uint32_t n) { *step += n; }
+__global__ void k_step_add(uint32_t* step, uint32_t n) { grid_begin(); *step += n; }
 
 // end of an epoch: its accumulated loss into losses[epoch], then the next epoch
 __global__ void k_epoch_end(double* loss_acc, float* losses, uint32_t* epoch) {
+  grid_begin();
   losses[*epoch] = float(*loss_acc);
   *loss_acc = 0;
   ++*epoch;
@@ -534,6 +543,7 @@ __global__ void k_epoch_end(double* loss_acc, float* losses, uint32_t* epoch) {
 // key = (16 bits of the score, high scores first) << 32 | location ordinal
 __global__ void k_rk_compose(const uint32_t* flag, const uint32_t* excl, const float* score, uint32_t n, uint64_t* rkey,
                              uint32_t* rval) {
+  grid_begin();
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const uint32_t loc = excl[i] + flag[i] - 1u;
@@ -546,6 +556,7 @@ __global__ void k_rk_compose(const uint32_t* flag, const uint32_t* excl, const f
 
 __global__ void k_rk_gather(const uint32_t* pos, uint32_t n, const uint64_t* key, const uint32_t* idx, uint64_t* key_out,
                             uint32_t* idx_out) {
+  grid_begin();
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const uint32_t p = pos[i];
@@ -554,6 +565,7 @@ __global__ void k_rk_gather(const uint32_t* pos, uint32_t n, const uint64_t* key
 }
 
 __global__ void k_stamp(unsigned long long* at) {
+  grid_begin();
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   *at = t;
@@ -562,7 +574,7 @@ __global__ void k_stamp(unsigned long long* at) {
 }  // namespace
 
 void stamp_now(unsigned long long* at, cudaStream_t s) {
-  k_stamp<<<1, 1, 0, s>>>(at);
+  launch(k_stamp, 1, 1, 0, s)(at);
   count_launch();
 }
 
@@ -586,22 +598,22 @@ void rank_features(const RankIn& in, uint32_t* tmp, size_t bits_words, float* fe
   uint32_t* bits = in.bits;
   cudaMemsetAsync(bits, 0, bits_words * 4, s);
   if (in.n_incs) {
-    k_rk_incs<<<nblk(in.n_incs, 256), 256, 0, s>>>(in.incs_idx, in.n_incs, bits);
+    launch(k_rk_incs, nblk(in.n_incs, 256), 256, 0, s)(in.incs_idx, in.n_incs, bits);
     count_launch();
   }
-  k_rk_flags<<<nblk(uint64_t(n) + 1, 256), 256, 0, s>>>(in.key, n, flag);
+  launch(k_rk_flags, nblk(uint64_t(n) + 1, 256), 256, 0, s)(in.key, n, flag);
   count_launch();
   scan_exclusive(flag, excl, size_t(n) + 1, n_loc_dev, scan_tmp, s);
-  k_rk_starts<<<nblk(n, 256), 256, 0, s>>>(flag, excl, n, loc_start);
+  launch(k_rk_starts, nblk(n, 256), 256, 0, s)(flag, excl, n, loc_start);
   count_launch();
   cudaMemsetAsync(cnt, 0, size_t(A_COUNT) * st * 4, s);
   cudaMemsetAsync(masks, 0, 2 * st * 8, s);
   AccArgs a{in.key, in.idx, in.info, flag, excl, loc_start, bits, n, uint32_t(st), cnt, masks};
-  k_rk_acc<<<nblk(uint64_t(nblk(n, 32)) * 32, 256), 256, 0, s>>>(a);
+  launch(k_rk_acc, nblk(uint64_t(nblk(n, 32)) * 32, 256), 256, 0, s)(a);
   count_launch();
   FinalArgs f{in.key, in.idx, loc_start, n_loc_dev, n, uint32_t(st), cnt, masks, in.acqrel, in.bar,
               in.n_acqrel, in.n_bar, feat, loc_key};
-  k_rk_final<<<nblk(n, 256), 256, 0, s>>>(f);
+  launch(k_rk_final, nblk(n, 256), 256, 0, s)(f);
   count_launch();
 }
 
@@ -612,7 +624,7 @@ void rank_scores(const float* theta, const float* feat, const uint32_t* n_dev, u
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const uint32_t tiles = nblk(n_bound, 16);
   const uint32_t grid = std::max(1u, std::min<uint32_t>(nblk(tiles, 8), uint32_t(sms) * 8));
-  k_mlp_fwd<<<grid, 256, 0, s>>>(theta, feat, n_dev, n_bound, score);
+  launch(k_mlp_fwd, grid, 256, 0, s)(theta, feat, n_dev, n_bound, score);
   count_launch();
 }
 
@@ -623,12 +635,12 @@ void rank_order(const RankIn& in, const uint32_t* tmp, const float* score, uint6
   const size_t st = size_t(n) + 1;
   const uint32_t* flag = tmp;
   const uint32_t* excl = flag + st;
-  k_rk_compose<<<nblk(n, 256), 256, 0, s>>>(flag, excl, score, n, rkey, rval);
+  launch(k_rk_compose, nblk(n, 256), 256, 0, s)(flag, excl, score, n, rkey, rval);
   count_launch();
   uint64_t mask = 0xFFFFull << 32;
   for (uint64_t v = n; v; v >>= 1) mask |= (mask & 0xFFFFFFFFull) << 1 | 1;
   const bool second = radix_sort_pairs(rkey, rval, rkey2, rval2, n, mask, sort_tmp, s);
-  k_rk_gather<<<nblk(n, 256), 256, 0, s>>>(second ? rval2 : rval, n, in.key, in.idx, key_out, idx_out);
+  launch(k_rk_gather, nblk(n, 256), 256, 0, s)(second ? rval2 : rval, n, in.key, in.idx, key_out, idx_out);
   count_launch();
 }
 
@@ -648,7 +660,7 @@ int rank_grad(const float* theta, const float* feat, const float* y, uint32_t n,
   if (!n) return GWCP_OK;
   // the CTAs' sums meet in float atomics, each a rounding: 128 rows per CTA keep their number
   // low (3,001 rows: an error of 0.9e-7 of the norm; with 16 rows per CTA, 2.0e-7)
-  k_mlp_grad<false><<<grad_ctas(n, 128), GR_THREADS, 0, s>>>(theta, feat, y, 0, n, pos_weight, 1.0f / float(n), grad, loss);
+  launch(k_mlp_grad<false>, grad_ctas(n, 128), GR_THREADS, 0, s)(theta, feat, y, 0, n, pos_weight, 1.0f / float(n), grad, loss);
   count_launch();
   return cudaGetLastError() == cudaSuccess ? GWCP_OK : GWCP_ERR_CUDA;
 }
@@ -665,15 +677,15 @@ int rank_epoch(float* theta, const float* feat, const float* y, uint32_t n, uint
   for (uint32_t q = 0; q < nb; ++q) {
     const uint32_t lo = q * batch, hi = uint32_t(std::min<uint64_t>(n, uint64_t(lo) + batch));
     const uint32_t ctas = grad_ctas(hi - lo, GR_ROWS);
-    k_mlp_grad<true><<<ctas, GR_THREADS, 0, s>>>(theta, feat, y, lo, hi, pos_weight,
+    launch(k_mlp_grad<true>, ctas, GR_THREADS, 0, s)(theta, feat, y, lo, hi, pos_weight,
                                                  1.0f / float(hi - lo) / float(nb), part, nullptr);
     count_launch();
-    k_adam<<<nblk(N_PARAMS + 1, 128), 128, 0, s>>>(theta, m, v, part, ctas, loss_acc, lr, ctr, q);
+    launch(k_adam, nblk(N_PARAMS + 1, 128), 128, 0, s)(theta, m, v, part, ctas, loss_acc, lr, ctr, q);
     count_launch();
   }
-  k_step_add<<<1, 1, 0, s>>>(ctr, nb);
+  launch(k_step_add, 1, 1, 0, s)(ctr, nb);
   count_launch();
-  k_epoch_end<<<1, 1, 0, s>>>(loss_acc, losses, ctr + 1);
+  launch(k_epoch_end, 1, 1, 0, s)(loss_acc, losses, ctr + 1);
   count_launch();
   return cudaGetLastError() == cudaSuccess ? GWCP_OK : GWCP_ERR_CUDA;
 }

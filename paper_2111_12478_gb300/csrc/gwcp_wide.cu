@@ -676,6 +676,7 @@ __global__ void __launch_bounds__(1024, MINB) k_prop_wide(const __grid_constant_
 // ---- check ---------------------------------------------------------------------------
 
 __global__ void k_wc_runflags(const uint64_t* key, uint32_t n, uint32_t* flag) {
+  grid_begin();
   const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p < n) flag[p] = (p == 0 || key[p] != key[p - 1]) ? 1u : 0u;
 }
@@ -687,6 +688,7 @@ __global__ void k_wc_runflags(const uint64_t* key, uint32_t n, uint32_t* flag) {
 __global__ void k_wc_compose(const uint32_t* run_excl, const uint32_t* flag, const uint32_t* idx,
                              const AccInfo* info, uint32_t n, uint64_t* ck, uint32_t* cv, uint32_t* s_who,
                              uint32_t* s_row, uint32_t* s_ep) {
+  grid_begin();
   const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
   const uint32_t run = run_excl[p] + flag[p] - 1;
@@ -701,15 +703,18 @@ __global__ void k_wc_compose(const uint32_t* run_excl, const uint32_t* flag, con
 // A location that no write-class access touches has no races (two reads never conflict):
 // its accesses are left out of the regrouping, so the check finds no partner groups there.
 __global__ void k_wc_runwrite(const uint64_t* ck, uint32_t n, uint32_t* run_w) {
+  grid_begin();
   const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p < n && ((ck[p] >> 13) & 3u) != C_READ) run_w[ck[p] >> 15] = 1u;
 }
 __global__ void k_wc_keep(const uint64_t* ck, uint32_t n, const uint32_t* run_w, uint32_t* keep) {
+  grid_begin();
   const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p < n) keep[p] = run_w[ck[p] >> 15];
 }
 __global__ void k_wc_compact(const uint64_t* ck, const uint32_t* cv, const uint32_t* keep, const uint32_t* kpos,
                              uint32_t n, uint64_t* ck2, uint32_t* cv2) {
+  grid_begin();
   const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p < n && keep[p]) {
     ck2[kpos[p]] = ck[p];
@@ -720,12 +725,14 @@ __global__ void k_wc_compact(const uint64_t* ck, const uint32_t* cv, const uint3
 // group starts over the sorted composite keys (the first *n_dev of n), and per (run, class)
 // group counts
 __global__ void k_wc_groupflags(const uint64_t* ck, uint32_t n, const uint32_t* n_dev, uint32_t* gflag) {
+  grid_begin();
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) gflag[i] = (i < *n_dev && (i == 0 || ck[i] != ck[i - 1])) ? 1u : 0u;
 }
 
 __global__ void k_wc_groups(const uint64_t* ck, const uint32_t* gflag, const uint32_t* gexcl, uint32_t n,
                             uint32_t* grp_lo, uint32_t* grp_agent, uint32_t* rc_cnt) {
+  grid_begin();
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n || !gflag[i]) return;
   const uint32_t gi = gexcl[i];
@@ -987,6 +994,7 @@ __device__ __forceinline__ uint32_t flush_warp(const WideCheckArgs& a, uint32_t 
 // walked here); otherwise the lanes of their warp share them (a ranked check keeps its order).
 template <int REP, bool ASIDE>
 __global__ void __launch_bounds__(kCheckThreads, 8) k_wc_check(const __grid_constant__ WideCheckArgs a) {
+  grid_begin();
   if (a.st->code) return;  // (the access records or clocks are incomplete)
   constexpr uint32_t kWarps = kCheckThreads / 32;
   __shared__ uint32_t s_cnt[kWarps];
@@ -1046,6 +1054,7 @@ __global__ void __launch_bounds__(kCheckThreads, 8) k_wc_check(const __grid_cons
 // at one hot location (neighbours in the order) spread over all SMs.
 template <int REP>
 __global__ void __launch_bounds__(kCheckThreads, 6) k_wc_big(const __grid_constant__ WideCheckArgs a) {
+  grid_begin();
   if (a.st->code) return;  // (the access records or clocks are incomplete)
   constexpr uint32_t kWarps = kCheckThreads / 32;
   __shared__ uint32_t s_cnt[kWarps];
@@ -1078,6 +1087,7 @@ __global__ void __launch_bounds__(kCheckThreads, 6) k_wc_big(const __grid_consta
 // location runs and (class, agent) groups of the composite keys (the first *n_dev keys)
 __global__ void k_gr_flags(const uint64_t* ck, uint32_t n, const uint32_t* n_dev, uint32_t* run_flag,
                            uint32_t* grp_flag) {
+  grid_begin();
   const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
   if (p >= *n_dev) {
@@ -1095,6 +1105,7 @@ __global__ void k_gr_flags(const uint64_t* ck, uint32_t n, const uint32_t* n_dev
 __global__ void k_gr_groups(const uint64_t* ck, const uint32_t* run_flag, const uint32_t* run_excl,
                             const uint32_t* gflag, const uint32_t* gexcl, const uint32_t* n_dev, uint32_t* grp_lo,
                             uint32_t* grp_agent, uint32_t* rc_off) {
+  grid_begin();
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   const uint32_t n = *n_dev;
   if (i >= n) return;
@@ -1117,6 +1128,7 @@ __global__ void k_gr_groups(const uint64_t* ck, const uint32_t* run_flag, const 
 // the fields of each access record the check needs, copied into the primary order
 __global__ void k_wc_fields(const uint32_t* idx, const AccInfo* info, const uint32_t* n_dev, uint32_t* s_who,
                             uint32_t* s_row, uint32_t* s_ep) {
+  grid_begin();
   const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= *n_dev) return;
   const AccInfo in = info[idx[p]];
@@ -1126,6 +1138,7 @@ __global__ void k_wc_fields(const uint32_t* idx, const AccInfo* info, const uint
 }
 
 __global__ void k_wc_grp_end(const uint32_t* n_groups, const uint32_t* n_dev, uint32_t* grp_lo) {
+  grid_begin();
   grp_lo[*n_groups] = *n_dev;
 }
 
@@ -1190,10 +1203,10 @@ void phaseI_wide_group(Bufs& b, const Geo& g, Sizes& z, uint32_t* tmp, cudaStrea
   const uint32_t n = z.n_acc;
   if (!n) return;
   p.begin("i_wide_group", double(n) * (8 + 4 + 16 + 12 * 3 * 5 + 16), s);
-  k_wc_runflags<<<nblk(n, 256), 256, 0, s>>>(b.acc_key, n, b.wc_flag);
+  launch(k_wc_runflags, nblk(n, 256), 256, 0, s)(b.acc_key, n, b.wc_flag);
   count_launch();
   scan_exclusive(b.wc_flag, b.wc_run, n, b.wc_run + n, tmp, s);
-  k_wc_compose<<<nblk(n, 256), 256, 0, s>>>(b.wc_run, b.wc_flag, b.acc_idx, b.acc_info, n, b.wc_key, b.wc_val,
+  launch(k_wc_compose, nblk(n, 256), 256, 0, s)(b.wc_run, b.wc_flag, b.acc_idx, b.acc_info, n, b.wc_key, b.wc_val,
                                             b.wc_who, b.wc_row, b.wc_ep);
   count_launch();
   // accesses of locations with a write-class access, compacted (count on the device, at
@@ -1203,12 +1216,12 @@ void phaseI_wide_group(Bufs& b, const Geo& g, Sizes& z, uint32_t* tmp, cudaStrea
   uint32_t* kpos = b.wc_gexcl;
   uint32_t* n_keep = b.wc_gexcl + n;
   cudaMemsetAsync(run_w, 0, (size_t(n) + 1) * 4, s);
-  k_wc_runwrite<<<nblk(n, 256), 256, 0, s>>>(b.wc_key, n, run_w);
+  launch(k_wc_runwrite, nblk(n, 256), 256, 0, s)(b.wc_key, n, run_w);
   count_launch();
-  k_wc_keep<<<nblk(n, 256), 256, 0, s>>>(b.wc_key, n, run_w, keep);
+  launch(k_wc_keep, nblk(n, 256), 256, 0, s)(b.wc_key, n, run_w, keep);
   count_launch();
   scan_exclusive(keep, kpos, n, n_keep, tmp, s);
-  k_wc_compact<<<nblk(n, 256), 256, 0, s>>>(b.wc_key, b.wc_val, keep, kpos, n, b.wc_key2, b.wc_val2);
+  launch(k_wc_compact, nblk(n, 256), 256, 0, s)(b.wc_key, b.wc_val, keep, kpos, n, b.wc_key2, b.wc_val2);
   count_launch();
   std::swap(b.wc_key, b.wc_key2);
   std::swap(b.wc_val, b.wc_val2);
@@ -1224,14 +1237,14 @@ void phaseI_wide_group(Bufs& b, const Geo& g, Sizes& z, uint32_t* tmp, cudaStrea
     std::swap(b.wc_key, b.wc_key2);
     std::swap(b.wc_val, b.wc_val2);
   }
-  k_wc_groupflags<<<nblk(n, 256), 256, 0, s>>>(b.wc_key, n, n_kept, b.wc_gflag);
+  launch(k_wc_groupflags, nblk(n, 256), 256, 0, s)(b.wc_key, n, n_kept, b.wc_gflag);
   count_launch();
   scan_exclusive(b.wc_gflag, b.wc_gexcl, n, b.wc_gexcl + n, tmp, s);
   cudaMemsetAsync(b.wc_rc, 0, (size_t(n) * 4 + 2) * 4, s);
-  k_wc_groups<<<nblk(n, 256), 256, 0, s>>>(b.wc_key, b.wc_gflag, b.wc_gexcl, n, b.wc_grp_lo, b.wc_grp_agent,
+  launch(k_wc_groups, nblk(n, 256), 256, 0, s)(b.wc_key, b.wc_gflag, b.wc_gexcl, n, b.wc_grp_lo, b.wc_grp_agent,
                                           b.wc_rc);
   count_launch();
-  k_wc_grp_end<<<1, 1, 0, s>>>(b.wc_gexcl + n, n_kept, b.wc_grp_lo);  // grp_lo[n_groups] = kept count
+  launch(k_wc_grp_end, 1, 1, 0, s)(b.wc_gexcl + n, n_kept, b.wc_grp_lo);  // grp_lo[n_groups] = kept count
   count_launch();
   scan_exclusive(b.wc_rc, b.wc_rc, size_t(n) * 4 + 1, nullptr, tmp, s);
   p.end();
@@ -1246,16 +1259,16 @@ void phaseI_grouped(Bufs& b, const Geo& g, Sizes& z, uint32_t* tmp, cudaStream_t
   const uint32_t n = z.n_kept;  // the accesses the written-location filter kept
   if (!n) return;
   p.begin("i_wide_group", double(n) * (8 + 4 * 4 + 16 + 12 + 16), s);  // ~ per access
-  k_gr_flags<<<nblk(n, 256), 256, 0, s>>>(b.acc_key, n, b.n_kept, b.wc_flag, b.wc_gflag);
+  launch(k_gr_flags, nblk(n, 256), 256, 0, s)(b.acc_key, n, b.n_kept, b.wc_flag, b.wc_gflag);
   count_launch();
   ScanBatch sb{};
   sb.job[0] = ScanJob{b.wc_flag, b.wc_run, b.wc_run + n, n};
   sb.job[1] = ScanJob{b.wc_gflag, b.wc_gexcl, b.wc_gexcl + n, n};
   scan_all(sb, 2, tmp, s);
-  k_gr_groups<<<nblk(n, 256), 256, 0, s>>>(b.acc_key, b.wc_flag, b.wc_run, b.wc_gflag, b.wc_gexcl, b.n_kept,
+  launch(k_gr_groups, nblk(n, 256), 256, 0, s)(b.acc_key, b.wc_flag, b.wc_run, b.wc_gflag, b.wc_gexcl, b.n_kept,
                                           b.wc_grp_lo, b.wc_grp_agent, b.wc_rc);
   count_launch();
-  k_wc_fields<<<nblk(n, 256), 256, 0, s>>>(b.acc_idx, b.acc_info, b.n_kept, b.wc_who, b.wc_row, b.wc_ep);
+  launch(k_wc_fields, nblk(n, 256), 256, 0, s)(b.acc_idx, b.acc_info, b.n_kept, b.wc_who, b.wc_row, b.wc_ep);
   count_launch();
   p.end();
 }
@@ -1305,12 +1318,12 @@ void phaseI_wide_check(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t
   if (!z.grouped)
     check = rep == REP_TILES ? k_wc_check<REP_TILES, false>
             : rep == REP_DENSE ? k_wc_check<REP_DENSE, false> : k_wc_check<REP_COMPRESSED, false>;
-  check<<<nblk(n, kCheckThreads), kCheckThreads, 0, s>>>(a);
+  launch(check, nblk(n, kCheckThreads), kCheckThreads, 0, s)(a);
   count_launch();
   if (z.grouped && 4 * g.W > a.big_groups) {  // fewer agents have no such access
     auto big = rep == REP_TILES ? k_wc_big<REP_TILES>
                : rep == REP_DENSE ? k_wc_big<REP_DENSE> : k_wc_big<REP_COMPRESSED>;
-    big<<<std::min<uint32_t>(nblk(n, 32), 152 * 6), kCheckThreads, 0, s>>>(a);
+    launch(big, std::min<uint32_t>(nblk(n, 32), 152 * 6), kCheckThreads, 0, s)(a);
     count_launch();
   }
   p.end();
