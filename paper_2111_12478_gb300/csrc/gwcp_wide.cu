@@ -964,11 +964,13 @@ __device__ __noinline__ uint32_t check_part(const WideCheckArgs& a, uint32_t p, 
 //   1M, 64              0.05    0.11    0.19    0.20
 //   1M, 64, ranked      0.047   0.074   0.172   0.172   (the lanes of the access's own warp)
 //   2M, 128             0.092   0.104   0.123   0.471
+//   3M, 64              0.121   0.195   0.254   0.326
 //   2.3M, 512           0.424   0.141   0.154   0.217
 //   5M, 256             1.145   0.850   0.274   0.344
 //   10M, 64             2.156   0.467   0.528   0.555
 //   5M, 512 threads     0.331   0.316   0.306   0.231
-inline uint32_t big_groups(uint32_t n) { return n <= (1u << 21) ? 48 : 96; }
+// (n counts the accesses that the written-location filter keeps, a tenth or two fewer.)
+inline uint32_t big_groups(uint32_t n) { return n <= 1500000 ? 48 : n <= 2200000 ? 64 : 96; }
 constexpr uint32_t kPieceGroups = 128;  // groups per item of k_wc_big: four per lane
 
 // appends the warp's staged races (one global atomic) and its test count; returns the races found
