@@ -462,6 +462,7 @@ struct Sizes {
   uint32_t pool_cap = 0;
   uint32_t n_chunks = 0;
   uint64_t race_cap = 0;
+  cudaEvent_t before_walk = nullptr;  // recorded when the plan is done, before the walkers' launch
   uint32_t check_ch = 512;  // accesses per chunk of the chunked check
   uint32_t big_cap = 0;  // partner check: items it may put aside
   uint64_t tile_cap = 0;      // wide clocks: tiles in the pool

@@ -1139,6 +1139,7 @@ int phaseG_propagate(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s
     count_launch();
   }
   p.end();
+  if (z.before_walk) cudaEventRecord(z.before_walk, s);
   if (g.nT) {
     // tile tables: each clock version and snapshot is a table (new tiles counted apart)
     p.begin("g_propagate", double(z.n_rows) * g.RW * 4 + double(z.n_cs) * 2 * g.RW * 4);
