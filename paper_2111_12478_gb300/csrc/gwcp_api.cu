@@ -397,19 +397,25 @@ int run(gwcp_ctx* c, cudaStream_t s) {
   if (oom) return GWCP_ERR_OOM;
 
   phaseA_scatter(b, g, z, s, c->prof);
-  // the access sort needs only the decoded accesses: it runs on the side stream beside the
-  // main stream's other phases (measured on the 8192-warp workload: it overlaps them, and
-  // the grouping ends before the propagation starts; with the side stream at a lower
-  // priority the sort drifts into the propagation and slows its latency-bound walkers)
+  // The access sort needs only the decoded accesses and runs on the side stream, as does the
+  // grouping of its result. Walkers that fill few SMs leave the others to it: it then starts
+  // with them, and the phases before them have the GPU to themselves (2.3M events, 512 agents:
+  // a pass 1.60 -> 1.49 ms; 5M, 256: 3.23 -> 2.97; 10M, 64: 13.33 -> 13.08; 250k, 256 threads:
+  // 0.83 -> 0.81). Walkers on most SMs would leave it nothing (50M events, 8192 agents: the
+  // sort beside them took 11.7 ms instead of 2.8), so there it runs beside the phases before.
   SideJoin side{c, s};
   cudaEventRecord(c->fork, s);
   cudaStreamWaitEvent(c->side, c->fork, 0);
   side.armed = true;
-  phaseH_sort(b, g, z, sort_mask, side_tmp, c->side, c->prof);
-  if (z.grouped) {  // the kept count sizes the grouping and the check (read before they are enqueued)
-    cudaMemcpyAsync(c->cnt_host + 15, b.n_kept, 4, cudaMemcpyDeviceToHost, c->side);
-    cudaEventRecord(c->kept_ev, c->side);
-  }
+  const bool late_sort = !g.nT && (g.apb <= 32 ? g.B : g.W / 8) <= 64;
+  auto sort_accesses = [&] {
+    phaseH_sort(b, g, z, sort_mask, side_tmp, c->side, c->prof);
+    if (z.grouped) {  // the kept count sizes the grouping and the check (read before they are enqueued)
+      cudaMemcpyAsync(c->cnt_host + 15, b.n_kept, 4, cudaMemcpyDeviceToHost, c->side);
+      cudaEventRecord(c->kept_ev, c->side);
+    }
+  };
+  if (!late_sort) sort_accesses();
   phaseB_sync(b, g, z, s, c->prof);
   phaseC_walk(b, g, z, s, c->prof);
   // forced compression at barriers renumbers the local times; barriers are validated in
@@ -553,12 +559,11 @@ int run(gwcp_ctx* c, cudaStream_t s) {
   phaseD_gaps(b, g, z, s, c->prof);
   c->acc_info_partial = z.wl_log2 != 0;
   // The access grouping and the check's carries need the access records (phase D), not clock
-  // values: they follow the sort on the side stream. With many accesses they start with the
-  // walkers, as they would fill the GPU in front of phase F's small kernels (50M events, 8192
-  // agents: phase F 0.95 ms beside the grouping, 0.13 before it; the pass 16.9 -> 16.6 ms).
-  // Otherwise they start at once (4M events, 4096 agents: 3.40 ms, 3.44 with the walkers; 10M
-  // events, 64 agents: no difference, the walkers' CTAs then wait for whole SMs).
-  if (z.n_acc >= (1u << 24))
+  // values: they follow the sort on the side stream. Where the sort runs early they start at
+  // once, but with many accesses they would fill the GPU in front of phase F's small kernels
+  // and start with the walkers (50M events, 8192 agents: phase F 0.95 ms beside the grouping,
+  // 0.13 before it, the pass 16.9 -> 16.6 ms; 4M, 4096: 3.40 ms at once, 3.44 with the walkers).
+  if (late_sort || z.n_acc >= (1u << 24))
     z.before_walk = c->fork2;
   else
     cudaEventRecord(c->fork2, s);
@@ -598,6 +603,7 @@ int run(gwcp_ctx* c, cudaStream_t s) {
     return rc ? rc : prc;
   }
   cudaStreamWaitEvent(c->side, c->fork2, 0);
+  if (late_sort) sort_accesses();
   if (z.grouped) {
     // the main stream has phases D to G queued; the sort has usually finished by now
     if (cudaEventSynchronize(c->kept_ev) != cudaSuccess) return GWCP_ERR_CUDA;
