@@ -1,4 +1,4 @@
-// Wide clocks (W > 1024 agents, up to 8192): clock propagation and race check over
+// Wide clocks (many agents, up to 8192): clock propagation and race check over
 // copy-on-write clock tiles.
 //
 // A clock of width W is cut into nT = ceil(W / 256) tiles of 256 u32 entries. Tiles live
