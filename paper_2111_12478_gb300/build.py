@@ -28,6 +28,7 @@ def _nvcc():
 def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(OUT, exist_ok=True)
     deps = [os.path.join(CSRC, f) for f in SOURCES] + [os.path.join(CSRC, "gwcp_internal.cuh"),
+                                                       os.path.join(CSRC, "gwcp_post.cuh"),
                                                        os.path.join(ROOT, "include", "gwcp.h")]
     if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= max(os.path.getmtime(d) for d in deps):
         return LIB

@@ -29,6 +29,7 @@
 #include <algorithm>
 
 #include "gwcp_internal.cuh"
+#include "gwcp_post.cuh"
 
 namespace gwcp {
 
@@ -154,14 +155,14 @@ __device__ __forceinline__ uint32_t merge_one(const WideArgs& a, uint32_t ia, ui
 // -> 17,000 cycles): 8192 warps, 50M events 16.7 -> 9.5 ms; 4096 warps, 4M 4.2 -> 1.86; 512
 // warps, 2.3M 2.2 -> 1.3. (The pairs of eight merges copied to shared memory ahead of the
 // one walker: 13.5 and 3.0 ms; four tiles per warp at a time: slower than one.)
-// A post is open while `next` is below kClosed; it is reused only after all its merges are
-// done, and opened by the store to `next` after everything else is written, so a helper that
-// comes late finds either no merge or one of the new post.
+// A post is reused only after all its merges are done, and opened by the store to `word`
+// after everything else is written. A walker that draws a merge thereby knows that the post
+// stays as it is until the merge is done; one that comes late draws nothing, or a merge of the
+// new post together with that post's own limit.
 struct Post {
-  uint32_t next, total, done, pad;  // merge to take next; merges; merges done
-  uint32_t ida[96], idb[96];        // the merges: my tile (then the result), the source's
+  uint32_t word, done, pad[2];  // merges and merges handed out (gwcp_post.cuh); merges done
+  uint32_t ida[96], idb[96];    // the merges: my tile (then the result), the source's
 };
-constexpr uint32_t kClosed = 0x40000000u;
 constexpr uint32_t kPosts = 4;  // per CTA; a walker that finds none free walks its merges alone
 
 struct __align__(16) Shared {  // a CTA's posts
@@ -176,12 +177,17 @@ struct __align__(16) Shared {  // a CTA's posts
 __device__ __forceinline__ bool take_merge(const WideArgs& a, Shared& sh, int b, TileAlloc& ta) {
   const int lane = threadIdx.x & 31;
   Post& q = sh.post[b];
-  uint32_t j = 0;
-  if (lane == 0) j = atomicAdd(&q.next, 1u);
-  j = __shfl_sync(0xffffffffu, j, 0);
-  const uint32_t total = *(volatile uint32_t*)&q.total;
-  if (j >= kClosed || j >= total) return false;
-  if (j + 1 == total && lane == 0) atomicAnd(&sh.open, ~(1u << b));
+  uint32_t w = kPostClosed;
+  if (lane == 0) {
+    w = *(volatile uint32_t*)&q.word;
+    if (post_left(w)) w = atomicAdd(&q.word, 1u);
+    __threadfence_block();
+  }
+  w = __shfl_sync(0xffffffffu, w, 0);
+  __syncwarp();
+  if (!post_left(w)) return false;
+  const uint32_t j = post_merge(w);
+  if (j + 1 == post_merges(w) && lane == 0) atomicAnd(&sh.open, ~(1u << b));
   bool fresh;
   const uint32_t id = merge_one(a, *(volatile uint32_t*)&q.ida[j], *(volatile uint32_t*)&q.idb[j], fresh, ta);
   ta.count(2, fresh ? 1u : 0u);
@@ -268,16 +274,13 @@ __device__ __noinline__ void merge_tables(const WideArgs& a, uint32_t (&my)[NT],
       post.idb[at[q]] = src[q];
     }
   }
-  if (lane == 0) {
-    post.total = total;
-    post.done = 0;
-  }
+  if (lane == 0) post.done = 0;
   __threadfence_block();
   __syncwarp();
   if (lane == 0) {
     atomicOr(&sh.open, 1u << b);  // (before the first merge can be taken: the last one taken clears it)
     __threadfence_block();
-    atomicExch(&post.next, 0u);
+    atomicExch(&post.word, post_open(total));
   }
   while (take_merge(a, sh, b, ta)) {
   }
@@ -292,7 +295,7 @@ __device__ __noinline__ void merge_tables(const WideArgs& a, uint32_t (&my)[NT],
     if (at[q] != NONE) my[q] = *(volatile uint32_t*)&post.ida[at[q]];
   __syncwarp();
   if (lane == 0) {
-    atomicExch(&post.next, kClosed);
+    atomicExch(&post.word, kPostClosed);
     atomicAnd(&sh.used, ~(1u << b));
   }
   dirty = true;
@@ -452,10 +455,7 @@ __global__ void __launch_bounds__(1024, MINB) k_prop_wide(const __grid_constant_
   if (threadIdx.x == 0) {
     start_code = *(volatile int*)&a.st->code;
     sh.used = sh.open = sh.arrived = 0;
-    for (uint32_t q = 0; q < kPosts; ++q) {
-      sh.post[q].next = kClosed;
-      sh.post[q].total = 0;
-    }
+    for (uint32_t q = 0; q < kPosts; ++q) sh.post[q].word = kPostClosed;
   }
   __syncthreads();
   if (start_code) return;
