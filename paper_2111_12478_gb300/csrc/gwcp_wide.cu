@@ -457,6 +457,9 @@ __global__ void __launch_bounds__(1024, MINB) k_prop_wide(const __grid_constant_
     sh.used = sh.open = sh.arrived = 0;
     for (uint32_t q = 0; q < kPosts; ++q) sh.post[q].word = kPostClosed;
   }
+  // a walker whose wait gave up goes on without waiting for its block: what it then reads of
+  // members that have not arrived is the zero tile and the local time 0
+  for (uint32_t i = threadIdx.x; i < apb * 96 + 32 + 96; i += blockDim.x) tabs[i] = 0;  // and nbuf, J
   __syncthreads();
   if (start_code) return;
   const bool act = lane < int(g.nT);
@@ -657,8 +660,9 @@ __global__ void __launch_bounds__(1024, MINB) k_prop_wide(const __grid_constant_
         hid = act ? J[32 + lane] : 0;
         jid = act ? J[64 + lane] : 0;
         joins += 2;  // this member's C_t and H_t joined into the block's
-        // J is rewritten only after the next barrier's first __syncthreads, which every
-        // member reaches after reading it here
+        // J is rewritten only after every member has arrived at the next barrier, after reading
+        // it here (or by a walker that has given up, with ids of this launch: the analysis has
+        // failed then, and every id that can be read is of a tile in the pool)
       }
       ++N;  // H_t[t] = N_t, implicit
     }
