@@ -270,8 +270,7 @@ int run(gwcp_ctx* c, cudaStream_t s) {
   // phase A's agent histogram, later phase D's index
   b.hist_a = b.d_index = get<uint32_t>(c, "d_index", std::max(hist_words, size_t(g.W) * z.d_nw), &oom);
   b.tile_cnt = get<uint32_t>(c, "tile_cnt", 4 * (size_t(z.ntA) + 1), &oom);
-  const size_t scan_need = std::max({scan_tmp_need(hist_words), radix_tmp_need(z.N + 1),
-                                     scan_tmp_need(z.N + 1)}) + 64;
+  size_t scan_need = std::max({scan_tmp_need(hist_words), radix_tmp_need(z.N + 1), scan_tmp_need(z.N + 1)}) + 64;
   b.scan_tmp = get<uint32_t>(c, "scan_tmp", scan_need, &oom);
   if (oom) return GWCP_ERR_OOM;
   DevStatus init{};
@@ -340,6 +339,10 @@ int run(gwcp_ctx* c, cudaStream_t s) {
   // compressed versions keep local times in 31 bits; a local time is at most 1 + n_sync
   if (z.compress && z.n_sync >= kCvExpanded - 1) return GWCP_ERR_UNSUPPORTED;
   const size_t ns1 = size_t(z.n_sync) + 1;
+  // (a barrier has an entry per member, up to 1024 times as many entries as events; the stream
+  // is idle here, so the scratch may move)
+  scan_need = std::max(scan_need, scan_tmp_need(ns1) + 64);
+  b.scan_tmp = get<uint32_t>(c, "scan_tmp", scan_need, &oom);
   b.sy_cnt = get<uint32_t>(c, "sy_cnt", z.nS / 512 + 2, &oom);  // one count per 512-entry chunk of S
   b.sy_spos = get<uint32_t>(c, "sy_spos", ns1, &oom);
   b.sy_idx = get<uint32_t>(c, "sy_idx", ns1, &oom);
