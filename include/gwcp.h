@@ -206,6 +206,13 @@ int gwcp_set_check_mode(gwcp_ctx* ctx, uint32_t mode);
  * (GWCP_ERR_TIMEOUT). Synchronous; allocates and frees a small buffer. */
 int gwcp_debug_wait_timeout(int device, uint32_t spin_limit, int* status);
 
+/* Test hook of failure detection: the analysis' radix sort on host arrays, by the key bits
+ * set in `mask` (stable; vals may be NULL), sorted in place. Its tiles wait for the digit
+ * counts of the tiles before them; a tile that has looked `poll_limit` times without news
+ * counts them itself, so the result is the same with every limit and the sort records no
+ * error. n < 2^30. Synchronous; allocates and frees device memory. */
+int gwcp_debug_sort(int device, uint64_t* keys, uint32_t* vals, uint64_t n, uint64_t mask, uint32_t poll_limit);
+
 /* Test hook of failure detection: caps the bytes of the buffers the context caches
  * (0 = no cap). A compute that would need more fails with GWCP_ERR_OOM, as on an exhausted
  * device, and leaves the context usable: after the cap is raised the next compute runs

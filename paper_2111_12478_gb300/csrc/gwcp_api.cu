@@ -1278,6 +1278,12 @@ int gwcp_debug_wait_timeout(int device, uint32_t spin_limit, int* status) {
   return wait_probe(spin_limit, status);
 }
 
+int gwcp_debug_sort(int device, uint64_t* keys, uint32_t* vals, uint64_t n, uint64_t mask, uint32_t poll_limit) {
+  if ((n && !keys) || n > kMaxEvents) return GWCP_ERR_ARGS;
+  if (cudaSetDevice(device) != cudaSuccess) return GWCP_ERR_CUDA;
+  return n ? debug_sort(keys, vals, n, mask, poll_limit) : GWCP_OK;
+}
+
 uint64_t gwcp_first_bad_index(const gwcp_ctx* c) { return c ? c->bad_index : ~0ull; }
 
 uint64_t gwcp_launch_count(void) { return gwcp::launch_count(); }

@@ -357,7 +357,7 @@ void phaseH_sort(Bufs& b, const Geo& g, const Sizes& z, uint64_t key_mask, uint3
     keep.shift = 15;
     keep.n_out = b.n_kept;
   }
-  if (radix_sort_pairs(b.acc_key, b.acc_idx, b.acc_key2, b.acc_idx2, z.n_acc, key_mask, tmp, s, nullptr, keep, b.st)) {
+  if (radix_sort_pairs(b.acc_key, b.acc_idx, b.acc_key2, b.acc_idx2, z.n_acc, key_mask, tmp, s, nullptr, keep)) {
     std::swap(b.acc_key, b.acc_key2);
     std::swap(b.acc_idx, b.acc_idx2);
   }
@@ -434,7 +434,7 @@ bool phaseI_sort_races(const Bufs& b, const Sizes& z, uint64_t n_races, cudaStre
   for (uint64_t v = z.N; v; v >>= 1) mask = (mask << 1) | 1;
   mask |= mask << 32;
   p.begin("i_race_sort", double(n) * 8 * 2);
-  bool second = radix_sort_pairs(b.races, nullptr, b.races2, nullptr, n, mask, b.scan_tmp, s, nullptr, {}, b.st);
+  bool second = radix_sort_pairs(b.races, nullptr, b.races2, nullptr, n, mask, b.scan_tmp, s);
   p.end();
   return second;
 }

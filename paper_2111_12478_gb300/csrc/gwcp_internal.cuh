@@ -282,21 +282,25 @@ void scan_exclusive(const uint32_t* in, uint32_t* out, size_t n, uint32_t* total
 void scan_all(const ScanBatch& b, int jobs, uint32_t* tmp, cudaStream_t s);
 // Stable LSD radix sort of (key, val) pairs on the bits set in `mask`, 8-bit digits.
 // Ping-pongs between (k0, v0) and (k1, v1); returns true if the result is in (k1, v1).
-// tmp must hold radix_tmp_need(n) u32. st (or null) gets GWCP_ERR_TIMEOUT if a bounded wait
-// between tiles gives up. With n_dev, only the first min(n, *n_dev) pairs are
+// tmp must hold radix_tmp_need(n) u32. With n_dev, only the first min(n, *n_dev) pairs are
 // sorted (a count known on the device only; n bounds it).
 // With keep.bits, the first pass keeps only the pairs whose bit wl_bit(key >> keep.shift,
 // keep.log2) is set in keep.bits (a stable filter folded into the sort); the kept count is
 // written to keep.n_out and bounds the later passes.
+// polls: looks at the tiles before it without news after which a tile goes on by itself (the
+// result is the same).
 struct RadixKeep {
   const uint32_t* bits = nullptr;
   uint32_t log2 = 0, shift = 0;
   uint32_t* n_out = nullptr;
 };
+constexpr uint32_t kSortPolls = 1u << 22;
 size_t radix_tmp_need(size_t n);
 bool radix_sort_pairs(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, size_t n, uint64_t mask,
                       uint32_t* tmp, cudaStream_t s, const uint32_t* n_dev = nullptr, RadixKeep keep = {},
-                      DevStatus* st = nullptr);
+                      uint32_t polls = kSortPolls);
+// a sort of host arrays (val may be null) with a poll limit: the test of the bounded wait
+int debug_sort(uint64_t* key, uint32_t* val, uint64_t n, uint64_t mask, uint32_t polls);
 // passes a sort on the bits of `mask` takes
 int radix_passes(uint64_t mask);
 

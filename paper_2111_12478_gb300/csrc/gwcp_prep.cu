@@ -1356,7 +1356,7 @@ void phaseA_scatter(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s,
     while ((1u << ab) < g.W) ++ab;
     const uint64_t mask = ((1ull << ab) - 1) << 32;
     const uint64_t* sorted =
-        radix_sort_pairs(b.s_key, nullptr, b.s_key2, nullptr, z.nS, mask, b.s_tmp, s, nullptr, {}, b.st) ? b.s_key2 : b.s_key;
+        radix_sort_pairs(b.s_key, nullptr, b.s_key2, nullptr, z.nS, mask, b.s_tmp, s) ? b.s_key2 : b.s_key;
     if (z.nS) {
       launch(k_aw_extract, blocks(z.nS, 256), 256, 0, s)(sorted, z.nS, b.S);
       count_launch();
@@ -1412,7 +1412,7 @@ void phaseC_forced(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t s, 
   count_launch();
   uint64_t mask = 0;  // keys 0..B (B: one-member barriers, left out of the walk)
   while (mask < g.B) mask = (mask << 1) | 1;
-  const bool second = radix_sort_pairs(b.fb_key, b.fb_val, b.fb_key2, b.fb_val2, n, mask, b.scan_tmp, s, nullptr, {}, b.st);
+  const bool second = radix_sort_pairs(b.fb_key, b.fb_val, b.fb_key2, b.fb_val2, n, mask, b.scan_tmp, s);
   const uint64_t* skey = second ? b.fb_key2 : b.fb_key;
   const uint32_t* spos = second ? b.fb_val2 : b.fb_val;
   launch(k_fb_rank, blocks(uint64_t(n) + 1, 256), 256, 0, s)(b.ev, g, b.bar, skey, spos, n, b.fb_rank, b.fb_off,
@@ -1461,7 +1461,7 @@ void phaseE_locks(Bufs& b, const Geo& g, const Sizes& z, uint64_t lock_mask, cud
   const uint32_t n = z.n_acqrel;
   if (!n) return;
   p.begin("e_sort", double(n) * 24);
-  if (radix_sort_pairs(b.lk_key, b.lk_k, b.lk_key2, b.lk_k2, n, lock_mask, b.scan_tmp, s, nullptr, {}, b.st)) {
+  if (radix_sort_pairs(b.lk_key, b.lk_k, b.lk_key2, b.lk_k2, n, lock_mask, b.scan_tmp, s)) {
     std::swap(b.lk_key, b.lk_key2);
     std::swap(b.lk_k, b.lk_k2);
   }
@@ -1526,7 +1526,7 @@ void phaseF_deps(Bufs& b, const Geo& g, const Sizes& z, uint64_t key_mask, cudaS
   const uint32_t n = z.n_exp;
   if (!n) return;
   p.begin("f_sort", double(n) * 24);
-  if (radix_sort_pairs(b.ex_key, b.ex_val, b.ex_key2, b.ex_val2, n, key_mask, b.scan_tmp, s, nullptr, {}, b.st)) {
+  if (radix_sort_pairs(b.ex_key, b.ex_val, b.ex_key2, b.ex_val2, n, key_mask, b.scan_tmp, s)) {
     std::swap(b.ex_key, b.ex_key2);
     std::swap(b.ex_val, b.ex_val2);
   }

@@ -158,7 +158,9 @@ __global__ void __launch_bounds__(SC_THREADS) k_scan_apply(const uint32_t* in, u
 // the tile. Against a histogram, a scan and a scatter kernel per digit this reads the keys
 // once per pass instead of twice and takes two launches plus one per digit instead of five
 // per digit. A tile reads the counts of LOOK tiles at a time: when all tiles start together,
-// tile i finds a complete prefix after about i / (2 LOOK) rounds of memory latency.
+// tile i finds a complete prefix after about i / (2 LOOK) rounds of memory latency. The wait is
+// bounded, and a tile that gives up counts its digits in the pairs before it itself: the sort
+// has one result, whatever the waits do, so it has no status and no caller reads one.
 // A digit takes the next eight varying bits of the key, in up to four separate runs, so the
 // number of passes is that of the varying bits alone (with runs of eight adjacent bits, the
 // composite keys of 64 agents took 6 passes instead of 5).
@@ -168,7 +170,6 @@ __global__ void __launch_bounds__(SC_THREADS) k_scan_apply(const uint32_t* in, u
 // for four blocks). Ranks by eight ballots; match.any measured 9% slower.
 constexpr int LOOK = 8;
 constexpr int kMaxPasses = 9;
-constexpr uint32_t kSweepSpins = 1u << 22;
 
 // a pair the filter of the first pass keeps
 __device__ __forceinline__ bool radix_kept(uint64_t key, const RadixKeep& kp) {
@@ -248,7 +249,7 @@ struct SweepArgs {
   uint32_t* counter;           // tiles handed out, in order
   uint32_t tag;                // this pass's tag of an own count; tag + 1: of a prefix
   RadixKeep kp;
-  DevStatus* st;
+  uint32_t polls;  // looks without news before a tile gives up
 };
 
 __device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long long* p) {
@@ -263,6 +264,30 @@ __device__ __forceinline__ void st_relaxed(unsigned long long* p, unsigned long 
 template <int THREADS, int ITEMS>
 constexpr size_t sweep_smem() {
   return size_t(THREADS) * ITEMS * 12 + size_t(THREADS / 32) * 256 * 4;
+}
+
+// What a tile that has given up does in the place of the rest of its wait: it counts the kept
+// pairs of each digit in front of it (cnt: 256 words), publishes its prefixes and sets glob,
+// by the whole block. Out of line, with all it needs computed again: no other tile pays for it.
+template <int THREADS>
+__device__ __noinline__ void count_before(const SweepArgs& a, size_t tile, size_t before, uint32_t* cnt,
+                                          const uint32_t* tile_off, uint32_t nvalid, uint32_t* glob) {
+  __shared__ uint32_t all;
+  const uint32_t tid = threadIdx.x;
+  if (tid < 256) cnt[tid] = 0;
+  __syncthreads();
+  for (size_t i = tid; i < before; i += THREADS) {
+    const uint64_t k = a.kin[i];
+    if (radix_kept(k, a.kp)) atomicAdd(&cnt[a.dig.of(k)], 1u);
+  }
+  __syncthreads();
+  const uint32_t dig_base = block_exclusive_scan<THREADS>(tid < 256 ? a.hist[tid] : 0u, &all);
+  if (tid < 256) {
+    const uint32_t own = (tid < 255 ? tile_off[tid + 1] : nvalid) - tile_off[tid];
+    st_relaxed(a.status + tile * 256 + tid, (static_cast<unsigned long long>(a.tag + 1) << 32) | (cnt[tid] + own));
+    glob[tid] = dig_base + cnt[tid];
+  }
+  __syncthreads();
 }
 
 // Warp w of a tile owns items [w * 32 * ITEMS, ..) of it, visited in rounds of 32 consecutive
@@ -372,22 +397,21 @@ __global__ void __launch_bounds__(THREADS, ITEMS <= 4 ? 6 : 4) k_sweep(const __g
       }
       if (used < 0) break;
       t -= used;
-      if (used == 0 && ++spins > kSweepSpins) {
+      if (used == 0 && ++spins > a.polls) {
         gone = true;
         break;
       }
     }
-    if (gone) {
+    if (gone)
       s_gone = 1;
-      if (a.st) atomicCAS(&a.st->code, 0, GWCP_ERR_TIMEOUT);
-    } else if (tile) {
+    else if (tile)
       st_relaxed(status + tid, (static_cast<unsigned long long>(a.tag + 1) << 32) | (excl + own));
-    }
     glob[tid] = dig_base + excl;
   }
   __syncthreads();
-  if (s_gone) return;
   const uint32_t nvalid = tot;
+  // (the input stays as it is until every tile of this pass is done)
+  if (s_gone) count_before<THREADS>(a, tile, size_t(tile) * TILE, cnt, tile_off, nvalid, glob);
   for (uint32_t i = tid; i < nvalid; i += THREADS) {
     const uint64_t key = sk[i];
     const uint32_t d = a.dig.of(key);
@@ -615,7 +639,7 @@ size_t radix_tmp_need(size_t n) {
 }
 
 bool radix_sort_pairs(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, size_t n, uint64_t mask,
-                      uint32_t* tmp, cudaStream_t s, const uint32_t* n_dev, RadixKeep keep, DevStatus* st) {
+                      uint32_t* tmp, cudaStream_t s, const uint32_t* n_dev, RadixKeep keep, uint32_t polls) {
   if (keep.bits) {
     if (n == 0) {
       cudaMemsetAsync(keep.n_out, 0, 4, s);
@@ -659,7 +683,7 @@ bool radix_sort_pairs(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, si
     a.counter = counters + p;
     a.tag = uint32_t(2 * p + 1);
     if (p == 0) a.kp = keep;
-    a.st = st;
+    a.polls = polls;
     if (tile == kSmallTile)
       launch_sweep<256, 4>(a, tiles, s);
     else
@@ -668,6 +692,32 @@ bool radix_sort_pairs(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, si
     in_second = !in_second;
   }
   return in_second;
+}
+
+int debug_sort(uint64_t* key, uint32_t* val, uint64_t n, uint64_t mask, uint32_t polls) {
+  unsigned char* mem = nullptr;
+  const size_t kb = n * 8, vb = val ? (n * 4 + 15) & ~size_t(15) : 0;
+  if (cudaMalloc(&mem, 2 * (kb + vb) + 512 + radix_tmp_need(n) * 4) != cudaSuccess) {
+    cudaGetLastError();
+    return GWCP_ERR_OOM;
+  }
+  // scratch first (256-byte aligned), then keys, then values
+  auto* tmp = reinterpret_cast<uint32_t*>(mem);
+  unsigned char* at = mem + ((radix_tmp_need(n) * 4 + 255) & ~size_t(255));
+  auto *k0 = reinterpret_cast<uint64_t*>(at), *k1 = reinterpret_cast<uint64_t*>(at + kb);
+  uint32_t *v0 = nullptr, *v1 = nullptr;
+  if (val) {
+    v0 = reinterpret_cast<uint32_t*>(at + 2 * kb);
+    v1 = reinterpret_cast<uint32_t*>(at + 2 * kb + vb);
+  }
+  cudaMemcpy(k0, key, kb, cudaMemcpyHostToDevice);
+  if (val) cudaMemcpy(v0, val, n * 4, cudaMemcpyHostToDevice);
+  const bool second = radix_sort_pairs(k0, v0, k1, v1, n, mask, tmp, nullptr, nullptr, {}, polls);
+  cudaMemcpy(key, second ? k1 : k0, kb, cudaMemcpyDeviceToHost);
+  if (val) cudaMemcpy(val, second ? v1 : v0, n * 4, cudaMemcpyDeviceToHost);
+  const int rc = cudaDeviceSynchronize() == cudaSuccess && cudaGetLastError() == cudaSuccess ? GWCP_OK : GWCP_ERR_CUDA;
+  cudaFree(mem);
+  return rc;
 }
 
 }  // namespace gwcp

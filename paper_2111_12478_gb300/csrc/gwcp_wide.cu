@@ -1239,7 +1239,7 @@ void phaseI_wide_group(Bufs& b, const Geo& g, Sizes& z, uint32_t* tmp, cudaStrea
   while ((1ull << rb) < n) ++rb;
   while ((1u << ab) < g.W) ++ab;
   const uint64_t mask = (((1ull << rb) - 1) << 15) | (3ull << 13) | ((1ull << ab) - 1);
-  if (radix_sort_pairs(b.wc_key, b.wc_val, b.wc_key2, b.wc_val2, n, mask, tmp, s, n_kept, {}, b.st)) {
+  if (radix_sort_pairs(b.wc_key, b.wc_val, b.wc_key2, b.wc_val2, n, mask, tmp, s, n_kept)) {
     std::swap(b.wc_key, b.wc_key2);
     std::swap(b.wc_val, b.wc_val2);
   }

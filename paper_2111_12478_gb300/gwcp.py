@@ -24,7 +24,7 @@ EXPORTS = ("gwcp_create", "gwcp_load_trace", "gwcp_compute_order", "gwcp_report_
            "gwcp_pool_run_batch", "gwcp_pool_set_active_lanes", "gwcp_pool_autotune", "gwcp_pool_now",
            "gwcp_pool_device_bytes", "gwcp_pool_destroy", "gwcp_set_ranker", "gwcp_location_features",
            "gwcp_rank_scores", "gwcp_rank_grad", "gwcp_rank_train", "gwcp_check_timeline", "gwcp_set_clock_mode",
-           "gwcp_pool_clock_modes", "gwcp_set_check_mode", "gwcp_debug_wait_timeout", "gwcp_pool_settings",
+           "gwcp_pool_clock_modes", "gwcp_set_check_mode", "gwcp_debug_wait_timeout", "gwcp_debug_sort", "gwcp_pool_settings",
            "gwcp_clock_bytes", "gwcp_debug_alloc_limit", "gwcp_counters_ex")
 CLOCKS_AUTO, CLOCKS_DENSE, CLOCKS_TILES, CLOCKS_COMPRESSED = 0, 1, 2, 3
 CHECK_AUTO, CHECK_CHUNKED, CHECK_SPARSE = 0, 1, 2
@@ -133,6 +133,8 @@ def load_library():
     L.gwcp_pool_clock_modes.restype = i32
     L.gwcp_debug_wait_timeout.argtypes = [i32, ctypes.c_uint32, ctypes.POINTER(ctypes.c_int)]
     L.gwcp_debug_wait_timeout.restype = i32
+    L.gwcp_debug_sort.argtypes = [i32, vp, vp, u64, u64, ctypes.c_uint32]
+    L.gwcp_debug_sort.restype = i32
     L.gwcp_set_check_mode.argtypes = [vp, ctypes.c_uint32]
     L.gwcp_set_check_mode.restype = i32
     L.gwcp_set_clock_mode.argtypes = [vp, ctypes.c_uint32]
@@ -386,6 +388,18 @@ def debug_wait_timeout(device: int, spin_limit: int) -> int:
     if rc:
         raise GwcpError(rc, "gwcp_debug_wait_timeout")
     return int(st.value)
+
+
+def debug_sort(device: int, keys: np.ndarray, vals: np.ndarray | None, mask: int, poll_limit: int) -> None:
+    """The analysis' stable radix sort of host arrays (uint64 keys, uint32 values or None) by the
+    key bits of `mask`, in place; a tile gives up its wait after `poll_limit` looks."""
+    for a, t in ((keys, np.uint64), (vals, np.uint32)):
+        if a is not None and (a.dtype != t or not a.flags.c_contiguous or len(a) != len(keys)):
+            raise ValueError("keys: contiguous uint64; vals: contiguous uint32 of the same length, or None")
+    rc = load_library().gwcp_debug_sort(device, keys.ctypes.data, vals.ctypes.data if vals is not None else None,
+                                        len(keys), mask, poll_limit)
+    if rc:
+        raise GwcpError(rc, "gwcp_debug_sort")
 
 
 def rank_scores(theta, feat, stream=None):

@@ -31,3 +31,13 @@ def test_tile_walker_clears_the_members_tables_first():
     layout = re.search(r"nbuf = tabs \+ apb \* (\d+);\s*uint32_t\* J = nbuf \+ (\d+);\s*uint32_t\* tcnt = J \+ (\d+)", head)
     clear = re.search(r"i < apb \* (\d+) \+ (\d+) \+ (\d+); i \+= blockDim\.x\)\s*tabs\[i\] = 0;", head)
     assert layout and clear and clear.groups() == layout.groups()
+
+
+def test_a_sort_tile_always_scatters():
+    # a tile that left without scattering would leave words of an earlier use in the output,
+    # which the next passes and phases take for keys and indices: the only early exit is that
+    # of a tile past the end, and the wait that gives up ends in a count of its own
+    body = kernel("k_sweep", source("gwcp_prims.cu"))
+    exits = re.findall(r"if \(([^;{]*)\)\s*return;", body)
+    assert exits == ["size_t(tile) * TILE >= n"]
+    assert re.search(r"if \(s_gone\) count_before<", body)
