@@ -627,8 +627,9 @@ __global__ void __launch_bounds__(MAXT, 1) k_propagate(const __grid_constant__ P
             red_max(at + Wc * 8 + brow<K>(j), J[j]);
           }
         }
-        // (no other member holds a larger value, so a plain store is enough)
-        if (lane < 2) asm volatile("st.shared.u32 [%0], %1;" ::"r"(buf + own), "r"(N) : "memory");
+        // (no other member holds a larger value, but other members' reductions of this word may
+        // be under way, so it is a reduction as well: a plain store could be lost to one)
+        if (lane < 2) red_max(buf + own, N);
         // a member with no other step since the last barrier is early: it works ahead
         if (!busy) ahead(p);
         changed = busy = false;

@@ -41,3 +41,10 @@ def test_a_sort_tile_always_scatters():
     exits = re.findall(r"if \(([^;{]*)\)\s*return;", body)
     assert exits == ["size_t(tile) * TILE >= n"]
     assert re.search(r"if \(s_gone\) count_before<", body)
+
+
+def test_barrier_rows_change_by_reductions_only():
+    # several members add to one word of a barrier buffer between two barriers: a plain store
+    # among their reductions is a race
+    body = kernel("k_propagate", source("gwcp_propagate.cu"))
+    assert "st.shared" not in body and "red_max(buf + own, N)" in body
