@@ -513,7 +513,7 @@ __global__ void __launch_bounds__(128) k_adam(float* theta, float* m, float* v, 
   if (p > N_PARAMS) return;
   double sum = 0;
 #pragma unroll 16
-  for (uint32_t c = 0; c < parts; ++c) sum += double(__ldg(grad + size_t(c) * GR_WORDS + p));
+  for (uint32_t c = 0; c < parts; ++c) sum += double(grad[size_t(c) * GR_WORDS + p]);
   if (p == N_PARAMS) {
     *loss_acc += sum;
     return;

@@ -48,3 +48,9 @@ def test_barrier_rows_change_by_reductions_only():
     # among their reductions is a race
     body = kernel("k_propagate", source("gwcp_propagate.cu"))
     assert "st.shared" not in body and "red_max(buf + own, N)" in body
+
+
+def test_no_read_only_load_of_what_the_kernel_ahead_writes():
+    # the Adam kernel's blocks are placed while the gradient kernel still writes the sums that
+    # they read: not data for the read-only path, which may load it ahead of the wait
+    assert "__ldg" not in kernel("k_adam", source("gwcp_rank.cu"))
