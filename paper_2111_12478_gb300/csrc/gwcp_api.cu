@@ -660,6 +660,7 @@ int run(gwcp_ctx* c, cudaStream_t s) {
     c->tile_cap_hint = 2 * z.tile_cap;  // the tile pool ran out: the caller runs again
     return kRerun;
   }
+  if (code) return code;  // (the walkers have not run, or not to their end: no pool size to learn from)
   if (z.compress) {
     // the walkers count every chunk they took, also past the end of the pool; the next run
     // sizes the pool from the count (with room for the chunks' varying tails)
@@ -676,7 +677,6 @@ int run(gwcp_ctx* c, cudaStream_t s) {
       if (!std::strcmp(r.name, "g_propagate"))
         r.bytes = 4.0 * double(c->st_host->spare[4]) + double(z.n_cs) * 2 * g.Wp * 4;
   }
-  if (code) return code;
   c->n_races = c->st_host->n_races;
   if (c->n_races > z.race_cap && c->opt.race_capacity == 0) {
     // automatic capacity: the race buffer was too small (a location read by many agents
