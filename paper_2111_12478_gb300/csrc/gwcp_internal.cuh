@@ -55,10 +55,12 @@ struct Event {
 };
 
 // Device-side status and counters (one per context).
+constexpr int kListSteps = 8;
 struct DevStatus {
   int code;                      // GWCP_OK or a GWCP_ERR_*
   int pad;
   unsigned long long bad_index;  // first offending event (atomicMin)
+  uint32_t long_lists[kListSteps];  // partner check: accesses with more than so many partner groups (list_step)
   unsigned long long key_or, key_and;    // over access location keys
   unsigned long long lock_or, lock_and;  // over acquire/release lock ids
   unsigned long long n_races;            // races found (may exceed the buffer)

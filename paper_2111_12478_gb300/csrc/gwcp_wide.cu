@@ -773,7 +773,6 @@ struct WideCheckArgs {
   uint32_t* chunk_races;         // and the races it found
   uint2* big;         // (position, piece | pieces << 16) items of k_wc_big
   uint32_t big_cap;   // items it holds
-  uint32_t big_groups;  // most groups that a lane walks itself
 };
 
 // position j in group gi of the latest member with gs[j] < x (gs ascends within a group:
@@ -958,23 +957,67 @@ __device__ __noinline__ uint32_t check_part(const WideCheckArgs& a, uint32_t p, 
   return check_merge<REP>(a, c, cur, end, s_cnt, s_buf);
 }
 
-// A lane walks its access's groups itself up to a limit (big_groups): below, lanes with
-// similar lists are better off each on its own (the reads of a hot location, whose group
-// count grows with the trace: cut by agent, every one of them would pay the searches that
-// place its parts). In a short trace the longest walk is the check's time, so the limit is
-// low there. The check (ms), by limit:
-//   accesses, agents    48      64      96      192
-//   200k, 256           0.045   0.045   0.061   0.111
-//   1M, 64              0.05    0.11    0.19    0.20
-//   1M, 64, ranked      0.047   0.074   0.172   0.172   (the lanes of the access's own warp)
-//   2M, 128             0.092   0.104   0.123   0.471
-//   3M, 64              0.121   0.195   0.254   0.326
-//   2.3M, 512           0.424   0.141   0.154   0.217
-//   5M, 256             1.145   0.850   0.274   0.344
-//   10M, 64             2.156   0.467   0.528   0.555
-//   5M, 512 threads     0.331   0.316   0.306   0.231
-// (n counts the accesses that the written-location filter keeps, a tenth or two fewer.)
-inline uint32_t big_groups(uint32_t n) { return n <= 1500000 ? 48 : n <= 2200000 ? 64 : 96; }
+// A lane walks its access's groups itself up to a limit; an access with more is put aside. The
+// longest walk left to a lane is a tail of about 1 us per group after everything else, so the
+// limit is low where it can be: but an access that is put aside costs the searches that place
+// its parts, and at the locations that most agents use nearly every access is as long as the
+// longest. So the limit is the lowest step that at most kAsideMost accesses of this trace are
+// above: about one for each warp of k_wc_big that the GPU holds. k_wc_fields (in the ranked order
+// k_wc_lists) counts them, beside the walkers. The check (ms) by limit, with the accesses above it:
+//   events, agents     32              48              64              96             192
+//   1M, 64        0.056  218      0.066  188      0.103  119      0.178    0     0.180    0
+//   2M, 128       0.334  83k      0.096  1717     0.106  424      0.125  377     0.480    0
+//   3M, 256       0.696  179k     0.524  122k     0.533  122k     0.170  603     0.244  507
+//   5M, 64        0.993  294k     0.766  200k     0.290  649      0.379  175     0.414    0
+//   8M, 128       2.286  674k     1.979  554k     1.319  317k     0.414  6629    0.795  188
+//   1M, 4096      0.215  42k      0.082  228      0.088  210      0.123  198     0.158  176
+//   3M, 512 thr.  0.205  57k      0.201  48k      0.201  42k      0.196  24k     0.226  3
+constexpr uint32_t kAsideMost = 8192;
+__host__ __device__ constexpr uint32_t list_step(int j) {
+  constexpr uint32_t step[kListSteps] = {32, 48, 64, 80, 96, 128, 192, 384};
+  return step[j];
+}
+__device__ __forceinline__ uint32_t list_limit(const DevStatus* st) {
+  uint32_t limit = list_step(kListSteps - 1);
+#pragma unroll
+  for (int j = kListSteps - 2; j >= 0; --j)
+    if (st->long_lists[j] <= kAsideMost) limit = list_step(j);  // (the counts fall from step to step)
+  return limit;
+}
+
+// The partner groups of an access of class cb in a run.
+__device__ __forceinline__ uint32_t list_length(const uint32_t* rc_off, uint32_t run, uint32_t cb) {
+  const uint32_t any_mask = conflict_classes(cb, false) | conflict_classes(cb, true);
+  uint32_t groups = 0, at = rc_off[run << 2];
+#pragma unroll
+  for (uint32_t q = 0; q < 4; ++q) {
+    const uint32_t next = rc_off[((run << 2) | q) + 1];
+    groups += (any_mask >> q) & 1u ? next - at : 0u;
+    at = next;
+  }
+  return groups;
+}
+// Counts the block's accesses above each step (every thread of it calls this).
+__device__ __forceinline__ void count_lists(uint32_t groups, DevStatus* st) {
+  __shared__ uint32_t s_over[kListSteps];
+  if (threadIdx.x < kListSteps) s_over[threadIdx.x] = 0;
+  if (!__syncthreads_or(groups > list_step(0))) return;
+#pragma unroll
+  for (int j = 0; j < kListSteps; ++j) {
+    const uint32_t over = __popc(__ballot_sync(0xffffffffu, groups > list_step(j)));
+    if ((threadIdx.x & 31) == 0 && over) atomicAdd(&s_over[j], over);
+  }
+  __syncthreads();
+  if (threadIdx.x < kListSteps && s_over[threadIdx.x]) atomicAdd(&st->long_lists[threadIdx.x], s_over[threadIdx.x]);
+}
+__global__ void __launch_bounds__(kCheckThreads) k_wc_lists(const uint32_t* flag, const uint32_t* run_excl,
+                                                            const uint32_t* s_who, const uint32_t* rc_off, uint32_t n,
+                                                            DevStatus* st) {
+  grid_begin();
+  const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
+  count_lists(p < n ? list_length(rc_off, run_excl[p] + flag[p] - 1, who_class(s_who[p])) : 0u, st);
+}
+
 constexpr uint32_t kPieceGroups = 128;  // groups per item of k_wc_big: four per lane
 
 // appends the warp's staged races (one global atomic) and its test count; returns the races found
@@ -1001,6 +1044,7 @@ __device__ __forceinline__ uint32_t flush_warp(const WideCheckArgs& a, uint32_t 
 template <int REP, bool ASIDE>
 __global__ void __launch_bounds__(kCheckThreads, 8) k_wc_check(const __grid_constant__ WideCheckArgs a) {
   grid_begin();
+  const uint32_t limit = list_limit(a.st);
   if (a.st->code) return;  // (the access records or clocks are incomplete)
   constexpr uint32_t kWarps = kCheckThreads / 32;
   __shared__ uint32_t s_cnt[kWarps];
@@ -1024,7 +1068,7 @@ __global__ void __launch_bounds__(kCheckThreads, 8) k_wc_check(const __grid_cons
     uint32_t groups = 0;
 #pragma unroll
     for (uint32_t q = 0; q < 4; ++q) groups += end[q] - cur[q];
-    big = groups > a.big_groups;
+    big = groups > limit;
     if constexpr (ASIDE) {
       if (big) {
         const uint32_t pieces = (groups + kPieceGroups - 1) / kPieceGroups;
@@ -1131,16 +1175,23 @@ __global__ void k_gr_groups(const uint64_t* ck, const uint32_t* run_flag, const 
   for (int64_t t = prev + 1; t <= int64_t(slot); ++t) rc_off[t] = gi;
 }
 
-// the fields of each access record the check needs, copied into the primary order
-__global__ void k_wc_fields(const uint32_t* idx, const AccInfo* info, const uint32_t* n_dev, uint32_t* s_who,
-                            uint32_t* s_row, uint32_t* s_ep) {
+// the fields of each access record the check needs, copied into the primary order; and the
+// counts of long lists
+__global__ void __launch_bounds__(kCheckThreads) k_wc_fields(const uint32_t* idx, const AccInfo* info, const uint32_t* n_dev,
+                                                             uint32_t* s_who, uint32_t* s_row, uint32_t* s_ep,
+                                                             const uint32_t* flag, const uint32_t* run_excl,
+                                                             const uint32_t* rc_off, DevStatus* st) {
   grid_begin();
   const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= *n_dev) return;
-  const AccInfo in = info[idx[p]];
-  s_who[p] = in.who;
-  s_row[p] = in.row;
-  s_ep[p] = in.epoch;
+  uint32_t groups = 0;
+  if (p < *n_dev) {
+    const AccInfo in = info[idx[p]];
+    s_who[p] = in.who;
+    s_row[p] = in.row;
+    s_ep[p] = in.epoch;
+    groups = list_length(rc_off, run_excl[p] + flag[p] - 1, who_class(in.who));
+  }
+  count_lists(groups, st);
 }
 
 __global__ void k_wc_grp_end(const uint32_t* n_groups, const uint32_t* n_dev, uint32_t* grp_lo) {
@@ -1253,6 +1304,8 @@ void phaseI_wide_group(Bufs& b, const Geo& g, Sizes& z, uint32_t* tmp, cudaStrea
   launch(k_wc_grp_end, 1, 1, 0, s)(b.wc_gexcl + n, n_kept, b.wc_grp_lo);  // grp_lo[n_groups] = kept count
   count_launch();
   scan_exclusive(b.wc_rc, b.wc_rc, size_t(n) * 4 + 1, nullptr, tmp, s);
+  launch(k_wc_lists, nblk(n, kCheckThreads), kCheckThreads, 0, s)(b.wc_flag, b.wc_run, b.wc_who, b.wc_rc, n, b.st);
+  count_launch();
   p.end();
 }
 
@@ -1274,7 +1327,8 @@ void phaseI_grouped(Bufs& b, const Geo& g, Sizes& z, uint32_t* tmp, cudaStream_t
   launch(k_gr_groups, nblk(n, 256), 256, 0, s)(b.acc_key, b.wc_flag, b.wc_run, b.wc_gflag, b.wc_gexcl, b.n_kept,
                                           b.wc_grp_lo, b.wc_grp_agent, b.wc_rc);
   count_launch();
-  launch(k_wc_fields, nblk(n, 256), 256, 0, s)(b.acc_idx, b.acc_info, b.n_kept, b.wc_who, b.wc_row, b.wc_ep);
+  launch(k_wc_fields, nblk(n, kCheckThreads), kCheckThreads, 0, s)(b.acc_idx, b.acc_info, b.n_kept, b.wc_who, b.wc_row,
+                                                              b.wc_ep, b.wc_flag, b.wc_run, b.wc_rc, b.st);
   count_launch();
   p.end();
 }
@@ -1313,7 +1367,6 @@ void phaseI_wide_check(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t
   a.row_words = z.compress ? g.B : g.RW;
   a.chunk_ns = b.chunk_ns;
   a.chunk_races = b.chunk_races;
-  a.big_groups = big_groups(n);
   a.big = reinterpret_cast<uint2*>(b.wc_big);
   a.big_cap = z.grouped ? z.big_cap : 0;
   p.begin("i_check", double(n) * (4 + 16 + 4 + 4 + 4 + 8));
@@ -1326,7 +1379,7 @@ void phaseI_wide_check(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t
             : rep == REP_DENSE ? k_wc_check<REP_DENSE, false> : k_wc_check<REP_COMPRESSED, false>;
   launch(check, nblk(n, kCheckThreads), kCheckThreads, 0, s)(a);
   count_launch();
-  if (z.grouped && 4 * g.W > a.big_groups) {  // fewer agents have no such access
+  if (z.grouped && 4 * g.W > list_step(0)) {  // fewer agents have no such access
     auto big = rep == REP_TILES ? k_wc_big<REP_TILES>
                : rep == REP_DENSE ? k_wc_big<REP_DENSE> : k_wc_big<REP_COMPRESSED>;
     launch(big, std::min<uint32_t>(nblk(n, 32), 152 * 6), kCheckThreads, 0, s)(a);
