@@ -147,6 +147,7 @@ void use_stream(gwcp_ctx* c, cudaStream_t s) {
 
 cudaError_t wait_stream(gwcp_ctx* c, cudaStream_t s);
 
+constexpr uint64_t kWaitForVerdict = uint64_t(1) << 23;  // events from which run() waits for the lock walk
 constexpr size_t kStageChunk = size_t(8) << 20;  // bytes per staging half
 
 // Device -> host copy of `bytes` into caller memory. Page-locked (or registered) memory
@@ -443,7 +444,10 @@ int run(gwcp_ctx* c, cudaStream_t s) {
   z.pool_cap = z.n_cs * slots + z.n_exp * 2 * slots + 64;
   b.dep_pool = get<uint32_t>(c, "dep_pool", z.pool_cap, &oom);
   // automatic capacity: at least what the race buffers of an earlier pass hold (a trace with
-  // more races than events would run its check twice on every pass)
+  // more races than events would run its check twice on every pass). The least capacity is
+  // 2^15 under 2^20: that pays for the buffers that the finer phase A and JN_t take in short
+  // traces (10k events: 20.4 MB, with 2^20 races 21.0, without those buffers 20.8), so a
+  // context fits where it fitted.
   z.race_cap = c->opt.race_capacity ? c->opt.race_capacity
                                     : std::max<uint64_t>({(1u << 20) - (1u << 15), z.N,
                                                           std::min(c->allocs["races"].second,
@@ -458,7 +462,11 @@ int run(gwcp_ctx* c, cudaStream_t s) {
   // The last validation (W3) and the acquires' dependency lists are done: no later phase runs
   // on an invalid trace or after an error (their inputs would be incomplete). In the grouped
   // order the kernels that follow see to that themselves and the host goes on without waiting
-  // (10 to 15 us); where the rest does not fit, the trace's own error comes first.
+  // (10 to 15 us); where the rest does not fit, the trace's own error comes first. A long trace
+  // is waited for: there the wait is a thousandth of the pass, and an invalid trace would be
+  // sorted and grouped to the end before it is refused (16M events, 8192 agents: 2.2 ms, as
+  // long as such a trace has ever taken; shorter ones are refused sooner than with the wait
+  // before the overlap: 10k events 0.44 -> 0.19 ms, 2M over 512 agents 1.10 -> 0.58).
   auto invalid = [&]() -> int {
     const int rc = read_status(c, s, nullptr, 0);
     if (rc) return rc;
@@ -469,7 +477,7 @@ int run(gwcp_ctx* c, cudaStream_t s) {
     const int rc = invalid();
     return rc ? rc : GWCP_ERR_OOM;
   };
-  if (code || !z.grouped)
+  if (code || !z.grouped || z.N >= kWaitForVerdict)
     if (int rc = invalid()) return rc;
 
   // ---- remaining buffers ------------------------------------------------------------

@@ -53,3 +53,26 @@ def test_trace_after_an_invalid_one(gw, mode):
         got, again = launches(gw, c, ev, geo)
         assert got <= want  # (one pass over the trace, as in a new context)
         assert np.array_equal(again, races)
+
+
+def test_long_invalid_trace_ends_at_the_lock_walk(gw):
+    def failing(n):
+        ev = np.zeros(n + 4, dtype=TG.EVENT_DTYPE)
+        rng = np.random.default_rng(n)
+        ev["agent"], ev["addr"] = rng.integers(0, 64, n + 4), 4 * rng.integers(0, 1000, n + 4)
+        ev["op"] = rng.choice([TG.READ, TG.WRITE], n + 4)
+        bad, geo = overlapping_sections(64, 8)
+        ev[n:] = bad
+        return ev, geo
+
+    taken = {}
+    for n in (100_000, 1 << 23):
+        ev, geo = failing(n)
+        with gw.Context(0) as c:
+            before = gw.launch_count()
+            c.load_trace(ev, *geo)
+            with pytest.raises(gw.GwcpError) as e:
+                c.compute_order()
+            taken[n] = gw.launch_count() - before
+        assert e.value.code == gw.ERR_INVALID_TRACE and e.value.bad_index == n + 1
+    assert taken[1 << 23] < taken[100_000]  # no sort, grouping or check behind the lock walk
