@@ -176,8 +176,9 @@ int gwcp_debug_clock(gwcp_ctx* ctx, uint64_t event_idx, int which, uint32_t* out
  *   the warp's 32 values. Release snapshots stay dense. num_agents <= 1024; the check is
  *   the sparse one. gwcp_clock_bytes reports the saving;
  * GWCP_CLOCKS_AUTO (default): where the trace allows tiles, tiles above 512 agents and, in
- *   blocks of more than 16, above 256 (where they are the faster on GB300), else dense. At 512
- *   agents, a dense analysis that runs out of device memory is run again with tiles.
+ *   blocks of more than 16, above 256 (where they are the faster on GB300), else dense. An
+ *   analysis that runs out of device memory is run again dense at 257 to 511 agents, and with
+ *   tiles at 512. With GWCP_CHECK_CHUNKED: dense below 512 agents, tiles from there.
  * Applies from the next gwcp_load_trace, which returns GWCP_ERR_UNSUPPORTED when the trace
  * does not allow the requested representation. */
 enum { GWCP_CLOCKS_AUTO = 0, GWCP_CLOCKS_DENSE = 1, GWCP_CLOCKS_TILES = 2, GWCP_CLOCKS_COMPRESSED = 3 };

@@ -69,7 +69,8 @@ struct gwcp_ctx {
   bool acc_info_partial = false;         // last compute wrote the kept accesses' records only
   uint64_t clock_words[3] = {};  // last compute: tiles, pool words taken, words written
   uint64_t tile_cap_hint = 0;  // wide clocks: pool size that the last run needed
-  bool tiles_if_oom = false;   // dense by choice, tiles when the device memory runs out
+  bool choose = false;      // automatic clocks, dense or tiles
+  bool fell_back = false;   // the choice for this trace ran out of device memory
   bool compressed = false;     // GWCP_CLOCKS_COMPRESSED was in force at gwcp_load_trace
   uint64_t cv_cap_hint = 0;    // compressed versions: pool words that the last run needed
   uint64_t alloc_limit = 0;    // gwcp_debug_alloc_limit: cap on the cached buffers' bytes (0 = none)
@@ -837,11 +838,9 @@ int gwcp_load_trace(gwcp_ctx* c, const gwcp_event* ev, uint64_t n, const gwcp_ge
   if (geo->num_agents > kMaxAgents && !tiles_ok) return GWCP_ERR_UNSUPPORTED;
   if (c->clock_mode == GWCP_CLOCKS_TILES && !tiles_ok) return GWCP_ERR_UNSUPPORTED;
   if (c->clock_mode == GWCP_CLOCKS_COMPRESSED && geo->num_agents > kMaxAgents) return GWCP_ERR_UNSUPPORTED;
-  const bool choose = c->clock_mode == GWCP_CLOCKS_AUTO && tiles_ok;
-  const bool tiles = geo->num_agents > kMaxAgents || c->clock_mode == GWCP_CLOCKS_TILES ||
-                     (choose && tiles_preferred(geo->num_agents, geo->agents_per_block));
-  // tiles hold less: the widest clocks that are dense by choice have them to fall back on
-  c->tiles_if_oom = choose && !tiles && geo->num_agents >= 512;
+  c->choose = c->clock_mode == GWCP_CLOCKS_AUTO && tiles_ok && geo->num_agents <= kMaxAgents;
+  c->fell_back = false;
+  const bool tiles = geo->num_agents > kMaxAgents || c->clock_mode == GWCP_CLOCKS_TILES;  // (or by choice: choose_tiles)
   cudaSetDevice(c->device);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   use_stream(c, s);
@@ -873,10 +872,21 @@ int gwcp_load_trace(gwcp_ctx* c, const gwcp_event* ev, uint64_t n, const gwcp_ge
   return GWCP_OK;
 }
 
+namespace {
+// Automatic clocks: the faster representation. The chunked check, which needs dense clocks, keeps
+// them below 512 agents; from there it would take twice a tile analysis, whose check is
+// the sparse one (2M events, 512 agents in blocks of 8: a pass 4.10 ms, with tiles 1.98).
+bool choose_tiles(const gwcp_ctx* c) {
+  return c->check_mode == GWCP_CHECK_CHUNKED ? c->g.W >= 512 : tiles_preferred(c->g.W, c->g.apb);
+}
+void set_tiles(gwcp_ctx* c, bool tiles) { c->g = make_geo(gwcp_geometry{c->g.W, c->g.apb, c->g.gran, 0}, tiles); }
+}  // namespace
+
 int gwcp_compute_order(gwcp_ctx* c, void* stream) {
   if (!c) return GWCP_ERR_ARGS;
   if (!c->has_trace) return GWCP_ERR_STATE;
   cudaSetDevice(c->device);
+  if (c->choose && !c->fell_back) set_tiles(c, choose_tiles(c));
   c->bad_index = ~0ull;
   c->n_races = 0;
   if (c->n == 0) {
@@ -890,13 +900,15 @@ int gwcp_compute_order(gwcp_ctx* c, void* stream) {
   int rc = run(c, static_cast<cudaStream_t>(stream));
   for (int attempt = 0; rc == kRerun && attempt < 6; ++attempt) rc = run(c, static_cast<cudaStream_t>(stream));
   if (rc == kRerun) rc = GWCP_ERR_OOM;
-  if (rc == GWCP_ERR_OOM && c->tiles_if_oom) {
-    c->tiles_if_oom = false;
+  // where the faster representation may hold more, the other one is there to fall back on: tiles
+  // at 512 agents, dense clocks below (a tile pool has 65,536 tiles at least)
+  if (rc == GWCP_ERR_OOM && c->choose && !c->fell_back && (c->g.nT ? c->g.W < 512 : c->g.W >= 512)) {
+    c->fell_back = true;
     cudaStreamSynchronize(static_cast<cudaStream_t>(stream));
-    for (auto& kv : c->allocs)  // what the dense attempt holds
+    for (auto& kv : c->allocs)  // what the attempt holds
       if (kv.second.first) cudaFreeAsync(kv.second.first, c->alloc_s);
     c->allocs.clear();
-    c->g = make_geo(gwcp_geometry{c->g.W, c->g.apb, c->g.gran, 0}, true);
+    set_tiles(c, c->g.nT == 0);
     return gwcp_compute_order(c, stream);
   }
   c->computed = true;
