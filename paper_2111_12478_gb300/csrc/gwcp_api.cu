@@ -465,9 +465,8 @@ int run(gwcp_ctx* c, cudaStream_t s) {
   // order the kernels that follow see to that themselves and the host goes on without waiting
   // (10 to 15 us); where the rest does not fit, the trace's own error comes first. A long trace
   // is waited for: there the wait is a thousandth of the pass, and an invalid trace would be
-  // sorted and grouped to the end before it is refused (16M events, 8192 agents: 2.2 ms, as
-  // long as such a trace has ever taken; shorter ones are refused sooner than with the wait
-  // before the overlap: 10k events 0.44 -> 0.19 ms, 2M over 512 agents 1.10 -> 0.58).
+  // sorted and grouped to the end before it is refused (16M events, 8192 agents: 2.23 ms without
+  // the wait, 1.75 with it; 2M, 512: 0.58 without; 10k, 64: 0.19 without).
   auto invalid = [&]() -> int {
     const int rc = read_status(c, s, nullptr, 0);
     if (rc) return rc;
