@@ -28,6 +28,7 @@ inline bool tiles_preferred(uint32_t agents, uint32_t per_block) {
 }
 constexpr uint32_t kSparseCheckFromAgents = 1;  // automatic check mode: partner groups (measured faster)
 constexpr uint32_t kMaxEvents = (1u << 30) - 1;
+constexpr uint32_t kSms = 152;  // SMs of a GB300: the grids of kernels that stride over their input
 constexpr size_t kMaxDynamicSmem = 200 * 1024;  // shared memory a walker's CTA may ask for
 // distinct scope ids one lock may be used with: 64, or 320 when the trace has more than
 // 63 blocks (a block-scoped lock may be used in every block)

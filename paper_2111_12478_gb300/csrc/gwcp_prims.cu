@@ -556,7 +556,7 @@ void fill_all(const FillBatch& b, cudaStream_t s) {
   size_t most = 0;
   for (int j = 0; j < b.n; ++j) most = std::max(most, b.job[j].words);
   if (!b.n) return;
-  launch(k_fill, unsigned(std::min<size_t>((most + 1023) / 1024, 152 * 8)), 256, 0, s)(b);
+  launch(k_fill, unsigned(std::min<size_t>((most + 1023) / 1024, kSms * 8)), 256, 0, s)(b);
   count_launch();
 }
 void read_back_to(const DevStatus* st, const ReadBack& r, DevStatus* st_out, uint32_t* val_out, cudaStream_t s) {
@@ -664,7 +664,7 @@ bool radix_sort_pairs(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, si
   uint32_t* counters = tmp + kMaxPasses * 256;
   auto* status = reinterpret_cast<unsigned long long*>((reinterpret_cast<uintptr_t>(tmp + kSweepHead) + 15) & ~uintptr_t(15));
   cudaMemsetAsync(tmp, 0, kSweepHead * 4, s);
-  const uint32_t hist_blocks = uint32_t(std::min<size_t>((n + 2047) / 2048, 152 * 4));
+  const uint32_t hist_blocks = uint32_t(std::min<size_t>((n + 2047) / 2048, kSms * 4));
   launch(k_sweep_hist, hist_blocks, HI_THREADS, 0, s)(k0, n, n_dev, pl, hist, reinterpret_cast<uint4*>(status),
                                                  size_t(tiles) * 128, keep);
   count_launch();

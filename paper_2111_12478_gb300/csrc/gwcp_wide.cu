@@ -1382,7 +1382,7 @@ void phaseI_wide_check(const Bufs& b, const Geo& g, const Sizes& z, cudaStream_t
   if (z.grouped && 4 * g.W > list_step(0)) {  // fewer agents have no such access
     auto big = rep == REP_TILES ? k_wc_big<REP_TILES>
                : rep == REP_DENSE ? k_wc_big<REP_DENSE> : k_wc_big<REP_COMPRESSED>;
-    launch(big, std::min<uint32_t>(nblk(n, 32), 152 * 6), kCheckThreads, 0, s)(a);
+    launch(big, std::min<uint32_t>(nblk(n, 32), kSms * 6), kCheckThreads, 0, s)(a);
     count_launch();
   }
   p.end();
