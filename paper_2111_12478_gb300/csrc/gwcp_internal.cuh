@@ -20,9 +20,11 @@ constexpr uint32_t kTileW = 256;           // entries per clock tile
 constexpr uint32_t kTabW = 32;             // words per published tile table (nT <= 32)
 // Automatic clock mode: tiles above 512 agents, and above 256 where a block has more than 16
 // (its walkers' CTA then leaves 64 registers per thread, and a clock of 16 words per lane
-// spills). Propagation, dense and tiles, ms: 512 agents in blocks of 8 (4M events) 1.29 and
-// 2.21, of 16 2.85 and 3.94, of 32 9.2 and 6.5; 600 in blocks of 8 2.46 and 2.20; 1024 in blocks
-// of 16 (3M) 3.06 and 1.80; 384 in blocks of 24 (2M) 4.5 and 3.2; 256 in blocks of 32 5.45 and 5.54.
+// spills). Propagation, dense and tiles, ms: 512 agents in blocks of 8 (4M events) 1.36 and
+// 2.27, of 16 2.91 and 4.06, of 32 (3M, as those below) 6.9 and 4.9; 600 in blocks of 8 1.77 and
+// 1.59; 768 in blocks of 4 1.08 and 1.02, of 8 1.48 and 1.37, of 16 3.90 and 2.10; 1024 in blocks
+// of 4 0.89 and 0.92, of 8 1.16 and 1.15, of 16 3.08 and 1.76; 384 in blocks of 24 (2M) 4.5 and
+// 3.2; 256 in blocks of 32 5.48 and 5.72.
 inline bool tiles_preferred(uint32_t agents, uint32_t per_block) {
   return agents > 512 || (agents > 256 && per_block > 16);
 }
